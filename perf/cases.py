@@ -19,6 +19,7 @@ from __future__ import annotations
 
 import math
 
+import numpy as np
 import torch
 
 from paper_1910_04732_b200 import binding as b
@@ -280,6 +281,93 @@ def run(state):
             b.compact_ranks(la, 0, HC, idx, k, z, P, Q, Pc, Qc)
         return [s["idx"], s["k"], s["z"], s["Pc"], s["Qc"]]
     return _run_train(s) if kind == "train" else _run_single(s)
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _uniforms(n, seed):
+    """Philox4x32-10, key = seed, counter = gate // 4: 23 bits of word gate % 4, centred in their interval."""
+    j = np.arange(n, dtype=np.uint64)
+    low, s = np.uint64(0xFFFFFFFF), np.uint64(32)
+    c, key = [(j >> np.uint64(2)) & low, j >> np.uint64(34), 0 * j, 0 * j], [np.uint64(seed), np.uint64(0)]
+    for _ in range(10):
+        p0, p1 = np.uint64(0xD2511F53) * c[0], np.uint64(0xCD9E8D57) * c[2]
+        c = [(p1 >> s) ^ c[1] ^ key[0], p1 & low, (p0 >> s) ^ c[3] ^ key[1], p0 & low]
+        key = [(key[0] + np.uint64(0x9E3779B9)) & low, (key[1] + np.uint64(0xBB67AE85)) & low]
+    bits = np.stack(c, axis=1)[np.arange(n), (j & np.uint64(3)).astype(np.int64)]
+    return ((bits >> np.uint64(9)).astype(np.float64) + 0.5) * 2.0 ** -23
+
+
+def _exact_gates(log_alpha, seed=7):
+    """(z, dz/dlog_alpha) of the sampled hard-concrete gates."""
+    u = torch.from_numpy(_uniforms(log_alpha.numel(), seed)).to(log_alpha.device)
+    beta, gamma, zeta = HC
+    s = torch.sigmoid((torch.log(u) - torch.log1p(-u) + log_alpha.double()) / beta)
+    bar = s * (zeta - gamma) + gamma
+    return bar.clamp(0.0, 1.0), torch.where((bar > 0) & (bar < 1), (zeta - gamma) * s * (1 - s) / beta, 0.0)
+
+
+def _exact_layer(X, dY, Q, P, z, dz):
+    """(Y, dX, dP, dQ, dlog_alpha) of one matrix."""
+    X, dY, Q, P = X.double(), dY.double(), Q.double(), P.double()
+    dH = dY @ P
+    M = dH.T @ X
+    return ((X @ Q.T) * z) @ P.T, dH @ (z[:, None] * Q), dY.T @ ((X @ Q.T) * z), z[:, None] * M, (Q * M).sum(1) * dz
+
+
+def _exact_l0(s):
+    """(out4, what the penalty adds to dlog_alpha)."""
+    thr = I.BETA * math.log(-I.GAMMA / I.ZETA)
+    pi = torch.sigmoid(s["log_alpha"].double() - thr)
+    size = torch.repeat_interleave(s["seg_size"].double(), s["seg_off"][1:] - s["seg_off"][:-1])
+    total, t, (l1, l2) = size.sum(), s["target"].double()[0], s["lam"].double()
+    diff = (pi * size).sum() / total - t
+    return torch.stack([diff + t, l1 * diff + l2 * diff * diff, diff, diff * diff]), (l1 + 2 * l2 * diff) * size / total * pi * (1 - pi)
+
+
+def _exact_export(s):
+    z = torch.zeros_like(s["z"], dtype=torch.float64)
+    Pc, Qc = [torch.zeros(t.shape, dtype=torch.float64, device="cuda") for t in s["Pc"]], [torch.zeros(t.shape, dtype=torch.float64, device="cuda") for t in s["Qc"]]
+    L, n = z.shape[:2]
+    for i, call in enumerate(s["calls"]):
+        layer, m, la, P, Q = i // n, i % n, call[0].double(), call[4], call[5]
+        pi = torch.sigmoid(la - I.BETA * math.log(-I.GAMMA / I.ZETA))
+        k = int(torch.floor(pi.sum() + 0.5))
+        idx = torch.sort(torch.sort(-la, stable=True).indices[:k]).values
+        z[layer, m, idx] = pi[idx]
+        Pc[m][layer, :, :k] = P[:, idx].double()
+        Qc[m][layer, :k] = pi[idx, None] * Q[idx].double()
+    return [None, None, z, Pc, Qc]
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits and without any rounding on the way (None for index lists and counts)."""
+    s = prepare(case, seed)
+    kind = s["kind"]
+    if kind == "infer":
+        return (s["X"].double() @ s["Qc"].double().T) @ s["Pc"].double().T
+    if kind == "export":
+        return _exact_export(s)
+    if kind == "embedding":
+        ids, z, dY, O = s["ids"].long(), s["z"].double(), s["dY"].double(), s["O"].double()
+        e, dH = s["E"][ids].double(), dY @ O.T
+        dE = torch.zeros(s["dE"].shape, dtype=torch.float64, device="cuda").index_add_(0, ids, dH * z)
+        return [(e * z) @ O, dE, (e * z).T @ dY, (e * dH).sum(0) * s["dz"].double()]
+    z, dz = _exact_gates(s["log_alpha"])
+    out4, penalty = _exact_l0(s)
+    if kind != "train":
+        parts = [_exact_layer(e["X"], e["dY"], s["Q"], s["P"], z, dz) for e in s["batches"]]
+        dP, dQ, dla = (sum(p[i] for p in parts) for i in (2, 3, 4))
+        return [None, [(p[0], p[1]) for p in parts], dP, dQ, dla + penalty, out4]
+    out = [[torch.empty(t.shape, dtype=torch.float64, device="cuda") for t in s[name]] for name in ("Y", "dX", "dP", "dQ")]
+    n, L, r, per = len(s["Y"]), s["Y"][0].shape[0], s["dP"][0].shape[2], 17 if s["active"] else 7
+    dla = torch.empty_like(z)
+    for i in range(L * n):
+        Q, P, X, dY = s["keep"][per * i:per * i + 4]
+        got = _exact_layer(X, dY, Q, P, z[i * r:i * r + r], dz[i * r:i * r + r])
+        for whole, part in zip(out, got):
+            whole[i % n][i // n] = part
+        dla[i * r:i * r + r] = got[4]
+    return [None, *out, dla + penalty, out4]
 
 
 # ------------------------------------------------------------------------------------------------ what a pass needs
