@@ -796,18 +796,55 @@ int launch_few_tokens(const void* A, int64_t lda, const void* B, int64_t ldb, vo
   return launch_skinny(A, lda, B, ldb, C, ldc, cs, T, N, K, st);
 }
 
-int launch_simt(const float* A, int64_t a_sm, int64_t a_sk, const float* B, int64_t b_sn, int64_t b_sk, float* C,
-                int64_t ldc, int64_t M, int64_t N, int64_t K, const float* col_scale, const float* row_scale,
-                int accumulate, cudaStream_t st) {
-  if (M <= 0 || N <= 0) return FLOP_OK;
-  if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
-  SimtGemmArgs a{A, a_sm, a_sk, B, b_sn, b_sk, C, ldc, (int)M, (int)N, (int)K, col_scale, row_scale, accumulate};
-  const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-  if (grid.y > 65535) return FLOP_ERR_UNSUPPORTED;
-  launch_k(simt_gemm_kernel, dim3(grid), dim3(256), (size_t)(0), st, a);
+// An operand of an fp32 product: a row-major matrix read along its rows (k_fast) or down its columns.
+struct SimtOperand { const float* ptr; int64_t ld; bool k_fast; };
+
+template <bool A_K, bool B_K, bool SCALE_K>
+int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
+  static bool configured[kMaxDevices] = {};
+  auto kern = simt::gemm_kernel<A_K, B_K, SCALE_K>;
+  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kSmemBytes));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3(simt::kThreads); cfg.dynamicSmemBytes = simt::kSmemBytes; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = grid.z;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_on() ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, kern, a);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
+}
+
+// fp32 product with the fields of `a` that the caller sets (outputs, gates, accumulate, row dot).  K is cut over a
+// cluster while the 64 x 64 tiles alone leave SMs idle and every CTA keeps at least two 32-wide k-blocks.
+int launch_simt(const SimtOperand& A, const SimtOperand& B, int64_t M, int64_t N, int64_t K, SimtGemmArgs a, cudaStream_t st) {
+  if (M <= 0 || N <= 0) return FLOP_OK;
+  if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
+  const int64_t tiles_n = (N + simt::BN - 1) / simt::BN, tiles_m = (M + simt::BM - 1) / simt::BM;
+  if (tiles_m > 65535) return FLOP_ERR_UNSUPPORTED;
+  const int num_kb = (int)((K + simt::BK - 1) / simt::BK);
+  int split = 1;
+  while (split < simt::kMaxSplit && tiles_m * tiles_n * split < num_sms() && num_kb >= 4 * split) split *= 2;
+  a.A = A.ptr; a.lda = A.ld; a.B = B.ptr; a.ldb = B.ld;
+  a.M = (int)M; a.N = (int)N; a.K = (int)K;
+  a.kb_per_split = (num_kb + split - 1) / split;
+  a.a_vec = aligned16(A.ptr) && A.ld % 4 == 0;
+  a.b_vec = aligned16(B.ptr) && B.ld % 4 == 0;
+  const dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, (unsigned)split);
+  if (A.k_fast && B.k_fast) return launch_simt_inst<true, true, false>(a, grid, st);
+  if (A.k_fast) return a.k_scale ? launch_simt_inst<true, false, true>(a, grid, st) : launch_simt_inst<true, false, false>(a, grid, st);
+  if (!B.k_fast) return launch_simt_inst<false, false, false>(a, grid, st);
+  return FLOP_ERR_UNSUPPORTED;
+}
+
+SimtGemmArgs simt_out(void* C, int64_t ldc, const float* col_scale = nullptr) {
+  SimtGemmArgs a{};
+  a.C = (float*)C; a.ldc = ldc; a.col_scale = col_scale;
+  return a;
 }
 
 template <typename T>
@@ -848,7 +885,7 @@ BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, 
   w.lddh = round_up(std::max<int64_t>(r, 1), 8);
   w.dH = ar.take((size_t)T * w.lddh * elt(dt));
   w.ldqz = round_up(std::max<int64_t>(d_in, 1), 8);
-  w.Qz = ar.take((size_t)r * w.ldqz * elt(dt));
+  w.Qz = dt == FLOP_BF16 ? ar.take((size_t)r * w.ldqz * 2) : nullptr;
   w.ld_slice_p = round_up(std::max<int64_t>(r, 1), 4);
   w.ld_slice_q = round_up(std::max<int64_t>(d_in, 1), 4);
   int sp = 1, sq = 1;
@@ -863,8 +900,9 @@ BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, 
   w.slice_elems_p = d_out * w.ld_slice_p;
   w.slice_elems_q = r * w.ld_slice_q;
   w.slices_p = dt == FLOP_BF16 ? (float*)ar.take((size_t)sp * w.slice_elems_p * 4) : nullptr;
-  w.slices_q = (float*)ar.take((size_t)sq * w.slice_elems_q * 4);
+  w.slices_q = dt == FLOP_BF16 ? (float*)ar.take((size_t)sq * w.slice_elems_q * 4) : nullptr;
   // room for the partials of any tile shape: the direct-epilogue path may use another N tile than plan_q
+  // (fp32 storage: one fp64 partial per 64-column tile)
   const int64_t part_cap = std::max<int64_t>(w.n_part, 2 * ((d_in + 63) / 64));
   w.dz_part = (float*)ar.take((size_t)part_cap * std::max<int64_t>(r, 1) * 4);
   w.dz_meta = (int*)ar.take(256);
@@ -915,18 +953,6 @@ int builtin_scratch(L0Scratch** out) {
 }
 
 }  // namespace
-
-template <typename TW, typename TQ>
-static int finalize_wgrad(const float* slices, int n_slices, int64_t slice_elems, int64_t ld_slice, int64_t M, int64_t N,
-                          const float* row_scale, void* out, int64_t ldo, int accumulate, const void* qdot, int64_t ldq,
-                          float* dz_out, cudaStream_t st) {
-  if (M <= 0) return FLOP_OK;
-  launch_k(wgrad_finalize_kernel<TW, TQ>, dim3((unsigned)M), dim3(256), (size_t)(0), st, slices, n_slices, slice_elems, ld_slice, (int)M, (int)N, row_scale,
-                                                            (TW*)out, ldo, accumulate, (const TQ*)qdot, ldq, dz_out);
-  count_launch();
-  FLOP_CUDA(cudaGetLastError());
-  return FLOP_OK;
-}
 
 // ====================================================================== C ABI
 extern "C" {
@@ -1188,8 +1214,8 @@ static int fwd_impl(const void* X, int64_t ldx, const void* Q, int64_t ldq, cons
     const TcPlan p2 = plan_tc(T, d_out, r, false, false);
     FLOP_TRY(launch_tc({H, ldh, false}, {P, ldp, false}, T, d_out, r, p2, store_epilogue(Y, ldy, nullptr), st));
   } else {
-    FLOP_TRY(launch_simt((const float*)X, ldx, 1, (const float*)Q, ldq, 1, (float*)H, ldh, T, r, d_in, z, nullptr, 0, st));
-    FLOP_TRY(launch_simt((const float*)H, ldh, 1, (const float*)P, ldp, 1, (float*)Y, ldy, T, d_out, r, nullptr, nullptr, 0, st));
+    FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Q, ldq, true}, T, r, d_in, simt_out(H, ldh, z), st));
+    FLOP_TRY(launch_simt({(const float*)H, ldh, true}, {(const float*)P, ldp, true}, T, d_out, r, simt_out(Y, ldy), st));
   }
   return FLOP_OK;
 }
@@ -1265,8 +1291,8 @@ int flop_compact_fwd(const void* X, int64_t ldx, const void* Qc, int64_t ldqc, c
     const TcPlan p2 = plan_tc(T, d_out, k, false, false);
     FLOP_TRY(launch_tc({w.H, w.ldh, false}, {Pc, ldpc, false}, T, d_out, k, p2, store_epilogue(Y, ldy, nullptr), st));
   } else {
-    FLOP_TRY(launch_simt((const float*)X, ldx, 1, (const float*)Qc, ldqc, 1, (float*)w.H, w.ldh, T, k, d_in, nullptr, nullptr, 0, st));
-    FLOP_TRY(launch_simt((const float*)w.H, w.ldh, 1, (const float*)Pc, ldpc, 1, (float*)Y, ldy, T, d_out, k, nullptr, nullptr, 0, st));
+    FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Qc, ldqc, true}, T, k, d_in, simt_out(w.H, w.ldh), st));
+    FLOP_TRY(launch_simt({(const float*)w.H, w.ldh, true}, {(const float*)Pc, ldpc, true}, T, d_out, k, simt_out(Y, ldy), st));
   }
   return FLOP_OK;
 }
@@ -1361,26 +1387,31 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     const float* Pf = (const float*)P; const float* Hf = (const float*)H_save;
     float* dHf = (float*)w.dH;
     // dH'[t,k] = sum_i dY[t,i] P[i,k]
-    FLOP_TRY(launch_simt(dYf, lddy, 1, Pf, 1, ldp, dHf, w.lddh, T, r, d_out, nullptr, nullptr, 0, st));
+    FLOP_TRY(launch_simt({dYf, lddy, true}, {Pf, ldp, false}, T, r, d_out, simt_out(dHf, w.lddh), st));
     // dP[i,k] = sum_t dY[t,i] H'[t,k]
-    if (dP) FLOP_TRY(launch_simt(dYf, 1, lddy, Hf, 1, ldh, (float*)dP, lddp, d_out, r, T, nullptr, nullptr, accumulate, st));
+    if (dP) {
+      SimtGemmArgs a = simt_out(dP, lddp);
+      a.accumulate = accumulate;
+      FLOP_TRY(launch_simt({dYf, lddy, false}, {Hf, ldh, false}, d_out, r, T, a, st));
+    }
     if (need_m) {
-      // M[k,j] = sum_t dH'[t,k] X[t,j] into the slice buffer, then the same finalisation as the tensor-core path
-      FLOP_TRY(launch_simt(dHf, 1, w.lddh, Xf, 1, ldx, w.slices_q, w.ld_slice_q, r, d_in, T, nullptr, nullptr, 0, st));
-      FLOP_TRY((finalize_wgrad<float, float>(w.slices_q, 1, w.slice_elems_q, w.ld_slice_q, r, d_in, z, dQ, lddq, accumulate,
-                                             dlog_alpha ? Q : nullptr, ldq, w.dz_part, st)));
+      // M[k,j] = sum_t dH'[t,k] X[t,j]; dQ = diag(z) M and the row dots <Q[k,:], M[k,:]> leave with the tile
+      SimtGemmArgs a = simt_out(dQ, lddq);
+      a.row_scale = z; a.accumulate = accumulate;
+      if (dlog_alpha) { a.qdot = Qf; a.ldq = ldq; a.dz_part = (double*)w.dz_part; a.dz_stride = r; }
+      FLOP_TRY(launch_simt({dHf, w.lddh, false}, {Xf, ldx, false}, r, d_in, T, a, st));
       if (dlog_alpha) {
-        launch_k(dalpha_kernel, dim3((unsigned)((r + 255) / 256)), dim3(256), (size_t)(0), st, w.dz_part, 1, r, dz_dla, (int)r, dlog_alpha, accumulate);
+        const int n_part = (int)((d_in + simt::BN - 1) / simt::BN);
+        launch_k(dalpha_f64_kernel, dim3((unsigned)((r + 255) / 256)), dim3(256), (size_t)(0), st, (const double*)w.dz_part, n_part, r, dz_dla, (int)r, dlog_alpha, accumulate);
         count_launch();
         FLOP_CUDA(cudaGetLastError());
       }
     }
     if (dX) {
-      launch_k(scale_rows_kernel<float>, dim3((unsigned)r), dim3(256), (size_t)(0), st, Qf, ldq, z, (int)r, (int)d_in, (float*)w.Qz, w.ldqz);
-      count_launch();
-      FLOP_CUDA(cudaGetLastError());
-      // dX[t,j] = sum_k dH'[t,k] Qz[k,j]
-      FLOP_TRY(launch_simt(dHf, w.lddh, 1, (const float*)w.Qz, 1, w.ldqz, (float*)dX, lddx, T, d_in, r, nullptr, nullptr, 0, st));
+      // dX[t,j] = sum_k dH'[t,k] z[k] Q[k,j], the gate applied to the rows of Q as they are read
+      SimtGemmArgs a = simt_out(dX, lddx);
+      a.k_scale = z;
+      FLOP_TRY(launch_simt({dHf, w.lddh, true}, {Qf, ldq, false}, T, d_in, r, a, st));
     }
   }
   return FLOP_OK;

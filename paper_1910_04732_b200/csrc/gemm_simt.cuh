@@ -1,78 +1,238 @@
 // fp32 FMA GEMM for the FLOP_F32 storage type: C[M,N] = sum_k A(m,k) B(n,k).
 //
-// The tensor cores have no true fp32 mode, and the fp32 configuration is held
-// to 1e-5 relative error, so this path multiplies and accumulates in fp32 on
-// the CUDA cores.  Operands are addressed by strides, which covers all six
-// GEMMs of the layer (forward, and the backward ones that contract over
-// tokens or over d_out) without transposes.  64x64x16 tiles, 4x4 per thread.
+// The tensor cores have no true fp32 mode, and the fp32 configuration is held to 1e-5 relative error, so this
+// path multiplies and accumulates in fp32 on the CUDA cores.  Every operand is a row-major matrix read either
+// along its rows (K-fast: k is the unit stride) or down its columns (MN-fast: m or n is), which covers all six
+// GEMMs of the layer without transposes; the two forms are template parameters, because they decide the
+// shared-memory layout.
+//
+// Bound: at the sizes of this configuration (outputs of 64..2048 x 128..768) by latency, not by the FMA units: the
+// 32 tiles of a 512 x 256 product leave 116 SMs idle, and a block that loads, waits and multiplies in turn spends
+// nine tenths of its time waiting.  Hence
+//   * cp.async into three shared-memory stages (64 x 32 floats of each operand), so that the loads of two k-blocks are
+//     in flight while a third is multiplied; 16-byte pieces where base and leading dimension allow them, else 4-byte;
+//   * a cluster of up to eight CTAs shares one 64 x 64 tile: each takes a slice of K, and every CTA adds up its rows of
+//     the tile from all slices through distributed shared memory, in rank order (the same bits on every run).
+// One 512 x 256 x 256 product took 26.6 us in the single-buffered unsplit form (64 x 64 x 16); forward and backward of that
+// matrix with its small launches went from 181.6 to 69.8 us.  4 x 4 results per thread: 64 FMAs per eight 16-byte
+// shared-memory reads, of which half are broadcasts.
+// The epilogue applies the gate of the column (H'), of the row (dQ) and the fused row dot <Q[m,:], C[m,:]> (dz), whose
+// partial sums stay in fp64; `k_scale` multiplies B(n,k) by z[k] as it is read, so that diag(z) Q is never written.
 #pragma once
 #include "common.cuh"
 
 namespace flop {
 
 struct SimtGemmArgs {
-  const float* A; int64_t a_sm, a_sk;   // A(m,k) = A[m*a_sm + k*a_sk]
-  const float* B; int64_t b_sn, b_sk;   // B(n,k) = B[n*b_sn + k*b_sk]
-  float* C; int64_t ldc;                // C[m*ldc + n]
+  const float* A; int64_t lda;          // A(m,k) = A[m*lda + k] (K-fast) or A[k*lda + m] (MN-fast)
+  const float* B; int64_t ldb;          // B(n,k) likewise
+  float* C; int64_t ldc;                // nullable when only the row dot is wanted; C[m*ldc + n]
   int M, N, K;
+  int kb_per_split;                     // 32-wide k-blocks per CTA of the cluster
+  int a_vec, b_vec;                     // operand rows are 16-byte aligned
   const float* col_scale;               // nullable: C[m,n] *= col_scale[n]
   const float* row_scale;               // nullable: C[m,n] *= row_scale[m]
+  const float* k_scale;                 // nullable: B(n,k) is multiplied by k_scale[k]
   int accumulate;                       // C += instead of C =
+  const float* qdot; int64_t ldq;       // nullable: dz_part[tile of n][m] = sum_n qdot[m,n] * C[m,n] before scaling
+  double* dz_part; int64_t dz_stride;
 };
 
-__global__ void __launch_bounds__(256)
-simt_gemm_kernel(SimtGemmArgs p) {
+namespace simt {
+
+constexpr int BM = 64, BN = 64, BK = 32, kThreads = 256, kStages = 3;
+constexpr int kRowK = BK + 4;                            // K-fast rows in shared memory: 144 bytes, conflict-free 16-byte reads
+constexpr int kOperandFloats = BM * kRowK;               // >= BK * BM, the MN-fast layout [k][64]
+constexpr int kStageFloats = 2 * kOperandFloats + BK;    // A, B, k_scale
+constexpr int kRowP = BN + 4;                            // rows of the partial tile
+constexpr int kSmemBytes = kStages * kStageFloats * 4;
+constexpr int kMaxSplit = 8;                             // portable cluster size
+static_assert(BM == BN && BM * kRowP <= kStages * kStageFloats, "partial tile reuses the stages");
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// bytes (0..16, or 0..4) are read, the rest of the piece is zero-filled; with bytes = 0 the source is not read
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy4(uint32_t dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// One operand's 64 x 32 block (rows from `row0` of `rows`, k from k0 below k_end) into shared memory.
+template <bool KFAST>
+__device__ __forceinline__ void load_block(const float* __restrict__ p, int64_t ld, int row0, int rows, int k0, int k_end, int vec,
+                                           uint32_t dst, int tid) {
+  if (vec) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = tid + i * kThreads;                   // 512 pieces of 16 bytes
+      if (KFAST) {
+        const int r = e >> 3, k = (e & 7) * 4;
+        const int left = row0 + r < rows ? min(4, k_end - (k0 + k)) : 0;
+        copy16(dst + (uint32_t)(r * kRowK + k) * 4u, left > 0 ? p + (int64_t)(row0 + r) * ld + k0 + k : p, max(left, 0) * 4);
+      } else {
+        const int k = e >> 4, r = (e & 15) * 4;
+        const int left = k0 + k < k_end ? min(4, rows - (row0 + r)) : 0;
+        copy16(dst + (uint32_t)(k * BM + r) * 4u, left > 0 ? p + (int64_t)(k0 + k) * ld + row0 + r : p, max(left, 0) * 4);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = tid + i * kThreads;                   // 2048 floats
+      const int r = KFAST ? e >> 5 : e & 63, k = KFAST ? e & 31 : e >> 6;
+      const bool in = row0 + r < rows && k0 + k < k_end;
+      const float* src = KFAST ? p + (int64_t)(row0 + r) * ld + k0 + k : p + (int64_t)(k0 + k) * ld + row0 + r;
+      copy4(dst + (uint32_t)(KFAST ? r * kRowK + k : k * BM + r) * 4u, in ? src : p, in ? 4 : 0);
+    }
+  }
+}
+
+template <bool A_K, bool B_K, bool SCALE_K>
+__global__ void __launch_bounds__(kThreads, 2)
+gemm_kernel(const SimtGemmArgs p) {
   pdl_wait();
   pdl_launch_dependents();
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
-  const int tid = threadIdx.x;
+  extern __shared__ __align__(16) float smem[];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int tm = (tid >> 4) * 4, tn = (tid & 15) * 4;
+  const int split = blockIdx.z, n_split = gridDim.z;      // the cluster spans z: split is the rank in it
+  const int kb0 = split * p.kb_per_split, kb1 = min((p.K + BK - 1) / BK, kb0 + p.kb_per_split);
+
+  auto load = [&](int kb) {
+    if (kb < kb1) {
+      const uint32_t st = smem_addr(smem + (kb % kStages) * kStageFloats);
+      load_block<A_K>(p.A, p.lda, m0, p.M, kb * BK, p.K, p.a_vec, st, tid);
+      load_block<B_K>(p.B, p.ldb, n0, p.N, kb * BK, p.K, p.b_vec, st + kOperandFloats * 4, tid);
+      if (SCALE_K && tid < BK) {
+        const bool in = kb * BK + tid < p.K;
+        copy4(st + (2 * kOperandFloats + tid) * 4, in ? p.k_scale + kb * BK + tid : p.k_scale, in ? 4 : 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");   // an empty group keeps the count of groups in step
+  };
+
   float acc[4][4] = {};
-  const bool a_kfast = p.a_sk == 1, b_kfast = p.b_sk == 1;
-  for (int k0 = 0; k0 < p.K; k0 += BK) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = tid + i * 256;   // 0..1023
-      int m, k;
-      if (a_kfast) { m = e >> 4; k = e & 15; } else { k = e >> 6; m = e & 63; }
-      const int gm = m0 + m, gk = k0 + k;
-      As[k][m] = (gm < p.M && gk < p.K) ? p.A[(int64_t)gm * p.a_sm + (int64_t)gk * p.a_sk] : 0.f;
-      int n, kb;
-      if (b_kfast) { n = e >> 4; kb = e & 15; } else { kb = e >> 6; n = e & 63; }
-      const int gn = n0 + n, gkb = k0 + kb;
-      Bs[kb][n] = (gn < p.N && gkb < p.K) ? p.B[(int64_t)gn * p.b_sn + (int64_t)gkb * p.b_sk] : 0.f;
+  for (int s = 0; s < kStages - 1; ++s) load(kb0 + s);
+  for (int kb = kb0; kb < kb1; ++kb) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    __syncthreads();                                       // block kb has landed; block kb - 1 has been read by everyone
+    load(kb + kStages - 1);
+    const float* As = smem + (kb % kStages) * kStageFloats;
+    const float* Bs = As + kOperandFloats;
+    const float* Zs = Bs + kOperandFloats;
+#pragma unroll
+    for (int k = 0; k < BK; k += 4) {
+      float a[4][4], b[4][4];                              // [row or column of the thread][k]
+      if (A_K) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(a[i]) = *reinterpret_cast<const float4*>(As + (ty + 16 * i) * kRowK + k);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(As + (k + c) * BM + ty * 4);
+          a[0][c] = v.x; a[1][c] = v.y; a[2][c] = v.z; a[3][c] = v.w;
+        }
+      }
+      if (B_K) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(b[j]) = *reinterpret_cast<const float4*>(Bs + (tx + 16 * j) * kRowK + k);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float4 v = *reinterpret_cast<const float4*>(Bs + (k + c) * BN + tx * 4);
+          b[0][c] = v.x; b[1][c] = v.y; b[2][c] = v.z; b[3][c] = v.w;
+        }
+      }
+      if (SCALE_K) {
+        const float4 z = *reinterpret_cast<const float4*>(Zs + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { b[j][0] *= z.x; b[j][1] *= z.y; b[j][2] *= z.z; b[j][3] *= z.w; }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i][c], b[j][c], acc[i][j]);
     }
-    __syncthreads();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();                                         // every stage has been read: the partial tile takes their place
 #pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[k][tm]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tn]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
+    for (int j = 0; j < 4; ++j)
+      smem[(A_K ? ty + 16 * i : ty * 4 + i) * kRowP + (B_K ? tx + 16 * j : tx * 4 + j)] = acc[i][j];
+  if (n_split > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
     __syncthreads();
   }
+  // this CTA finishes rows [split, split + 1) * BM / n_split of the tile, 16 lanes per row, 4 columns each
+  const int rows = BM / n_split;
+  const bool c_vec = (reinterpret_cast<uintptr_t>(p.C) & 15) == 0 && (p.ldc & 3) == 0;
+  for (int lr = ty; lr < rows; lr += 16) {
+    const int r = split * rows + lr, gm = m0 + r, gn = n0 + tx * 4;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint32_t at = smem_addr(smem + r * kRowP + tx * 4);
+    for (int s = 0; s < n_split; ++s) {
+      uint32_t peer;
+      float x, y, z, w;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(s));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x), "=f"(y), "=f"(z), "=f"(w) : "r"(peer) : "memory");
+      v[0] += x; v[1] += y; v[2] += z; v[3] += w;
+    }
+    if (p.qdot) {
+      double dot = 0.0;
+      if (gm < p.M)
+        for (int j = 0; j < 4; ++j)
+          if (gn + j < p.N) dot += (double)v[j] * (double)p.qdot[(int64_t)gm * p.ldq + gn + j];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + tm + i;
-    if (gm >= p.M) continue;
-    const float rs = p.row_scale ? p.row_scale[gm] : 1.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tn + j;
-      if (gn >= p.N) continue;
-      float v = acc[i][j] * rs;
-      if (p.col_scale) v *= p.col_scale[gn];
+      for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);   // rows is 8..64: warps are in the loop as a whole
+      if (tx == 0 && gm < p.M) p.dz_part[(int64_t)blockIdx.x * p.dz_stride + gm] = dot;
+    }
+    if (p.C && gm < p.M) {
+      const float rs = p.row_scale ? p.row_scale[gm] : 1.f;
       float* c = p.C + (int64_t)gm * p.ldc + gn;
-      *c = p.accumulate ? *c + v : v;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        v[j] *= rs;
+        if (p.col_scale && gn + j < p.N) v[j] *= p.col_scale[gn + j];
+      }
+      if (c_vec && gn + 4 <= p.N) {
+        float4 w = make_float4(v[0], v[1], v[2], v[3]);
+        if (p.accumulate) { const float4 o = *reinterpret_cast<const float4*>(c); w.x += o.x; w.y += o.y; w.z += o.z; w.w += o.w; }
+        *reinterpret_cast<float4*>(c) = w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (gn + j < p.N) c[j] = p.accumulate ? c[j] + v[j] : v[j];
+      }
     }
   }
+  if (n_split > 1) {       // no CTA leaves while another still reads its shared memory
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+
+}  // namespace simt
+
+// dlog_alpha[k] (=|+=) dz_dla[k] * sum_p dz_part[p][k], fp64 partials of the fp32 path added in order.
+__global__ void __launch_bounds__(256)
+dalpha_f64_kernel(const double* __restrict__ dz_part, int n_part, int64_t part_stride, const float* __restrict__ dz_dla, int r,
+                  float* __restrict__ dlog_alpha, int accumulate) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= r) return;
+  double s = 0.0;
+  for (int p = 0; p < n_part; ++p) s += dz_part[(int64_t)p * part_stride + k];
+  const float v = (float)s * dz_dla[k];
+  dlog_alpha[k] = accumulate ? dlog_alpha[k] + v : v;
 }
 
 }  // namespace flop
