@@ -954,6 +954,22 @@ int builtin_scratch(L0Scratch** out) {
 
 }  // namespace
 
+template <typename T>
+static int launch_compact_fused(const float* in, int mode, double thr, int64_t r, int32_t* idx, int32_t* k_dev, float* z_det, const void* P,
+                                int64_t ldp, const void* Q, int64_t ldq, int64_t d_in, int64_t d_out, void* Pc, int64_t ldpc, void* Qc,
+                                int64_t ldqc, cudaStream_t st) {
+  const int vec_q = aligned16(Q) && aligned16(Qc) && (ldq * sizeof(T)) % 16 == 0 && (ldqc * sizeof(T)) % 16 == 0;
+  const int pair_p = reinterpret_cast<uintptr_t>(Pc) % (2 * sizeof(T)) == 0 && ldpc % 2 == 0;
+  const int64_t rows = d_out + (d_in > 0 ? r : 0);                           // a warp each, at most four blocks per SM
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms() * 4));
+  auto kern = r <= 4 * kFusedThreads ? compact_fused_kernel<T, 4> : compact_fused_kernel<T, kFusedMaxR / kFusedThreads>;
+  launch_k(kern, dim3((unsigned)grid), dim3(kFusedThreads), (size_t)0, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
+           (const T*)Q, ldq, (int)d_in, (int)d_out, (T*)Pc, ldpc, (T*)Qc, ldqc, vec_q, pair_p);
+  count_launch();
+  FLOP_CUDA(cudaGetLastError());
+  return FLOP_OK;
+}
+
 // ====================================================================== C ABI
 extern "C" {
 
@@ -2077,6 +2093,12 @@ int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t h
   }
   cudaStream_t st = (cudaStream_t)stream;
   const double thr = (double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta);
+  if (r <= kFusedMaxR) {   // every block repeats the selection; beyond, the repetition would cost more than a launch
+    const int64_t pd = gather ? d_out : 0, qd = gather ? d_in : 0;
+    if (pd > INT32_MAX / 2 || qd > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
+    return dt == FLOP_BF16 ? launch_compact_fused<bf16>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st)
+                           : launch_compact_fused<float>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st);
+  }
   launch_k(compact_select_kernel, dim3(1), dim3(kSelThreads), (size_t)(0), st, log_alpha_or_z, mode, thr, (int)r, idx, k_dev, z_det);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
