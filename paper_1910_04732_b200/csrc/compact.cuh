@@ -1,6 +1,6 @@
 // Deterministic inference mask and rank compaction (Sections 4.4 and 4.1).
 //
-// Ranks up to kFusedMaxR: compact_fused_kernel does all of the following in one launch.  Larger ranks:
+// Ranks up to kFusedMaxR with P up to kFusedMaxBytes: compact_fused_kernel does all of the following in one launch.  Else:
 //   compact_select_kernel : one block.  mode 0: pi_j in fp64, k = floor(sum pi + 1/2),
 //       exact top-k of log_alpha by a 4-pass radix select on order-preserving
 //       keys (ties -> lower index), then a block scan (warp shuffles) that
@@ -306,7 +306,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 }
 
 // ---------------------------------------------------------------------------------------------
-// Selection and both gathers in one launch, for ranks up to kFusedMaxR.
+// Selection and both gathers in one launch.
 //
 // Bound: latency.  The factors of one matrix are 1-10 MB (0.2-1.5 us of memory time), but the selection is a chain
 // of dependent steps, and as a launch of its own (one block of 1024 threads, 13 us) it kept 147 SMs waiting.  Here
@@ -320,12 +320,18 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // a load touches only a few lines, and a row needs neither staging nor a barrier.
 // Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (three launches each: 13.0 + 4.0 + 5.8 us
 // of GPU time); what is left there is the caller's time per call.
-constexpr int kFusedMaxR = 4096;
+// Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
+// saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74), and for long P the staged
+// gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
+constexpr int kFusedMaxR = 1024;
+constexpr int64_t kFusedMaxBytes = 16 << 20;
 constexpr int kFusedThreads = 256, kFusedWarps = kFusedThreads / 32;
 
 template <typename T> struct alignas(2 * sizeof(T)) Pair2 { T e[2]; };
 
-template <typename T, int kKeys>   // gates per thread: r <= kKeys * kFusedThreads
+constexpr int kKeys = kFusedMaxR / kFusedThreads;   // gates per thread
+
+template <typename T>
 __global__ void __launch_bounds__(kFusedThreads)
 compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, int32_t* __restrict__ idx, int32_t* __restrict__ k_dev,
                      float* __restrict__ z_det, const T* __restrict__ P, int64_t ldp, const T* __restrict__ Q, int64_t ldq, int d_in,

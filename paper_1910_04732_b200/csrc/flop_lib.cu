@@ -962,8 +962,7 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
   const int pair_p = reinterpret_cast<uintptr_t>(Pc) % (2 * sizeof(T)) == 0 && ldpc % 2 == 0;
   const int64_t rows = d_out + (d_in > 0 ? r : 0);                           // a warp each, at most four blocks per SM
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms() * 4));
-  auto kern = r <= 4 * kFusedThreads ? compact_fused_kernel<T, 4> : compact_fused_kernel<T, kFusedMaxR / kFusedThreads>;
-  launch_k(kern, dim3((unsigned)grid), dim3(kFusedThreads), (size_t)0, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
+  launch_k(compact_fused_kernel<T>, dim3((unsigned)grid), dim3(kFusedThreads), (size_t)0, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
            (const T*)Q, ldq, (int)d_in, (int)d_out, (T*)Pc, ldpc, (T*)Qc, ldqc, vec_q, pair_p);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
@@ -2093,9 +2092,8 @@ int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t h
   }
   cudaStream_t st = (cudaStream_t)stream;
   const double thr = (double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta);
-  if (r <= kFusedMaxR) {   // every block repeats the selection; beyond, the repetition would cost more than a launch
-    const int64_t pd = gather ? d_out : 0, qd = gather ? d_in : 0;
-    if (pd > INT32_MAX / 2 || qd > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
+  const int64_t pd = gather ? d_out : 0, qd = gather ? d_in : 0;
+  if (r <= kFusedMaxR && pd <= kFusedMaxBytes / (int64_t)(std::max<int64_t>(r, 1) * elt(dt)) && qd <= INT32_MAX) {
     return dt == FLOP_BF16 ? launch_compact_fused<bf16>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st)
                            : launch_compact_fused<float>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st);
   }

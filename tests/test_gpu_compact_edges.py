@@ -1,5 +1,4 @@
-"""Selection and gathers in one launch: ranks at the edges of its two key counts (1024, 4096) and of the ranks it serves, odd
-numbers of survivors, outputs whose rows allow no paired stores, ties at the cut.  A gather moves values: exact."""
+"""Selection and gathers in one launch (ranks up to 1024) and in three: ranks at word, block and route edges, odd numbers of survivors, outputs whose rows allow no paired stores, ties at the cut.  A gather moves values: exact."""
 import numpy as np
 import pytest
 import torch
@@ -18,7 +17,7 @@ def b():
     return binding
 
 
-@pytest.mark.parametrize("r", [1, 31, 256, 257, 1023, 1024, 1025, 4095, 4096, 4097])
+@pytest.mark.parametrize("r", [1, 31, 256, 257, 1023, 1024, 1025, 4097])
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("odd_ld", [False, True])
 @pytest.mark.parametrize("ties", [False, True])
@@ -39,6 +38,6 @@ def test_mask_and_compact_factors(b, r, dtype, odd_ld, ties):
     assert np.max(np.abs(host(zd) - zo)) < 1e-7
     Pco, Qco = O.compact_ranks(host(P), host(Q), idxo, host(zd))
     assert np.array_equal(host(Pc)[:, :k], Pco) and np.all(np.isnan(host(Pc)[:, k:])) and np.all(np.isnan(host(Qc)[k:]))
-    if k:      # one rounding of each product: half an ulp, 2^-9 (bf16) or 2^-24 (fp32) relative
-        assert np.all(np.abs(host(Qc)[:k] - Qco) <= (2.0 ** -8.9 if dtype == "bf16" else 2.0 ** -23.9) * np.abs(Qco))
+    if k:      # one rounding of each product to 8 (bf16) or 24 (fp32) significant bits: at most 2^-8 or 2^-24 relative
+        assert np.all(np.abs(host(Qc)[:k] - Qco) <= (2.0 ** -8 if dtype == "bf16" else 2.0 ** -24) * np.abs(Qco))
     assert b.device_status() == b.OK
