@@ -1,46 +1,73 @@
 // Gated adaptive embedding of one word cluster (Section 4.2 of the paper): E~ = E G O.
 // The lookup replaces the first GEMM of the gated layer by a row gather; the projection with O
 // and the backward products are the tensor-core GEMMs used everywhere else.
-//   embed_gather_kernel : H'[t, :] = E[ids[t], :] * z                       (one warp per token)
+//   embed_gather_kernel : H'[t, :] = E[ids[t], :] * z
 //   embed_bwd_kernel    : dE[ids[t], :] += dH'[t, :] * z   (fp32 atomic adds: rows repeat across tokens)
 //                         part[b][k]    = sum over the block's tokens of E[ids[t], k] dH'[t, k]
-//                         (the per-block partial sums of dz are then added in block order)
+//   embed_finish_kernel : dlog_alpha from the per-block partial sums, and dO from the split-K slices of its GEMM
+//
+// The two token kernels are bound by the latency of a chain: token -> row of E -> store or atomic add.  A warp
+// therefore takes kEmbTokens tokens at once and has all their ids, then all their rows in flight before it uses the first;
+// rows narrower than 32 pieces of 8 columns share the warp (LPT lanes per token), so that no lane idles at
+// 64 or 128 columns.  Walking eight tokens one after another, one warp per SM scheduler, took 33.5 us for 16 384 tokens of
+// 256 columns, and adding up 256 partial vectors by one thread per column another 17 us.
 #pragma once
 #include "common.cuh"
+#include "wgrad.cuh"
 
 namespace flop {
 
 constexpr int kEmbWarps = 8;
-constexpr int kEmbTokensPerWarp = 8;   // tokens a warp walks in the backward kernel
+constexpr int kEmbTokens = 4;   // tokens a warp has in flight (per lane group)
+// Tokens of a backward block.  Fixed for every width, so that the partial sums (one vector per block) have one size.
+constexpr int kEmbBlockTokens = 32;
 
+// Lanes that share a token's row: 8 columns per lane and pass.
+inline int embed_lanes(int64_t d_i) { return d_i <= 64 ? 8 : d_i <= 128 ? 16 : 32; }
+
+template <int LPT>
 __global__ void __launch_bounds__(32 * kEmbWarps)
 embed_gather_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __restrict__ E, int64_t lde, int n_rows,
                     const float* __restrict__ z, int d_i, __nv_bfloat16* __restrict__ H, int64_t ldh) {
   pdl_wait();
   pdl_launch_dependents();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kEmbWarps + warp;
-  if (t >= T) return;
-  const int w = min(max(ids[t], 0), n_rows - 1);      // out-of-range ids are clamped, never dereferenced
-  const __nv_bfloat16* e = E + (int64_t)w * lde;
-  __nv_bfloat16* h = H + (int64_t)t * ldh;
-  for (int k = lane * 8; k < d_i; k += 32 * 8) {
-    if (k + 8 <= d_i) {
-      uint4 raw = *reinterpret_cast<const uint4*>(e + k);
-      __nv_bfloat16* v = reinterpret_cast<__nv_bfloat16*>(&raw);
+  constexpr int G = 32 / LPT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPT, l = lane % LPT;
+  const int t0 = (blockIdx.x * kEmbWarps + warp) * (kEmbTokens * G) + grp;       // this lane group: t0, t0 + G, ...
+  int w[kEmbTokens];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = __float2bfloat16_rn(__bfloat162float(v[i]) * __ldg(z + k + i));
-      *reinterpret_cast<uint4*>(h + k) = raw;
+  for (int i = 0; i < kEmbTokens; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;   // out-of-range ids are clamped, never dereferenced
+  for (int k = l * 8; k < d_i; k += LPT * 8) {
+    if (k + 8 <= d_i) {
+      uint4 raw[kEmbTokens];
+#pragma unroll
+      for (int i = 0; i < kEmbTokens; ++i)
+        if (t0 + i * G < T) raw[i] = *reinterpret_cast<const uint4*>(E + (int64_t)w[i] * lde + k);
+      float zk[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) zk[j] = __ldg(z + k + j);
+#pragma unroll
+      for (int i = 0; i < kEmbTokens; ++i) {
+        if (t0 + i * G < T) {
+          __nv_bfloat16* v = reinterpret_cast<__nv_bfloat16*>(&raw[i]);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = __float2bfloat16_rn(__bfloat162float(v[j]) * zk[j]);
+          *reinterpret_cast<uint4*>(H + (int64_t)(t0 + i * G) * ldh + k) = raw[i];
+        }
+      }
     } else {
-      for (int i = k; i < d_i; ++i) h[i] = __float2bfloat16_rn(__bfloat162float(e[i]) * z[i]);
+      for (int i = 0; i < kEmbTokens; ++i)
+        if (t0 + i * G < T)
+          for (int j = k; j < d_i; ++j)
+            H[(int64_t)(t0 + i * G) * ldh + j] = __float2bfloat16_rn(__bfloat162float(E[(int64_t)w[i] * lde + j]) * z[j]);
     }
   }
 }
 
-// Block b handles tokens [b * 64, b * 64 + 64): warp w its 8 consecutive tokens.  A lane owns 8
-// consecutive columns of every 256-column chunk (16-byte loads of dH' and E), so the per-column
-// partial sums of dz need no cross-lane step; the eight warps' partials are added in warp order
-// through shared memory.  dE takes 16-byte vector atomic adds when its rows allow them.
+// Block b handles tokens [b * 32, b * 32 + 32).  A lane owns 8 consecutive columns of every LPT * 8 columns (16-byte
+// loads of dH' and E); the lane groups' and the warps' partial sums of dz are added in a fixed order (shuffles, then
+// shared memory in warp order).  dE takes 16-byte vector atomic adds when its rows allow them.
+template <int LPT>
 __global__ void __launch_bounds__(32 * kEmbWarps)
 embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __restrict__ E, int64_t lde, int n_rows,
                  const float* __restrict__ z, int d_i, const __nv_bfloat16* __restrict__ dH, int64_t lddh,
@@ -48,59 +75,127 @@ embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __
   pdl_wait();
   pdl_launch_dependents();
   extern __shared__ float red[];   // [kEmbWarps][d_i]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t0 = (blockIdx.x * kEmbWarps + warp) * kEmbTokensPerWarp;
+  constexpr int G = 32 / LPT;                                        // tokens side by side in a warp
+  constexpr int kIn = kEmbBlockTokens / kEmbWarps / G > 0 ? kEmbBlockTokens / kEmbWarps / G : 1;   // ... and one after another, in flight together
+  static_assert(kIn * G * kEmbWarps == kEmbBlockTokens, "a block's tokens are dealt out evenly");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPT, l = lane % LPT;
+  const int t0 = blockIdx.x * kEmbBlockTokens + warp * (kIn * G) + grp;
   const bool vec_de = dE && (reinterpret_cast<uintptr_t>(dE) & 15) == 0 && (ldde % 4) == 0;
-  for (int k = lane * 8; k < d_i; k += 32 * 8) {
-    const int nk = min(8, d_i - k);
-    float zk[8], acc[8];
+  int w[kIn];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { zk[i] = i < nk ? z[k + i] : 0.f; acc[i] = 0.f; }
-    for (int i = 0; i < kEmbTokensPerWarp; ++i) {
-      const int t = t0 + i;
-      if (t >= T) break;
-      const int w = min(max(ids[t], 0), n_rows - 1);
-      float gv[8], ev[8];
-      if (nk == 8) {   // rows of dH' and E are 16-byte aligned (ld % 8 == 0)
-        const uint4 graw = *reinterpret_cast<const uint4*>(dH + (int64_t)t * lddh + k);
-        const uint4 eraw = *reinterpret_cast<const uint4*>(E + (int64_t)w * lde + k);
-        const __nv_bfloat162* gh = reinterpret_cast<const __nv_bfloat162*>(&graw);
-        const __nv_bfloat162* eh = reinterpret_cast<const __nv_bfloat162*>(&eraw);
+  for (int i = 0; i < kIn; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;
+  for (int k0 = 0; k0 < d_i; k0 += LPT * 8) {
+    const int k = k0 + l * 8, nk = min(8, d_i - k);                  // nk <= 0: no column for this lane in the last pass
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (nk == 8) {   // rows of dH' and E are 16-byte aligned (ld % 8 == 0)
+      uint4 graw[kIn], eraw[kIn];
+#pragma unroll
+      for (int i = 0; i < kIn; ++i) {
+        graw[i] = eraw[i] = make_uint4(0, 0, 0, 0);
+        if (t0 + i * G < T) {
+          graw[i] = __ldcs(reinterpret_cast<const uint4*>(dH + (int64_t)(t0 + i * G) * lddh + k));
+          eraw[i] = *reinterpret_cast<const uint4*>(E + (int64_t)w[i] * lde + k);
+        }
+      }
+      float zk[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) zk[j] = __ldg(z + k + j);
+#pragma unroll
+      for (int i = 0; i < kIn; ++i) {
+        const __nv_bfloat162* gh = reinterpret_cast<const __nv_bfloat162*>(&graw[i]);
+        const __nv_bfloat162* eh = reinterpret_cast<const __nv_bfloat162*>(&eraw[i]);
+        float gv[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const float2 a = __bfloat1622float2(gh[j]), c = __bfloat1622float2(eh[j]);
-          gv[2 * j] = a.x; gv[2 * j + 1] = a.y; ev[2 * j] = c.x; ev[2 * j + 1] = c.y;
+          gv[2 * j] = a.x; gv[2 * j + 1] = a.y;
+          acc[2 * j] = fmaf(c.x, a.x, acc[2 * j]);
+          acc[2 * j + 1] = fmaf(c.y, a.y, acc[2 * j + 1]);
         }
-      } else {
+        if (dE && t0 + i * G < T) {
+          float* o = dE + (int64_t)w[i] * ldde + k;
+          if (vec_de) {
+            atomicAdd(reinterpret_cast<float4*>(o), make_float4(gv[0] * zk[0], gv[1] * zk[1], gv[2] * zk[2], gv[3] * zk[3]));
+            atomicAdd(reinterpret_cast<float4*>(o + 4), make_float4(gv[4] * zk[4], gv[5] * zk[5], gv[6] * zk[6], gv[7] * zk[7]));
+          } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          gv[j] = j < nk ? __bfloat162float(dH[(int64_t)t * lddh + k + j]) : 0.f;
-          ev[j] = j < nk ? __bfloat162float(E[(int64_t)w * lde + k + j]) : 0.f;
+            for (int j = 0; j < 8; ++j)
+              if (zk[j] != 0.f) atomicAdd(o + j, gv[j] * zk[j]);
+          }
         }
       }
+    } else if (nk > 0) {
+      for (int i = 0; i < kIn; ++i) {
+        const int t = t0 + i * G;
+        if (t >= T) break;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = fmaf(ev[j], gv[j], acc[j]);
-      if (dE) {
-        float* o = dE + (int64_t)w * ldde + k;
-        if (vec_de && nk == 8) {
-          atomicAdd(reinterpret_cast<float4*>(o), make_float4(gv[0] * zk[0], gv[1] * zk[1], gv[2] * zk[2], gv[3] * zk[3]));
-          atomicAdd(reinterpret_cast<float4*>(o + 4), make_float4(gv[4] * zk[4], gv[5] * zk[5], gv[6] * zk[6], gv[7] * zk[7]));
-        } else {
-          for (int j = 0; j < nk; ++j)
-            if (zk[j] != 0.f) atomicAdd(o + j, gv[j] * zk[j]);
+        for (int j = 0; j < 8; ++j) {
+          if (j < nk) {
+            const float gj = __bfloat162float(dH[(int64_t)t * lddh + k + j]), zj = z[k + j];
+            acc[j] = fmaf(__bfloat162float(E[(int64_t)w[i] * lde + k + j]), gj, acc[j]);
+            if (dE && zj != 0.f) atomicAdd(dE + (int64_t)w[i] * ldde + k + j, gj * zj);
+          }
         }
       }
     }
-    for (int j = 0; j < nk; ++j) red[warp * d_i + k + j] = acc[j];
+#pragma unroll
+    for (int o = LPT; o < 32; o <<= 1)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+    if (grp == 0)
+      for (int j = 0; j < nk; ++j) red[warp * d_i + k + j] = acc[j];
   }
   __syncthreads();
   if (part) {
     for (int k = threadIdx.x; k < d_i; k += blockDim.x) {
       float s = 0.f;
-      for (int w = 0; w < kEmbWarps; ++w) s += red[w * d_i + k];
+      for (int w8 = 0; w8 < kEmbWarps; ++w8) s += red[w8 * d_i + k];
       part[(int64_t)blockIdx.x * d_i + k] = s;
     }
   }
+}
+
+// Blocks [0, dla_blocks): 32 gates each, dlog_alpha[k] (=|+=) dz_dla[k] * sum of the n_part partial vectors (a warp adds
+// a run of consecutive vectors, the runs are added in warp order).  The other blocks: dO (=|+=) the ordered sum of the
+// split-K slices, four columns per thread.
+struct EmbedFinish {
+  const float* part; int n_part, d_i; const float* dz_dla; float* dla; int dla_blocks;
+  const float* slices; int n_slices; int64_t slice_elems, ld_slice; void* dO; int64_t lddo; int d;
+  int accumulate;
+};
+
+template <typename TW>
+__global__ void __launch_bounds__(256)
+embed_finish_kernel(const EmbedFinish a) {
+  pdl_wait();
+  pdl_launch_dependents();
+  if ((int)blockIdx.x < a.dla_blocks) {
+    __shared__ float run[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * 32 + lane;
+    const int per = (a.n_part + 7) / 8, p1 = min(a.n_part, (warp + 1) * per);
+    float s = 0.f;
+    if (k < a.d_i) {
+#pragma unroll 8
+      for (int p = warp * per; p < p1; ++p) s += a.part[(int64_t)p * a.d_i + k];
+    }
+    run[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && k < a.d_i) {
+      s = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += run[w][lane];
+      const float v = s * a.dz_dla[k];
+      a.dla[k] = a.accumulate ? a.dla[k] + v : v;
+    }
+    return;
+  }
+  constexpr int al = sizeof(TW) == 4 ? 15 : 7;
+  const bool vec = (reinterpret_cast<uintptr_t>(a.dO) & al) == 0 && a.lddo % 4 == 0;
+  const int c4 = (a.d + 3) >> 2;
+  const int64_t units = (int64_t)a.d_i * c4, step = (int64_t)(gridDim.x - a.dla_blocks) * blockDim.x;
+  for (int64_t u = (int64_t)(blockIdx.x - a.dla_blocks) * blockDim.x + threadIdx.x; u < units; u += step)
+    reduce_unit<TW>(a.slices, a.n_slices, a.slice_elems, a.ld_slice, (int)(u / c4), (int)(u % c4) * 4, a.d, 1.f, (TW*)a.dO, a.lddo,
+                    a.accumulate, vec);
 }
 
 }  // namespace flop

@@ -969,6 +969,29 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
   return FLOP_OK;
 }
 
+// Room for the split-K slices of dO: the query knows the tokens and the cluster's width but not the output width d, so
+// it reserves 8 bytes per element of dH' (2 T / d slices of d_i x d floats), at most 64 MB; the call splits no finer.
+static size_t embedding_slice_bytes(int64_t T, int64_t d_i) {
+  return (size_t)std::min<int64_t>(64ll << 20, T * round_up(std::max<int64_t>(d_i, 1), 8) * 8);
+}
+static int64_t embedding_blocks(int64_t T) { return (T + kEmbBlockTokens - 1) / kEmbBlockTokens; }
+template <int LPT>
+static void launch_embed_gather(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
+                                void* H, int64_t ldh, cudaStream_t st) {
+  constexpr int per_block = kEmbWarps * kEmbTokens * (32 / LPT);
+  launch_k(embed_gather_kernel<LPT>, dim3((unsigned)((T + per_block - 1) / per_block)), dim3(32 * kEmbWarps), (size_t)0, st, ids, (int)T,
+           (const bf16*)E, lde, (int)n_rows, z, (int)d_i, (bf16*)H, ldh);
+}
+template <int LPT>
+static int launch_embed_bwd(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
+                            const bf16* dH, int64_t lddh, float* dE, int64_t ldde, float* part, cudaStream_t st) {
+  const size_t smem = (size_t)kEmbWarps * d_i * 4;
+  if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(embed_bwd_kernel<LPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  launch_k(embed_bwd_kernel<LPT>, dim3((unsigned)embedding_blocks(T)), dim3(32 * kEmbWarps), smem, st, ids, (int)T, (const bf16*)E, lde,
+           (int)n_rows, z, (int)d_i, dH, lddh, dE, ldde, part);
+  return FLOP_OK;
+}
+
 // ====================================================================== C ABI
 extern "C" {
 
@@ -1997,9 +2020,9 @@ int flop_agp_gates(const float* g, int64_t n, const int64_t* seg_off, int32_t n_
 // ---- gated adaptive embedding of one word cluster (Section 4.2): Y = (E[ids] * z) O
 static size_t embedding_ws_bytes(int64_t T, int64_t d_i) {
   Arena ar{nullptr, 0, 0};
-  ar.take((size_t)T * round_up(std::max<int64_t>(d_i, 1), 8) * 2);                                   // dH'
-  const int64_t blocks = (T + kEmbWarps * kEmbTokensPerWarp - 1) / (kEmbWarps * kEmbTokensPerWarp);
-  ar.take((size_t)std::max<int64_t>(blocks, 1) * std::max<int64_t>(d_i, 1) * 4);                     // dz partials
+  ar.take((size_t)T * round_up(std::max<int64_t>(d_i, 1), 8) * 2);                                              // dH'
+  ar.take((size_t)std::max<int64_t>(embedding_blocks(T), 1) * std::max<int64_t>(d_i, 1) * 4);                   // dz partials
+  ar.take(embedding_slice_bytes(T, d_i));                                                                       // dO slices
   return align_up(ar.used, 256);
 }
 
@@ -2015,8 +2038,10 @@ int flop_gated_embedding_fwd(const int32_t* ids, int64_t T, const void* E, int64
   if (!bf16_ok(E, lde) || !bf16_ok(O, ldo) || !bf16_ok(Y, ldy) || !bf16_ok(H_save, ldh)) return FLOP_ERR_UNSUPPORTED;
   if (T > INT32_MAX || n_rows > INT32_MAX || d_i > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
   cudaStream_t st = (cudaStream_t)stream;
-  launch_k(embed_gather_kernel, dim3((unsigned)((T + kEmbWarps - 1) / kEmbWarps)), dim3(32 * kEmbWarps), (size_t)0, st, ids, (int)T,
-           (const bf16*)E, lde, (int)n_rows, z, (int)d_i, (bf16*)H_save, ldh);
+  const int lanes = embed_lanes(d_i);
+  if (lanes == 8)       launch_embed_gather<8>(ids, T, E, lde, n_rows, z, d_i, H_save, ldh, st);
+  else if (lanes == 16) launch_embed_gather<16>(ids, T, E, lde, n_rows, z, d_i, H_save, ldh, st);
+  else                  launch_embed_gather<32>(ids, T, E, lde, n_rows, z, d_i, H_save, ldh, st);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   // Y[T, d] = H'[T, d_i] O[d_i, d]: B(n, k) = O[k, n] is read "transposed" (MN-major)
@@ -2050,27 +2075,52 @@ int flop_gated_embedding_bwd(const void* dY, int64_t lddy, const int32_t* ids, i
   Arena ar{(unsigned char*)ws, ws_bytes, 0};
   const int64_t lddh = round_up(d_i, 8);
   bf16* dH = (bf16*)ar.take((size_t)T * lddh * 2);
-  const int64_t blocks = (T + kEmbWarps * kEmbTokensPerWarp - 1) / (kEmbWarps * kEmbTokensPerWarp);
+  const int64_t blocks = embedding_blocks(T);
   float* part = (float*)ar.take((size_t)blocks * d_i * 4);
+  const size_t slice_bytes = embedding_slice_bytes(T, d_i);
+  float* slices = (float*)ar.take(slice_bytes);
+  EmbedFinish fin{};
+  fin.accumulate = accumulate; fin.d_i = (int)d_i; fin.d = (int)d;
   // dH'[T, d_i] = dY[T, d] O^T: B(n = k_dim, k = j) = O[n, j] (K-major as stored)
   FLOP_TRY(launch_tc({dY, lddy, false}, {O, ldo, false}, T, d_i, d, plan_tc(T, d_i, d, false, false),
                      store_epilogue(dH, lddh, nullptr), st));
   if (dO) {
-    // dO[d_i, d] = H'^T dY: contraction over tokens, written in place when the output allows 16-byte vectors
-    TcPlan pl = plan_tc(d_i, d, T, false, true);
-    FLOP_TRY(launch_tc({H_save, ldh, true}, {dY, lddy, true}, d_i, d, T, pl, wgrad_epilogue(dO, lddo, wgrad_dt, nullptr, accumulate), st));
+    // dO[d_i, d] = H'^T dY: contraction over the tokens.  A cluster's few tiles cannot fill the machine, so K is split as
+    // far as the cost model wants and the workspace allows; unsplit, the result is written in place.
+    TcPlan pl = plan_tc(d_i, d, T, true, true);
+    const int64_t ld_slice = round_up(d, 4), max_splits = (int64_t)(slice_bytes / ((size_t)d_i * ld_slice * 4));
+    if (pl.splits > max_splits) {
+      if (max_splits >= 2) {
+        pl.kb_per_split = (int)((pl.num_kb + max_splits - 1) / max_splits);
+        pl.splits = (pl.num_kb + pl.kb_per_split - 1) / pl.kb_per_split;
+      } else {
+        pl = plan_tc(d_i, d, T, false, true);
+      }
+    }
+    TcEpilogue e = wgrad_epilogue(dO, lddo, wgrad_dt, nullptr, accumulate);
+    if (pl.splits > 1) {
+      e = TcEpilogue{};
+      e.kind = tc::EPI_SLICE; e.slices = slices; e.slice_elems = d_i * ld_slice; e.ld_slice = ld_slice;
+      fin.slices = slices; fin.n_slices = pl.splits; fin.slice_elems = e.slice_elems; fin.ld_slice = ld_slice; fin.dO = dO; fin.lddo = lddo;
+    }
+    FLOP_TRY(launch_tc({H_save, ldh, true}, {dY, lddy, true}, d_i, d, T, pl, e, st));
   }
   if (dE || dlog_alpha) {
-    const size_t smem = (size_t)kEmbWarps * d_i * 4;
-    if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(embed_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_k(embed_bwd_kernel, dim3((unsigned)blocks), dim3(32 * kEmbWarps), smem, st, ids, (int)T, (const bf16*)E, lde, (int)n_rows, z,
-             (int)d_i, (const bf16*)dH, lddh, dE, ldde, dlog_alpha ? part : nullptr);
+    const int lanes = embed_lanes(d_i);
+    float* dz = dlog_alpha ? part : nullptr;
+    FLOP_TRY(lanes == 8    ? launch_embed_bwd<8>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st)
+             : lanes == 16 ? launch_embed_bwd<16>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st)
+                           : launch_embed_bwd<32>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st));
     count_launch();
-    if (dlog_alpha) {
-      launch_k(dalpha_kernel, dim3((unsigned)((d_i + 255) / 256)), dim3(256), (size_t)0, st, (const float*)part, (int)blocks, d_i, dz_dla,
-               (int)d_i, dlog_alpha, accumulate);
-      count_launch();
-    }
+    FLOP_CUDA(cudaGetLastError());
+  }
+  if (dlog_alpha) { fin.part = part; fin.n_part = (int)blocks; fin.dz_dla = dz_dla; fin.dla = dlog_alpha; fin.dla_blocks = (int)((d_i + 31) / 32); }
+  if (dlog_alpha || fin.slices) {
+    const int64_t units = fin.slices ? d_i * ((d + 3) / 4) : 0;
+    const int grid = fin.dla_blocks + (int)std::min<int64_t>((units + 255) / 256, (int64_t)num_sms() * 8);
+    if (wgrad_dt == FLOP_BF16) launch_k(embed_finish_kernel<bf16>, dim3((unsigned)grid), dim3(256), (size_t)0, st, fin);
+    else                       launch_k(embed_finish_kernel<float>, dim3((unsigned)grid), dim3(256), (size_t)0, st, fin);
+    count_launch();
     FLOP_CUDA(cudaGetLastError());
   }
   return FLOP_OK;

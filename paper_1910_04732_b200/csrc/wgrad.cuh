@@ -6,21 +6,6 @@
 
 namespace flop {
 
-// dlog_alpha[k] (=|+=) dz_dla[k] * sum_p dz_part[p][k], partials added in order.
-__global__ void __launch_bounds__(256)
-dalpha_kernel(const float* __restrict__ dz_part, int n_part, int64_t part_stride, const float* __restrict__ dz_dla,
-              int r, float* __restrict__ dlog_alpha, int accumulate) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= r) return;
-  float s = 0.f;
-  for (int p = 0; p < n_part; ++p) s += dz_part[(int64_t)p * part_stride + k];
-  const float v = s * dz_dla[k];
-  dlog_alpha[k] = accumulate ? dlog_alpha[k] + v : v;
-}
-
-
 // One launch that finishes the backward pass of the tensor-core path:
 //   dP[i,k]      (=|+=) sum_s slices_p[s][i,k]                      (d_out x r)
 //   dQ[k,j]      (=|+=) z[k] * sum_s slices_q[s][k,j]               (r x d_in)
