@@ -29,8 +29,7 @@
 #include "l0_lagrangian.cuh"
 #include "wgrad.cuh"
 #include "active_ranks.cuh"
-#include "gemm_small_t.cuh"
-#include "gemm_skinny.cuh"
+#include "gemm_few.cuh"
 #include "agp.cuh"
 #include "embedding.cuh"
 
@@ -67,14 +66,14 @@ inline bool debug_on() {
 //   FLOP_TC_BN / FLOP_TC_STAGES / FLOP_TC_CTA2 (1 force pairs, 2 forbid)     tile shape of single GEMMs
 //   FLOP_TC_GROUP_BN / FLOP_TC_GROUP_CTA2, FLOP_TC_WGRAD_BN / FLOP_TC_WGRAD_CTA2   tile shape of grouped launches
 //   FLOP_NO_TMA_STORE=1    bf16 output tiles by per-thread stores    FLOP_NO_SCHED=1   round-robin tile order
-//   FLOP_NO_SMALL_T=1, FLOP_NO_SKINNY=1   few-token forward kernels off
+//   FLOP_NO_FEW=1          few-token forward kernel off
 //   FLOP_STAGE_MERGE=0     backward in three launches per stage instead of two shared ones
 //   FLOP_GATHER_PIPE=0     plain P gather kernel                     FLOP_NO_CHAIN=1   chained calls run unchained
 //   FLOP_CHAIN_STAGES=2    chained calls put dependent products in ONE launch (default 1: a launch per stage)
 //   FLOP_SCHED_EPI=c       per-tile fixed cost (SM cycles) in the tile schedule's cost model instead of 400 + 4 bn
 struct Tuning {
   int no_pdl = 0, tc_bn = 0, tc_stages = 0, tc_cta2 = 0, no_tma_store = 0, no_sched = 0, group_bn = 0, group_cta2 = 0,
-      wgrad_bn = 0, wgrad_cta2 = 0, no_small_t = 0, no_skinny = 0, stage_merge = 1, gather_pipe = 1, no_chain = 0, chain_stages = 1, sched_epi = 0;
+      wgrad_bn = 0, wgrad_cta2 = 0, no_few = 0, stage_merge = 1, gather_pipe = 1, no_chain = 0, chain_stages = 1, sched_epi = 0;
 };
 inline const Tuning& tuning() {
   static const Tuning t = [] {
@@ -84,7 +83,7 @@ inline const Tuning& tuning() {
     v.no_pdl = get("FLOP_NO_PDL", 0); v.tc_bn = get("FLOP_TC_BN", 0); v.tc_stages = get("FLOP_TC_STAGES", 0);
     v.tc_cta2 = get("FLOP_TC_CTA2", 0); v.no_tma_store = get("FLOP_NO_TMA_STORE", 0); v.no_sched = get("FLOP_NO_SCHED", 0);
     v.group_bn = get("FLOP_TC_GROUP_BN", 0); v.group_cta2 = get("FLOP_TC_GROUP_CTA2", 0); v.wgrad_bn = get("FLOP_TC_WGRAD_BN", 0);
-    v.wgrad_cta2 = get("FLOP_TC_WGRAD_CTA2", 0); v.no_small_t = get("FLOP_NO_SMALL_T", 0); v.no_skinny = get("FLOP_NO_SKINNY", 0);
+    v.wgrad_cta2 = get("FLOP_TC_WGRAD_CTA2", 0); v.no_few = get("FLOP_NO_FEW", 0);
     v.stage_merge = get("FLOP_STAGE_MERGE", 1); v.gather_pipe = get("FLOP_GATHER_PIPE", 1); v.no_chain = get("FLOP_NO_CHAIN", 0);
     v.chain_stages = get("FLOP_CHAIN_STAGES", 1); v.sched_epi = get("FLOP_SCHED_EPI", 0);
 #endif
@@ -732,68 +731,49 @@ int launch_chain_fwd(const void* X, int64_t ldx, const void* Q, int64_t ldq, con
   return FLOP_OK;
 }
 
-// Few-token forward product C = (A B^T) * col_scale on the CUDA cores (see gemm_small_t.cuh).
-// Returns FLOP_ERR_UNSUPPORTED when the shape does not fit (the caller then uses the tensor-core path).
-template <int TT>
-int launch_small_t_inst(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, bf16* C, int64_t ldc, const float* cs, int T,
-                        int N, int K, int k_pad, size_t smem, cudaStream_t st) {
+// Forward product for few tokens (see gemm_few.cuh).  `second`: A is what the launch before on the stream wrote, and that
+// launch wrote nothing else.
+template <int MT, int NT>
+int launch_few_inst(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, bf16* C, int64_t ldc, const float* cs, int T, int N, int K,
+                    bool second, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
-  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(small_t_gemm_kernel<TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-  const int grid = std::min((N + kSmallTWarps - 1) / kSmallTWarps, num_sms() * 4);
-  launch_k(small_t_gemm_kernel<TT>, dim3(grid), dim3(32 * kSmallTWarps), smem, st, A, lda, B, ldb, C, ldc, cs, T, N, K, k_pad);
+  constexpr int smem = few::smem_bytes(MT, NT);
+  if (smem > 48 * 1024 && first_use_on_device(configured)) {
+    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  }
+  const dim3 grid((unsigned)((N + 16 * MT - 1) / (16 * MT)), (unsigned)((T + 8 * NT - 1) / (8 * NT)));
+  launch_k(second ? few::gemm_kernel<MT, NT, true> : few::gemm_kernel<MT, NT, false>, grid, dim3(few::kThreads), (size_t)smem, st, A, lda, B,
+           ldb, C, ldc, cs, T, N, K);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
 }
-int launch_small_t(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T,
-                   int64_t N, int64_t K, cudaStream_t st) {
-  const int off = tuning().no_small_t;
-  if (off || T < 1 || T > kSmallTMax || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
-  int tt = 1;
-  while (tt < T) tt *= 2;
-  const int k_pad = (int)round_up(K, 256);                 // every lane's 8-element step stays inside the row
-  const size_t smem = (size_t)tt * k_pad * 2;
-  if (smem > (size_t)kSmemBudget) return FLOP_ERR_UNSUPPORTED;
+int64_t few_blocks(int64_t T, int64_t N) { return ((N + 31) / 32) * ((T + 63) / 64); }
+int launch_few(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
+               int64_t K, bool second, cudaStream_t st) {
   const bf16* a = (const bf16*)A; const bf16* b = (const bf16*)B; bf16* c = (bf16*)C;
-  switch (tt) {
-    case 1: return launch_small_t_inst<1>(a, lda, b, ldb, c, ldc, cs, (int)T, (int)N, (int)K, k_pad, smem, st);
-    case 2: return launch_small_t_inst<2>(a, lda, b, ldb, c, ldc, cs, (int)T, (int)N, (int)K, k_pad, smem, st);
-    default: return launch_small_t_inst<4>(a, lda, b, ldb, c, ldc, cs, (int)T, (int)N, (int)K, k_pad, smem, st);
-  }
+  const int t = (int)T, n = (int)N, k = (int)K;
+  if (T <= 8) return launch_few_inst<1, 1>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (T <= 16) return launch_few_inst<1, 2>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (T <= 32) return launch_few_inst<1, 4>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  // 32 weight rows per block read half as many token rows in all; 16 where 32 would leave half of the SMs idle
+  if (few_blocks(T, N) * 2 >= num_sms()) return launch_few_inst<2, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  return launch_few_inst<1, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
 }
-
-// Forward product for 5..16 tokens with warp-level tensor-core instructions (see gemm_skinny.cuh).
-template <int MT>
-int launch_skinny_inst(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, bf16* C, int64_t ldc, const float* cs, int T, int N,
-                       int K, int k_pad, size_t smem, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
-  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(skinny_gemm_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-  const int groups = (N + 7) / 8;
-  const int grid = std::min((groups + kSkinnyWarps - 1) / kSkinnyWarps, num_sms() * 2);
-  launch_k(skinny_gemm_kernel<MT>, dim3(grid), dim3(32 * kSkinnyWarps), smem, st, A, lda, B, ldb, C, ldc, cs, T, N, K, k_pad);
-  count_launch();
-  FLOP_CUDA(cudaGetLastError());
-  return FLOP_OK;
+// Whether a product takes the few-token kernel: up to 32 tokens, and beyond while its 32 x 64 blocks are one round over the
+// SMs.  Both products of a pair in a replayed graph, us, this kernel / tcgen05 tiles: 1024 -> 358 -> 4096 at 16, 64, 128 tokens
+// 4.7 / 11.9, 9.2 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024 tokens 16.2 / 26.6; at two rounds
+// it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
+bool few_ok(int64_t T, int64_t N, int64_t K) {
+  if (T < 1 || T > 1024 || N > INT32_MAX / 2 || K > INT32_MAX / 2 || tuning().no_few) return false;
+  return T <= 32 || few_blocks(T, N) <= num_sms();
 }
-int launch_skinny(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
-                  int64_t K, cudaStream_t st) {
-  const int off = tuning().no_skinny;
-  if (off || T < 1 || T > kSkinnyMaxT || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
-  const int mt = (int)((T + 15) / 16);
-  const int k_pad = (int)round_up(K, 32);
-  const size_t smem = (size_t)16 * mt * (k_pad + kSkinnyPad) * 2;
-  if (smem > (size_t)kSmemBudget) return FLOP_ERR_UNSUPPORTED;
-  const bf16* a = (const bf16*)A; const bf16* b = (const bf16*)B; bf16* c = (bf16*)C;
-  switch (mt) {
-    case 1: return launch_skinny_inst<1>(a, lda, b, ldb, c, ldc, cs, (int)T, (int)N, (int)K, k_pad, smem, st);
-    default: return FLOP_ERR_UNSUPPORTED;
-  }
-}
-// Few-token forward: CUDA-core streaming up to 4 tokens, warp-level tensor cores up to 16.
-int launch_few_tokens(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T,
-                      int64_t N, int64_t K, cudaStream_t st) {
-  if (T <= kSmallTMax) return launch_small_t(A, lda, B, ldb, C, ldc, cs, T, N, K, st);
-  return launch_skinny(A, lda, B, ldb, C, ldc, cs, T, N, K, st);
+// Forward product C = (A B^T) * col_scale of a layer, in the form the sizes call for.
+int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
+                       int64_t K, bool second, cudaStream_t st) {
+  if (few_ok(T, N, K)) return launch_few(A, lda, B, ldb, C, ldc, cs, T, N, K, second, st);
+  return launch_tc({A, lda, false}, {B, ldb, false}, T, N, K, plan_tc(T, N, K, false, false), store_epilogue(C, ldc, cs), st);
 }
 
 // An operand of an fp32 product: a row-major matrix read along its rows (k_fast) or down its columns.
@@ -1236,21 +1216,8 @@ static int fwd_impl(const void* X, int64_t ldx, const void* Q, int64_t ldq, cons
       if (r > 0) FLOP_TRY(zero_2d<bf16>(H, ldh, T, r, st));
       return FLOP_OK;
     }
-    if (T <= kSkinnyMaxT) {   // a few tokens: the weights are streamed once (CUDA cores up to 4 tokens, warp-level MMA up to 16)
-      const int rc = launch_few_tokens(X, ldx, Q, ldq, H, ldh, z, T, r, d_in, st);
-      if (rc == FLOP_OK) {
-        const int rc2 = launch_few_tokens(H, ldh, P, ldp, Y, ldy, nullptr, T, d_out, r, st);
-        if (rc2 != FLOP_ERR_UNSUPPORTED) return rc2;
-      } else if (rc != FLOP_ERR_UNSUPPORTED) {
-        return rc;
-      }
-    }
-    // GEMM1: H' = (X Q^T) * z, gate applied to column k in the epilogue
-    const TcPlan p1 = plan_tc(T, r, d_in, false, false);
-    FLOP_TRY(launch_tc({X, ldx, false}, {Q, ldq, false}, T, r, d_in, p1, store_epilogue(H, ldh, z), st));
-    // GEMM2: Y = H' P^T
-    const TcPlan p2 = plan_tc(T, d_out, r, false, false);
-    FLOP_TRY(launch_tc({H, ldh, false}, {P, ldp, false}, T, d_out, r, p2, store_epilogue(Y, ldy, nullptr), st));
+    FLOP_TRY(launch_fwd_product(X, ldx, Q, ldq, H, ldh, z, T, r, d_in, false, st));           // H' = (X Q^T) * z
+    FLOP_TRY(launch_fwd_product(H, ldh, P, ldp, Y, ldy, nullptr, T, d_out, r, true, st));     // Y = H' P^T
   } else {
     FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Q, ldq, true}, T, r, d_in, simt_out(H, ldh, z), st));
     FLOP_TRY(launch_simt({(const float*)H, ldh, true}, {(const float*)P, ldp, true}, T, d_out, r, simt_out(Y, ldy), st));
@@ -1315,19 +1282,8 @@ int flop_compact_fwd(const void* X, int64_t ldx, const void* Qc, int64_t ldqc, c
   const FwdWs w = plan_fwd_ws(ar, T, k, dt);
   if (dt == FLOP_BF16) {
     if (!bf16_ok(Y, ldy) || !bf16_ok(X, ldx) || !bf16_ok(Qc, ldqc) || !bf16_ok(Pc, ldpc)) return FLOP_ERR_UNSUPPORTED;
-    if (T <= kSkinnyMaxT) {
-      const int rc = launch_few_tokens(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, st);
-      if (rc == FLOP_OK) {
-        const int rc2 = launch_few_tokens(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, st);
-        if (rc2 != FLOP_ERR_UNSUPPORTED) return rc2;
-      } else if (rc != FLOP_ERR_UNSUPPORTED) {
-        return rc;
-      }
-    }
-    const TcPlan p1 = plan_tc(T, k, d_in, false, false);
-    FLOP_TRY(launch_tc({X, ldx, false}, {Qc, ldqc, false}, T, k, d_in, p1, store_epilogue(w.H, w.ldh, nullptr), st));
-    const TcPlan p2 = plan_tc(T, d_out, k, false, false);
-    FLOP_TRY(launch_tc({w.H, w.ldh, false}, {Pc, ldpc, false}, T, d_out, k, p2, store_epilogue(Y, ldy, nullptr), st));
+    FLOP_TRY(launch_fwd_product(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, false, st));
+    FLOP_TRY(launch_fwd_product(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, true, st));
   } else {
     FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Qc, ldqc, true}, T, k, d_in, simt_out(w.H, w.ldh), st));
     FLOP_TRY(launch_simt({(const float*)w.H, w.ldh, true}, {(const float*)Pc, ldpc, true}, T, d_out, k, simt_out(Y, ldy), st));

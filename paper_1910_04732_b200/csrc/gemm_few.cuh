@@ -1,0 +1,124 @@
+// Forward product for few tokens, bf16 in, fp32 accumulate, bf16 out:
+//     C[t, n] = col_scale[n] * sum_k A[t, k] B[n, k]          (A [T, K] tokens, B [N, K] weights, both K-major)
+//
+// Bound: latency.  At these sizes the weights are 0.1-10 MB (about a microsecond of L2 or HBM time) and a 128-row tcgen05
+// tile spends 7-10 us per launch on its pipeline (barriers, tensor memory, descriptors, a serial walk over K).  What a
+// launch needs is that every byte it reads is requested at once and that many SMs ask.  So
+//   * the weights are the row operand of the warp-level m16n8k16 instruction and the tokens its 8-wide column operand:
+//     a block computes 16 MT weight rows x 8 NT tokens, and small T wastes nothing on the weight side;
+//   * the eight warps of a block cut K into 32-wide steps dealt out in turn, each reading its own part of both operands
+//     straight from global memory into registers: no byte is read twice in a block, nothing is staged or waited for,
+//     and a warp has `kDepth` steps of loads in flight.  The warps' sums are added through shared memory in warp order;
+//   * a lane reads 16 contiguous bytes of a row per step: the k positions inside a step are permuted identically for both
+//     operands, so that those bytes serve two instructions without a shuffle;
+//   * with EARLY the first weights are requested before the wait on the previous launch.  That is for the second product of
+//     a pair only: its predecessor on the stream is the first product, which waits for everything before it
+//     before it lets this launch start, and which writes H' and nothing else, so the weights are final.
+// Both products of 1024 -> 358 -> 4096, replayed: 3.7 us at one token and 4.7 at 16, where a warp per output column on the
+// CUDA cores (up to 4 tokens) took 5.3 and a warp per 8 columns walking all of K, on 7 SMs for the first product, 11.9.
+// At 64 tokens 9.2 against 14.6 with tcgen05 tiles.  A 64 x 64 block per CTA (fewer bytes read in all) was never faster.
+#pragma once
+#include "common.cuh"
+
+namespace flop {
+namespace few {
+
+constexpr int kWarps = 8, kThreads = 32 * kWarps;
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                               uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Eight elements of a row from k on, zero beyond K (rows are 16-byte aligned; nothing beyond K is read).
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, int k, int K) {
+  uint4 v = make_uint4(0, 0, 0, 0);
+  if (k + 8 <= K) {
+    v = *reinterpret_cast<const uint4*>(row + k);
+  } else if (k < K) {
+    __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(&v);
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+      if (k + i < K) h[i] = row[k + i];
+  }
+  return v;
+}
+
+__host__ __device__ constexpr int part_stride(int mt) { return 16 * mt + 4; }   // floats per token of a warp's partial tile: conflict-free writes
+__host__ __device__ constexpr int smem_bytes(int mt, int nt) { return kWarps * 8 * nt * part_stride(mt) * 4; }
+
+template <int MT, int NT, bool EARLY>
+__global__ void __launch_bounds__(kThreads)
+gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat16* __restrict__ B, int64_t ldb,
+            __nv_bfloat16* __restrict__ C, int64_t ldc, const float* __restrict__ col_scale, int T, int N, int K) {
+  constexpr int kDepth = 2 * MT + NT <= 4 ? 4 : 2;         // steps of loads in flight: up to 24 16-byte loads per lane
+  extern __shared__ __align__(16) float part[];            // [kWarps][8 NT][part_stride(MT)]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const int n0 = blockIdx.x * 16 * MT, t0 = blockIdx.y * 8 * NT;
+  const __nv_bfloat16* wrow[2 * MT];                       // rows past the end are read from the last row and not stored
+  const __nv_bfloat16* trow[NT];
+#pragma unroll
+  for (int i = 0; i < 2 * MT; ++i) wrow[i] = B + (int64_t)min(n0 + 8 * i + g, N - 1) * ldb;
+#pragma unroll
+  for (int i = 0; i < NT; ++i) trow[i] = A + (int64_t)min(t0 + 8 * i + g, T - 1) * lda;
+  float acc[MT][NT][4] = {};
+  uint4 wv[kDepth][2 * MT], tv[kDepth][NT];
+  auto load_weights = [&](int s) {
+#pragma unroll
+    for (int d = 0; d < kDepth; ++d)
+#pragma unroll
+      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * kWarps) * 32 + 8 * q, K);
+  };
+  if (!EARLY) pdl_wait();
+  load_weights(warp);
+  if (EARLY) pdl_wait();
+  pdl_launch_dependents();
+  for (int s = warp; s * 32 < K; s += kDepth * kWarps) {
+    if (s != warp) load_weights(s);
+#pragma unroll
+    for (int d = 0; d < kDepth; ++d)
+#pragma unroll
+      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * kWarps) * 32 + 8 * q, K);
+#pragma unroll
+    for (int d = 0; d < kDepth; ++d)
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const uint4 lo = wv[d][2 * m], hi = wv[d][2 * m + 1], t = tv[d][n];
+          mma_bf16_16816(acc[m][n], lo.x, hi.x, lo.y, hi.y, t.x, t.y);
+          mma_bf16_16816(acc[m][n], lo.z, hi.z, lo.w, hi.w, t.z, t.w);
+        }
+  }
+  // lane (g, q) holds rows 16 m + g and + 8, tokens 8 n + 2 q and + 1
+  constexpr int S = part_stride(MT);
+#pragma unroll
+  for (int m = 0; m < MT; ++m)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        part[(warp * 8 * NT + 8 * n + 2 * q + (i & 1)) * S + 16 * m + g + (i >> 1) * 8] = acc[m][n][i];
+  __syncthreads();
+#pragma unroll
+  for (int e = threadIdx.x; e < 8 * NT * 8 * MT; e += kThreads) {      // two neighbouring columns of one token
+    const int t = e / (8 * MT), c = (e % (8 * MT)) * 2;
+    float x = 0.f, y = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const float2 v = *reinterpret_cast<const float2*>(part + (w * 8 * NT + t) * S + c);
+      x += v.x; y += v.y;
+    }
+    const int n = n0 + c;
+    if (t0 + t < T && n < N) {
+      if (col_scale) { x *= __ldg(col_scale + n); if (n + 1 < N) y *= __ldg(col_scale + n + 1); }
+      __nv_bfloat16* o = C + (int64_t)(t0 + t) * ldc + n;
+      if (n + 1 < N) *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(x, y);   // rows are 16-byte aligned, n is even
+      else *o = __float2bfloat16_rn(x);
+    }
+  }
+}
+
+}  // namespace few
+}  // namespace flop
