@@ -769,10 +769,10 @@ bool few_ok(int64_t T, int64_t N, int64_t K) {
   if (T < 1 || T > 1024 || N > INT32_MAX / 2 || K > INT32_MAX / 2 || tuning().no_few) return false;
   return T <= 32 || few_blocks(T, N) <= num_sms();
 }
-// Forward product C = (A B^T) * col_scale of a layer, in the form the sizes call for.
+// Forward product C = (A B^T) * col_scale of a layer, in the form the sizes call for.  `few`: the few-token kernel may serve it.
 int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
-                       int64_t K, bool second, cudaStream_t st) {
-  if (few_ok(T, N, K)) return launch_few(A, lda, B, ldb, C, ldc, cs, T, N, K, second, st);
+                       int64_t K, bool few, bool second, cudaStream_t st) {
+  if (few && few_ok(T, N, K)) return launch_few(A, lda, B, ldb, C, ldc, cs, T, N, K, second, st);
   return launch_tc({A, lda, false}, {B, ldb, false}, T, N, K, plan_tc(T, N, K, false, false), store_epilogue(C, ldc, cs), st);
 }
 
@@ -1216,8 +1216,10 @@ static int fwd_impl(const void* X, int64_t ldx, const void* Q, int64_t ldq, cons
       if (r > 0) FLOP_TRY(zero_2d<bf16>(H, ldh, T, r, st));
       return FLOP_OK;
     }
-    FLOP_TRY(launch_fwd_product(X, ldx, Q, ldq, H, ldh, z, T, r, d_in, false, st));           // H' = (X Q^T) * z
-    FLOP_TRY(launch_fwd_product(H, ldh, P, ldp, Y, ldy, nullptr, T, d_out, r, true, st));     // Y = H' P^T
+    // From 17 tokens on a training forward keeps the tiles, and so the bits, of the grouped call.
+    const bool few = T <= 16;
+    FLOP_TRY(launch_fwd_product(X, ldx, Q, ldq, H, ldh, z, T, r, d_in, few, false, st));          // H' = (X Q^T) * z
+    FLOP_TRY(launch_fwd_product(H, ldh, P, ldp, Y, ldy, nullptr, T, d_out, r, few, true, st));    // Y = H' P^T
   } else {
     FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Q, ldq, true}, T, r, d_in, simt_out(H, ldh, z), st));
     FLOP_TRY(launch_simt({(const float*)H, ldh, true}, {(const float*)P, ldp, true}, T, d_out, r, simt_out(Y, ldy), st));
@@ -1282,8 +1284,8 @@ int flop_compact_fwd(const void* X, int64_t ldx, const void* Qc, int64_t ldqc, c
   const FwdWs w = plan_fwd_ws(ar, T, k, dt);
   if (dt == FLOP_BF16) {
     if (!bf16_ok(Y, ldy) || !bf16_ok(X, ldx) || !bf16_ok(Qc, ldqc) || !bf16_ok(Pc, ldpc)) return FLOP_ERR_UNSUPPORTED;
-    FLOP_TRY(launch_fwd_product(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, false, st));
-    FLOP_TRY(launch_fwd_product(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, true, st));
+    FLOP_TRY(launch_fwd_product(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, true, false, st));
+    FLOP_TRY(launch_fwd_product(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, true, true, st));
   } else {
     FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Qc, ldqc, true}, T, k, d_in, simt_out(w.H, w.ldh), st));
     FLOP_TRY(launch_simt({(const float*)w.H, w.ldh, true}, {(const float*)Pc, ldpc, true}, T, d_out, k, simt_out(Y, ldy), st));
