@@ -1,13 +1,17 @@
-"""Thin ctypes binding over the C ABI in include/flop.h.
+"""Thin binding over the C ABI in include/flop.h.
 
 Argument marshalling only: torch tensors provide device memory and the
 current CUDA stream; every step of the path runs in the library's kernels.
+The calls on one matrix read their arguments in native code
+(csrc/binding_native.cpp), because they can be shorter than their own
+marshalling; everything else goes through ctypes.
 If the library is missing or a call fails this module raises -- there is no
 CPU fallback.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -150,6 +154,25 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
+_native_module = None
+
+
+def _native():
+    """The native half of the binding (csrc/binding_native.cpp), loaded on first use."""
+    global _native_module
+    if _native_module is None:
+        load_library()
+        path = os.path.join(_HERE, "_binding_native.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build it with `python -m paper_1910_04732_b200.build` "
+                               "(there is no CPU fallback)")
+        spec = importlib.util.spec_from_file_location("paper_1910_04732_b200._binding_native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native_module = module
+    return _native_module
+
+
 def plan_tile_schedule(cost, units: int):
     """Host-only: (unit of every work item, largest unit load, largest load of the round-robin deal)."""
     n = len(cost)
@@ -281,9 +304,7 @@ def tc_gemm(A, a_mn_major: bool, B, b_mn_major: bool, M: int, N: int, K: int, D=
 
 def gate_sample(log_alpha: torch.Tensor, hc, seed: int, offset: int, z: torch.Tensor,
                 mask: Optional[torch.Tensor] = None, dz_dla: Optional[torch.Tensor] = None) -> None:
-    n = log_alpha.numel()
-    _check(load_library().flop_gate_sample(_ptr(log_alpha), n, _hc(hc), seed, offset, _ptr(z), _ptr(mask),
-                                           _ptr(dz_dla), _stream()), "flop_gate_sample")
+    _check(_native().gate_sample(log_alpha, hc, seed, offset, z, mask, dz_dla), "flop_gate_sample")
 
 
 def gate_sample_devoff(log_alpha: torch.Tensor, hc, seed: int, offset: int, offset_dev: torch.Tensor, z: torch.Tensor,
@@ -296,25 +317,12 @@ def gate_sample_devoff(log_alpha: torch.Tensor, hc, seed: int, offset: int, offs
 
 
 def gated_lowrank_fwd(X, Q, P, z, Y, H_save=None, ws=None) -> None:
-    T, d_in = X.shape
-    d_out, r = P.shape
-    _check(load_library().flop_gated_lowrank_fwd(
-        _ptr(X), _ld(X), _ptr(Q), _ld(Q), _ptr(P), _ld(P), _ptr(z), _ptr(Y), _ld(Y),
-        _ptr(H_save), _ld(H_save) if H_save is not None else 0, T, d_in, d_out, r, _dt(X),
-        _ptr(ws), ws.numel() if ws is not None else 0, _stream()), "flop_gated_lowrank_fwd")
+    _check(_native().gated_lowrank_fwd(X, Q, P, z, Y, H_save, ws), "flop_gated_lowrank_fwd")
 
 
 def gated_lowrank_bwd(dY, X, Q, P, z, dz_dla, H_save, dX, dP, dQ, dlog_alpha, ws, accumulate: bool = False) -> None:
-    T, d_in = X.shape
-    d_out, r = P.shape
-    wdt = _dt(dP) if dP is not None else (_dt(dQ) if dQ is not None else _dt(X))
-    _check(load_library().flop_gated_lowrank_bwd(
-        _ptr(dY), _ld(dY), _ptr(X), _ld(X), _ptr(Q), _ld(Q), _ptr(P), _ld(P), _ptr(z), _ptr(dz_dla),
-        _ptr(H_save), _ld(H_save),
-        _ptr(dX), _ld(dX) if dX is not None else 0, _ptr(dP), _ld(dP) if dP is not None else 0,
-        _ptr(dQ), _ld(dQ) if dQ is not None else 0, _ptr(dlog_alpha), int(accumulate),
-        T, d_in, d_out, r, _dt(X), wdt, _ptr(ws), ws.numel() if ws is not None else 0, _stream()),
-        "flop_gated_lowrank_bwd")
+    _check(_native().gated_lowrank_bwd(dY, X, Q, P, z, dz_dla, H_save, dX, dP, dQ, dlog_alpha, ws, accumulate),
+           "flop_gated_lowrank_bwd")
 
 
 def _p(t: Optional[torch.Tensor]):
@@ -430,10 +438,8 @@ def gated_lowrank_bwd_chained(problems, sync: torch.Tensor, accumulate: bool = F
 
 def expected_l0_lagrangian(log_alpha, seg_off, seg_size, hc, target, lam, out4, seg_expected=None,
                            dlog_alpha=None, ws=None) -> None:
-    _check(load_library().flop_expected_l0_lagrangian(
-        _ptr(log_alpha), log_alpha.numel(), _ptr(seg_off), _ptr(seg_size), seg_size.numel(), _hc(hc),
-        _ptr(target), _ptr(lam), _ptr(out4), _ptr(seg_expected), _ptr(dlog_alpha),
-        _ptr(ws), ws.numel() if ws is not None else 0, _stream()), "flop_expected_l0_lagrangian")
+    _check(_native().expected_l0_lagrangian(log_alpha, seg_off, seg_size, hc, target, lam, out4, seg_expected, dlog_alpha, ws),
+           "flop_expected_l0_lagrangian")
 
 
 def expected_l0_lagrangian_noalloc(log_alpha, seg_off, seg_size, hc, target, lam, out4, seg_expected=None,
@@ -449,20 +455,12 @@ def expected_l0_lagrangian_noalloc(log_alpha, seg_off, seg_size, hc, target, lam
 
 
 def gated_embedding_fwd(ids, E, O, z, Y, H_save) -> None:
-    T, (n_rows, d_i), d = ids.numel(), E.shape, O.shape[1]
-    _check(load_library().flop_gated_embedding_fwd(_ptr(ids), T, _ptr(E), _ld(E), n_rows, _ptr(O), _ld(O), _ptr(z), _ptr(Y),
-                                                   _ld(Y), _ptr(H_save), _ld(H_save), d_i, d, _dt(E), _stream()),
-           "flop_gated_embedding_fwd")
+    _check(_native().gated_embedding_fwd(ids, E, O, z, Y, H_save), "flop_gated_embedding_fwd")
 
 
 def gated_embedding_bwd(dY, ids, E, O, z, dz_dla, H_save, dE, dO, dlog_alpha, ws, accumulate: bool = False) -> None:
-    T, (n_rows, d_i), d = ids.numel(), E.shape, O.shape[1]
-    wdt = _dt(dO) if dO is not None else BF16
-    _check(load_library().flop_gated_embedding_bwd(
-        _ptr(dY), _ld(dY), _ptr(ids), T, _ptr(E), _ld(E), n_rows, _ptr(O), _ld(O), _ptr(z), _ptr(dz_dla), _ptr(H_save),
-        _ld(H_save), _ptr(dE), _ld(dE) if dE is not None else 0, _ptr(dO), _ld(dO) if dO is not None else 0,
-        _ptr(dlog_alpha), int(accumulate), d_i, d, _dt(E), wdt, _ptr(ws), ws.numel() if ws is not None else 0, _stream()),
-        "flop_gated_embedding_bwd")
+    _check(_native().gated_embedding_bwd(dY, ids, E, O, z, dz_dla, H_save, dE, dO, dlog_alpha, ws, accumulate),
+           "flop_gated_embedding_bwd")
 
 
 def agp_gates(g, seg_off, sparsity, l1: float, z, mask=None, dz_dg=None, seg_l1=None, dg=None) -> None:
@@ -473,20 +471,8 @@ def agp_gates(g, seg_off, sparsity, l1: float, z, mask=None, dz_dg=None, seg_l1=
 
 
 def compact_ranks(log_alpha_or_z, mode: int, hc, idx, k_dev, z_det=None, P=None, Q=None, Pc=None, Qc=None) -> None:
-    r = log_alpha_or_z.numel()
-    d_in = Q.shape[1] if Q is not None else 0
-    d_out = P.shape[0] if P is not None else 0
-    dt = _dt(P) if P is not None else F32
-    _check(load_library().flop_compact_ranks(
-        _ptr(log_alpha_or_z), mode, _hc(hc), r, _ptr(P), _ld(P) if P is not None else 0,
-        _ptr(Q), _ld(Q) if Q is not None else 0, d_in, d_out, dt, _ptr(idx), _ptr(k_dev), _ptr(z_det),
-        _ptr(Pc), _ld(Pc) if Pc is not None else 0, _ptr(Qc), _ld(Qc) if Qc is not None else 0,
-        None, 0, _stream()), "flop_compact_ranks")
+    _check(_native().compact_ranks(log_alpha_or_z, mode, hc, idx, k_dev, z_det, P, Q, Pc, Qc), "flop_compact_ranks")
 
 
 def compact_fwd(X, Qc, Pc, Y, k: int, ws) -> None:
-    T, d_in = X.shape
-    d_out = Pc.shape[0]
-    _check(load_library().flop_compact_fwd(
-        _ptr(X), _ld(X), _ptr(Qc), _ld(Qc), _ptr(Pc), _ld(Pc), _ptr(Y), _ld(Y), T, d_in, d_out, k, _dt(X),
-        _ptr(ws), ws.numel() if ws is not None else 0, _stream()), "flop_compact_fwd")
+    _check(_native().compact_fwd(X, Qc, Pc, Y, k, ws), "flop_compact_fwd")
