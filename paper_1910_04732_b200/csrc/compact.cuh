@@ -319,13 +319,14 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // columns of P are read straight from global memory, two per lane: neighbouring lanes read neighbouring survivors, so
 // a load touches only a few lines, and a row needs neither staging nor a barrier.
 // Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (three launches each: 13.0 + 4.0 + 5.8 us
-// of GPU time); what is left there is the caller's time per call.
+// of GPU time).  Blocks of 256 threads, four per SM, repeated the fp64 probabilities twice as often: 706 us against 650 us
+// with 512 threads and two per SM (both with the binding's calls at 4 us).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
 // saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74), and for long P the staged
 // gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
 constexpr int kFusedMaxR = 1024;
 constexpr int64_t kFusedMaxBytes = 16 << 20;
-constexpr int kFusedThreads = 256, kFusedWarps = kFusedThreads / 32;
+constexpr int kFusedThreads = 512, kFusedWarps = kFusedThreads / 32;
 
 template <typename T> struct alignas(2 * sizeof(T)) Pair2 { T e[2]; };
 
@@ -350,12 +351,11 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
   for (int i = my_warp; i < d_out; i += warps)
     for (int b = lane * 128; b < r * (int)sizeof(T); b += 32 * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(P + (int64_t)i * ldp) + b));
-#pragma unroll
-  for (int p = 0; p < 4; ++p) hist[p][tid] = 0;
+  for (int i = tid; i < 4 * 256; i += kFusedThreads) (&hist[0][0])[i] = 0;
   pdl_wait();
   pdl_launch_dependents();
 
-  // gate n of this thread is n * 256 + tid: word n * 8 + warp of the ballots, bit lane
+  // gate n of this thread is n * kFusedThreads + tid: word n * kFusedWarps + warp of the ballots, bit lane
   float v[kKeys], zv[kKeys];
   double sum = 0.0;
 #pragma unroll
@@ -375,9 +375,7 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
     sum = warp_sum_f64(sum);
     if (lane == 0) red[warp] = sum;
     __syncthreads();   // histograms are zero, warp sums are there
-    sum = 0.0;
-#pragma unroll
-    for (int w = 0; w < kFusedWarps; ++w) sum += red[w];
+    sum = warp_sum_f64(lane < kFusedWarps ? red[lane] : 0.0);
     k = max(0, min(r, (int)floor(sum + 0.5)));
     uint32_t prefix = 0, pmask = 0;
     int need = k;       // rank (1-based, from the top) still to be located inside the prefix class
