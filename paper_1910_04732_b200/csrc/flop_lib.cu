@@ -684,6 +684,52 @@ GroupShape plan_group(const std::vector<Mnk>& jobs, bool b_mn_major, bool wgrad 
   return best;
 }
 
+// Estimated SM cycles of one launch: the largest of its longest tile and its mean load per CTA (or pair), plus what a launch
+// costs before its first and after its last k-block (about 5 us).  A tile costs its k-blocks at the slower of MMA
+// issue and shared-memory fill, plus its epilogue.
+struct LaunchCost {
+  int cta2;
+  double total = 0.0, longest = 0.0;
+  void add(int64_t M, int64_t N, int64_t K, int bn, int splits = 1) {
+    const int bm = cta2 ? tc::BM2 : tc::BM;
+    const int64_t num_kb = (K + tc::BK - 1) / tc::BK, kbps = (num_kb + splits - 1) / splits;
+    const double bytes = cta2 ? (double)tc::stage_bytes2(bn) : (double)tc::stage_bytes(bn);
+    const double tile = (double)kbps * std::max(2.0 * bn, bytes / 50.0) + 600.0 + 10.0 * bn;
+    total += (double)((M + bm - 1) / bm) * (double)((N + bn - 1) / bn) * splits * tile;
+    longest = std::max(longest, tile);
+  }
+  void add(int64_t M, int64_t N, int64_t K, const TcPlan& pl) { add(M, N, K, pl.bn, std::max(pl.splits, 1)); }
+  double cycles() const { return longest <= 0.0 ? 0.0 : std::max(longest, total / (cta2 ? num_sms() / 2 : num_sms())) + 9000.0; }
+};
+constexpr double kSmallLaunchCycles = 4000.0;   // a small kernel between GEMMs
+
+// Whether the backward pass of these problems is faster as two shared launches -- {dH', dP}, then {dQ, dX}, every tile a CTA
+// pair's, no split-K -- than as one launch per product with the weight gradients split over the tokens, and with which
+// N tiles.  Splitting wins when there are many tokens and few tiles (a tile then walks all tokens alone while
+// most of the machine waits); otherwise the shared launches save three launches, the fp32 slices and the pass
+// that adds them up.
+struct MergedShape { int bn_h, bn_p, bn_q, bn_x; double cycles; };
+MergedShape plan_merged(const flop_bwd_problem_t* pr, int n) {
+  MergedShape best{0, 0, 0, 0, 1e300};
+  double half[2] = {1e300, 1e300};
+  for (int a = 0; a < 2; ++a)
+    for (int b = 0; b < 2; ++b) {
+      const int bn0 = a ? 256 : 128, bn1 = b ? 256 : 128;
+      LaunchCost first{1}, second{1};
+      for (int i = 0; i < n; ++i) {
+        const flop_bwd_problem_t& p = pr[i];
+        first.add(p.T, p.r, p.d_out, bn0);
+        if (p.dP) first.add(p.d_out, p.r, p.T, bn1);
+        if (p.dQ || p.dlog_alpha) second.add(p.r, p.d_in, p.T, bn0);
+        if (p.dX) second.add(p.T, p.d_in, p.r, bn1);
+      }
+      if (first.cycles() < half[0]) { half[0] = first.cycles(); best.bn_h = bn0; best.bn_p = bn1; }
+      if (second.cycles() < half[1]) { half[1] = second.cycles(); best.bn_q = bn0; best.bn_x = bn1; }
+    }
+  best.cycles = half[0] + half[1] + 2 * kSmallLaunchCycles;
+  return best;
+}
+
 // Weight gradient written straight from the GEMM epilogue (no split-K, no fp32 slices).
 TcEpilogue wgrad_epilogue(void* out, int64_t ldo, int wgrad_dt, const float* row_scale, int accumulate) {
   TcEpilogue e{};
@@ -1293,6 +1339,9 @@ int flop_compact_fwd(const void* X, int64_t ldx, const void* Qc, int64_t ldqc, c
   return FLOP_OK;
 }
 
+static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate, int dt, int wgrad_dt, void* sync, size_t sync_bytes,
+                            void* stream, double single_cycles);
+
 int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t ldx, const void* Q, int64_t ldq,
                            const void* P, int64_t ldp, const float* z, const float* dz_dla, const void* H_save,
                            int64_t ldh, void* dX, int64_t lddx, void* dP, int64_t lddp, void* dQ, int64_t lddq,
@@ -1332,6 +1381,25 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
   const BwdWs w = plan_bwd_ws(ar, T, d_in, d_out, r, dt);
   const bool need_m = dQ || dlog_alpha;   // M = dH'^T X feeds both dQ and dz
 
+  if (dt == FLOP_BF16 && (!dP || wgrad_direct_ok(dP, lddp, wgrad_dt)) && (!dQ || wgrad_direct_ok(dQ, lddq, wgrad_dt)) &&
+      T <= INT32_MAX && d_in <= INT32_MAX && d_out <= INT32_MAX && r <= INT32_MAX) {
+    // The two shared launches of the grouped call when they are estimated faster than a launch per product.
+    const TcPlan ph = plan_tc(T, r, d_out, false, true), px = plan_tc(T, d_in, r, false, true);
+    LaunchCost ch{ph.cta2}, cp{w.plan_p.cta2}, cq{w.plan_q.cta2}, cx{px.cta2};
+    ch.add(T, r, d_out, ph);
+    if (dP) cp.add(d_out, r, T, w.plan_p);
+    if (need_m) cq.add(r, d_in, T, w.plan_q);
+    if (dX) cx.add(T, d_in, r, px);
+    double slice_bytes = 0.0;
+    if (dP && w.plan_p.splits > 1) slice_bytes += 8.0 * w.plan_p.splits * (double)d_out * r;
+    if (need_m && w.plan_q.splits > 1) slice_bytes += 8.0 * w.plan_q.splits * (double)r * d_in;
+    const double separate = ch.cycles() + cp.cycles() + cq.cycles() + cx.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0;
+    const flop_bwd_problem_t one{dY, lddy, X, ldx, Q, ldq, P, ldp, z, dz_dla, H_save, ldh, dX, lddx, dP, lddp, dQ, lddq, dlog_alpha,
+                                 T, d_in, d_out, r, ws, ws_bytes, nullptr, nullptr, 0, 0};
+    Arena grouped{nullptr, 0, 0};
+    if (plan_merged(&one, 1).cycles < separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes)
+      return bwd_grouped_impl(&one, 1, accumulate, dt, wgrad_dt, nullptr, 0, stream, separate);
+  }
   if (dt == FLOP_BF16) {
     // dH' = dY P            (A = dY K-major over d_out; B(n=k_rank, k=i) = P[i, k_rank]: MN-major)
     const TcPlan ph = plan_tc(T, r, d_out, false, true);
@@ -1513,8 +1581,9 @@ int flop_sync_bytes(size_t* out_bytes) {
   return FLOP_OK;
 }
 
+// single_cycles: estimate of the other form of the call (a launch per product) when the caller has one of its own, else 0.
 static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate, int dt, int wgrad_dt, void* sync,
-                            size_t sync_bytes, void* stream) {
+                            size_t sync_bytes, void* stream, double single_cycles) {
   if (n < 0 || (n > 0 && !pr) || !valid_dt(dt) || !valid_dt(wgrad_dt)) return FLOP_ERR_INVALID_ARG;
   FLOP_TRY(check_sync(sync, sync_bytes));
   if (dt == FLOP_F32 && wgrad_dt != FLOP_F32) return FLOP_ERR_UNSUPPORTED;
@@ -1575,20 +1644,42 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
     const GroupShape swp = plan_group(mw, true, true, true);
     if (swp.bn != 0 && swp.items >= num_sms() / 2) sw = swp;
   }
-  if (sw.bn == 0 || sw.items < (sw.cta2 ? num_sms() / 2 : num_sms())) direct = false;
+  MergedShape mg{0, 0, 0, 0, 1e300};
+  if (sw.bn == 0 || sw.items < (sw.cta2 ? num_sms() / 2 : num_sms())) {
+    if (direct && n > 0 && !sync && 2 * n <= tc::kMaxGroup) {
+      mg = plan_merged(pr, n);
+      if (single_cycles <= 0.0) {     // the other form of this call: a launch per product, weight gradients split, a finishing pass
+        LaunchCost h{s3.cta2}, p{0}, q{0}, x{s6.cta2};
+        double slice_bytes = 0.0;
+        for (int i = 0; i < n; ++i) {
+          const flop_bwd_problem_t& a = pr[i];
+          h.add(a.T, a.r, a.d_out, s3.bn);
+          if (a.dP) { p.add(a.d_out, a.r, a.T, wss[i].plan_p); slice_bytes += 8.0 * wss[i].plan_p.splits * a.d_out * a.r; }
+          if (a.dQ || a.dlog_alpha) { q.add(a.r, a.d_in, a.T, wss[i].plan_q); slice_bytes += 8.0 * wss[i].plan_q.splits * a.r * a.d_in; }
+          if (a.dX) x.add(a.T, a.d_in, a.r, s6.bn);
+        }
+        single_cycles = h.cycles() + p.cycles() + q.cycles() + x.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0;
+      }
+    }
+    if (mg.cycles >= single_cycles) { direct = false; mg.bn_h = 0; }
+  } else if (single_cycles > 0.0 && sync == nullptr) {
+    mg = plan_merged(pr, n);          // a single call that comes here asked for the merged form
+  }
   auto direct_plan = [&](int64_t M, int64_t N, int64_t K) { return fixed_plan(M, N, K, sw.bn, sw.cta2); };
   for (int i = 0; i < n; ++i) {
     const flop_bwd_problem_t& a = pr[i];
     const BwdWs& w = wss[i];
     const bool need_m = a.dQ || a.dlog_alpha;
-    TcJob j3{{a.dY, a.lddy, false}, {a.P, a.ldp, true}, a.T, a.r, a.d_out, fixed_plan(a.T, a.r, a.d_out, s3.bn, s3.cta2),
+    TcJob j3{{a.dY, a.lddy, false}, {a.P, a.ldp, true}, a.T, a.r, a.d_out,
+             mg.bn_h ? fixed_plan(a.T, a.r, a.d_out, mg.bn_h, 1) : fixed_plan(a.T, a.r, a.d_out, s3.bn, s3.cta2),
              store_epilogue(w.dH, w.lddh, nullptr)};
     j3.dyn_n = a.r_dev;
     g3.push_back(j3);
     int n_part = w.n_part;
     if (a.dP) {
       if (direct) {
-        TcJob j{{a.dY, a.lddy, true}, {a.H_save, a.ldh, true}, a.d_out, a.r, a.T, direct_plan(a.d_out, a.r, a.T),
+        TcJob j{{a.dY, a.lddy, true}, {a.H_save, a.ldh, true}, a.d_out, a.r, a.T,
+                mg.bn_h ? fixed_plan(a.d_out, a.r, a.T, mg.bn_p, 1) : direct_plan(a.d_out, a.r, a.T),
                 wgrad_epilogue(a.dP, a.lddp, wgrad_dt, nullptr, accumulate)};
         j.dyn_n = a.r_dev;
         g4.push_back(j);
@@ -1606,7 +1697,7 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
       if (direct) {
         // dQ = diag(z) (dH'^T X) stored in place (dQ may be absent when only dlog_alpha is wanted: then
         // the product still runs for the fused row dots and its values go to the slice buffer)
-        pl = direct_plan(a.r, a.d_in, a.T);
+        pl = mg.bn_h ? fixed_plan(a.r, a.d_in, a.T, mg.bn_q, 1) : direct_plan(a.r, a.d_in, a.T);
         if (a.dQ) e = wgrad_epilogue(a.dQ, a.lddq, wgrad_dt, a.z, accumulate);
         else      e = wgrad_epilogue(w.slices_q, w.ld_slice_q, FLOP_F32, nullptr, 0);
         n_part = 2 * pl.tiles_n;
@@ -1628,7 +1719,8 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
     f.dz_part = w.dz_part; f.n_part = n_part; f.dz_dla = a.dz_dla; f.dlog_alpha = a.defer_dlog_alpha ? nullptr : a.dlog_alpha; f.accumulate = accumulate;
     fin.push_back(f);
     if (a.dX) {
-      TcJob j6{{w.dH, w.lddh, false}, {a.Qz ? a.Qz : w.Qz, a.Qz ? a.ldqz : w.ldqz, true}, a.T, a.d_in, a.r, fixed_plan(a.T, a.d_in, a.r, s6.bn, s6.cta2),
+      TcJob j6{{w.dH, w.lddh, false}, {a.Qz ? a.Qz : w.Qz, a.Qz ? a.ldqz : w.ldqz, true}, a.T, a.d_in, a.r,
+               mg.bn_h ? fixed_plan(a.T, a.d_in, a.r, mg.bn_x, 1) : fixed_plan(a.T, a.d_in, a.r, s6.bn, s6.cta2),
                store_epilogue(a.dX, a.lddx, nullptr)};
       j6.dyn_k = a.r_dev;
       g6.push_back(j6);
@@ -1765,13 +1857,13 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
 }
 
 int flop_gated_lowrank_bwd_grouped(const flop_bwd_problem_t* pr, int n, int accumulate, int dt, int wgrad_dt, void* stream) {
-  return bwd_grouped_impl(pr, n, accumulate, dt, wgrad_dt, nullptr, 0, stream);
+  return bwd_grouped_impl(pr, n, accumulate, dt, wgrad_dt, nullptr, 0, stream, 0.0);
 }
 
 int flop_gated_lowrank_bwd_chained(const flop_bwd_problem_t* pr, int n, int accumulate, int dt, int wgrad_dt, void* sync,
                                    size_t sync_bytes, void* stream) {
   if (!sync) return FLOP_ERR_WORKSPACE;
-  return bwd_grouped_impl(pr, n, accumulate, dt, wgrad_dt, sync, sync_bytes, stream);
+  return bwd_grouped_impl(pr, n, accumulate, dt, wgrad_dt, sync, sync_bytes, stream, 0.0);
 }
 
 int flop_dlog_alpha_finish_grouped(const flop_bwd_problem_t* pr, int n, int accumulate, int dt, void* stream) {
