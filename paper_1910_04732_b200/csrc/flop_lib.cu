@@ -209,7 +209,7 @@ struct TcPlan {
   int cta2;   // 1: pairs of CTAs compute 256 x bn tiles (gemm2_group_kernel); 0: one CTA per 128 x bn tile
 };
 
-constexpr int kSmemBudget = 227 * 1024 - 1024;   // opt-in maximum minus room for the static __shared__ variables
+constexpr int kSmemBudget = 227 * 1024 - 1024;   // opt-in maximum minus room for the static __shared__ variables (item table: 768 bytes)
 constexpr int kSmemBarrierBytes = 384;   // pipeline barriers (8 x (2 x 8 + 5) bytes) and the chained kernel's queue ring (160 bytes)
 constexpr int kSmemFixed = 1024 + (int)tc::kStoreBufTotal + kSmemBarrierBytes;   // alignment slack + epilogue staging + barriers
 
@@ -430,6 +430,7 @@ int add_problem(tc::GroupParams& gp, const TcJob& j, std::vector<double>& item_c
   p.qdot = j.ep.qdot; p.ldq = j.ep.ldq; p.dz_part = j.ep.dz_part; p.dz_stride = j.ep.dz_stride; p.dz_meta = j.ep.dz_meta;
   p.wg_out = j.ep.wg_out; p.wg_f32 = j.ep.wg_f32; p.row_scale = j.ep.row_scale; p.accumulate = j.ep.accumulate;
   p.dyn_m = j.dyn_m; p.dyn_n = j.dyn_n; p.dyn_k = j.dyn_k;
+  if (j.dyn_m || j.dyn_n || j.dyn_k) gp.any_dyn = 1;
   p.link = j.link;
   // bf16 tiles that are plainly overwritten leave through a TMA store (64 x 32 boxes of the output)
   void* tma_dst = j.ep.kind == tc::EPI_STORE ? (void*)j.ep.out

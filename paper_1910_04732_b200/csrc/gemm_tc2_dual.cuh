@@ -33,10 +33,10 @@ __device__ __forceinline__ bool pair_produce_item(const GroupParams& gp, const G
                                                   uint32_t sbytes, const PairBars& bars, int& stage, uint32_t& phase,
                                                   volatile int* abort_flag) {
   const GroupProblem& pr = gp.prob[it.g];
-  const int half_n = pr.p.bn >> 1;
+  const int half_n = it.bn >> 1;
   const uint32_t tx = kATileBytes + (uint32_t)half_n * BK * 2;
   const int m_base = it.tm * BM2 + (int)rank * BM;
-  const int n_base = it.tn * pr.p.bn + (int)rank * half_n;
+  const int n_base = it.tn * it.bn + (int)rank * half_n;
   for (int kb = it.kb0; kb < it.kb1; ++kb) {
     if (!mbar_wait2(bars.empty(stage), phase ^ 1u, abort_flag)) return false;
     const uint32_t sa = smem_base + (uint32_t)stage * sbytes, sb = sa + kATileBytes;
@@ -65,7 +65,7 @@ template <bool A_MN, bool B_MN>
 __device__ __forceinline__ bool pair_mma_item(const GroupParams& gp, const GroupItem& it, uint32_t smem_base, uint32_t sbytes,
                                               const PairBars& bars, uint32_t tmem_base, int& stage, uint32_t& phase, int& acc,
                                               uint32_t& acc_phase, volatile int* abort_flag) {
-  const uint32_t idesc = instr_desc2(A_MN, B_MN, gp.prob[it.g].p.bn);
+  const uint32_t idesc = instr_desc2(A_MN, B_MN, it.bn);
   if (!mbar_wait2(bars.tempty(acc), acc_phase ^ 1u, abort_flag)) return false;
   tcgen05_fence_after();
   const uint32_t d_tmem = tmem_base + (uint32_t)acc * acc_stride(gp.bn_max);
@@ -98,11 +98,13 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
   const PairBars bars{store_base + kStoreBufTotal};
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
+  __shared__ ItemTable s_items;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const WorkRange wr = work_range(gp, pair, npairs);
+  const int n_items = work_count(wr);
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -117,6 +119,7 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
     if (gp.prob[lane].p.tma_store) prefetch_tmap(&gp.prob[lane].tout);
   }
   if (warp == 1) tmem_alloc2(smem_u32(&s_tmem_base), kTmemCols);
+  if (warp == 2 && !gp.any_dyn) fill_item_table(gp, wr, lane, BM2, s_items);
   tcgen05_fence_before();
   __syncthreads();
   cluster_sync_all();            // both CTAs' barriers exist before either signals the other
@@ -125,6 +128,10 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
   volatile int* abort_flag = &s_abort;
   pdl_wait();
   pdl_launch_dependents();
+  if (gp.any_dyn) {
+    if (warp == 2) fill_item_table(gp, wr, lane, BM2, s_items);
+    __syncthreads();
+  }
   if (gp.stamp && blockIdx.x == 0 && threadIdx.x == 0) gp.stamp[0] = global_ns();
 
   if (warp == 0) {
@@ -133,10 +140,10 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM2);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM2);
         if (!it.active) continue;
-        if (gp.prob[it.g].p.kind == 0) ok = pair_produce_item<A0, B0>(gp, it, rank, smem_base, sbytes, bars, stage, phase, abort_flag);
+        if (it.kind == 0) ok = pair_produce_item<A0, B0>(gp, it, rank, smem_base, sbytes, bars, stage, phase, abort_flag);
         else                           ok = pair_produce_item<A1, B1>(gp, it, rank, smem_base, sbytes, bars, stage, phase, abort_flag);
       }
       if (!ok || *abort_flag) {
@@ -154,10 +161,10 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM2);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM2);
         if (!it.active) continue;
-        if (gp.prob[it.g].p.kind == 0)
+        if (it.kind == 0)
           ok = pair_mma_item<A0, B0>(gp, it, smem_base, sbytes, bars, tmem_base, stage, phase, acc, acc_phase, abort_flag);
         else
           ok = pair_mma_item<A1, B1>(gp, it, smem_base, sbytes, bars, tmem_base, stage, phase, acc, acc_phase, abort_flag);
@@ -168,8 +175,8 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-      const GroupItem it = work_item(gp, wi, BM2);
+    for (int i = 0; i < n_items && ok; ++i) {
+      const GroupItem it = item_at(gp, wr, s_items, i, BM2);
       if (!it.active) continue;
       const Params& p = gp.prob[it.g].p;
       if (!mbar_wait2(bars.tfull(acc), acc_phase, abort_flag)) { ok = false; }
@@ -179,7 +186,7 @@ gemm2_dual_kernel(const __grid_constant__ GroupParams gp) {
       const uint32_t sbuf = store_base + (uint32_t)(warp - 2) * kStoreBufBytes, t_acc = tmem_base + (uint32_t)acc * acc_stride(gp.bn_max);
       const int row0 = it.tm * BM2 + (int)rank * BM;
       const uint32_t rel = map_to_cta(bars.tempty(acc), 0);
-      if (p.kind == 0) run_epilogue<E0, true>(p, &gp.prob[it.g].tout, sbuf, t_acc, row0, it.tn * p.bn, it.n_limit, it.split, it.tn, warp, lane, rel);
+      if (it.kind == 0) run_epilogue<E0, true>(p, &gp.prob[it.g].tout, sbuf, t_acc, row0, it.tn * p.bn, it.n_limit, it.split, it.tn, warp, lane, rel);
       else             run_epilogue<E1, true>(p, &gp.prob[it.g].tout, sbuf, t_acc, row0, it.tn * p.bn, it.n_limit, it.split, it.tn, warp, lane, rel);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }

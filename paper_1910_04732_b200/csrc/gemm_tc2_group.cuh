@@ -28,11 +28,13 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
   const uint32_t exit_bar = bar_base + 8u * (uint32_t)(2 * kMaxStages + 4);
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
+  __shared__ ItemTable s_items;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const WorkRange wr = work_range(gp, pair, npairs);
+  const int n_items = work_count(wr);
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -47,6 +49,7 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
     if (gp.prob[lane].p.tma_store) prefetch_tmap(&gp.prob[lane].tout);
   }
   if (warp == 1) tmem_alloc2(smem_u32(&s_tmem_base), kTmemCols);
+  if (warp == 2 && !gp.any_dyn) fill_item_table(gp, wr, lane, BM2, s_items);
   tcgen05_fence_before();
   __syncthreads();
   cluster_sync_all();            // both CTAs' barriers exist before either signals the other
@@ -55,6 +58,10 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
   volatile int* abort_flag = &s_abort;
   pdl_wait();
   pdl_launch_dependents();
+  if (gp.any_dyn) {
+    if (warp == 2) fill_item_table(gp, wr, lane, BM2, s_items);
+    __syncthreads();
+  }
   if (gp.stamp && blockIdx.x == 0 && threadIdx.x == 0) gp.stamp[0] = global_ns();
 
   if (warp == 0) {
@@ -63,14 +70,14 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM2);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM2);
         if (!it.active) continue;
         const GroupProblem& pr = gp.prob[it.g];
-        const int half_n = pr.p.bn >> 1;
+        const int half_n = it.bn >> 1;
         const uint32_t tx = kATileBytes + (uint32_t)half_n * BK * 2;
         const int m_base = it.tm * BM2 + (int)rank * BM;
-        const int n_base = it.tn * pr.p.bn + (int)rank * half_n;
+        const int n_base = it.tn * it.bn + (int)rank * half_n;
         for (int kb = it.kb0; kb < it.kb1; ++kb) {
           if (!mbar_wait2(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t sa = smem_base + (uint32_t)stage * sbytes, sb = sa + kATileBytes;
@@ -107,10 +114,10 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM2);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM2);
         if (!it.active) continue;
-        const uint32_t idesc = instr_desc2(A_MN, B_MN, gp.prob[it.g].p.bn);
+        const uint32_t idesc = instr_desc2(A_MN, B_MN, it.bn);
         if (!mbar_wait2(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * acc_stride(gp.bn_max);
@@ -137,8 +144,8 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-      const GroupItem it = work_item(gp, wi, BM2);
+    for (int i = 0; i < n_items && ok; ++i) {
+      const GroupItem it = item_at(gp, wr, s_items, i, BM2);
         if (!it.active) continue;
       const Params& p = gp.prob[it.g].p;
       if (!mbar_wait2(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; }

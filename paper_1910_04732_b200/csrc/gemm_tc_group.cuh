@@ -42,6 +42,7 @@ struct GroupParams {
   // Chained launches only (gemm_tc2_chain.cuh): the zero-initialised sync area, the words in use (the last
   // unit to finish clears them) and the arrivals that complete the launch's side work (0: none).
   unsigned* sync; int sync_words; unsigned side_need;
+  int any_dyn;      // 1: some problem carries device-side sizes, so items can only be decoded after the dependency wait
   // Which work items each persistent unit walks (schedule.cuh); n_units == 0: round-robin.
   Schedule sched;
 };
@@ -60,7 +61,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-struct GroupItem { int g, tm, tn, split, kb0, kb1, n_limit; bool active; };
+struct GroupItem { int g, tm, tn, split, kb0, kb1, n_limit, bn, kind; bool active; };
 
 // Work item w of the group; bm = rows of D per tile (128, or 256 for a CTA pair).  When a problem
 // carries device-side sizes the item may lie outside the effective extent (active = false: every
@@ -68,7 +69,7 @@ struct GroupItem { int g, tm, tn, split, kb0, kb1, n_limit; bool active; };
 __device__ __forceinline__ GroupItem decode_problem_item(const GroupParams& gp, int g, int w, int bm) {
   const Params& p = gp.prob[g].p;
   const WorkItem it = decode(p, w - gp.prob[g].work_begin);
-  GroupItem o{g, it.tm, it.tn, it.split, it.kb0, it.kb1, p.N, true};
+  GroupItem o{g, it.tm, it.tn, it.split, it.kb0, it.kb1, p.N, p.bn, p.kind, true};
   if (p.dyn_m || p.dyn_n || p.dyn_k) {
     const int m_eff = p.dyn_m ? max(1, min(p.M, __ldg(p.dyn_m))) : p.M;
     const int n_eff = p.dyn_n ? max(1, min(p.N, __ldg(p.dyn_n))) : p.N;
@@ -95,6 +96,31 @@ __device__ __forceinline__ GroupItem work_item(const GroupParams& gp, int i, int
   return decode_group(gp, i, bm);
 }
 
+// The first kItemTable work items of a unit, decoded once into shared memory by one warp (an item per lane) while the launch
+// before still runs.  A decode is a chain of dependent loads from the 21 KB parameter block, most of them misses of the
+// small constant cache: 1200 cycles, which the TMA thread and the MMA thread each paid between two tiles, with nothing to
+// hide it -- a quarter of a 12-k-block tile's period (8750 cycles of which 6750 main loop), a third of a 7-k-block one's --
+// and once more before the first load of a launch.  Training steps (BERT / Transformer-XL / SRU shapes): 3114 -> 2915,
+// 4231 -> 4107, 7694 -> 7403 us; two micro-batches 134 -> 126.  Items beyond the table are decoded by each role as it gets to them.
+constexpr int kItemTable = 32;
+struct ItemTable { int tm[kItemTable], tn[kItemTable], kb0[kItemTable], kb1[kItemTable], n_limit[kItemTable]; uint32_t packed[kItemTable]; };
+
+__device__ __forceinline__ int work_count(const WorkRange& wr) { return wr.last > wr.first ? (wr.last - wr.first + wr.step - 1) / wr.step : 0; }
+__device__ __forceinline__ void fill_item_table(const GroupParams& gp, const WorkRange& wr, int lane, int bm, ItemTable& t) {
+  if (lane >= work_count(wr)) return;
+  const GroupItem it = work_item(gp, wr.first + lane * wr.step, bm);
+  t.tm[lane] = it.tm; t.tn[lane] = it.tn; t.kb0[lane] = it.kb0; t.kb1[lane] = it.active ? it.kb1 : it.kb0; t.n_limit[lane] = it.n_limit;
+  t.packed[lane] = (uint32_t)it.g | ((uint32_t)it.bn << 5) | ((uint32_t)it.kind << 14) | ((uint32_t)it.split << 16);   // g < 32, bn <= 256, split < 65536
+}
+// Item i of the unit.
+__device__ __forceinline__ GroupItem item_at(const GroupParams& gp, const WorkRange& wr, const ItemTable& t, int i, int bm) {
+  if (i >= kItemTable) return work_item(gp, wr.first + i * wr.step, bm);
+  const uint32_t k = t.packed[i];
+  GroupItem o{(int)(k & 31u), t.tm[i], t.tn[i], (int)(k >> 16), t.kb0[i], t.kb1[i], t.n_limit[i], (int)((k >> 5) & 511u), (int)((k >> 14) & 1u), true};
+  o.active = o.kb0 < o.kb1;
+  return o;
+}
+
 template <bool A_MN, bool B_MN, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_group_kernel(const __grid_constant__ GroupParams gp) {
@@ -109,9 +135,11 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
   auto tempty_bar = [&](int a) { return bar_base + 8u * (uint32_t)(2 * kMaxStages + 2 + a); };
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
+  __shared__ ItemTable s_items;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WorkRange wr = work_range(gp, (int)blockIdx.x, (int)gridDim.x);
+  const int n_items = work_count(wr);
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -125,6 +153,7 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
     if (gp.prob[lane].p.tma_store) prefetch_tmap(&gp.prob[lane].tout);
   }
   if (warp == 1) tmem_alloc(smem_u32(&s_tmem_base), kTmemCols);
+  if (warp == 2 && !gp.any_dyn) fill_item_table(gp, wr, lane, BM, s_items);
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
@@ -132,6 +161,10 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
   volatile int* abort_flag = &s_abort;
   pdl_wait();
   pdl_launch_dependents();
+  if (gp.any_dyn) {
+    if (warp == 2) fill_item_table(gp, wr, lane, BM, s_items);
+    __syncthreads();
+  }
   if (gp.stamp && blockIdx.x == 0 && threadIdx.x == 0) gp.stamp[0] = global_ns();
 
   if (warp == 0) {
@@ -141,11 +174,11 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
       uint32_t phase = 0;
       int armed = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM);
         if (!it.active) continue;
         const GroupProblem& pr = gp.prob[it.g];
-        const int bn = pr.p.bn;
+        const int bn = it.bn;
         const uint32_t tx = kATileBytes + (uint32_t)bn * BK * 2;
         for (int kb = it.kb0; kb < it.kb1; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
@@ -188,10 +221,10 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-        const GroupItem it = work_item(gp, wi, BM);
+      for (int i = 0; i < n_items && ok; ++i) {
+        const GroupItem it = item_at(gp, wr, s_items, i, BM);
         if (!it.active) continue;
-        const uint32_t idesc = instr_desc(A_MN, B_MN, gp.prob[it.g].p.bn);
+        const uint32_t idesc = instr_desc(A_MN, B_MN, it.bn);
         if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)acc * acc_stride(gp.bn_max);
@@ -218,8 +251,8 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
-    for (int wi = wr.first; wi < wr.last && ok; wi += wr.step) {
-      const GroupItem it = work_item(gp, wi, BM);
+    for (int i = 0; i < n_items && ok; ++i) {
+      const GroupItem it = item_at(gp, wr, s_items, i, BM);
         if (!it.active) continue;
       const Params& p = gp.prob[it.g].p;
       if (!mbar_wait(tfull_bar(acc), acc_phase, abort_flag)) { ok = false; }
