@@ -405,8 +405,8 @@ int launch_dual_inst(const tc::GroupParams& gp, double flops, cudaStream_t st) {
 }
 
 // Fills the next problem slot of a launch from a job: tensor maps, sizes, epilogue, work-list position; appends
-// the cost of each of its work items (SM cycles, the model of plan_group) for the schedule.
-int add_problem(tc::GroupParams& gp, const TcJob& j, std::vector<double>& item_cost, double& flops) {
+// its work items with their cost (SM cycles, the model of plan_group) for the schedule.
+int add_problem(tc::GroupParams& gp, const TcJob& j, std::vector<tc::ItemGroup>& groups, double& flops) {
   if (j.M > INT32_MAX || j.N > INT32_MAX || j.K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
   const bool kind1 = j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_WGRAD;
   tc::GroupProblem& pr = gp.prob[gp.n];
@@ -441,11 +441,14 @@ int add_problem(tc::GroupParams& gp, const TcJob& j, std::vector<double>& item_c
   gp.total_work += p.tiles_m * p.tiles_n * p.splits;
   const double bytes = j.pl.cta2 ? (double)tc::stage_bytes2(p.bn) : (double)tc::stage_bytes(p.bn);
   const double per_kb = std::max(2.0 * p.bn, bytes / 50.0), epi = tuning().sched_epi > 0 ? (double)tuning().sched_epi : 400.0 + 4.0 * p.bn;
-  if (item_cost.size() <= (size_t)tc::kMaxSched)
-    for (int sp = 0; sp < p.splits; ++sp) {
-      const int kbs = std::min(p.kb_per_split, p.num_kb - sp * p.kb_per_split);
-      item_cost.insert(item_cost.end(), (size_t)p.tiles_m * p.tiles_n, kbs * per_kb + epi);
-    }
+  for (int sp = 0; sp < p.splits; ++sp) {
+    const int kbs = std::min(p.kb_per_split, p.num_kb - sp * p.kb_per_split), tiles = p.tiles_m * p.tiles_n, first = pr.work_begin + sp * tiles;
+    const double cost = kbs * per_kb + epi;
+    // a group per position along an extent that only the device knows, else one
+    if (j.dyn_n)      for (int tn = 0; tn < p.tiles_n; ++tn) groups.push_back(tc::ItemGroup{cost, tn, gp.n, first + tn, p.tiles_m, p.tiles_n});
+    else if (j.dyn_m) for (int tm = 0; tm < p.tiles_m; ++tm) groups.push_back(tc::ItemGroup{cost, tm, gp.n, first + tm * p.tiles_n, p.tiles_n, 1});
+    else              groups.push_back(tc::ItemGroup{cost, 0, gp.n, first, tiles, 1});
+  }
   gp.bn_max = std::max(gp.bn_max, p.bn);
   flops += 2.0 * j.M * (double)j.N * j.K;
   ++gp.n;
@@ -468,7 +471,8 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
     double flops = 0.0;
     const TcJob& first = jobs[i];
     bool uniform = true, dual_ok = true;   // one kind of problem / the two kinds gemm2_dual_kernel is built for
-    std::vector<double> item_cost;
+    std::vector<tc::ItemGroup> groups;
+    groups.reserve(64);
     for (; i < jobs.size() && gp.n < tc::kMaxGroup; ++i) {
       const TcJob& j = jobs[i];
       if (j.M <= 0 || j.N <= 0 || j.K <= 0) continue;
@@ -477,7 +481,7 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
       const bool kind0 = !j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_STORE;
       const bool kind1 = j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_WGRAD;
       if (!(kind0 || kind1) || !j.pl.cta2) dual_ok = false;
-      FLOP_TRY(add_problem(gp, j, item_cost, flops));
+      FLOP_TRY(add_problem(gp, j, groups, flops));
     }
     if (gp.n == 0) continue;
     const int cta2 = first.pl.cta2;
@@ -488,22 +492,12 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
     // round-robin order.
     {
       const int units = std::min(gp.total_work, cta2 ? num_sms() / 2 : num_sms());
+      // every entry also names its problem, so that no role has to search for it
+      static_assert(tc::kMaxSched <= (1 << tc::kSchedProblemShift) && tc::kMaxGroup <= (1 << (16 - tc::kSchedProblemShift)), "entry bits");
       double rr = 0.0;
-      if (tuning().no_sched || (int)item_cost.size() != gp.total_work) {
-        gp.sched.n_units = 0;
-      } else {
-        const double lpt = tc::build_schedule(item_cost, units, &gp.sched, &rr);
-        if (lpt < 0.0 || lpt > 0.97 * rr) gp.sched.n_units = 0;
-        if (gp.sched.n_units) {     // every entry also names its problem, so that no role has to search for it
-          static_assert(tc::kMaxSched <= (1 << tc::kSchedProblemShift) && tc::kMaxGroup <= (1 << (16 - tc::kSchedProblemShift)), "entry bits");
-          for (int i = 0; i < gp.total_work; ++i) {
-            const int w = gp.sched.item[i];
-            int g = 0;
-            for (int k = 1; k < gp.n; ++k)
-              if (w >= gp.prob[k].work_begin) g = k;
-            gp.sched.item[i] = (uint16_t)((g << tc::kSchedProblemShift) | w);
-          }
-        }
+      if (!tuning().no_sched && gp.total_work <= tc::kMaxSched && (gp.any_dyn || !tc::round_robin_is_good(groups, units, &rr))) {
+        const double lpt = tc::deal_groups(groups, gp.total_work, units, tc::kSchedProblemShift, &gp.sched);
+        if (lpt < 0.0 || (!gp.any_dyn && lpt > 0.97 * rr)) gp.sched.n_units = 0;
       }
     }
     const bool a_mn = first.A.mn_major, b_mn = first.B.mn_major;
@@ -563,14 +557,14 @@ int launch_tc_chain(const std::vector<TcJob>& jobs, const std::vector<int>& dep_
   tc::GroupParams gp;
   memset(&gp, 0, sizeof(gp));
   double flops = 0.0;
-  std::vector<double> item_cost;
+  std::vector<tc::ItemGroup> groups;
   struct Item { int job, tm; };
   std::vector<Item> items;
   bool side = false;
   for (size_t i = 0; i < jobs.size(); ++i) {
     const TcJob& j = jobs[i];
     if (i > 0 && j.stage < jobs[i - 1].stage) return FLOP_ERR_INVALID_ARG;
-    FLOP_TRY(add_problem(gp, j, item_cost, flops));
+    FLOP_TRY(add_problem(gp, j, groups, flops));
     for (int tm = 0; tm < j.pl.tiles_m; ++tm)
       for (int tn = 0; tn < j.pl.tiles_n; ++tn) items.push_back(Item{(int)i, tm});
     if (j.link.sw_qz) side = true;
@@ -583,7 +577,10 @@ int launch_tc_chain(const std::vector<TcJob>& jobs, const std::vector<int>& dep_
   // queue, long before short.
   gp.sched.n_units = 0;
   const int n = (int)items.size();
-  if ((int)item_cost.size() == n && n == gp.total_work && n <= tc::kMaxSched) {
+  if (n == gp.total_work && n <= tc::kMaxSched) {
+    std::vector<double> item_cost((size_t)n, 0.0);
+    for (const tc::ItemGroup& g : groups)
+      for (int i = 0; i < g.count; ++i) item_cost[(size_t)(g.first + i * g.stride)] = g.cost;
     const int64_t kCostMax = (int64_t)1 << 30;
     auto inv_cost = [&](int i) { return kCostMax - std::min<int64_t>(kCostMax - 1, (int64_t)item_cost[(size_t)i]); };
     std::vector<int> stage((size_t)n);

@@ -49,17 +49,19 @@ gemm2_group_kernel(const __grid_constant__ GroupParams gp) {
     if (gp.prob[lane].p.tma_store) prefetch_tmap(&gp.prob[lane].tout);
   }
   if (warp == 1) tmem_alloc2(smem_u32(&s_tmem_base), kTmemCols);
-  if (warp == 2 && !gp.any_dyn) fill_item_table(gp, wr, lane, BM2, s_items);
+  if (warp == 2) fill_item_table(gp, wr, lane, s_items);
   tcgen05_fence_before();
   __syncthreads();
   cluster_sync_all();            // both CTAs' barriers exist before either signals the other
   tcgen05_fence_after();
   const uint32_t tmem_base = s_tmem_base;
   volatile int* abort_flag = &s_abort;
+  ItemSizes sizes{};
+  if (gp.any_dyn && warp == 2) sizes = item_sizes(gp, s_items, lane, min(n_items, kItemTable));
   pdl_wait();
   pdl_launch_dependents();
   if (gp.any_dyn) {
-    if (warp == 2) fill_item_table(gp, wr, lane, BM2, s_items);
+    if (warp == 2) apply_item_sizes(sizes, lane, BM2, s_items);
     __syncthreads();
   }
   if (gp.stamp && blockIdx.x == 0 && threadIdx.x == 0) gp.stamp[0] = global_ns();

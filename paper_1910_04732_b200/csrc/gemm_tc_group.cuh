@@ -66,10 +66,13 @@ struct GroupItem { int g, tm, tn, split, kb0, kb1, n_limit, bn, kind; bool activ
 // Work item w of the group; bm = rows of D per tile (128, or 256 for a CTA pair).  When a problem
 // carries device-side sizes the item may lie outside the effective extent (active = false: every
 // role skips it, so stage and accumulator phases stay in step) or have a shorter K loop.
-__device__ __forceinline__ GroupItem decode_problem_item(const GroupParams& gp, int g, int w, int bm) {
+__device__ __forceinline__ GroupItem decode_static_item(const GroupParams& gp, int g, int w) {
   const Params& p = gp.prob[g].p;
   const WorkItem it = decode(p, w - gp.prob[g].work_begin);
-  GroupItem o{g, it.tm, it.tn, it.split, it.kb0, it.kb1, p.N, p.bn, p.kind, true};
+  return GroupItem{g, it.tm, it.tn, it.split, it.kb0, it.kb1, p.N, p.bn, p.kind, true};
+}
+__device__ __forceinline__ void apply_device_sizes(const GroupParams& gp, int bm, GroupItem& o) {
+  const Params& p = gp.prob[o.g].p;
   if (p.dyn_m || p.dyn_n || p.dyn_k) {
     const int m_eff = p.dyn_m ? max(1, min(p.M, __ldg(p.dyn_m))) : p.M;
     const int n_eff = p.dyn_n ? max(1, min(p.N, __ldg(p.dyn_n))) : p.N;
@@ -78,6 +81,10 @@ __device__ __forceinline__ GroupItem decode_problem_item(const GroupParams& gp, 
     o.kb1 = min(o.kb1, (k_eff + BK - 1) / BK);
     o.active = o.tm * bm < m_eff && o.tn * p.bn < n_eff && o.kb0 < o.kb1;
   }
+}
+__device__ __forceinline__ GroupItem decode_problem_item(const GroupParams& gp, int g, int w, int bm) {
+  GroupItem o = decode_static_item(gp, g, w);
+  apply_device_sizes(gp, bm, o);
   return o;
 }
 __device__ __forceinline__ GroupItem decode_group(const GroupParams& gp, int w, int bm) {
@@ -106,11 +113,41 @@ constexpr int kItemTable = 32;
 struct ItemTable { int tm[kItemTable], tn[kItemTable], kb0[kItemTable], kb1[kItemTable], n_limit[kItemTable]; uint32_t packed[kItemTable]; };
 
 __device__ __forceinline__ int work_count(const WorkRange& wr) { return wr.last > wr.first ? (wr.last - wr.first + wr.step - 1) / wr.step : 0; }
-__device__ __forceinline__ void fill_item_table(const GroupParams& gp, const WorkRange& wr, int lane, int bm, ItemTable& t) {
-  if (lane >= work_count(wr)) return;
-  const GroupItem it = work_item(gp, wr.first + lane * wr.step, bm);
+__device__ __forceinline__ void store_item(ItemTable& t, int lane, const GroupItem& it) {
   t.tm[lane] = it.tm; t.tn[lane] = it.tn; t.kb0[lane] = it.kb0; t.kb1[lane] = it.active ? it.kb1 : it.kb0; t.n_limit[lane] = it.n_limit;
   t.packed[lane] = (uint32_t)it.g | ((uint32_t)it.bn << 5) | ((uint32_t)it.kind << 14) | ((uint32_t)it.split << 16);   // g < 32, bn <= 256, split < 65536
+}
+// Before the dependency wait: an item per lane, without the sizes that only the device knows.
+__device__ __forceinline__ void fill_item_table(const GroupParams& gp, const WorkRange& wr, int lane, ItemTable& t) {
+  if (lane >= work_count(wr)) return;
+  const int i = wr.first + lane * wr.step;
+  int w = i, g = 0;
+  if (gp.sched.n_units) {
+    const int e = (int)gp.sched.item[i];
+    g = e >> kSchedProblemShift; w = e & ((1 << kSchedProblemShift) - 1);
+  } else {
+    for (int k = 1; k < gp.n && w >= gp.prob[k].work_begin; ++k) g = k;
+  }
+  store_item(t, lane, decode_static_item(gp, g, w));
+}
+// After it (launches with such sizes only): the effective extents; an item outside them becomes empty (kb1 = kb0).
+// The capacities and pointers were touched while the launch before still ran, so this is one round of loads.
+struct ItemSizes { const int *m, *n, *k; int M, N, K; };
+__device__ __forceinline__ ItemSizes item_sizes(const GroupParams& gp, const ItemTable& t, int lane, int n_items) {
+  ItemSizes z{nullptr, nullptr, nullptr, 0, 0, 0};
+  if (lane < n_items) {
+    const Params& p = gp.prob[t.packed[lane] & 31u].p;
+    z = ItemSizes{p.dyn_m, p.dyn_n, p.dyn_k, p.M, p.N, p.K};
+  }
+  return z;
+}
+__device__ __forceinline__ void apply_item_sizes(const ItemSizes& z, int lane, int bm, ItemTable& t) {
+  if (!z.m && !z.n && !z.k) return;
+  const int m_eff = z.m ? max(1, min(z.M, __ldg(z.m))) : z.M, n_eff = z.n ? max(1, min(z.N, __ldg(z.n))) : z.N;
+  const int k_eff = z.k ? max(1, min(z.K, __ldg(z.k))) : z.K, bn = (int)((t.packed[lane] >> 5) & 511u);
+  if (z.n) t.n_limit[lane] = min(z.N, (n_eff + 63) & ~63);
+  const int kb0 = t.kb0[lane], kb1 = min(t.kb1[lane], (k_eff + BK - 1) / BK);
+  t.kb1[lane] = t.tm[lane] * bm < m_eff && t.tn[lane] * bn < n_eff ? max(kb0, kb1) : kb0;
 }
 // Item i of the unit.
 __device__ __forceinline__ GroupItem item_at(const GroupParams& gp, const WorkRange& wr, const ItemTable& t, int i, int bm) {
@@ -153,16 +190,18 @@ gemm_group_kernel(const __grid_constant__ GroupParams gp) {
     if (gp.prob[lane].p.tma_store) prefetch_tmap(&gp.prob[lane].tout);
   }
   if (warp == 1) tmem_alloc(smem_u32(&s_tmem_base), kTmemCols);
-  if (warp == 2 && !gp.any_dyn) fill_item_table(gp, wr, lane, BM, s_items);
+  if (warp == 2) fill_item_table(gp, wr, lane, s_items);
   tcgen05_fence_before();
   __syncthreads();
   tcgen05_fence_after();
   const uint32_t tmem_base = s_tmem_base;
   volatile int* abort_flag = &s_abort;
+  ItemSizes sizes{};
+  if (gp.any_dyn && warp == 2) sizes = item_sizes(gp, s_items, lane, min(n_items, kItemTable));
   pdl_wait();
   pdl_launch_dependents();
   if (gp.any_dyn) {
-    if (warp == 2) fill_item_table(gp, wr, lane, BM, s_items);
+    if (warp == 2) apply_item_sizes(sizes, lane, BM, s_items);
     __syncthreads();
   }
   if (gp.stamp && blockIdx.x == 0 && threadIdx.x == 0) gp.stamp[0] = global_ns();

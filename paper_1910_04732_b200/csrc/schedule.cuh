@@ -16,9 +16,6 @@
 
 #ifndef __CUDACC_RTC__
 #include <algorithm>
-#include <functional>
-#include <queue>
-#include <utility>
 #include <vector>
 #endif
 
@@ -35,49 +32,83 @@ struct Schedule {
   uint16_t item[kMaxSched];          // work-list indices
 };
 
-// Longest-processing-time assignment of `cost.size()` work items to `units` units.  Items of equal
-// cost keep their work-list order (neighbouring tiles share operand tiles in L2).  Returns the
-// largest unit load; `rr_makespan` receives the largest load of the round-robin deal for comparison.
+// Work items of equal cost: first, first + stride, ... (count of them), of one problem.
+struct ItemGroup { double cost; int rank, problem, first, count, stride; };
+
+// Longest-processing-time assignment of the items of `groups` to `units` units: groups of a lower rank first, within a rank the
+// costlier first (ties keep list order, so that neighbouring tiles share operand tiles in L2), every item to the least
+// loaded unit.  Returns the largest unit load and fills the table; `shift` > 0 adds the problem index to the entries.
+// rank is 0 except in launches whose tile count only the device knows: there it is the index of a tile along the extent that
+// may end early.  Any prefix of the ranks is then balanced, whereas one list over all tiles leaves units with several live
+// tiles next to units with none once the later tiles turn out empty (open components only, BERT shapes, a quarter of the
+// gates open: the backward launches 39.5 -> 32.1 and 44.9 -> 39.8 us).
+// Groups rather than items are sorted, the heap holds plain pairs and nothing is allocated per unit: a table is built for
+// every launch, and at 500 items the item-wise form took longer than the launch it was for.
+inline double deal_groups(std::vector<ItemGroup>& groups, int n, int units, int shift, Schedule* out) {
+  out->n_units = 0;
+  if (n <= 0 || n > kMaxSched || units <= 0 || units > kMaxUnits) return -1.0;
+  std::stable_sort(groups.begin(), groups.end(), [](const ItemGroup& a, const ItemGroup& b) { return a.rank != b.rank ? a.rank < b.rank : a.cost > b.cost; });
+  struct Slot { double load; int unit; };
+  Slot heap[kMaxUnits];              // least loaded first, ties to the lower unit index
+  for (int u = 0; u < units; ++u) heap[u] = Slot{0.0, u};
+  uint8_t owner[kMaxSched];
+  uint16_t entry[kMaxSched];
+  int held[kMaxUnits + 1] = {};
+  int pos = 0;
+  for (const ItemGroup& g : groups)
+    for (int i = 0; i < g.count; ++i, ++pos) {
+      const int u = heap[0].unit;
+      owner[pos] = (uint8_t)u;
+      entry[pos] = (uint16_t)((shift ? g.problem << shift : 0) | (g.first + i * g.stride));
+      ++held[u];
+      const Slot s{heap[0].load + g.cost, u};
+      int at = 0;
+      for (;;) {                     // sift the unit down from the top
+        int c = 2 * at + 1;
+        if (c >= units) break;
+        if (c + 1 < units && (heap[c + 1].load < heap[c].load || (heap[c + 1].load == heap[c].load && heap[c + 1].unit < heap[c].unit))) ++c;
+        if (s.load < heap[c].load || (s.load == heap[c].load && s.unit < heap[c].unit)) break;
+        heap[at] = heap[c];
+        at = c;
+      }
+      heap[at] = s;
+    }
+  double makespan = 0.0;
+  for (int u = 0; u < units; ++u) makespan = std::max(makespan, heap[u].load);
+  int next[kMaxUnits], sum = 0;
+  for (int u = 0; u < units; ++u) { out->begin[u] = (uint16_t)sum; next[u] = sum; sum += held[u]; }
+  for (int u = units; u <= kMaxUnits; ++u) out->begin[u] = (uint16_t)sum;
+  for (int i = 0; i < pos; ++i) out->item[next[owner[i]]++] = entry[i];
+  out->n_units = units;
+  return makespan;
+}
+
+// Largest load of the round-robin deal (item i to unit i % units); true when it is within 3 % of the lower bound
+// max(mean load, longest item), so that a table has nothing to gain.  `groups` in work-list order.
+inline bool round_robin_is_good(const std::vector<ItemGroup>& groups, int units, double* rr_makespan) {
+  double load[kMaxUnits] = {};
+  double total = 0.0, longest = 0.0, rr = 0.0;
+  for (const ItemGroup& g : groups) {
+    for (int i = 0; i < g.count; ++i) load[(g.first + i * g.stride) % units] += g.cost;
+    total += g.cost * g.count;
+    longest = std::max(longest, g.cost);
+  }
+  for (int u = 0; u < units; ++u) rr = std::max(rr, load[u]);
+  if (rr_makespan) *rr_makespan = rr;
+  return rr <= 1.03 * std::max(total / units, longest);
+}
+
+// The same for a plain list of costs (item i costs cost[i]); returns the largest unit load, or -1 without a table.
 inline double build_schedule(const std::vector<double>& cost, int units, Schedule* out, double* rr_makespan) {
   const int n = (int)cost.size();
   out->n_units = 0;
-  if (rr_makespan) {
-    std::vector<double> load((size_t)std::max(units, 1), 0.0);
-    for (int i = 0; i < n; ++i) load[(size_t)(i % std::max(units, 1))] += cost[(size_t)i];
-    *rr_makespan = load.empty() ? 0.0 : *std::max_element(load.begin(), load.end());
-  }
-  if (n == 0 || n > kMaxSched || units <= 0 || units > kMaxUnits) return -1.0;
-  if (rr_makespan) {
-    // Nothing to gain when round-robin is already within 3 % of the lower bound max(mean load, longest item):
-    // skip the sort (this keeps the host cost of the common equal-tile launches at one pass over the list).
-    double total = 0.0, longest = 0.0;
-    for (int i = 0; i < n; ++i) { total += cost[(size_t)i]; longest = std::max(longest, cost[(size_t)i]); }
-    if (*rr_makespan <= 1.03 * std::max(total / units, longest)) return -1.0;
-  }
-  std::vector<int> order((size_t)n);
-  for (int i = 0; i < n; ++i) order[(size_t)i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[(size_t)a] > cost[(size_t)b]; });
-  typedef std::pair<double, int> LoadUnit;   // least loaded first, ties to the lower unit index
-  std::priority_queue<LoadUnit, std::vector<LoadUnit>, std::greater<LoadUnit>> heap;
-  for (int u = 0; u < units; ++u) heap.push(LoadUnit(0.0, u));
-  std::vector<std::vector<int>> lists((size_t)units);
-  double makespan = 0.0;
-  for (int i = 0; i < n; ++i) {
-    LoadUnit lu = heap.top();
-    heap.pop();
-    lists[(size_t)lu.second].push_back(order[(size_t)i]);
-    lu.first += cost[(size_t)order[(size_t)i]];
-    makespan = std::max(makespan, lu.first);
-    heap.push(lu);
-  }
-  int pos = 0;
-  for (int u = 0; u < units; ++u) {
-    out->begin[u] = (uint16_t)pos;
-    for (int w : lists[(size_t)u]) out->item[pos++] = (uint16_t)w;
-  }
-  for (int u = units; u <= kMaxUnits; ++u) out->begin[u] = (uint16_t)pos;
-  out->n_units = units;
-  return makespan;
+  if (rr_makespan) *rr_makespan = 0.0;
+  if (units <= 0 || units > kMaxUnits) return -1.0;
+  std::vector<ItemGroup> groups;
+  groups.reserve((size_t)n);
+  for (int i = 0; i < n; ++i) groups.push_back(ItemGroup{cost[(size_t)i], 0, 0, i, 1, 1});
+  if (round_robin_is_good(groups, units, rr_makespan) && rr_makespan) return -1.0;
+  return deal_groups(groups, n, units, 0, out);
 }
 
 // Queue of a chained launch (gemm_tc2_chain.cuh): the work list holds the tiles of two stages, a tile of the
