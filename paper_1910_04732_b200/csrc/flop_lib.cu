@@ -906,7 +906,8 @@ struct BwdWs {
 };
 BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, int dt, bool grouped = false) {
   BwdWs w{};
-  w.lddh = round_up(std::max<int64_t>(r, 1), 8);
+  // rows of dH' start on 128-byte lines: a TMA box row is 128 bytes, and one that straddles two lines costs two L2 requests
+  w.lddh = round_up(std::max<int64_t>(r, 1), dt == FLOP_BF16 ? 64 : 8);
   w.dH = ar.take((size_t)T * w.lddh * elt(dt));
   w.ldqz = round_up(std::max<int64_t>(d_in, 1), 8);
   w.Qz = dt == FLOP_BF16 ? ar.take((size_t)r * w.ldqz * 2) : nullptr;
