@@ -1017,6 +1017,24 @@ static int launch_embed_bwd(const int32_t* ids, int64_t T, const void* E, int64_
   return FLOP_OK;
 }
 
+static bool l0_small_ok(int64_t n, int32_t n_seg) { return n > 0 && n_seg > 0 && n <= kL0SmallMax && n <= kL0SmallPerSeg * n_seg; }
+static int launch_l0_small(const float* log_alpha, int64_t n, const int64_t* seg_off, const float* seg_size, int32_t n_seg, float thr,
+                           const float* target, const float* lambda, float* out4, float* seg_expected, float* dlog_alpha, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kL0SmallCtas); cfg.blockDim = dim3(kL0SmallThreads); cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kL0SmallCtas; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_on() ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, l0_small_kernel, log_alpha, seg_off, seg_size, (int)n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, n);
+  count_launch();
+  FLOP_CUDA(cudaGetLastError());
+  return FLOP_OK;
+}
+
 // ====================================================================== C ABI
 extern "C" {
 
@@ -2002,6 +2020,7 @@ int flop_expected_l0_lagrangian(const float* log_alpha, int64_t n, const int64_t
   cudaStream_t st = (cudaStream_t)stream;
   L0Scratch* sc = (L0Scratch*)ws;
   const float thr = (float)((double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta));
+  if (l0_small_ok(n, n_seg)) return launch_l0_small(log_alpha, n, seg_off, seg_size, n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, st);
   const int64_t chunks = (n + kL0Chunk - 1) / kL0Chunk + n_seg;
   if (chunks > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
   if (chunks > 0 && n_seg > 0) {
@@ -2032,10 +2051,11 @@ int flop_expected_l0_lagrangian_noalloc(const float* log_alpha, int64_t n, const
   }
   if (n_seg > 0 && (!seg_off || !seg_size)) return FLOP_ERR_INVALID_ARG;
   if (n > 0 && !log_alpha) return FLOP_ERR_INVALID_ARG;
-  L0Scratch* sc = nullptr;
-  FLOP_TRY(builtin_scratch(&sc));
   cudaStream_t st = (cudaStream_t)stream;
   const float thr = (float)((double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta));
+  if (l0_small_ok(n, n_seg)) return launch_l0_small(log_alpha, n, seg_off, seg_size, n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, st);
+  L0Scratch* sc = nullptr;
+  FLOP_TRY(builtin_scratch(&sc));
   const int64_t chunks = (n + kL0Chunk - 1) / kL0Chunk + n_seg;
   // Nothing in the scratch has to start at zero: every chunk sum that the finalisation reads and
   // the gradient coefficient are rewritten by this call before they are read.

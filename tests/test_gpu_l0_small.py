@@ -1,0 +1,41 @@
+"""The one-launch expected-L0 call on both sides of its limits (65 536 gates, 2048 per segment on average), with empty and
+uneven segments, against the oracle.  out4 is formed in fp64 from probabilities good to a few fp32 ulp, the gradient adds one fp32
+product to what is there: relative 2e-6."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flop_oracle as O
+from tests._util import HC, host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def b():
+    from paper_1910_04732_b200 import build, binding
+    build.build()
+    binding.load_library()
+    return binding
+
+
+@pytest.mark.parametrize("sizes", [[1], [31, 0, 33], [256], [2048], [2049], [768] * 72, [0, 5000, 1, 0, 7], [512] * 128, [512] * 128 + [1], [3] * 4000])
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_against_the_oracle(b, sizes, noalloc):
+    g = np.random.default_rng(len(sizes))
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n, a, size = int(off[-1]), g.normal(0.5, 2.0, int(off[-1])).astype(np.float32), g.uniform(100, 3000, len(sizes)).astype(np.float32)
+    dev = lambda v: torch.from_numpy(np.asarray(v)).cuda()
+    out4, seg, dla = torch.full((4,), float("nan"), device="cuda"), torch.full((len(sizes),), float("nan"), device="cuda"), dev(np.linspace(-1, 1, n).astype(np.float32))
+    args = (dev(a), dev(off), dev(size), HC, dev(np.float32([0.4])), dev(np.float32([0.3, 1.7])), out4, seg, dla)
+    if noalloc:
+        b.expected_l0_lagrangian_noalloc(*args)
+    else:
+        b.expected_l0_lagrangian(*args, b.alloc_workspace(b.workspace_bytes(b.OP_L0, n, 0, 0, len(sizes), b.F32)))
+    assert b.device_status() == b.OK
+    want = O.expected_l0_lagrangian(a, off, size, *HC, float(np.float32(0.4)), float(np.float32(0.3)), float(np.float32(1.7)))
+    ref = np.array([want["s"], want["g"], want["dg_dlambda1"], want["dg_dlambda2"]])
+    assert np.all(np.abs(host(out4) - ref) <= 2e-6 * np.maximum(np.abs(ref), want["s"]))
+    assert np.all(np.abs(host(seg) - want["seg_expected"]) <= 2e-6 * np.maximum(want["seg_expected"], 1.0))
+    base = np.linspace(-1, 1, n).astype(np.float32).astype(np.float64)
+    assert np.all(np.abs(host(dla) - (base + want["dlog_alpha"])) <= 1e-6 * (np.abs(base) + np.abs(want["dlog_alpha"])) + 2e-6 * np.abs(want["dlog_alpha"]) + 1e-12)
