@@ -380,9 +380,10 @@ int launch_group_inst(const tc::GroupParams& gp, int cta2, double flops, cudaStr
 
 // A launch whose problems are of two kinds: bf16 stores with (K-major A, MN-major B) and in-place weight
 // gradients with both operands MN-major (the two steps of the grouped backward pass).  CTA pairs only.
+template <bool B0_MN, int E1>   // B operand of the stores; epilogue of the products that contract over tokens
 int launch_dual_inst(const tc::GroupParams& gp, double flops, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
-  auto kern = tc::gemm2_dual_kernel<false, true, tc::EPI_STORE, true, true, tc::EPI_WGRAD>;
+  auto kern = tc::gemm2_dual_kernel<false, B0_MN, tc::EPI_STORE, true, true, E1>;
   if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
   {
     GemmTimer timer(st, flops);
@@ -408,7 +409,7 @@ int launch_dual_inst(const tc::GroupParams& gp, double flops, cudaStream_t st) {
 // its work items with their cost (SM cycles, the model of plan_group) for the schedule.
 int add_problem(tc::GroupParams& gp, const TcJob& j, std::vector<tc::ItemGroup>& groups, double& flops) {
   if (j.M > INT32_MAX || j.N > INT32_MAX || j.K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
-  const bool kind1 = j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_WGRAD;
+  const bool kind1 = j.A.mn_major && j.B.mn_major && j.ep.kind != tc::EPI_STORE;
   tc::GroupProblem& pr = gp.prob[gp.n];
   pr.p.kind = kind1 ? 1 : 0;
   if (!j.A.mn_major) FLOP_TRY(make_tmap(&pr.ta, j.A.ptr, j.M, j.K, j.A.ld, tc::BK, tc::BM));
@@ -470,7 +471,9 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
     memset(&gp, 0, sizeof(gp));
     double flops = 0.0;
     const TcJob& first = jobs[i];
-    bool uniform = true, dual_ok = true;   // one kind of problem / the two kinds gemm2_dual_kernel is built for
+    // one kind of problem / the two pairs of kinds gemm2_dual_kernel is built for: the layer's backward pass (MN-major B, weight
+    // gradients in place) and the embedding's (K-major B, split-K slices)
+    bool uniform = true, dual_ok = true, dual_emb = true;
     std::vector<tc::ItemGroup> groups;
     groups.reserve(64);
     for (; i < jobs.size() && gp.n < tc::kMaxGroup; ++i) {
@@ -481,6 +484,9 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
       const bool kind0 = !j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_STORE;
       const bool kind1 = j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_WGRAD;
       if (!(kind0 || kind1) || !j.pl.cta2) dual_ok = false;
+      const bool emb0 = !j.A.mn_major && !j.B.mn_major && j.ep.kind == tc::EPI_STORE;
+      const bool emb1 = j.A.mn_major && j.B.mn_major && j.ep.kind == tc::EPI_SLICE;
+      if (!(emb0 || emb1) || !j.pl.cta2) dual_emb = false;
       FLOP_TRY(add_problem(gp, j, groups, flops));
     }
     if (gp.n == 0) continue;
@@ -502,7 +508,7 @@ int launch_tc_group(const std::vector<TcJob>& jobs, cudaStream_t st) {
     }
     const bool a_mn = first.A.mn_major, b_mn = first.B.mn_major;
     int rc = FLOP_ERR_UNSUPPORTED;
-    if (!uniform) rc = dual_ok ? launch_dual_inst(gp, flops, st) : FLOP_ERR_INVALID_ARG;
+    if (!uniform) rc = dual_ok ? launch_dual_inst<true, tc::EPI_WGRAD>(gp, flops, st) : dual_emb ? launch_dual_inst<false, tc::EPI_SLICE>(gp, flops, st) : FLOP_ERR_INVALID_ARG;
     else if (!a_mn && !b_mn && first.ep.kind == tc::EPI_STORE) rc = launch_group_inst<false, false, tc::EPI_STORE>(gp, cta2, flops, st);
     else if (!a_mn && b_mn && first.ep.kind == tc::EPI_STORE) rc = launch_group_inst<false, true, tc::EPI_STORE>(gp, cta2, flops, st);
     else if (a_mn && b_mn && first.ep.kind == tc::EPI_SLICE) rc = launch_group_inst<true, true, tc::EPI_SLICE>(gp, cta2, flops, st);
@@ -2150,29 +2156,58 @@ int flop_gated_embedding_bwd(const void* dY, int64_t lddy, const int32_t* ids, i
   float* slices = (float*)ar.take(slice_bytes);
   EmbedFinish fin{};
   fin.accumulate = accumulate; fin.d_i = (int)d_i; fin.d = (int)d;
-  // dH'[T, d_i] = dY[T, d] O^T: B(n = k_dim, k = j) = O[n, j] (K-major as stored)
-  FLOP_TRY(launch_tc({dY, lddy, false}, {O, ldo, false}, T, d_i, d, plan_tc(T, d_i, d, false, false),
-                     store_epilogue(dH, lddh, nullptr), st));
+  // dH'[T, d_i] = dY[T, d] O^T: B(n = k_dim, k = j) = O[n, j] (K-major as stored); dO[d_i, d] = H'^T dY contracts over the
+  // tokens.  The two need nothing of each other, so they share a launch when that is estimated faster: dH' alone is one
+  // uneven round of tiles, and dO's split tiles fill it up.
+  const int64_t ld_slice = round_up(d, 4), max_splits = (int64_t)(slice_bytes / ((size_t)d_i * ld_slice * 4));
+  const TcPlan ph = plan_tc(T, d_i, d, false, false);
+  TcPlan po = plan_tc(d_i, d, T, true, true);
+  if (po.splits > max_splits) {     // no finer than the workspace allows
+    if (max_splits >= 2) {
+      po.kb_per_split = (int)((po.num_kb + max_splits - 1) / max_splits);
+      po.splits = (po.num_kb + po.kb_per_split - 1) / po.kb_per_split;
+    } else {
+      po = plan_tc(d_i, d, T, false, true);
+    }
+  }
+  auto slice_epilogue = [&](int splits) {
+    TcEpilogue e{};
+    e.kind = tc::EPI_SLICE; e.slices = slices; e.slice_elems = d_i * ld_slice; e.ld_slice = ld_slice;
+    fin.slices = slices; fin.n_slices = splits; fin.slice_elems = e.slice_elems; fin.ld_slice = ld_slice; fin.dO = dO; fin.lddo = lddo;
+    return e;
+  };
+  const auto slice_pass = [&](int splits) { return splits > 1 ? 8.0 * splits * (double)d_i * d / 3000.0 : 0.0; };
+  TcPlan mh{}, mo{};
+  double merged = 1e300;
   if (dO) {
-    // dO[d_i, d] = H'^T dY: contraction over the tokens.  A cluster's few tiles cannot fill the machine, so K is split as
-    // far as the cost model wants and the workspace allows; unsplit, the result is written in place.
-    TcPlan pl = plan_tc(d_i, d, T, true, true);
-    const int64_t ld_slice = round_up(d, 4), max_splits = (int64_t)(slice_bytes / ((size_t)d_i * ld_slice * 4));
-    if (pl.splits > max_splits) {
-      if (max_splits >= 2) {
-        pl.kb_per_split = (int)((pl.num_kb + max_splits - 1) / max_splits);
-        pl.splits = (pl.num_kb + pl.kb_per_split - 1) / pl.kb_per_split;
-      } else {
-        pl = plan_tc(d_i, d, T, false, true);
+    LaunchCost ch{ph.cta2}, co{po.cta2};
+    ch.add(T, d_i, d, ph);
+    co.add(d_i, d, T, po);
+    const double separate = ch.cycles() + co.cycles() + slice_pass(po.splits);
+    const int num_kb = (int)((T + tc::BK - 1) / tc::BK);
+    for (int a = 0; a < 4; ++a)
+      for (int sp = 2; sp <= std::min<int64_t>(32, std::min<int64_t>(max_splits, num_kb)); ++sp) {
+        const int bn_h = a & 1 ? 256 : 128, bn_o = a & 2 ? 256 : 128, kbps = (num_kb + sp - 1) / sp;
+        if ((num_kb + kbps - 1) / kbps != sp) continue;
+        LaunchCost both{1};
+        both.add(T, d_i, d, bn_h);
+        both.add(d_i, d, T, bn_o, sp);
+        const double c = both.cycles() + slice_pass(sp);
+        if (c >= merged || c >= separate) continue;
+        merged = c;
+        mh = fixed_plan(T, d_i, d, bn_h, 1);
+        mo = fixed_plan(d_i, d, T, bn_o, 1);
+        mo.splits = sp; mo.kb_per_split = kbps;
       }
-    }
-    TcEpilogue e = wgrad_epilogue(dO, lddo, wgrad_dt, nullptr, accumulate);
-    if (pl.splits > 1) {
-      e = TcEpilogue{};
-      e.kind = tc::EPI_SLICE; e.slices = slices; e.slice_elems = d_i * ld_slice; e.ld_slice = ld_slice;
-      fin.slices = slices; fin.n_slices = pl.splits; fin.slice_elems = e.slice_elems; fin.ld_slice = ld_slice; fin.dO = dO; fin.lddo = lddo;
-    }
-    FLOP_TRY(launch_tc({H_save, ldh, true}, {dY, lddy, true}, d_i, d, T, pl, e, st));
+  }
+  if (mo.splits > 1) {
+    FLOP_TRY(launch_tc_group({TcJob{{dY, lddy, false}, {O, ldo, false}, T, d_i, d, mh, store_epilogue(dH, lddh, nullptr)},
+                              TcJob{{H_save, ldh, true}, {dY, lddy, true}, d_i, d, T, mo, slice_epilogue(mo.splits)}}, st));
+  } else {
+    FLOP_TRY(launch_tc({dY, lddy, false}, {O, ldo, false}, T, d_i, d, ph, store_epilogue(dH, lddh, nullptr), st));
+    if (dO)   // unsplit, the result is written in place
+      FLOP_TRY(launch_tc({H_save, ldh, true}, {dY, lddy, true}, d_i, d, T, po,
+                         po.splits > 1 ? slice_epilogue(po.splits) : wgrad_epilogue(dO, lddo, wgrad_dt, nullptr, accumulate), st));
   }
   if (dE || dlog_alpha) {
     const int lanes = embed_lanes(d_i);
