@@ -84,8 +84,11 @@ inline double deal_groups(std::vector<ItemGroup>& groups, int n, int units, int 
 }
 
 // Largest load of the round-robin deal (item i to unit i % units); true when it is within 3 % of the lower bound
-// max(mean load, longest item), so that a table has nothing to gain.  `groups` in work-list order.
+// max(mean load, longest item), so that a table has nothing to gain, and when a table could not name the units at all (more
+// than kMaxUnits).  `groups` in work-list order.
 inline bool round_robin_is_good(const std::vector<ItemGroup>& groups, int units, double* rr_makespan) {
+  if (rr_makespan) *rr_makespan = 0.0;
+  if (units <= 0 || units > kMaxUnits) return true;
   double load[kMaxUnits] = {};
   double total = 0.0, longest = 0.0, rr = 0.0;
   for (const ItemGroup& g : groups) {
