@@ -111,6 +111,20 @@ inline void launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline int64_t round_up(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// A caller's buffer, from its first byte to one past its last (nothing when the pointer is null).  A launch whose blocks read what
+// another of its blocks writes needs its outputs apart from its inputs; a sequence of launches often does not, so a call
+// whose buffers overlap keeps the sequence.
+struct Span {
+  uintptr_t lo = 0, hi = 0;
+  Span() = default;
+  Span(const void* p, int64_t rows, int64_t cols, int64_t ld, size_t elem) {
+    if (!p || rows <= 0 || cols <= 0) return;
+    lo = reinterpret_cast<uintptr_t>(p);
+    hi = lo + (size_t)((rows - 1) * ld + cols) * elem;
+  }
+  bool meets(const Span& o) const { return lo < o.hi && o.lo < hi; }
+};
 inline bool valid_dt(int dt) { return dt == FLOP_F32 || dt == FLOP_BF16; }
 inline size_t elt(int dt) { return dt == FLOP_BF16 ? 2 : 4; }
 inline bool valid_hc(const flop_hc_params_t& hc) { return hc.beta > 0.f && hc.gamma < 0.f && hc.zeta > 1.f; }
@@ -2247,7 +2261,14 @@ int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t h
   cudaStream_t st = (cudaStream_t)stream;
   const double thr = (double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta);
   const int64_t pd = gather ? d_out : 0, qd = gather ? d_in : 0;
-  if (r <= kFusedMaxR && pd <= kFusedMaxBytes / (int64_t)(std::max<int64_t>(r, 1) * elt(dt)) && qd <= INT32_MAX) {
+  // In one launch every block reads the gates and its rows while others already write results; the three launches finish
+  // reading first (the gates may become z_det in place, and P its own surviving columns).
+  const Span in(log_alpha_or_z, 1, r, r, 4), p_in(P, pd, r, ldp, elt(dt)), q_in(Q, r, qd, ldq, elt(dt));
+  const Span out[5] = {Span(idx, 1, r, r, 4), Span(k_dev, 1, 1, 1, 4), Span(z_det, 1, r, r, 4),
+                       Span(Pc, pd, std::min(r, ldpc), ldpc, elt(dt)), Span(Qc, r, qd, ldqc, elt(dt))};
+  bool apart = true;
+  for (const Span& o : out) apart = apart && !o.meets(in) && !o.meets(p_in) && !o.meets(q_in);
+  if (apart && r <= kFusedMaxR && pd <= kFusedMaxBytes / (int64_t)(std::max<int64_t>(r, 1) * elt(dt)) && qd <= INT32_MAX) {
     return dt == FLOP_BF16 ? launch_compact_fused<bf16>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st)
                            : launch_compact_fused<float>(log_alpha_or_z, mode, thr, r, idx, k_dev, z_det, P, ldp, Q, ldq, qd, pd, Pc, ldpc, Qc, ldqc, st);
   }
