@@ -748,6 +748,25 @@ MergedShape plan_merged(const flop_bwd_problem_t* pr, int n) {
   return best;
 }
 
+// Whether the shared launches may stand in for the launches per product: the first writes dP while dH' still reads dY and P (and
+// X and Q are read after it), the second writes dX and dQ while the other of the two still reads X and Q.  One after another,
+// dX may take the place of X, and split weight gradients the place of anything but Q.
+bool merged_apart(const flop_bwd_problem_t* pr, int n, int wgrad_dt) {
+  for (int i = 0; i < n; ++i) {
+    const flop_bwd_problem_t& a = pr[i];
+    const Span dP(a.dP, a.d_out, a.r, a.lddp, elt(wgrad_dt)), dQ(a.dQ, a.r, a.d_in, a.lddq, elt(wgrad_dt)), dX(a.dX, a.T, a.d_in, a.lddx, 2);
+    for (int j = 0; j < n; ++j) {
+      const flop_bwd_problem_t& o = pr[j];
+      const Span X(o.X, o.T, o.d_in, o.ldx, 2), Q(o.Q, o.r, o.d_in, o.ldq, 2);
+      for (const Span& in : {Span(o.dY, o.T, o.d_out, o.lddy, 2), Span(o.P, o.d_out, o.r, o.ldp, 2), Span(o.H_save, o.T, o.r, o.ldh, 2)})
+        if (dP.meets(in)) return false;
+      for (const Span& in : {X, Q})
+        if (dP.meets(in) || dQ.meets(in) || dX.meets(in)) return false;
+    }
+  }
+  return true;
+}
+
 // Weight gradient written straight from the GEMM epilogue (no split-K, no fp32 slices).
 TcEpilogue wgrad_epilogue(void* out, int64_t ldo, int wgrad_dt, const float* row_scale, int accumulate) {
   TcEpilogue e{};
@@ -1434,7 +1453,8 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     const flop_bwd_problem_t one{dY, lddy, X, ldx, Q, ldq, P, ldp, z, dz_dla, H_save, ldh, dX, lddx, dP, lddp, dQ, lddq, dlog_alpha,
                                  T, d_in, d_out, r, ws, ws_bytes, nullptr, nullptr, 0, 0};
     Arena grouped{nullptr, 0, 0};
-    if (plan_merged(&one, 1).cycles < separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes)
+    if (plan_merged(&one, 1).cycles < separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes &&
+        merged_apart(&one, 1, wgrad_dt))
       return bwd_grouped_impl(&one, 1, accumulate, dt, wgrad_dt, nullptr, 0, stream, separate);
   }
   if (dt == FLOP_BF16) {
@@ -1683,7 +1703,7 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
   }
   MergedShape mg{0, 0, 0, 0, 1e300};
   if (sw.bn == 0 || sw.items < (sw.cta2 ? num_sms() / 2 : num_sms())) {
-    if (direct && n > 0 && !sync && 2 * n <= tc::kMaxGroup) {
+    if (direct && n > 0 && !sync && 2 * n <= tc::kMaxGroup && merged_apart(pr, n, wgrad_dt)) {
       mg = plan_merged(pr, n);
       if (single_cycles <= 0.0) {     // the other form of this call: a launch per product, weight gradients split, a finishing pass
         LaunchCost h{s3.cta2}, p{0}, q{0}, x{s6.cta2};
