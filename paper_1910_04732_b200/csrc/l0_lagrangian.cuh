@@ -211,10 +211,12 @@ constexpr int kL0SmallCtas = 8, kL0SmallThreads = 512, kL0SmallWarps = kL0SmallT
 
 __global__ void __launch_bounds__(kL0SmallThreads)
 l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__ seg_off, const float* __restrict__ seg_size, int n_seg,
-                float thr, const float* __restrict__ target, const float* __restrict__ lambda, float* __restrict__ out4,
-                float* __restrict__ seg_expected, float* __restrict__ dlog_alpha, int64_t n) {
+                float thr, const float* target, const float* lambda, float* out4, float* __restrict__ seg_expected,
+                float* __restrict__ dlog_alpha, int64_t n) {
   pdl_wait();
   pdl_launch_dependents();
+  // read by every CTA before the cluster's barrier: CTA 0 writes out4 after it, which may lie on the same memory
+  const double goal = (double)target[0], l1 = (double)lambda[0], l2 = (double)lambda[1];
   __shared__ double red_w[kL0SmallWarps], red_s[kL0SmallWarps];
   __shared__ __align__(16) double total[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x;
@@ -262,8 +264,7 @@ l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__
     weighted += a; size_sum += b;
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // the totals have been read (waited for at the end)
-  const double s = size_sum > 0.0 ? weighted / size_sum : 0.0, diff = s - (double)target[0];
-  const double l1 = (double)lambda[0], l2 = (double)lambda[1];
+  const double s = size_sum > 0.0 ? weighted / size_sum : 0.0, diff = s - goal;
   if (cta == 0 && tid == 0) {
     out4[0] = (float)s;
     out4[1] = (float)(l1 * diff + l2 * diff * diff);

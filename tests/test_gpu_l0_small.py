@@ -39,3 +39,22 @@ def test_against_the_oracle(b, sizes, noalloc):
     assert np.all(np.abs(host(seg) - want["seg_expected"]) <= 2e-6 * np.maximum(want["seg_expected"], 1.0))
     base = np.linspace(-1, 1, n).astype(np.float32).astype(np.float64)
     assert np.all(np.abs(host(dla) - (base + want["dlog_alpha"])) <= 1e-6 * (np.abs(base) + np.abs(want["dlog_alpha"])) + 2e-6 * np.abs(want["dlog_alpha"]) + 1e-12)
+
+
+@pytest.mark.parametrize("at", [0, 2, 3])
+def test_results_over_the_multipliers(b, at):
+    """out4 on the same memory as lambda (and target): every block has read them before the results are written."""
+    sizes = [768] * 72
+    g = np.random.default_rng(7)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    a, size = g.normal(0.5, 2.0, int(off[-1])).astype(np.float32), g.uniform(100, 3000, len(sizes)).astype(np.float32)
+    want = O.expected_l0_lagrangian(a, off, size, *HC, float(np.float32(0.4)), float(np.float32(0.3)), float(np.float32(1.7)))
+    dev = lambda v: torch.from_numpy(np.asarray(v)).cuda()
+    ws = b.alloc_workspace(b.workspace_bytes(b.OP_L0, a.size, 0, 0, len(sizes), b.F32))
+    la, offd, sized = dev(a), dev(off), dev(size)
+    for _ in range(50):
+        buf, dla = dev(np.float32([9, 9, 0.3, 1.7, 0.4, 9, 9, 9])), torch.zeros(a.size, device="cuda")
+        b.expected_l0_lagrangian(la, offd, sized, HC, buf[4:5], buf[2:4], buf[at:at + 4], None, dla, ws)
+        assert abs(float(buf[at]) - want["s"]) <= 2e-6 * want["s"]
+        assert np.all(np.abs(host(dla) - want["dlog_alpha"]) <= 3e-6 * np.abs(want["dlog_alpha"]) + 1e-12)
+    assert b.device_status() == b.OK
