@@ -2093,9 +2093,10 @@ int flop_expected_l0_lagrangian_noalloc(const float* log_alpha, int64_t n, const
   if (n > 0 && !log_alpha) return FLOP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const float thr = (float)((double)hc.beta * log(-(double)hc.gamma / (double)hc.zeta));
-  if (l0_small_ok(n, n_seg)) return launch_l0_small(log_alpha, n, seg_off, seg_size, n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, st);
+  // Looked up by every call, also by one that needs no scratch: the first call on a device is the one outside any capture.
   L0Scratch* sc = nullptr;
   FLOP_TRY(builtin_scratch(&sc));
+  if (l0_small_ok(n, n_seg)) return launch_l0_small(log_alpha, n, seg_off, seg_size, n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, st);
   const int64_t chunks = (n + kL0Chunk - 1) / kL0Chunk + n_seg;
   // Nothing in the scratch has to start at zero: every chunk sum that the finalisation reads and
   // the gradient coefficient are rewritten by this call before they are read.

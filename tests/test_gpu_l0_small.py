@@ -1,6 +1,10 @@
 """The one-launch expected-L0 call on both sides of its limits (65 536 gates, 2048 per segment on average), with empty and
 uneven segments, against the oracle.  out4 is formed in fp64 from probabilities good to a few fp32 ulp, the gradient adds one fp32
 product to what is there: relative 2e-6."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -58,3 +62,36 @@ def test_results_over_the_multipliers(b, at):
         assert abs(float(buf[at]) - want["s"]) <= 2e-6 * want["s"]
         assert np.all(np.abs(host(dla) - want["dlog_alpha"]) <= 3e-6 * np.abs(want["dlog_alpha"]) + 1e-12)
     assert b.device_status() == b.OK
+
+
+CAPTURE_AFTER_SMALL = """
+import torch
+from paper_1910_04732_b200 import binding as b
+hc = (2.0 / 3.0, -0.1, 1.1)
+def table(sizes):
+    n = sum(sizes)
+    off = torch.cumsum(torch.tensor([0] + sizes), 0).cuda()
+    return (torch.linspace(-3, 3, n, device="cuda"), off, torch.full((len(sizes),), 100.0, device="cuda"), hc, torch.tensor([0.5], device="cuda"),
+            torch.tensor([0.3, 1.7], device="cuda"), torch.zeros(4, device="cuda"), torch.zeros(len(sizes), device="cuda"), torch.zeros(n, device="cuda"))
+small, large = table([64]), table([2048] * 40)
+b.expected_l0_lagrangian_noalloc(*small)
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):
+    b.expected_l0_lagrangian_noalloc(*large)
+g.replay()
+torch.cuda.synchronize()
+want = table([2048] * 40)
+b.expected_l0_lagrangian(*want, b.alloc_workspace(b.workspace_bytes(b.OP_L0, 81920, 0, 0, 40, b.F32)))
+assert torch.equal(large[6], want[6]) and torch.equal(large[8], want[8]) and float(large[6][0]) > 0
+assert b.device_status() == b.OK
+print("captured")
+"""
+
+
+def test_first_call_small_then_a_larger_one_captured(b):
+    """The first call on a device looks up the built-in scratch even when it needs none, so that a later call may be captured.
+    In a process of its own: the lookup happens once per process."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", CAPTURE_AFTER_SMALL], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "captured", r.stderr[-2000:]
