@@ -62,20 +62,24 @@ int64_t integer(PyObject* o) {
   if (v == (unsigned long long)-1 && PyErr_Occurred()) throw Stop{};
   return (int64_t)v;
 }
-int truth(PyObject* o) {
-  const int v = PyObject_IsTrue(o);
-  if (v < 0) throw Stop{};
-  return v;
+int flag(PyObject* o) {   // int(o)
+  PyObject* v = PyNumber_Long(o);
+  if (!v) throw Stop{};
+  const unsigned long m = PyLong_AsUnsignedLongMask(v);
+  Py_DECREF(v);
+  return (int)m;
 }
 flop_hc_params_t hard_concrete(PyObject* o) {
   float v[3];
   for (int i = 0; i < 3; ++i) {
-    PyObject* e = PySequence_GetItem(o, i);
-    if (!e) throw Stop{};
-    const double d = PyFloat_AsDouble(e);
-    Py_DECREF(e);
-    if (d == -1.0 && PyErr_Occurred()) throw Stop{};
-    v[i] = (float)d;
+    PyObject* at = PyLong_FromLong(i);
+    PyObject* e = at ? PyObject_GetItem(o, at) : nullptr;   // float(o[i]), whatever o is
+    Py_XDECREF(at);
+    PyObject* d = e ? PyNumber_Float(e) : nullptr;
+    Py_XDECREF(e);
+    if (!d) throw Stop{};
+    v[i] = (float)PyFloat_AS_DOUBLE(d);
+    Py_DECREF(d);
   }
   return flop_hc_params_t{v[0], v[1], v[2]};
 }
@@ -128,7 +132,7 @@ FLOP_METHOD(gated_lowrank_bwd, 13) {   // dY, X, Q, P, z, dz_dla, H_save, dX, dP
   const int dt = storage(required(a[1]));
   const int wdt = a[8] != Py_None ? storage(required(a[8])) : a[9] != Py_None ? storage(required(a[9])) : dt;
   const float *z = ptr<float>(a[4]), *dz = ptr<float>(a[5]); float* dla = ptr<float>(a[10]);
-  void* ws = ptr(a[11]); const size_t wb = numel(a[11]); const int acc = truth(a[12]);
+  void* ws = ptr(a[11]); const size_t wb = numel(a[11]); const int acc = flag(a[12]);
   void* st = stream();
   return call([&] {
     return flop_gated_lowrank_bwd(dY.p, dY.ld, X.p, X.ld, Q.p, Q.ld, P.p, P.ld, z, dz, H.p, H.ld, dX.p, dX.ld, dP.p, dP.ld, dQ.p, dQ.ld, dla, acc,
@@ -163,7 +167,7 @@ FLOP_METHOD(gated_embedding_bwd, 12) {   // dY, ids, E, O, z, dz_dla, H_save, dE
   const int dt = storage(required(a[2])), wdt = a[8] != Py_None ? storage(required(a[8])) : (int)FLOP_BF16;
   const int64_t T = required(a[1]).numel();
   const int32_t* ids = ptr<int32_t>(a[1]); const float *z = ptr<float>(a[4]), *dz = ptr<float>(a[5]); float* dla = ptr<float>(a[9]);
-  void* ws = ptr(a[10]); const size_t wb = numel(a[10]); const int acc = truth(a[11]);
+  void* ws = ptr(a[10]); const size_t wb = numel(a[10]); const int acc = flag(a[11]);
   void* st = stream();
   return call([&] {
     return flop_gated_embedding_bwd(dY.p, dY.ld, ids, T, E.p, E.ld, E.rows, O.p, O.ld, z, dz, H.p, H.ld, (float*)dE.p, dE.ld, dO.p, dO.ld, dla, acc,

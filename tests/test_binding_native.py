@@ -32,3 +32,29 @@ def test_every_native_call_has_its_python_name():
     assert len(names) == 8 and all(callable(getattr(b, n)) and "flop_" + n in b.EXPORTS for n in names)
     with pytest.raises(TypeError):
         native.compact_fwd(X)
+
+
+HC = (0.5, -0.25, 1.25)      # exact in every form
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hc", [list(HC), torch.tensor(HC), torch.tensor(HC).numpy(), dict(enumerate(HC)), [str(v) for v in HC]])
+def test_constants_in_any_form_that_can_be_indexed(hc):
+    la, z, want = torch.linspace(-3, 3, 64, device="cuda"), torch.zeros(64, device="cuda"), torch.zeros(64, device="cuda")
+    b.gate_sample(la, HC, 1, 2, want)
+    b.gate_sample(la, hc, 1, 2, z)
+    assert torch.equal(z, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("accumulate,adds", [(False, False), (0, False), (0.5, False), ("0", False), (True, True), (2, True), (torch.tensor(1), True)])
+def test_accumulate_is_an_integer(accumulate, adds):
+    x = torch.ones(8, 8, device="cuda")
+    v, dP, dQ, dla = torch.ones(8, device="cuda"), 3 * x, 3 * x, 3 * v
+    b.gated_lowrank_bwd(x, x, x, x, v, v, x, None, dP, dQ, dla, b.alloc_workspace(b.workspace_bytes(b.OP_BWD, 8, 8, 8, 8, b.F32)), accumulate)
+    assert torch.all(dP == 8 + 3 * adds) and torch.all(dQ == 64 + 3 * adds) and torch.all(dla == 512 + 3 * adds)
+
+
+def test_accumulate_that_is_no_integer_is_refused():
+    with pytest.raises(TypeError):
+        b.gated_lowrank_bwd(X, X, X, X, None, None, X, None, None, None, None, None, None)
