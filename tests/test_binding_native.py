@@ -50,7 +50,8 @@ def test_constants_in_any_form_that_can_be_indexed(hc):
 @pytest.mark.parametrize("accumulate,adds", [(False, False), (0, False), (0.5, False), ("0", False), (True, True), (2, True), (torch.tensor(1), True)])
 def test_accumulate_is_an_integer(accumulate, adds):
     x = torch.ones(8, 8, device="cuda")
-    v, dP, dQ, dla = torch.ones(8, device="cuda"), 3 * x, 3 * x, 3 * v
+    v = torch.ones(8, device="cuda")
+    dP, dQ, dla = 3 * x, 3 * x, 3 * v
     b.gated_lowrank_bwd(x, x, x, x, v, v, x, None, dP, dQ, dla, b.alloc_workspace(b.workspace_bytes(b.OP_BWD, 8, 8, 8, 8, b.F32)), accumulate)
     assert torch.all(dP == 8 + 3 * adds) and torch.all(dQ == 64 + 3 * adds) and torch.all(dla == 512 + 3 * adds)
 
