@@ -1056,7 +1056,7 @@ static int launch_embed_bwd(const int32_t* ids, int64_t T, const void* E, int64_
   return FLOP_OK;
 }
 
-static bool l0_small_ok(int64_t n, int32_t n_seg) { return n > 0 && n_seg > 0 && n <= kL0SmallMax && n <= kL0SmallPerSeg * n_seg; }
+static bool l0_small_ok(int64_t n, int32_t n_seg) { return n > 0 && n_seg > 0 && n <= kL0SmallMax; }
 static int launch_l0_small(const float* log_alpha, int64_t n, const int64_t* seg_off, const float* seg_size, int32_t n_seg, float thr,
                            const float* target, const float* lambda, float* out4, float* seg_expected, float* dlog_alpha, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
@@ -1068,7 +1068,10 @@ static int launch_l0_small(const float* log_alpha, int64_t n, const int64_t* seg
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl_on() ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, l0_small_kernel, log_alpha, seg_off, seg_size, (int)n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, n);
+  const int run = l0_small_run((int)n);
+  static_assert(kL0SmallMax <= 16 * kL0SmallCtas * kL0SmallThreads, "the longest run fits the registers");
+  auto kern = run <= 32 ? l0_small_kernel<1> : run <= 128 ? l0_small_kernel<4> : run <= 256 ? l0_small_kernel<8> : l0_small_kernel<16>;
+  cudaLaunchKernelEx(&cfg, kern, log_alpha, seg_off, seg_size, (int)n_seg, thr, target, lambda, out4, seg_expected, dlog_alpha, (int)n, run, l0_small_inverse(run));
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;

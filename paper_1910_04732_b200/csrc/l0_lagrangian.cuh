@@ -201,29 +201,70 @@ l0_finalize_kernel(const int64_t* __restrict__ seg_off, const float* __restrict_
   }
 }
 
-// All three passes in one launch for up to kL0SmallMax gates with segments of kL0SmallPerSeg gates on average: the gates of a
-// whole model, where the three launches above are bound by their latencies (5.2 + 10.5 + 5.1 us for 72 segments of 768
-// gates).  One cluster of eight CTAs; a warp takes segments w, w + 128, ...; the CTAs exchange their totals through distributed
-// shared memory and each finishes the scalar part by itself, so nothing passes through global memory and no scratch
-// is needed.  Every sum has a fixed order.  The table is checked as in l0_finalize_kernel, before anything is written.
-constexpr int64_t kL0SmallMax = 65536, kL0SmallPerSeg = 2048;
+// All three passes in one launch for up to kL0SmallMax gates: the gates of a whole model, where the three launches above are
+// bound by their latencies (5.2 + 10.5 + 5.1 us for 72 segments of 768 gates).  One cluster of eight CTAs.  The gates are dealt
+// to the 128 warps in equal runs whatever the segments are: a warp takes the pieces of segments that lie in its run, reads the
+// table 32 entries at a time and leaves short segments to single lanes, so that neither one long segment nor many short or
+// empty ones make a chain (a warp per segment took 243 us where one segment held 65 000 gates).  The CTAs exchange
+// their totals through distributed shared memory and each finishes the scalar part by itself, so nothing passes through global
+// memory and no scratch is needed.  Every sum has a fixed order.  The table is checked as in l0_finalize_kernel, before
+// anything is written.
+constexpr int64_t kL0SmallMax = 65536;
 constexpr int kL0SmallCtas = 8, kL0SmallThreads = 512, kL0SmallWarps = kL0SmallThreads / 32;
+inline int l0_small_run(int n) { return (n + kL0SmallCtas * kL0SmallThreads - 1) / (kL0SmallCtas * kL0SmallThreads) * 32; }   // gates per warp
+inline uint32_t l0_small_inverse(int run) { return (uint32_t)(0x100000000ull / (uint64_t)run + 1); }   // j / run == (j * inverse) >> 32 for j <= kL0SmallMax + run
 
-__global__ void __launch_bounds__(kL0SmallThreads)
+// The pieces of segments in gates [pos, end) of a warp's run, in order; `s` is the segment that holds gate pos.  A segment of
+// fewer than 32 gates that lies in the run as a whole goes to one lane, lane_piece(segment, first gate, one past the last, size);
+// every other piece to the warp, warp_piece(segment, its first gate, one past its last, the same of the piece, size).
+template <typename L, typename W>
+__device__ __forceinline__ void l0_for_pieces(const int64_t* __restrict__ seg_off, const float* __restrict__ seg_size, int n_seg, int s, int pos,
+                                              int end, int lane, L&& lane_piece, W&& warp_piece) {
+  bool more = pos < end;
+  for (; more && s < n_seg; s += 32) {
+    int lo = end, hi = end;
+    float size = 0.f;
+    if (s + lane < n_seg) { lo = (int)seg_off[s + lane]; hi = (int)seg_off[s + lane + 1]; size = seg_size[s + lane]; }
+    const bool mine = lo >= pos && lo < hi && hi <= end && hi - lo < 32;
+    if (mine) lane_piece(s + lane, lo, hi, size);
+    unsigned todo = __ballot_sync(0xffffffffu, !mine && max(lo, pos) < min(hi, end));
+    more = __shfl_sync(0xffffffffu, hi, 31) < end;
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int seg_lo = __shfl_sync(0xffffffffu, lo, l), seg_hi = __shfl_sync(0xffffffffu, hi, l);
+      warp_piece(s + l, seg_lo, seg_hi, max(seg_lo, pos), min(seg_hi, end), __shfl_sync(0xffffffffu, size, l));
+    }
+  }
+}
+
+// STEPS: gates per lane of a run, 32 STEPS >= run.
+template <int STEPS>
+__global__ void __launch_bounds__(kL0SmallThreads, 1)
 l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__ seg_off, const float* __restrict__ seg_size, int n_seg,
                 float thr, const float* target, const float* lambda, float* out4, float* __restrict__ seg_expected,
-                float* __restrict__ dlog_alpha, int64_t n) {
+                float* __restrict__ dlog_alpha, int n, int run, uint32_t run_inv) {
   pdl_wait();
   pdl_launch_dependents();
   // read by every CTA before the cluster's barrier: CTA 0 writes out4 after it, which may lie on the same memory
   const double goal = (double)target[0], l1 = (double)lambda[0], l2 = (double)lambda[1];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x;
+  const int me = cta * kL0SmallWarps + warp, pos = min(n, me * run), end = min(n, pos + run);
+  float a[STEPS];                       // gate pos + 32 i + lane: the whole run is on its way before the table is read
+#pragma unroll
+  for (int i = 0; i < STEPS; ++i) a[i] = pos + 32 * i + lane < end ? log_alpha[pos + 32 * i + lane] : 0.f;
   __shared__ double red_w[kL0SmallWarps], red_s[kL0SmallWarps];
   __shared__ __align__(16) double total[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x;
+  __shared__ double head[kL0SmallWarps];        // a warp's sum over the segment that began before its run
+  __shared__ int s_first[kL0SmallWarps];        // the segment that holds the first gate of a warp's run
+  auto warp_of = [&](int j) { return (int)__umulhi((uint32_t)j, run_inv); };   // j / run
   int bad = 0;
   for (int s = tid; s < n_seg; s += kL0SmallThreads) {
     const int64_t lo = seg_off[s], hi = seg_off[s + 1];
-    bad |= lo < 0 || hi < lo || hi > n || (s == 0 && lo != 0) || (s == n_seg - 1 && hi != n);
+    if (lo < 0 || hi < lo || hi > n || (s == 0 && lo != 0) || (s == n_seg - 1 && hi != n)) { bad = 1; continue; }
+    if (lo == hi) continue;
+    const int g1 = min(warp_of((int)hi - 1), cta * kL0SmallWarps + kL0SmallWarps - 1);
+    for (int g = max(warp_of((int)lo + run - 1), cta * kL0SmallWarps); g <= g1; ++g) s_first[g - cta * kL0SmallWarps] = s;
   }
   if (__syncthreads_or(bad)) {     // every CTA takes the same decision
     if (cta == 0 && tid == 0) {
@@ -233,17 +274,41 @@ l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__
     }
     return;
   }
-  double weighted = 0.0, size_sum = 0.0;
-  for (int s = cta * kL0SmallWarps + warp; s < n_seg; s += kL0SmallCtas * kL0SmallWarps) {
-    const int64_t lo = seg_off[s], hi = seg_off[s + 1];
+  const int s0 = pos < end ? s_first[warp] : n_seg;
+  double weighted = 0.0, size_sum = 0.0, tail = 0.0;
+  int tail_seg = -1, tail_end = 0;              // the segment that goes on in the next warps' runs
+  int lanes = 0;                                // some sums are spread over the lanes
+  l0_for_pieces(seg_off, seg_size, n_seg, s0, pos, end, lane, [&](int s, int lo, int hi, float size) {
+    lanes = 1;
     double v = 0.0;
 #pragma unroll 4
-    for (int64_t j = lo + lane; j < hi; j += 32) v += (double)l0_pi(log_alpha[j], thr);
+    for (int j = lo; j < hi; ++j) v += (double)l0_pi(log_alpha[j], thr);
+    weighted += (double)size * v;
+    size_sum += (double)size * (double)(hi - lo);
+    if (seg_expected) seg_expected[s] = (float)v;
+  }, [&](int s, int seg_lo, int seg_hi, int lo, int hi, float size) {
+    double v = 0.0;
+#pragma unroll
+    for (int i = 0; i < STEPS; ++i) {
+      const int j = pos + 32 * i + lane;
+      if (j >= lo && j < hi) v += (double)l0_pi(a[i], thr);
+    }
     v = warp_sum_f64(v);
-    if (lane == 0 && seg_expected) seg_expected[s] = (float)v;
-    const double size = (double)seg_size[s];
-    weighted += size * v;
-    size_sum += size * (double)(hi - lo);
+    if (lane == 0) {
+      weighted += (double)size * v;
+      size_sum += (double)size * (double)(hi - lo);
+    }
+    if (lo > seg_lo) {
+      if (lane == 0) head[warp] = v;
+    } else if (hi < seg_hi) {
+      tail = v; tail_seg = s; tail_end = seg_hi;
+    } else if (seg_expected && lane == 0) {
+      seg_expected[s] = (float)v;
+    }
+  });
+  if (__any_sync(0xffffffffu, lanes)) {
+    weighted = warp_sum_f64(weighted);
+    size_sum = warp_sum_f64(size_sum);
   }
   if (lane == 0) { red_w[warp] = weighted; red_s[warp] = size_sum; }
   __syncthreads();
@@ -253,6 +318,9 @@ l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__
     total[0] = weighted; total[1] = size_sum;
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if (seg_expected)                             // segments without gates
+    for (int s = cta * kL0SmallThreads + tid; s < n_seg; s += kL0SmallCtas * kL0SmallThreads)
+      if (seg_off[s] == seg_off[s + 1]) seg_expected[s] = 0.f;
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   weighted = 0.0; size_sum = 0.0;
   const uint32_t at = (uint32_t)__cvta_generic_to_shared(total);
@@ -262,6 +330,18 @@ l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(c));
     asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "r"(peer) : "memory");
     weighted += a; size_sum += b;
+  }
+  if (seg_expected && tail_seg >= 0) {          // the rest of the segment that began in this run
+    double v = 0.0;
+    for (int g = me + 1 + lane; g <= warp_of(tail_end - 1); g += 32) {
+      uint32_t peer;
+      double h;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"((uint32_t)__cvta_generic_to_shared(head + g % kL0SmallWarps)), "r"(g / kL0SmallWarps));
+      asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(h) : "r"(peer) : "memory");
+      v += h;
+    }
+    v = warp_sum_f64(v) + tail;
+    if (lane == 0) seg_expected[tail_seg] = (float)v;
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // the totals have been read (waited for at the end)
   const double s = size_sum > 0.0 ? weighted / size_sum : 0.0, diff = s - goal;
@@ -273,15 +353,22 @@ l0_small_kernel(const float* __restrict__ log_alpha, const int64_t* __restrict__
   }
   if (dlog_alpha) {
     const double coef = size_sum > 0.0 ? (l1 + 2.0 * l2 * diff) / size_sum : 0.0;
-    for (int g = cta * kL0SmallWarps + warp; g < n_seg; g += kL0SmallCtas * kL0SmallWarps) {
-      const int64_t lo = seg_off[g], hi = seg_off[g + 1];
-      const float w = (float)(coef * (double)seg_size[g]);
+    auto gradient = [&](float alpha, float w) {
+      const float e = __expf(-fabsf(alpha - thr)), q = __fdividef(1.0f, 1.0f + e);   // as in l0_chunk_kernel<true>
+      return w * e * q * q;
+    };
+    l0_for_pieces(seg_off, seg_size, n_seg, s0, pos, end, lane, [&](int, int lo, int hi, float size) {
+      const float w = (float)(coef * (double)size);
 #pragma unroll 4
-      for (int64_t j = lo + lane; j < hi; j += 32) {
-        const float e = __expf(-fabsf(log_alpha[j] - thr)), q = __fdividef(1.0f, 1.0f + e);   // as in l0_chunk_kernel<true>
-        dlog_alpha[j] += w * e * q * q;
+      for (int j = lo; j < hi; ++j) dlog_alpha[j] += gradient(log_alpha[j], w);
+    }, [&](int, int, int, int lo, int hi, float size) {
+      const float w = (float)(coef * (double)size);
+#pragma unroll
+      for (int i = 0; i < STEPS; ++i) {
+        const int j = pos + 32 * i + lane;
+        if (j >= lo && j < hi) dlog_alpha[j] += gradient(a[i], w);
       }
-    }
+    });
   }
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

@@ -1,5 +1,5 @@
-"""The one-launch expected-L0 call on both sides of its limits (65 536 gates, 2048 per segment on average), with empty and
-uneven segments, against the oracle.  out4 is formed in fp64 from probabilities good to a few fp32 ulp, the gradient adds one fp32
+"""The one-launch expected-L0 call on both sides of its limit (65 536 gates), with empty and uneven segments, segments that cross
+the runs its warps take and tables of mostly empty segments, against the oracle.  out4 is formed in fp64 from probabilities good to a few fp32 ulp, the gradient adds one fp32
 product to what is there: relative 2e-6."""
 import os
 import subprocess
@@ -23,7 +23,9 @@ def b():
     return binding
 
 
-@pytest.mark.parametrize("sizes", [[1], [31, 0, 33], [256], [2048], [2049], [768] * 72, [0, 5000, 1, 0, 7], [512] * 128, [512] * 128 + [1], [3] * 4000])
+@pytest.mark.parametrize("sizes", [[1], [31, 0, 33], [256], [2048], [2049], [768] * 72, [0, 5000, 1, 0, 7], [512] * 128, [512] * 128 + [1], [3] * 4000,
+                                   [65000] + [1] * 31, [1] * 31 + [65000], [0] * 4000 + [40000] + [0] * 90, [20000, 0, 1, 30000, 0], [511, 513, 512, 1, 3000],
+                                   [65536], [33, 0, 4063] * 16])
 @pytest.mark.parametrize("noalloc", [False, True])
 def test_against_the_oracle(b, sizes, noalloc):
     g = np.random.default_rng(len(sizes))
@@ -62,6 +64,29 @@ def test_results_over_the_multipliers(b, at):
         assert abs(float(buf[at]) - want["s"]) <= 2e-6 * want["s"]
         assert np.all(np.abs(host(dla) - want["dlog_alpha"]) <= 3e-6 * np.abs(want["dlog_alpha"]) + 1e-12)
     assert b.device_status() == b.OK
+
+
+def _time_us(b, sizes):
+    off = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), device="cuda")
+    n, zeros = int(off[-1]), lambda k: torch.zeros(k, device="cuda")
+    args = (zeros(n), off, torch.ones(len(sizes), device="cuda"), HC, zeros(1), zeros(2), zeros(4), zeros(len(sizes)), zeros(n),
+            b.alloc_workspace(b.workspace_bytes(b.OP_L0, n, 0, 0, len(sizes), b.F32)))
+    best = float("inf")
+    for _ in range(5):
+        a, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            b.expected_l0_lagrangian(*args)
+        e.record()
+        e.synchronize()
+        best = min(best, a.elapsed_time(e) * 50)
+    return best
+
+
+@pytest.mark.parametrize("sizes", [[65000] + [1] * 31, [32000, 32000] + [1] * 40, [1] * 100 + [32768]])
+def test_an_uneven_table_costs_about_what_an_even_one_does(b, sizes):
+    """One long segment took sixteen times as long when a warp walked a whole segment; three times leaves room for noise."""
+    assert _time_us(b, sizes) < 3 * _time_us(b, [sum(sizes) // 64] * 64)
 
 
 CAPTURE_AFTER_SMALL = """
