@@ -816,41 +816,66 @@ int launch_chain_fwd(const void* X, int64_t ldx, const void* Q, int64_t ldq, con
 
 // Forward product for few tokens (see gemm_few.cuh).  `second`: A is what the launch before on the stream wrote, and that
 // launch wrote nothing else.
-template <int MT, int NT>
+template <int MT, int NT, int KS>
 int launch_few_inst(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, bf16* C, int64_t ldc, const float* cs, int T, int N, int K,
                     bool second, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
   constexpr int smem = few::smem_bytes(MT, NT);
   if (smem > 48 * 1024 && first_use_on_device(configured)) {
-    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, KS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, KS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   }
-  const dim3 grid((unsigned)((N + 16 * MT - 1) / (16 * MT)), (unsigned)((T + 8 * NT - 1) / (8 * NT)));
-  launch_k(second ? few::gemm_kernel<MT, NT, true> : few::gemm_kernel<MT, NT, false>, grid, dim3(few::kThreads), (size_t)smem, st, A, lda, B,
+  constexpr int rows = 16 * MT * (few::kWarps / KS);       // weight rows per block
+  const dim3 grid((unsigned)((N + rows - 1) / rows), (unsigned)((T + 8 * NT - 1) / (8 * NT)));
+  launch_k(second ? few::gemm_kernel<MT, NT, KS, true> : few::gemm_kernel<MT, NT, KS, false>, grid, dim3(few::kThreads), (size_t)smem, st, A, lda, B,
            ldb, C, ldc, cs, T, N, K);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
 }
+template <int NT>
+int launch_few_cut(int ks, const bf16* a, int64_t lda, const bf16* b, int64_t ldb, bf16* c, int64_t ldc, const float* cs, int t, int n, int k, bool second,
+                   cudaStream_t st) {
+  if (ks == 8) return launch_few_inst<1, NT, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (ks == 4) return launch_few_inst<1, NT, 4>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (ks == 2) return launch_few_inst<1, NT, 2>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  return launch_few_inst<1, NT, 1>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+}
 int64_t few_blocks(int64_t T, int64_t N) { return ((N + 31) / 32) * ((T + 63) / 64); }
+// Warps that K is cut over for up to 32 tokens: as many as leave the blocks of 128 / ks weight rows one round on the SMs (three
+// resident blocks each, two with the registers of 16 tokens).  Second product of a pair, with its small first one, in a replayed
+// graph, us, ks = 8 / by this rule: 100 000 outputs, K = 32 at 1, 8, 16 tokens 18.8 / 4.7, 19.0 / 4.8, 30.3 / 7.5; 16 384 outputs, K = 150
+// 6.8 / 3.7, 6.9 / 3.9, 10.2 / 4.8.  Large weights are a matter of bytes in flight, not of rounds, and the whole block on K has the most
+// (up to 8 tokens: 100 000 outputs, K = 1024, 8 tokens 35.7 / 40.3 with ks = 1).
+int few_cut(int64_t T, int64_t N, int64_t K) {
+  if (T <= 8 && K >= 1024 && N * K >= 40000000) return few::kWarps;
+  const int64_t round = (int64_t)num_sms() * (T > 8 && T <= 16 ? 2 : 3);
+  int ks = few::kWarps;
+  while (ks > 1 && (N * ks + 16 * few::kWarps - 1) / (16 * few::kWarps) > round) ks /= 2;
+  return ks;
+}
 int launch_few(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
                int64_t K, bool second, cudaStream_t st) {
   const bf16* a = (const bf16*)A; const bf16* b = (const bf16*)B; bf16* c = (bf16*)C;
   const int t = (int)T, n = (int)N, k = (int)K;
-  if (T <= 8) return launch_few_inst<1, 1>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (T <= 16) return launch_few_inst<1, 2>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (T <= 32) return launch_few_inst<1, 4>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (T <= 8) return launch_few_cut<1>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (T <= 16) return launch_few_cut<2>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (T <= 32) return launch_few_cut<4>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
   // 32 weight rows per block read half as many token rows in all; 16 where 32 would leave half of the SMs idle
-  if (few_blocks(T, N) * 2 >= num_sms()) return launch_few_inst<2, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  return launch_few_inst<1, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  if (few_blocks(T, N) * 2 >= num_sms()) return launch_few_inst<2, 8, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+  return launch_few_inst<1, 8, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
 }
-// Whether a product takes the few-token kernel: up to 32 tokens, and beyond while its 32 x 64 blocks are one round over the
-// SMs.  Both products of a pair in a replayed graph, us, this kernel / tcgen05 tiles: 1024 -> 358 -> 4096 at 16, 64, 128 tokens
+// Whether a product takes the few-token kernel.  Up to 16 tokens always.  Up to 32 unless the weights are wide and large: every
+// group of 16 weight rows reads the tokens again, which a tcgen05 tile of 128 or 256 columns does not (32 tokens, K = 1024, us, this
+// kernel / tcgen05 tiles: 8192 outputs 8.1 / 11.2, 16 384 12.3 / 12.4, 32 768 20.0 / 15.1, 100 000 62.2 / 46.2).  Beyond, while its 32 x 64
+// blocks are one round over the SMs.  Both products of a pair in a replayed graph: 1024 -> 358 -> 4096 at 16, 64, 128 tokens
 // 4.7 / 11.9, 9.2 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024 tokens 16.2 / 26.6; at two rounds
 // it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
 bool few_ok(int64_t T, int64_t N, int64_t K) {
   if (T < 1 || T > 1024 || N > INT32_MAX / 2 || K > INT32_MAX / 2 || tuning().no_few) return false;
-  return T <= 32 || few_blocks(T, N) <= num_sms();
+  if (T <= 16) return true;
+  if (T <= 32) return N < 16384 || N * K < 10000000;
+  return few_blocks(T, N) <= num_sms();
 }
 // Forward product C = (A B^T) * col_scale of a layer, in the form the sizes call for.  `few`: the few-token kernel may serve it.
 int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,

@@ -5,10 +5,12 @@
 // tile spends 7-10 us per launch on its pipeline (barriers, tensor memory, descriptors, a serial walk over K).  What a
 // launch needs is that every byte it reads is requested at once and that many SMs ask.  So
 //   * the weights are the row operand of the warp-level m16n8k16 instruction and the tokens its 8-wide column operand:
-//     a block computes 16 MT weight rows x 8 NT tokens, and small T wastes nothing on the weight side;
-//   * the eight warps of a block cut K into 32-wide steps dealt out in turn, each reading its own part of both operands
-//     straight from global memory into registers: no byte is read twice in a block, nothing is staged or waited for,
-//     and a warp has `kDepth` steps of loads in flight.  The warps' sums are added through shared memory in warp order;
+//     a group of KS warps computes 16 MT weight rows x 8 NT tokens, and small T wastes nothing on the weight side;
+//   * KS of the eight warps of a block cut K into 32-wide steps dealt out in turn, each reading its own part of both operands
+//     straight from global memory into registers: no byte is read twice by them, nothing is staged or waited for,
+//     and a warp has `kDepth` steps of loads in flight.  Their sums are added through shared memory in warp order.  The
+//     8 / KS groups of warps take other weight rows: a narrow output needs all eight on K to fill the machine, a wide one has
+//     rows enough, and with a short K the cut would leave warps without a step (the host picks KS);
 //   * a lane reads 16 contiguous bytes of a row per step: the k positions inside a step are permuted identically for both
 //     operands, so that those bytes serve two instructions without a shuffle;
 //   * with EARLY the first weights are requested before the wait on the previous launch.  That is for the second product of
@@ -48,14 +50,15 @@ __device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, in
 __host__ __device__ constexpr int part_stride(int mt) { return 16 * mt + 4; }   // floats per token of a warp's partial tile: conflict-free writes
 __host__ __device__ constexpr int smem_bytes(int mt, int nt) { return kWarps * 8 * nt * part_stride(mt) * 4; }
 
-template <int MT, int NT, bool EARLY>
+template <int MT, int NT, int KS, bool EARLY>
 __global__ void __launch_bounds__(kThreads)
 gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat16* __restrict__ B, int64_t ldb,
             __nv_bfloat16* __restrict__ C, int64_t ldc, const float* __restrict__ col_scale, int T, int N, int K) {
   constexpr int kDepth = 2 * MT + NT <= 4 ? 4 : 2;         // steps of loads in flight: up to 24 16-byte loads per lane
-  extern __shared__ __align__(16) float part[];            // [kWarps][8 NT][part_stride(MT)]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  const int n0 = blockIdx.x * 16 * MT, t0 = blockIdx.y * 8 * NT;
+  constexpr int kGroups = kWarps / KS;                     // groups of weight rows side by side in the block, KS warps each
+  extern __shared__ __align__(16) float part[];            // [kGroups][KS][8 NT][part_stride(MT)]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3, k_warp = warp % KS;
+  const int n0 = (blockIdx.x * kGroups + warp / KS) * 16 * MT, t0 = blockIdx.y * 8 * NT;
   const __nv_bfloat16* wrow[2 * MT];                       // rows past the end are read from the last row and not stored
   const __nv_bfloat16* trow[NT];
 #pragma unroll
@@ -68,18 +71,18 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
 #pragma unroll
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
-      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * kWarps) * 32 + 8 * q, K);
+      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * KS) * 32 + 8 * q, K);
   };
   if (!EARLY) pdl_wait();
-  load_weights(warp);
+  load_weights(k_warp);
   if (EARLY) pdl_wait();
   pdl_launch_dependents();
-  for (int s = warp; s * 32 < K; s += kDepth * kWarps) {
-    if (s != warp) load_weights(s);
+  for (int s = k_warp; s * 32 < K; s += kDepth * KS) {
+    if (s != k_warp) load_weights(s);
 #pragma unroll
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
-      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * kWarps) * 32 + 8 * q, K);
+      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * KS) * 32 + 8 * q, K);
 #pragma unroll
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
@@ -102,15 +105,15 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
         part[(warp * 8 * NT + 8 * n + 2 * q + (i & 1)) * S + 16 * m + g + (i >> 1) * 8] = acc[m][n][i];
   __syncthreads();
 #pragma unroll
-  for (int e = threadIdx.x; e < 8 * NT * 8 * MT; e += kThreads) {      // two neighbouring columns of one token
-    const int t = e / (8 * MT), c = (e % (8 * MT)) * 2;
+  for (int e = threadIdx.x; e < kGroups * 8 * NT * 8 * MT; e += kThreads) {      // two neighbouring columns of one token
+    const int grp = e / (8 * NT * 8 * MT), t = e / (8 * MT) % (8 * NT), c = (e % (8 * MT)) * 2;
     float x = 0.f, y = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      const float2 v = *reinterpret_cast<const float2*>(part + (w * 8 * NT + t) * S + c);
+    for (int w = 0; w < KS; ++w) {
+      const float2 v = *reinterpret_cast<const float2*>(part + ((grp * KS + w) * 8 * NT + t) * S + c);
       x += v.x; y += v.y;
     }
-    const int n = n0 + c;
+    const int n = (blockIdx.x * kGroups + grp) * 16 * MT + c;
     if (t0 + t < T && n < N) {
       if (col_scale) { x *= __ldg(col_scale + n); if (n + 1 < N) y *= __ldg(col_scale + n + 1); }
       __nv_bfloat16* o = C + (int64_t)(t0 + t) * ldc + n;
