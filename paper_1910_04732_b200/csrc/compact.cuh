@@ -315,7 +315,9 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the k-th largest is found by four 256-bin histogram passes with ONE barrier each (four histograms zeroed up front, every
 // warp searches the bins by itself), and positions come from ballots and one scan over 32-gate words.
 // A warp then takes one row at a time: P rows first (their number is known before the selection, so the rows are
-// prefetched into L2 while the previous launch on the stream still runs), then the surviving rows of Q.  Surviving
+// prefetched into L2 while the previous launch on the stream still runs), then the surviving rows of Q in pieces of at most
+// kFusedPiece elements (a warp per whole row took 45 us for 400 rows of 30 000 bf16, the gather in its own launch 23 with
+// the selection, and in pieces it takes 16).  Surviving
 // columns of P are read straight from global memory, two per lane: neighbouring lanes read neighbouring survivors, so
 // a load touches only a few lines, and a row needs neither staging nor a barrier.
 // Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (three launches each: 13.0 + 4.0 + 5.8 us
@@ -326,6 +328,8 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
 constexpr int kFusedMaxR = 1024;
 constexpr int64_t kFusedMaxBytes = 16 << 20;
+constexpr int kFusedPiece = 4096;
+inline int fused_pieces(int64_t d_in) { return (int)((d_in + kFusedPiece - 1) / kFusedPiece); }   // of a row of Q
 constexpr int kFusedThreads = 512, kFusedWarps = kFusedThreads / 32;
 
 template <typename T> struct alignas(2 * sizeof(T)) Pair2 { T e[2]; };
@@ -336,7 +340,7 @@ template <typename T>
 __global__ void __launch_bounds__(kFusedThreads)
 compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, int32_t* __restrict__ idx, int32_t* __restrict__ k_dev,
                      float* __restrict__ z_det, const T* __restrict__ P, int64_t ldp, const T* __restrict__ Q, int64_t ldq, int d_in,
-                     int d_out, T* __restrict__ Pc, int64_t ldpc, T* __restrict__ Qc, int64_t ldqc, int vec_q, int pair_p) {
+                     int d_out, T* __restrict__ Pc, int64_t ldpc, T* __restrict__ Qc, int64_t ldqc, int vec_q, int pair_p, int pieces) {
   constexpr int kWords = kKeys * kFusedWarps;
   constexpr int kWordsPerLane = (kWords + 31) / 32;
   __shared__ __align__(16) int hist[4][256];
@@ -488,7 +492,8 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
   __syncthreads();
 
   constexpr int V = Vec16<T>::n;
-  for (int t = my_warp; t < d_out + (d_in > 0 ? k : 0); t += warps) {
+  const int piece = ((d_in + max(pieces, 1) - 1) / max(pieces, 1) + 63) & ~63;
+  for (int t = my_warp; t < d_out + k * pieces; t += warps) {
     if (t < d_out) {                       // Pc[t, :] = P[t, idx]
       const T* p = P + (int64_t)t * ldp;
       T* o = Pc + (int64_t)t * ldpc;
@@ -509,20 +514,20 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
         for (int c = lane; c < k; c += 32) o[c] = p[s_idx[c]];
       }
     } else {                               // Qc[c, :] = z[idx[c]] * Q[idx[c], :]
-      const int c = t - d_out;
+      const int c = (t - d_out) / pieces, j0 = (t - d_out - c * pieces) * piece, j1 = min(d_in, j0 + piece);
       const float g = s_z[c];
       const T* q = Q + (int64_t)s_idx[c] * ldq;
       T* o = Qc + (int64_t)c * ldqc;
-      const int full = vec_q ? d_in / V * V : 0;
+      const int full = vec_q ? j1 / V * V : j0;
 #pragma unroll 4
-      for (int j = lane * V; j < full; j += 32 * V) {
+      for (int j = j0 + lane * V; j < full; j += 32 * V) {
         uint4 raw = *reinterpret_cast<const uint4*>(q + j);
         T* e = reinterpret_cast<T*>(&raw);
 #pragma unroll
         for (int i = 0; i < V; ++i) e[i] = from_f32<T>(to_f32<T>(e[i]) * g);
         *reinterpret_cast<uint4*>(o + j) = raw;
       }
-      for (int j = full + lane; j < d_in; j += 32) o[j] = from_f32<T>(to_f32<T>(q[j]) * g);
+      for (int j = max(full, j0) + lane; j < j1; j += 32) o[j] = from_f32<T>(to_f32<T>(q[j]) * g);
     }
   }
 }

@@ -41,3 +41,26 @@ def test_mask_and_compact_factors(b, r, dtype, odd_ld, ties):
     if k:      # one rounding of each product to 8 (bf16) or 24 (fp32) significant bits: at most 2^-8 or 2^-24 relative
         assert np.all(np.abs(host(Qc)[:k] - Qco) <= (2.0 ** -8 if dtype == "bf16" else 2.0 ** -24) * np.abs(Qco))
     assert b.device_status() == b.OK
+
+
+@pytest.mark.parametrize("d_in", [4095, 4096, 4097, 8193, 30001])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("odd_ld", [False, True])
+def test_rows_of_q_in_pieces(b, d_in, dtype, odd_ld):
+    """Rows longer than 4096 elements are gathered in pieces; with and without 16-byte vectors."""
+    g = np.random.default_rng(d_in)
+    r, d_out, tdt = 100, 5, torch.bfloat16 if dtype == "bf16" else torch.float32
+    z = np.where(g.random(r) < 0.4, g.uniform(0.05, 1.0, r), 0.0).astype(np.float32)
+    P, Q = to_dev(g.standard_normal((d_out, r)), dtype), to_dev(g.standard_normal((r, d_in)), dtype)
+    Pc, Qc = empty_dev(d_out, r, tdt), torch.full((r, d_in + (9 if odd_ld else 24)), float("nan"), dtype=tdt, device="cuda")[:, :d_in]
+    if not odd_ld:
+        Qc = empty_dev(r, d_in, tdt)
+    idx, kd = torch.full((r,), -1, dtype=torch.int32, device="cuda"), torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    b.compact_ranks(torch.from_numpy(z).cuda(), 1, HC, idx, kd, None, P, Q, Pc, Qc)
+    k, idxo = O.active_ranks(z)
+    assert int(kd.item()) == k and np.array_equal(idx.cpu().numpy()[:k], idxo)
+    Pco, Qco = O.compact_ranks(host(P), host(Q), idxo, z.astype(np.float64))
+    got = host(Qc)
+    assert np.array_equal(host(Pc)[:, :k], Pco) and np.all(np.isnan(got[k:]))
+    assert np.all(np.abs(got[:k] - Qco) <= (2.0 ** -8 if dtype == "bf16" else 2.0 ** -24) * np.abs(Qco))      # one rounding of each product
+    assert b.device_status() == b.OK
