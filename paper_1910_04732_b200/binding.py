@@ -17,6 +17,8 @@ from typing import Optional
 
 import torch
 
+from . import build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libflop_b200.so")
 
@@ -162,7 +164,7 @@ def _native():
     global _native_module
     if _native_module is None:
         load_library()
-        path = os.path.join(_HERE, "_binding_native.so")
+        path = build.native_path()
         if not os.path.exists(path):
             raise RuntimeError(f"{path} is missing: build it with `python -m paper_1910_04732_b200.build` "
                                "(there is no CPU fallback)")

@@ -59,3 +59,12 @@ def test_accumulate_is_an_integer(accumulate, adds):
 def test_accumulate_that_is_no_integer_is_refused():
     with pytest.raises(TypeError):
         b.gated_lowrank_bwd(X, X, X, X, None, None, X, None, None, None, None, None, None)
+
+
+def test_a_module_of_another_torch_is_not_loaded(monkeypatch):
+    assert build.native_up_to_date()
+    monkeypatch.setattr(torch, "__version__", "0.0.0+other")
+    monkeypatch.setattr(b, "_native_module", None)
+    assert not build.native_up_to_date()
+    with pytest.raises(RuntimeError, match="0.0.0"):
+        b._native()
