@@ -86,12 +86,18 @@ flop_hc_params_t hard_concrete(PyObject* o) {
 void* stream() { return (void*)c10::cuda::getCurrentCUDAStream().stream(); }
 size_t numel(PyObject* o) { const at::Tensor* t = tensor(o); return t ? (size_t)t->numel() : 0; }
 
-// Runs the library call without the interpreter lock and returns its status as a Python integer.
+// Runs the library call without the interpreter lock and returns its status as a Python integer.  The lock is back before an
+// exception (the library's planners allocate on the host) leaves the call and becomes a Python one.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
 template <typename F> PyObject* call(F&& f) {
   int status;
-  Py_BEGIN_ALLOW_THREADS
-  status = f();
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked u;
+    status = f();
+  }
   return PyLong_FromLong(status);
 }
 
