@@ -7,7 +7,7 @@
 //   embed_finish_kernel : dlog_alpha from the per-block partial sums, and dO from the split-K slices of its GEMM
 //
 // The two token kernels are bound by the latency of a chain: token -> row of E -> store or atomic add.  A warp
-// therefore takes kEmbTokens tokens at once and has all their ids, then all their rows in flight before it uses the first;
+// therefore takes four tokens at once and has all their ids, then all their rows in flight before it uses the first;
 // rows narrower than 32 pieces of 8 columns share the warp (LPT lanes per token), so that no lane idles at
 // 64 or 128 columns.  Walking eight tokens one after another, one warp per SM scheduler, took 33.5 us for 16 384 tokens of
 // 256 columns, and adding up 256 partial vectors by one thread per column another 17 us.
@@ -18,14 +18,15 @@
 namespace flop {
 
 constexpr int kEmbWarps = 8;
-constexpr int kEmbTokens = 4;   // tokens a warp has in flight (per lane group)
 // Tokens of a backward block.  Fixed for every width, so that the partial sums (one vector per block) have one size.
 constexpr int kEmbBlockTokens = 32;
 
 // Lanes that share a token's row: 8 columns per lane and pass.
 inline int embed_lanes(int64_t d_i) { return d_i <= 64 ? 8 : d_i <= 128 ? 16 : 32; }
 
-template <int LPT>
+// TOK: tokens a lane group has in flight.  Few tokens are spread over the SMs instead, one per lane group (32 tokens of 2048 columns and
+// the product after it: 15.8 us, 17.5 with four).
+template <int LPT, int TOK>
 __global__ void __launch_bounds__(32 * kEmbWarps)
 embed_gather_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __restrict__ E, int64_t lde, int n_rows,
                     const float* __restrict__ z, int d_i, __nv_bfloat16* __restrict__ H, int64_t ldh) {
@@ -33,21 +34,21 @@ embed_gather_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16*
   pdl_launch_dependents();
   constexpr int G = 32 / LPT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPT, l = lane % LPT;
-  const int t0 = (blockIdx.x * kEmbWarps + warp) * (kEmbTokens * G) + grp;       // this lane group: t0, t0 + G, ...
-  int w[kEmbTokens];
+  const int t0 = (blockIdx.x * kEmbWarps + warp) * (TOK * G) + grp;       // this lane group: t0, t0 + G, ...
+  int w[TOK];
 #pragma unroll
-  for (int i = 0; i < kEmbTokens; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;   // out-of-range ids are clamped, never dereferenced
+  for (int i = 0; i < TOK; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;   // out-of-range ids are clamped, never dereferenced
   for (int k = l * 8; k < d_i; k += LPT * 8) {
     if (k + 8 <= d_i) {
-      uint4 raw[kEmbTokens];
+      uint4 raw[TOK];
 #pragma unroll
-      for (int i = 0; i < kEmbTokens; ++i)
+      for (int i = 0; i < TOK; ++i)
         if (t0 + i * G < T) raw[i] = *reinterpret_cast<const uint4*>(E + (int64_t)w[i] * lde + k);
       float zk[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) zk[j] = __ldg(z + k + j);
 #pragma unroll
-      for (int i = 0; i < kEmbTokens; ++i) {
+      for (int i = 0; i < TOK; ++i) {
         if (t0 + i * G < T) {
           __nv_bfloat16* v = reinterpret_cast<__nv_bfloat16*>(&raw[i]);
 #pragma unroll
@@ -56,7 +57,7 @@ embed_gather_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16*
         }
       }
     } else {
-      for (int i = 0; i < kEmbTokens; ++i)
+      for (int i = 0; i < TOK; ++i)
         if (t0 + i * G < T)
           for (int j = k; j < d_i; ++j)
             H[(int64_t)(t0 + i * G) * ldh + j] = __float2bfloat16_rn(__bfloat162float(E[(int64_t)w[i] * lde + j]) * z[j]);
@@ -83,15 +84,20 @@ embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPT, l = lane % LPT;
   const int t0 = blockIdx.x * kEmbBlockTokens + warp * (kIn * G) + grp;
   const bool vec_de = dE && (reinterpret_cast<uintptr_t>(dE) & 15) == 0 && (ldde % 4) == 0;
+  const bool live = blockIdx.x * kEmbBlockTokens + warp * (kIn * G) < T;   // warps past the last token have nothing to add
+  if (!live)
+    for (int k = lane; k < d_i; k += 32) red[warp * d_i + k] = 0.f;
   int w[kIn];
 #pragma unroll
   for (int i = 0; i < kIn; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;
-  for (int k0 = 0; k0 < d_i; k0 += LPT * 8) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int k0 = 0; live && k0 < d_i; k0 += LPT * 8) {
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, zk[2][4];
     uint2 graw[2][kIn], eraw[2][kIn];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int k = k0 + h * (LPT * 4) + l * 4;                      // rows of dH' and E are 16-byte aligned (ld % 8 == 0)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) zk[h][j] = k + 4 <= d_i ? __ldg(z + k + j) : 0.f;
 #pragma unroll
       for (int i = 0; i < kIn; ++i) {
         graw[h][i] = eraw[h][i] = make_uint2(0, 0);
@@ -105,9 +111,6 @@ embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __
     for (int h = 0; h < 2; ++h) {
       const int k = k0 + h * (LPT * 4) + l * 4, nk = min(4, d_i - k);   // nk <= 0: no column for this lane here
       if (nk == 4) {
-        float zk[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) zk[j] = __ldg(z + k + j);
 #pragma unroll
         for (int i = 0; i < kIn; ++i) {
           const __nv_bfloat162* gh = reinterpret_cast<const __nv_bfloat162*>(&graw[h][i]);
@@ -119,13 +122,13 @@ embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __
           acc[4 * h + 3] = fmaf(e1.y, g1.y, acc[4 * h + 3]);
           if (dE && t0 + i * G < T) {
             float* o = dE + (int64_t)w[i] * ldde + k;
-            const float d[4] = {g0.x * zk[0], g0.y * zk[1], g1.x * zk[2], g1.y * zk[3]};
+            const float d[4] = {g0.x * zk[h][0], g0.y * zk[h][1], g1.x * zk[h][2], g1.y * zk[h][3]};
             if (vec_de) {
               atomicAdd(reinterpret_cast<float4*>(o), make_float4(d[0], d[1], d[2], d[3]));
             } else {
 #pragma unroll
               for (int j = 0; j < 4; ++j)
-                if (zk[j] != 0.f) atomicAdd(o + j, d[j]);
+                if (zk[h][j] != 0.f) atomicAdd(o + j, d[j]);
             }
           }
         }

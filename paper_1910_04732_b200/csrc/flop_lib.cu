@@ -1068,8 +1068,9 @@ static int64_t embedding_blocks(int64_t T) { return (T + kEmbBlockTokens - 1) / 
 template <int LPT>
 static void launch_embed_gather(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
                                 void* H, int64_t ldh, cudaStream_t st) {
-  constexpr int per_block = kEmbWarps * kEmbTokens * (32 / LPT);
-  launch_k(embed_gather_kernel<LPT>, dim3((unsigned)((T + per_block - 1) / per_block)), dim3(32 * kEmbWarps), (size_t)0, st, ids, (int)T,
+  const int64_t groups = kEmbWarps * (32 / LPT), tokens = T <= groups * num_sms() ? 1 : 4;   // one round of blocks, or four tokens in flight
+  const dim3 grid((unsigned)((T + groups * tokens - 1) / (groups * tokens)));
+  launch_k(tokens == 1 ? embed_gather_kernel<LPT, 1> : embed_gather_kernel<LPT, 4>, grid, dim3(32 * kEmbWarps), (size_t)0, st, ids, (int)T,
            (const bf16*)E, lde, (int)n_rows, z, (int)d_i, (bf16*)H, ldh);
 }
 template <int LPT>

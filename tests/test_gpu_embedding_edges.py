@@ -51,3 +51,20 @@ def test_widths_and_token_counts(b, d_i, T, d, wdt, accumulate):
     assert rel_fro(host(dE), want) < 4e-3                                            # dH' is rounded to bf16 before it is summed
     size = np.sum(np.abs(Eh[idn] * dH), axis=0) * host(dz)
     assert np.all(np.abs(host(dla) - (np.sum(Eh[idn] * dH, axis=0) * host(dz) + off)) <= 2.0 ** -7 * size + 1e-6)
+
+
+@pytest.mark.parametrize("d_i,line", [(40, 4736), (100, 2368), (300, 1184), (2048, 1184)])
+@pytest.mark.parametrize("over", [0, 1])
+def test_lookup_on_both_sides_of_one_round(b, d_i, line, over):
+    """One token per lane group while that is one round of blocks over 148 SMs, four in flight beyond: one rounding to 8 bits."""
+    T, n_rows, d = line + over, 70, 24
+    g = np.random.default_rng(T)
+    E, Om = to_dev(g.standard_normal((n_rows, d_i)), "bf16"), to_dev(g.standard_normal((d_i, d)) / np.sqrt(d_i), "bf16")
+    ids = torch.from_numpy(g.integers(-3, n_rows + 3, T).astype(np.int32)).cuda()
+    z = torch.from_numpy(g.uniform(0.2, 1.0, d_i).astype(np.float32)).cuda()
+    Y, H = empty_dev(T, d, torch.bfloat16), empty_dev(T, d_i, torch.bfloat16)
+    b.gated_embedding_fwd(ids, E, Om, z, Y, H)
+    rows = host(E)[np.clip(ids.cpu().numpy(), 0, n_rows - 1)] * host(z)
+    assert np.all(np.abs(host(H) - rows) <= 2.0 ** -8 * np.abs(rows))
+    assert_close(Y, host(H) @ host(Om), "bf16", "Y")
+    assert b.device_status() == b.OK
