@@ -1483,7 +1483,10 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     const flop_bwd_problem_t one{dY, lddy, X, ldx, Q, ldq, P, ldp, z, dz_dla, H_save, ldh, dX, lddx, dP, lddp, dQ, lddq, dlog_alpha,
                                  T, d_in, d_out, r, ws, ws_bytes, nullptr, nullptr, 0, 0};
     Arena grouped{nullptr, 0, 0};
-    if (plan_merged(&one, 1).cycles < separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes &&
+    // Without dP or dX the shared form saves one launch or none, and gives up the split: the estimate has to be clearly lower
+    // (768 -> 3072 at 4096 tokens, dX and dlog_alpha: a launch per product 55 us, shared 65, estimated at 51 and 49).
+    const double margin = need_m && !(dP && dX) ? 0.84 : 1.0;
+    if (plan_merged(&one, 1).cycles < margin * separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes &&
         merged_apart(&one, 1, wgrad_dt))
       return bwd_grouped_impl(&one, 1, accumulate, dt, wgrad_dt, nullptr, 0, stream, separate);
   }
@@ -1745,7 +1748,8 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
           if (a.dQ || a.dlog_alpha) { q.add(a.r, a.d_in, a.T, wss[i].plan_q); slice_bytes += 8.0 * wss[i].plan_q.splits * a.r * a.d_in; }
           if (a.dX) x.add(a.T, a.d_in, a.r, s6.bn);
         }
-        single_cycles = h.cycles() + p.cycles() + q.cycles() + x.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0;
+        // 0.96: level estimates go to the launches per product (six matrices 256 -> 256 at 9000 tokens: 92 us, shared 104, estimated at 0.98)
+        single_cycles = 0.96 * (h.cycles() + p.cycles() + q.cycles() + x.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0);
       }
     }
     if (mg.cycles >= single_cycles) { direct = false; mg.bn_h = 0; }
