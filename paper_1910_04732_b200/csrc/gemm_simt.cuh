@@ -122,8 +122,7 @@ gemm_kernel(const SimtGemmArgs p) {
     const float* As = smem + (kb % kStages) * kStageFloats;
     const float* Bs = As + kOperandFloats;
     const float* Zs = Bs + kOperandFloats;
-#pragma unroll
-    for (int k = 0; k < BK; k += 4) {
+    auto multiply = [&](int k) {
       float a[4][4], b[4][4];                              // [row or column of the thread][k]
       if (A_K) {
 #pragma unroll
@@ -156,6 +155,13 @@ gemm_kernel(const SimtGemmArgs p) {
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i][c], b[j][c], acc[i][j]);
+    };
+    if (kb * BK + BK <= p.K) {
+#pragma unroll
+      for (int k = 0; k < BK; k += 4) multiply(k);
+    } else {                                               // the zeros beyond K need no FMAs (K = 33: 36 of 64 steps are left)
+#pragma unroll 1
+      for (int k = 0; kb * BK + k < p.K; k += 4) multiply(k);
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
