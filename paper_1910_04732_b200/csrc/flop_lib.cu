@@ -968,10 +968,11 @@ struct BwdWs {
   TcPlan plan_p, plan_q;
   size_t bytes;
 };
-BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, int dt, bool grouped = false) {
+BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, int dt, bool grouped = false, bool tight = false) {
   BwdWs w{};
-  // rows of dH' start on 128-byte lines: a TMA box row is 128 bytes, and one that straddles two lines costs two L2 requests
-  w.lddh = round_up(std::max<int64_t>(r, 1), dt == FLOP_BF16 ? 64 : 8);
+  // rows of dH' start on 128-byte lines: a TMA box row is 128 bytes, and one that straddles two lines costs two L2 requests.
+  // `tight`: on 16-byte pieces, for a workspace that has no room for the lines.
+  w.lddh = round_up(std::max<int64_t>(r, 1), dt == FLOP_BF16 && !tight ? 64 : 8);
   w.dH = ar.take((size_t)T * w.lddh * elt(dt));
   w.ldqz = round_up(std::max<int64_t>(d_in, 1), 8);
   w.Qz = dt == FLOP_BF16 ? ar.take((size_t)r * w.ldqz * 2) : nullptr;
@@ -999,17 +1000,27 @@ BwdWs plan_bwd_ws(Arena& ar, int64_t T, int64_t d_in, int64_t d_out, int64_t r, 
   return w;
 }
 
-size_t l0_ws_bytes(int64_t n, int64_t n_seg) {
-  const int64_t chunks = (n + kL0Chunk - 1) / kL0Chunk + n_seg;
-  return sizeof(L0Scratch) + (size_t)std::max<int64_t>(chunks, 1) * sizeof(double);
-}
-
 int check_ws(const void* ws, size_t ws_bytes, size_t need) {
   if (need == 0) return FLOP_OK;
   if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255) != 0 || ws_bytes < need) return FLOP_ERR_WORKSPACE;
   return FLOP_OK;
 }
 
+// The layout in the caller's workspace: the one the query sizes, or the tight one where only that fits.
+int place_bwd_ws(BwdWs& w, void* ws, size_t ws_bytes, int64_t T, int64_t d_in, int64_t d_out, int64_t r, int dt, bool grouped) {
+  Arena ar{(unsigned char*)ws, ws_bytes, 0};
+  w = plan_bwd_ws(ar, T, d_in, d_out, r, dt, grouped);
+  if (ws_bytes < w.bytes) {
+    ar.used = 0;
+    w = plan_bwd_ws(ar, T, d_in, d_out, r, dt, grouped, true);
+  }
+  return check_ws(ws, ws_bytes, w.bytes);
+}
+
+size_t l0_ws_bytes(int64_t n, int64_t n_seg) {
+  const int64_t chunks = (n + kL0Chunk - 1) / kL0Chunk + n_seg;
+  return sizeof(L0Scratch) + (size_t)std::max<int64_t>(chunks, 1) * sizeof(double);
+}
 
 // ------------------------------------------------------------------ built-in scratch (no-allocation entry point)
 // Scratch of flop_expected_l0_lagrangian_noalloc: a fixed device array that is part of the
@@ -1461,10 +1472,8 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     }
     return FLOP_OK;
   }
-  Arena probe{nullptr, 0, 0};
-  FLOP_TRY(check_ws(ws, ws_bytes, plan_bwd_ws(probe, T, d_in, d_out, r, dt).bytes));
-  Arena ar{(unsigned char*)ws, ws_bytes, 0};
-  const BwdWs w = plan_bwd_ws(ar, T, d_in, d_out, r, dt);
+  BwdWs w;
+  FLOP_TRY(place_bwd_ws(w, ws, ws_bytes, T, d_in, d_out, r, dt, false));
   const bool need_m = dQ || dlog_alpha;   // M = dH'^T X feeds both dQ and dz
 
   if (dt == FLOP_BF16 && (!dP || wgrad_direct_ok(dP, lddp, wgrad_dt)) && (!dQ || wgrad_direct_ok(dQ, lddq, wgrad_dt)) &&
@@ -1486,7 +1495,7 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     // Without dP or dX the shared form saves one launch or none, and gives up the split: the estimate has to be clearly lower
     // (768 -> 3072 at 4096 tokens, dX and dlog_alpha: a launch per product 55 us, shared 65, estimated at 51 and 49).
     const double margin = need_m && !(dP && dX) ? 0.84 : 1.0;
-    if (plan_merged(&one, 1).cycles < margin * separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true).bytes &&
+    if (plan_merged(&one, 1).cycles < margin * separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true, true).bytes &&
         merged_apart(&one, 1, wgrad_dt))
       return bwd_grouped_impl(&one, 1, accumulate, dt, wgrad_dt, nullptr, 0, stream, separate);
   }
@@ -1709,10 +1718,8 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
     if ((a.dX && !bf16_ok(a.dX, a.lddx)) || !bf16_ok(a.dY, a.lddy) || !bf16_ok(a.X, a.ldx) || !bf16_ok(a.Q, a.ldq) ||
         !bf16_ok(a.P, a.ldp) || !bf16_ok(a.H_save, a.ldh) || (a.Qz && !bf16_ok(a.Qz, a.ldqz)))
       return FLOP_ERR_UNSUPPORTED;
-    Arena probe{nullptr, 0, 0};
-    FLOP_TRY(check_ws(a.ws, a.ws_bytes, plan_bwd_ws(probe, a.T, a.d_in, a.d_out, a.r, dt, true).bytes));
-    Arena ar{(unsigned char*)a.ws, a.ws_bytes, 0};
-    wss.push_back(plan_bwd_ws(ar, a.T, a.d_in, a.d_out, a.r, dt, true));
+    wss.emplace_back();
+    FLOP_TRY(place_bwd_ws(wss.back(), a.ws, a.ws_bytes, a.T, a.d_in, a.d_out, a.r, dt, true));
     if ((a.dP && !wgrad_direct_ok(a.dP, a.lddp, wgrad_dt)) || (a.dQ && !wgrad_direct_ok(a.dQ, a.lddq, wgrad_dt))) direct = false;
   }
   // One tile shape per stage for all problems of the call.  The weight gradients go direct when
@@ -1971,10 +1978,8 @@ int flop_dlog_alpha_finish_grouped(const flop_bwd_problem_t* pr, int n, int accu
       DlaFinish& o = g.a[g.n];
       if (!a.dlog_alpha || a.T == 0 || a.r == 0 || a.d_in == 0 || a.d_out == 0) { o.r = 0; continue; }
       if (!a.dz_dla) return FLOP_ERR_INVALID_ARG;
-      Arena probe{nullptr, 0, 0};
-      FLOP_TRY(check_ws(a.ws, a.ws_bytes, plan_bwd_ws(probe, a.T, a.d_in, a.d_out, a.r, dt, true).bytes));
-      Arena ar{(unsigned char*)a.ws, a.ws_bytes, 0};
-      const BwdWs w = plan_bwd_ws(ar, a.T, a.d_in, a.d_out, a.r, dt, true);
+      BwdWs w;
+      FLOP_TRY(place_bwd_ws(w, a.ws, a.ws_bytes, a.T, a.d_in, a.d_out, a.r, dt, true));
       o.dz_part = w.dz_part; o.n_part = w.dz_meta; o.cap = (int)std::max<int64_t>(w.n_part, 2 * ((a.d_in + 63) / 64));
       o.dz_dla = a.dz_dla; o.dla = a.dlog_alpha; o.r = (int)a.r;
       max_r = std::max(max_r, o.r);
