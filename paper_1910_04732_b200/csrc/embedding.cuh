@@ -65,7 +65,7 @@ embed_gather_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16*
   }
 }
 
-// Block b handles tokens [b * 32, b * 32 + 32).  A lane owns two groups of 4 consecutive columns of every LPT * 8 columns, LPT * 4
+// Block b handles `runs` x 32 consecutive tokens: one run, or two where the workspace holds half as many partial sums.  A lane owns two groups of 4 consecutive columns of every LPT * 8 columns, LPT * 4
 // apart, so that a 16-byte vector atomic add of the warp covers 512 contiguous bytes of a row of dE: with 8 consecutive columns
 // per lane every 32-byte sector was visited twice, by half each time, and the atomic units of the L2 bound the kernel
 // (30.6 us for 16 384 tokens of 256 columns, about 19 now).  The lane groups' and the warps' partial sums of dz are added in a fixed order (shuffles, then shared
@@ -74,7 +74,7 @@ template <int LPT>
 __global__ void __launch_bounds__(32 * kEmbWarps)
 embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __restrict__ E, int64_t lde, int n_rows,
                  const float* __restrict__ z, int d_i, const __nv_bfloat16* __restrict__ dH, int64_t lddh,
-                 float* __restrict__ dE, int64_t ldde, float* __restrict__ part) {
+                 float* __restrict__ dE, int64_t ldde, float* __restrict__ part, int runs) {
   pdl_wait();
   pdl_launch_dependents();
   extern __shared__ float red[];   // [kEmbWarps][d_i]
@@ -82,76 +82,80 @@ embed_bwd_kernel(const int32_t* __restrict__ ids, int T, const __nv_bfloat16* __
   constexpr int kIn = kEmbBlockTokens / kEmbWarps / G > 0 ? kEmbBlockTokens / kEmbWarps / G : 1;   // ... and one after another, in flight together
   static_assert(kIn * G * kEmbWarps == kEmbBlockTokens, "a block's tokens are dealt out evenly");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPT, l = lane % LPT;
-  const int t0 = blockIdx.x * kEmbBlockTokens + warp * (kIn * G) + grp;
   const bool vec_de = dE && (reinterpret_cast<uintptr_t>(dE) & 15) == 0 && (ldde % 4) == 0;
-  const bool live = blockIdx.x * kEmbBlockTokens + warp * (kIn * G) < T;   // warps past the last token have nothing to add
-  if (!live)
-    for (int k = lane; k < d_i; k += 32) red[warp * d_i + k] = 0.f;
-  int w[kIn];
-#pragma unroll
-  for (int i = 0; i < kIn; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;
-  for (int k0 = 0; live && k0 < d_i; k0 += LPT * 8) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, zk[2][4];
-    uint2 graw[2][kIn], eraw[2][kIn];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = k0 + h * (LPT * 4) + l * 4;                      // rows of dH' and E are 16-byte aligned (ld % 8 == 0)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) zk[h][j] = k + 4 <= d_i ? __ldg(z + k + j) : 0.f;
-#pragma unroll
-      for (int i = 0; i < kIn; ++i) {
-        graw[h][i] = eraw[h][i] = make_uint2(0, 0);
-        if (k + 4 <= d_i && t0 + i * G < T) {
-          graw[h][i] = __ldcs(reinterpret_cast<const uint2*>(dH + (int64_t)(t0 + i * G) * lddh + k));
-          eraw[h][i] = *reinterpret_cast<const uint2*>(E + (int64_t)w[i] * lde + k);
-        }
-      }
+  for (int run = 0; run < runs; ++run) {
+    const int first = (blockIdx.x * runs + run) * kEmbBlockTokens + warp * (kIn * G), t0 = first + grp;
+    if (first >= T) {              // warps past the last token have nothing to add
+      if (run == 0)
+        for (int k = lane; k < d_i; k += 32) red[warp * d_i + k] = 0.f;
+      break;
     }
+    int w[kIn];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = k0 + h * (LPT * 4) + l * 4, nk = min(4, d_i - k);   // nk <= 0: no column for this lane here
-      if (nk == 4) {
+    for (int i = 0; i < kIn; ++i) w[i] = t0 + i * G < T ? min(max(ids[t0 + i * G], 0), n_rows - 1) : 0;
+    for (int k0 = 0; k0 < d_i; k0 += LPT * 8) {
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, zk[2][4];
+      uint2 graw[2][kIn], eraw[2][kIn];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + h * (LPT * 4) + l * 4;                      // rows of dH' and E are 16-byte aligned (ld % 8 == 0)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) zk[h][j] = k + 4 <= d_i ? __ldg(z + k + j) : 0.f;
 #pragma unroll
         for (int i = 0; i < kIn; ++i) {
-          const __nv_bfloat162* gh = reinterpret_cast<const __nv_bfloat162*>(&graw[h][i]);
-          const __nv_bfloat162* eh = reinterpret_cast<const __nv_bfloat162*>(&eraw[h][i]);
-          const float2 g0 = __bfloat1622float2(gh[0]), g1 = __bfloat1622float2(gh[1]), e0 = __bfloat1622float2(eh[0]), e1 = __bfloat1622float2(eh[1]);
-          acc[4 * h] = fmaf(e0.x, g0.x, acc[4 * h]);
-          acc[4 * h + 1] = fmaf(e0.y, g0.y, acc[4 * h + 1]);
-          acc[4 * h + 2] = fmaf(e1.x, g1.x, acc[4 * h + 2]);
-          acc[4 * h + 3] = fmaf(e1.y, g1.y, acc[4 * h + 3]);
-          if (dE && t0 + i * G < T) {
-            float* o = dE + (int64_t)w[i] * ldde + k;
-            const float d[4] = {g0.x * zk[h][0], g0.y * zk[h][1], g1.x * zk[h][2], g1.y * zk[h][3]};
-            if (vec_de) {
-              atomicAdd(reinterpret_cast<float4*>(o), make_float4(d[0], d[1], d[2], d[3]));
-            } else {
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (zk[h][j] != 0.f) atomicAdd(o + j, d[j]);
-            }
-          }
-        }
-      } else if (nk > 0) {
-        for (int i = 0; i < kIn; ++i) {
-          const int t = t0 + i * G;
-          if (t >= T) break;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            if (j < nk) {
-              const float gj = __bfloat162float(dH[(int64_t)t * lddh + k + j]), zj = z[k + j];
-              acc[4 * h + j] = fmaf(__bfloat162float(E[(int64_t)w[i] * lde + k + j]), gj, acc[4 * h + j]);
-              if (dE && zj != 0.f) atomicAdd(dE + (int64_t)w[i] * ldde + k + j, gj * zj);
-            }
+          graw[h][i] = eraw[h][i] = make_uint2(0, 0);
+          if (k + 4 <= d_i && t0 + i * G < T) {
+            graw[h][i] = __ldcs(reinterpret_cast<const uint2*>(dH + (int64_t)(t0 + i * G) * lddh + k));
+            eraw[h][i] = *reinterpret_cast<const uint2*>(E + (int64_t)w[i] * lde + k);
           }
         }
       }
 #pragma unroll
-      for (int o = LPT; o < 32; o <<= 1)
+      for (int h = 0; h < 2; ++h) {
+        const int k = k0 + h * (LPT * 4) + l * 4, nk = min(4, d_i - k);   // nk <= 0: no column for this lane here
+        if (nk == 4) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[4 * h + j] += __shfl_xor_sync(0xffffffffu, acc[4 * h + j], o);
-      if (grp == 0)
-        for (int j = 0; j < nk; ++j) red[warp * d_i + k + j] = acc[4 * h + j];
+          for (int i = 0; i < kIn; ++i) {
+            const __nv_bfloat162* gh = reinterpret_cast<const __nv_bfloat162*>(&graw[h][i]);
+            const __nv_bfloat162* eh = reinterpret_cast<const __nv_bfloat162*>(&eraw[h][i]);
+            const float2 g0 = __bfloat1622float2(gh[0]), g1 = __bfloat1622float2(gh[1]), e0 = __bfloat1622float2(eh[0]), e1 = __bfloat1622float2(eh[1]);
+            acc[4 * h] = fmaf(e0.x, g0.x, acc[4 * h]);
+            acc[4 * h + 1] = fmaf(e0.y, g0.y, acc[4 * h + 1]);
+            acc[4 * h + 2] = fmaf(e1.x, g1.x, acc[4 * h + 2]);
+            acc[4 * h + 3] = fmaf(e1.y, g1.y, acc[4 * h + 3]);
+            if (dE && t0 + i * G < T) {
+              float* o = dE + (int64_t)w[i] * ldde + k;
+              const float d[4] = {g0.x * zk[h][0], g0.y * zk[h][1], g1.x * zk[h][2], g1.y * zk[h][3]};
+              if (vec_de) {
+                atomicAdd(reinterpret_cast<float4*>(o), make_float4(d[0], d[1], d[2], d[3]));
+              } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  if (zk[h][j] != 0.f) atomicAdd(o + j, d[j]);
+              }
+            }
+          }
+        } else if (nk > 0) {
+          for (int i = 0; i < kIn; ++i) {
+            const int t = t0 + i * G;
+            if (t >= T) break;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+              if (j < nk) {
+                const float gj = __bfloat162float(dH[(int64_t)t * lddh + k + j]), zj = z[k + j];
+                acc[4 * h + j] = fmaf(__bfloat162float(E[(int64_t)w[i] * lde + k + j]), gj, acc[4 * h + j]);
+                if (dE && zj != 0.f) atomicAdd(dE + (int64_t)w[i] * ldde + k + j, gj * zj);
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int o = LPT; o < 32; o <<= 1)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[4 * h + j] += __shfl_xor_sync(0xffffffffu, acc[4 * h + j], o);
+        if (grp == 0)
+          for (int j = 0; j < nk; ++j) red[warp * d_i + k + j] = (run ? red[warp * d_i + k + j] : 0.f) + acc[4 * h + j];
+      }
     }
   }
   __syncthreads();

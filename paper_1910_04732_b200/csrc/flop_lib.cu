@@ -1075,7 +1075,8 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
 static size_t embedding_slice_bytes(int64_t T, int64_t d_i) {
   return (size_t)std::min<int64_t>(64ll << 20, T * round_up(std::max<int64_t>(d_i, 1), 8) * 8);
 }
-static int64_t embedding_blocks(int64_t T) { return (T + kEmbBlockTokens - 1) / kEmbBlockTokens; }
+// Blocks of the token kernel, and vectors of partial sums; runs: 32-token runs per block.
+static int64_t embedding_blocks(int64_t T, int runs = 1) { return (T + kEmbBlockTokens * runs - 1) / (kEmbBlockTokens * runs); }
 template <int LPT>
 static void launch_embed_gather(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
                                 void* H, int64_t ldh, cudaStream_t st) {
@@ -1086,11 +1087,11 @@ static void launch_embed_gather(const int32_t* ids, int64_t T, const void* E, in
 }
 template <int LPT>
 static int launch_embed_bwd(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
-                            const bf16* dH, int64_t lddh, float* dE, int64_t ldde, float* part, cudaStream_t st) {
+                            const bf16* dH, int64_t lddh, float* dE, int64_t ldde, float* part, int runs, cudaStream_t st) {
   const size_t smem = (size_t)kEmbWarps * d_i * 4;
   if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(embed_bwd_kernel<LPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  launch_k(embed_bwd_kernel<LPT>, dim3((unsigned)embedding_blocks(T)), dim3(32 * kEmbWarps), smem, st, ids, (int)T, (const bf16*)E, lde,
-           (int)n_rows, z, (int)d_i, dH, lddh, dE, ldde, part);
+  launch_k(embed_bwd_kernel<LPT>, dim3((unsigned)embedding_blocks(T, runs)), dim3(32 * kEmbWarps), smem, st, ids, (int)T, (const bf16*)E, lde,
+           (int)n_rows, z, (int)d_i, dH, lddh, dE, ldde, part, runs);
   return FLOP_OK;
 }
 
@@ -2167,13 +2168,14 @@ int flop_agp_gates(const float* g, int64_t n, const int64_t* seg_off, int32_t n_
 }
 
 // ---- gated adaptive embedding of one word cluster (Section 4.2): Y = (E[ids] * z) O
-static size_t embedding_ws_bytes(int64_t T, int64_t d_i) {
+static size_t embedding_ws_need(int64_t T, int64_t d_i, int runs, bool slices) {
   Arena ar{nullptr, 0, 0};
-  ar.take((size_t)T * round_up(std::max<int64_t>(d_i, 1), 8) * 2);                                              // dH'
-  ar.take((size_t)std::max<int64_t>(embedding_blocks(T), 1) * std::max<int64_t>(d_i, 1) * 4);                   // dz partials
-  ar.take(embedding_slice_bytes(T, d_i));                                                                       // dO slices
-  return align_up(ar.used, 256);
+  ar.take((size_t)T * round_up(std::max<int64_t>(d_i, 1), 8) * 2);                                                    // dH'
+  ar.take((size_t)std::max<int64_t>(embedding_blocks(T, runs), 1) * std::max<int64_t>(d_i, 1) * 4);                   // dz partials
+  if (slices) ar.take(embedding_slice_bytes(T, d_i));                                                                 // dO slices
+  return ar.used;
 }
+static size_t embedding_ws_bytes(int64_t T, int64_t d_i) { return align_up(embedding_ws_need(T, d_i, 1, true), 256); }
 
 int flop_gated_embedding_fwd(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const void* O,
                              int64_t ldo, const float* z, void* Y, int64_t ldy, void* H_save, int64_t ldh, int64_t d_i,
@@ -2220,13 +2222,15 @@ int flop_gated_embedding_bwd(const void* dY, int64_t lddy, const int32_t* ids, i
   if (T > INT32_MAX || n_rows > INT32_MAX || d_i > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
   if ((size_t)kEmbWarps * d_i * 4 > (size_t)kSmemBudget) return FLOP_ERR_UNSUPPORTED;
   if (dO && !wgrad_direct_ok(dO, lddo, wgrad_dt)) return FLOP_ERR_UNSUPPORTED;   // dO is written in place with 16-byte stores
-  FLOP_TRY(check_ws(ws, ws_bytes, embedding_ws_bytes(T, d_i)));
+  // A vector of dz partials per 32 tokens, and the rest of the workspace for slices of dO; one per 64 tokens in a smaller one.
+  const int runs = ws_bytes >= embedding_ws_need(T, d_i, 1, false) ? 1 : 2;
+  FLOP_TRY(check_ws(ws, ws_bytes, embedding_ws_need(T, d_i, runs, false)));
   Arena ar{(unsigned char*)ws, ws_bytes, 0};
   const int64_t lddh = round_up(d_i, 8);
   bf16* dH = (bf16*)ar.take((size_t)T * lddh * 2);
-  const int64_t blocks = embedding_blocks(T);
+  const int64_t blocks = embedding_blocks(T, runs);
   float* part = (float*)ar.take((size_t)blocks * d_i * 4);
-  const size_t slice_bytes = embedding_slice_bytes(T, d_i);
+  const size_t used = align_up(ar.used, 256), slice_bytes = std::min(embedding_slice_bytes(T, d_i), ws_bytes > used ? ws_bytes - used : 0);
   float* slices = (float*)ar.take(slice_bytes);
   EmbedFinish fin{};
   fin.accumulate = accumulate; fin.d_i = (int)d_i; fin.d = (int)d;
@@ -2286,9 +2290,9 @@ int flop_gated_embedding_bwd(const void* dY, int64_t lddy, const int32_t* ids, i
   if (dE || dlog_alpha) {
     const int lanes = embed_lanes(d_i);
     float* dz = dlog_alpha ? part : nullptr;
-    FLOP_TRY(lanes == 8    ? launch_embed_bwd<8>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st)
-             : lanes == 16 ? launch_embed_bwd<16>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st)
-                           : launch_embed_bwd<32>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, st));
+    FLOP_TRY(lanes == 8    ? launch_embed_bwd<8>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, runs, st)
+             : lanes == 16 ? launch_embed_bwd<16>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, runs, st)
+                           : launch_embed_bwd<32>(ids, T, E, lde, n_rows, z, d_i, dH, lddh, dE, ldde, dz, runs, st));
     count_launch();
     FLOP_CUDA(cudaGetLastError());
   }
