@@ -85,7 +85,7 @@ def test_pruned_inference_config(b, dtype):
     assert np.all(np.isnan(host(Pc)[:, k:])) and np.all(np.isnan(host(Qc)[k:]))     # the rest is untouched
     assert rel_fro(host(Qc)[:k], Qco) < (4e-3 if dtype == "bf16" else 1e-6)
     tol = 2e-2 if dtype == "bf16" else 1e-5
-    for T in (1, 3, 4, 5, 9, 16, 17, 64, 256, 4096):   # 1..4: CUDA-core streaming, 5..16: warp-level MMA, above: tcgen05
+    for T in (1, 3, 4, 5, 9, 16, 17, 64, 256, 4096):   # 1..64: the few-token kernel (gated only to 16), above: also tcgen05 tiles
         X = to_dev(prob["X"][:T], dtype)
         Y = empty_dev(T, m.d_out, tdt)
         ws = b.alloc_workspace(b.workspace_bytes(b.OP_COMPACT_FWD, T, m.d_in, m.d_out, k, b.BF16 if dtype == "bf16" else b.F32))
@@ -109,10 +109,13 @@ def test_compact_fwd_with_no_survivors(b):
 @pytest.mark.parametrize("r,d_out,d_in,keep", [
     (1024, 40003, 16, 0.35),    # 8 rows per stage, more groups than buffers per block (buffers reused, parity flips), ragged last group
     (16384, 1003, 8, 0.40),     # one 32 KB row per stage, two buffers
-    (64, 777, 24, 0.5),         # 16 rows per stage, tiny rows
-    (1024, 517, 8, 0.001),      # one or two survivors: the scalar tail of a row
+    (64, 140000, 24, 0.5),      # 16 rows per stage, tiny rows
+    (64, 777, 24, 0.5),         # tiny rows in one launch with the selection
+    (1024, 9000, 8, 0.001),     # one or two survivors: the scalar tail of a row
+    (1024, 517, 8, 0.001),      # the same in one launch
     (1032, 300, 8, 1.0),        # every component survives
-    (1020, 300, 8, 0.35),       # rows that are not 16-byte multiples: the plain kernel
+    (1020, 9000, 8, 0.35),      # rows that are not 16-byte multiples: the plain kernel
+    (1020, 300, 8, 0.35),       # the same in one launch
 ])
 def test_gather_of_survivors_is_exact(b, r, d_out, d_in, keep):
     """P_c = P[:, idx] and Q_c = diag(z) Q[idx, :] for a supplied gate vector (mode 1): a pure gather on the P side,
