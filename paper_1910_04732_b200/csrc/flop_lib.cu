@@ -848,7 +848,7 @@ int64_t few_blocks(int64_t T, int64_t N) { return ((N + 31) / 32) * ((T + 63) / 
 // 6.8 / 3.7, 6.9 / 3.9, 10.2 / 4.8.  Large weights are a matter of bytes in flight, not of rounds, and the whole block on K has the most
 // (up to 8 tokens: 100 000 outputs, K = 1024, 8 tokens 35.7 / 40.3 with ks = 1).
 int few_cut(int64_t T, int64_t N, int64_t K) {
-  if (T <= 8 && K >= 1024 && N * K >= 40000000) return few::kWarps;
+  if (N <= 2048 || (T <= 8 && K >= 1024 && N * K >= 40000000)) return few::kWarps;   // 2048: at most 128 blocks, fewer than SMs
   const int64_t round = (int64_t)num_sms() * (T > 8 && T <= 16 ? 2 : 3);
   int ks = few::kWarps;
   while (ks > 1 && (N * ks + 16 * few::kWarps - 1) / (16 * few::kWarps) > round) ks /= 2;
@@ -908,7 +908,8 @@ int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
 }
 
 // fp32 product with the fields of `a` that the caller sets (outputs, gates, accumulate, row dot).  K is cut over a
-// cluster while the 64 x 64 tiles alone leave SMs idle and every CTA keeps at least two 32-wide k-blocks.
+// cluster while the 64 x 64 tiles alone leave SMs idle and a CTA has two 32-wide k-blocks on average (they are rounded up, so the
+// last CTAs of a cluster can have fewer, or none, and add zeros).
 int launch_simt(const SimtOperand& A, const SimtOperand& B, int64_t M, int64_t N, int64_t K, SimtGemmArgs a, cudaStream_t st) {
   if (M <= 0 || N <= 0) return FLOP_OK;
   if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
@@ -1756,8 +1757,8 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
           if (a.dQ || a.dlog_alpha) { q.add(a.r, a.d_in, a.T, wss[i].plan_q); slice_bytes += 8.0 * wss[i].plan_q.splits * a.r * a.d_in; }
           if (a.dX) x.add(a.T, a.d_in, a.r, s6.bn);
         }
-        // 0.96: level estimates go to the launches per product (six matrices 256 -> 256 at 9000 tokens: 92 us, shared 104, estimated at 0.98)
-        single_cycles = 0.96 * (h.cycles() + p.cycles() + q.cycles() + x.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0);
+        // 0.975: level estimates go to the launches per product (six matrices 256 -> 256 at 9000 tokens: 92 us, shared 104, estimated at 0.98)
+        single_cycles = 0.975 * (h.cycles() + p.cycles() + q.cycles() + x.cycles() + kSmallLaunchCycles + slice_bytes / 3000.0);
       }
     }
     if (mg.cycles >= single_cycles) { direct = false; mg.bn_h = 0; }
