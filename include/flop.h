@@ -43,7 +43,7 @@ typedef enum {
   FLOP_OK = 0,
   FLOP_ERR_INVALID_ARG = 1, /* null pointer, negative size, ld too small, bad enum; a bad device-side table */
   FLOP_ERR_UNSUPPORTED = 2, /* alignment / leading-dimension / size limit of the kernels   */
-  FLOP_ERR_WORKSPACE = 3,   /* ws is NULL, misaligned or smaller than flop_workspace_bytes */
+  FLOP_ERR_WORKSPACE = 3,   /* ws is NULL, misaligned or too small (flop_workspace_bytes is always enough) */
   FLOP_ERR_CUDA = 4,        /* a CUDA runtime/driver call failed                           */
   FLOP_ERR_TIMEOUT = 5      /* a bounded device-side wait gave up                          */
 } flop_status_t;
@@ -368,7 +368,8 @@ int flop_expected_l0_lagrangian_noalloc(const float* log_alpha, int64_t n, const
  *             repeat across tokens: clear dE before the first call of a step; the order of the adds
  *             is not fixed, so dE is reproducible only to fp32 rounding),
  *             dlog_alpha = dz_dla * sum_t E[ids[t], :] dH'[t, :]  (fixed summation order).
- *   Any of dE, dO, dlog_alpha may be NULL.  dO is written in place with 16-byte stores: its pointer must be
+ *   Any of dE, dO, dlog_alpha may be NULL.  dO is written with 16-byte stores (by its product, or by the pass that adds
+ *   up its split-K slices in ws; a ws without room for slices keeps the product unsplit): its pointer must be
  *   16-byte aligned and lddo a multiple of 8 (bf16) or 4 (fp32) elements, else FLOP_ERR_UNSUPPORTED (checked
  *   before anything is launched).  Workspace: flop_workspace_bytes(FLOP_OP_EMBEDDING_BWD, T,
  *   0, 0, d_i, dt).  The tied softmax side of the same cluster, logits = ((h O^T) * z) E^T, is
@@ -402,7 +403,8 @@ int flop_agp_gates(const float* g, int64_t n, const int64_t* seg_off, int32_t n_
  * (nullable) and, when P/Q/Pc/Qc are given (all or none),
  *     Pc[d_out, k] = P[:, idx]          (ld ldpc >= max k the caller allows, e.g. r)
  *     Qc[k, d_in]  = diag(z[idx]) Q[idx, :]   (the gate is absorbed into Q)
- * Columns >= k of Pc and rows >= k of Qc are left untouched.  r <= 65536. */
+ * Columns >= k of Pc and rows >= k of Qc are left untouched.  r <= 65536.  z_det may be the
+ * input vector itself, and Pc may be P (same ld). */
 int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t hc, int64_t r,
                        const void* P, int64_t ldp, const void* Q, int64_t ldq, int64_t d_in,
                        int64_t d_out, int dt, int32_t* idx, int32_t* k_dev, float* z_det, void* Pc,

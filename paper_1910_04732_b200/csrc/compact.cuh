@@ -320,7 +320,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the selection, and in pieces it takes 16).  Surviving
 // columns of P are read straight from global memory, two per lane: neighbouring lanes read neighbouring survivors, so
 // a load touches only a few lines, and a row needs neither staging nor a barrier.
-// Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (three launches each: 13.0 + 4.0 + 5.8 us
+// Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (calls of 12 us; three launches each: 13.0 + 4.0 + 5.8 us
 // of GPU time).  Blocks of 256 threads, four per SM, repeated the fp64 probabilities twice as often: 706 us against 650 us
 // with 512 threads and two per SM (both with the binding's calls at 4 us).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
