@@ -9,6 +9,8 @@
 //   gather_p_kernel : Pc[i, c] = P[i, idx[c]]  (each P row is read once, coalesced,
 //       into shared memory and the surviving columns are written out coalesced)
 #pragma once
+#include <float.h>
+
 #include "common.cuh"
 
 namespace flop {
@@ -311,18 +313,19 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // Bound: latency.  The factors of one matrix are 1-10 MB (0.2-1.5 us of memory time), but the selection is a chain
 // of dependent steps, and as a launch of its own (one block of 1024 threads, 13 us) it kept 147 SMs waiting.  Here
 // every block repeats the selection in its own shared memory -- r gates are 4 KB, L2-resident after the first block --
-// and goes straight on to its rows.  What makes the repetition cheap: keys stay in registers (kKeys per thread),
-// the k-th largest is found by four 256-bin histogram passes with ONE barrier each (four histograms zeroed up front, every
-// warp searches the bins by itself), and positions come from ballots and one scan over 32-gate words.
+// and goes straight on to its rows.  What makes the repetition cheap: gates stay in registers (kKeys per thread), ordinary
+// gates need no fp64 and one histogram (select_fast; the rest goes to select_general), and positions come from ballots and a scan
+// of the 32 words by every warp.  The fp64 probabilities are evaluated only where they are results: one per row of Q_c, by the warp
+// that scales it, and z_det spread over the blocks.
 // A warp then takes one row at a time: P rows first (their number is known before the selection, so the rows are
-// prefetched into L2 while the previous launch on the stream still runs), then the surviving rows of Q in pieces of at most
+// prefetched into L2 while the previous launch on the stream still runs, and the warp's first one is staged in shared memory
+// during the selection), then the surviving rows of Q in pieces of at most
 // kFusedPiece elements (a warp per whole row took 45 us for 400 rows of 30 000 bf16, the gather in its own launch 23 with
-// the selection, and in pieces it takes 16).  Surviving
-// columns of P are read straight from global memory, two per lane: neighbouring lanes read neighbouring survivors, so
-// a load touches only a few lines, and a row needs neither staging nor a barrier.
-// Measured: the 72 matrices of a BERT-base-shaped model in 991 us instead of 1364 (calls of 12 us; three launches each: 13.0 + 4.0 + 5.8 us
-// of GPU time).  Blocks of 256 threads, four per SM, repeated the fp64 probabilities twice as often: 706 us against 650 us
-// with 512 threads and two per SM (both with the binding's calls at 4 us).
+// the selection, and in pieces it takes 16).  Surviving columns of further rows of P are read straight from global memory, two
+// per lane: neighbouring lanes read neighbouring survivors, so a load touches only a few lines.
+// Measured, the 72 matrices of a BERT-base-shaped model: three launches each 1364 us (13.0 + 4.0 + 5.8 us of GPU time per matrix);
+// one launch with four histogram passes and all probabilities in fp64 643 us; this form 444 us.  Held to 40 or 32 registers, so that
+// more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
 // saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74), and for long P the staged
 // gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
@@ -335,199 +338,304 @@ constexpr int kFusedThreads = 512, kFusedWarps = kFusedThreads / 32;
 template <typename T> struct alignas(2 * sizeof(T)) Pair2 { T e[2]; };
 
 constexpr int kKeys = kFusedMaxR / kFusedThreads;   // gates per thread
+constexpr int kFusedWords = kKeys * kFusedWarps;    // 32-gate words, one per lane of a warp that scans them
+static_assert(kFusedWords == 32, "a warp scans all words at once");
+constexpr int kFineBins = 1024, kCloseGates = 64;
+// Shared memory for one row of P per warp, staged while the selection runs.
+template <typename T> __host__ __device__ constexpr size_t fused_row_bytes(int64_t r) { return ((size_t)r * sizeof(T) + 15) & ~(size_t)15; }
+
+// Exclusive prefix of `count` over the lanes and, in *total, the sum.
+__device__ __forceinline__ int warp_exclusive_scan(int count, int lane, int* total) {
+  int inc = count;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += up;
+  }
+  *total = __shfl_sync(0xffffffffu, inc, 31);
+  return inc - count;
+}
+// The bin among 32, counted from lane 0 up, that holds item `need` (1-based); *need becomes its rank inside the bin.
+// -1 when there are fewer items.
+__device__ __forceinline__ int warp_find(int count, int lane, int* need) {
+  int total;
+  const int before = warp_exclusive_scan(count, lane, &total);
+  const unsigned who = __ballot_sync(0xffffffffu, before < *need && *need <= before + count);
+  const int at = who ? __ffs(who) - 1 : 0;
+  *need -= __shfl_sync(0xffffffffu, before, at);
+  return who ? at : -1;
+}
+
+struct FusedShared {
+  __align__(16) int hist[kFineBins];           // fine bins of the fast selection, or four times 256 of the general one
+  int coarse[32];
+  unsigned long long close[kCloseGates];
+  double red[kFusedWarps];
+  uint32_t lo[kFusedWarps], hi[kFusedWarps], fixed[kFusedWarps], words[kFusedWords];
+  int n_close;
+  __align__(16) unsigned short idx[kFusedMaxR];
+  float v[kFusedMaxR];
+};
+
+// P(z > 0) as the deterministic gate, evaluated in fp64 (out of line: it is needed once per row and must not cost the kernel registers).
+__device__ __noinline__ float probability(float a, double thr) { return (float)(1.0 / (1.0 + exp(-((double)a - thr)))); }
+
+// Which of this thread's gates are among the k = floor(sum of probabilities + 1/2) largest, for any input (NaN, infinities, all
+// equal, sums next to a half): k from fp64 probabilities, the k-th largest by four histogram passes over the gates' bits.
+// Bit n of the result: gate n is kept.
+__device__ __noinline__ unsigned select_general(FusedShared& sh, float v0, float v1, double thr, int r) {
+  static_assert(kKeys == 2, "two gates per thread");
+  const float v[kKeys] = {v0, v1};
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __syncthreads();
+  for (int i = tid; i < kFineBins; i += kFusedThreads) sh.hist[i] = 0;
+  double sum = 0.0;
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n)
+    if (n * kFusedThreads + tid < r) sum += 1.0 / (1.0 + exp(-((double)v[n] - thr)));
+  sum = warp_sum_f64(sum);
+  if (lane == 0) sh.red[warp] = sum;
+  __syncthreads();   // histograms are zero, warp sums are there
+  sum = warp_sum_f64(lane < kFusedWarps ? sh.red[lane] : 0.0);
+  const int k = max(0, min(r, (int)floor(sum + 0.5)));
+  uint32_t prefix = 0, pmask = 0;
+  int need = k;       // rank (1-based, from the top) still to be located inside the prefix class
+#pragma unroll 1
+  for (int pass = 0; pass < 4; ++pass) {
+    const int shift = 24 - 8 * pass;
+    int* hist = sh.hist + 256 * pass;
+#pragma unroll
+    for (int n = 0; n < kKeys; ++n) {
+      const uint32_t key = order_key(v[n]);
+      if (n * kFusedThreads + tid < r && (key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
+    }
+    __syncthreads();
+    // lane l holds bins 255 - 8 l .. 248 - 8 l, so that a scan over the lanes counts from the top
+    int total = 0;
+    for (int i = 0; i < 8; ++i) total += hist[255 - 8 * lane - i];
+    int left = need;
+    const int at = warp_find(total, lane, &left);      // (none when k is 0)
+    if (at >= 0) {
+      int bin = 255 - 8 * at;
+      for (; left > hist[bin]; --bin) left -= hist[bin];
+      prefix |= (uint32_t)bin << shift;
+      need = left;
+    }
+    pmask |= 255u << shift;
+  }
+  // of the gates equal to the k-th largest, the `need` lowest indices are kept
+  unsigned keep = 0, eq = 0;
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    const bool in_range = n * kFusedThreads + tid < r && k > 0;
+    if (in_range && order_key(v[n]) > prefix) keep |= 1u << n;
+    if (in_range && order_key(v[n]) == prefix) eq |= 1u << n;
+    const uint32_t word = __ballot_sync(0xffffffffu, (eq >> n) & 1u);
+    if (lane == 0) sh.words[n * kFusedWarps + warp] = word;
+  }
+  __syncthreads();
+  const uint32_t word = sh.words[lane];
+  int total;
+  const int before = warp_exclusive_scan(__popc(word), lane, &total);
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    const int w = n * kFusedWarps + warp;
+    const int rank = __shfl_sync(0xffffffffu, before, w) + __popc(__shfl_sync(0xffffffffu, word, w) & ((1u << lane) - 1u));
+    if (((eq >> n) & 1u) && rank < need) keep |= 1u << n;
+  }
+  __syncthreads();   // the words are written again
+  return keep;
+}
+
+// The same decision for ordinary gates in a third of the time; false (for the whole block) when it is not certain here.
+//   k: probabilities in fp32, added as 20-bit fixed point (order-free, one instruction per warp).  A gate is off by at most half a
+//      unit of rounding and 0.42 of fp32 error (|x| e^-|x| times a few 2^-24, and two units in the last place of the quotient), so
+//      the sum is off by less than r units, and floor(sum + 1/2) is that of fp64 unless the sum lies within r + 16 units of a half.
+//   k-th largest: 1024 bins between the smallest and the largest gate (finite ones; the map to a bin is monotone in fp32 arithmetic),
+//      found through 32 coarse sums; the gates of its bin, a few, are ranked against one another on (value, lower index first).
+__device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kKeys], unsigned& keep, float thr, int r) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t lo = 0xffffffffu, hi = 0u, fixed = 0u;
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n)
+    if (n * kFusedThreads + tid < r) {
+      const uint32_t key = order_key(v[n]);
+      lo = min(lo, key); hi = max(hi, fabsf(v[n]) <= FLT_MAX ? key : 0xffffffffu);     // the key of no finite gate
+      fixed += __float2uint_rn(__fdividef(1048576.f, 1.f + __expf(thr - v[n])));
+    }
+  lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi); fixed = __reduce_add_sync(0xffffffffu, fixed);
+  if (lane == 0) { sh.lo[warp] = lo; sh.hi[warp] = hi; sh.fixed[warp] = fixed; }
+  __syncthreads();     // (the bins are zero by now as well)
+  lo = __reduce_min_sync(0xffffffffu, sh.lo[lane % kFusedWarps]);
+  hi = __reduce_max_sync(0xffffffffu, sh.hi[lane % kFusedWarps]);
+  fixed = __reduce_add_sync(0xffffffffu, lane < kFusedWarps ? sh.fixed[lane] : 0u) + (1u << 19);
+  const uint32_t part = fixed & 0xfffffu, margin = (uint32_t)r + 16u;
+  if (r == 0 || hi == 0xffffffffu || part <= margin || part >= 0x100000u - margin) return false;
+  int need = min(r, (int)(fixed >> 20));
+  auto value = [](uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); };
+  const float low = value(lo), scale = (kFineBins - 0.25f) / (value(hi) - low);
+  int bin[kKeys];      // counted from the largest gate down
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    bin[n] = kFineBins - 1 - max(0, min(kFineBins - 1, (int)((v[n] - low) * scale)));
+    if (n * kFusedThreads + tid < r) atomicAdd(&sh.hist[bin[n]], 1);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 32 / kFusedWarps; ++i) {
+    const int c = warp * (32 / kFusedWarps) + i, sum = __reduce_add_sync(0xffffffffu, sh.hist[32 * c + lane]);
+    if (lane == 0) sh.coarse[c] = sum;
+  }
+  __syncthreads();
+  int cut = -1;        // bin of the k-th largest; none when k is 0
+  if (need > 0) {
+    const int c = warp_find(sh.coarse[lane], lane, &need);
+    cut = 32 * c + warp_find(sh.hist[32 * c + lane], lane, &need);
+  }
+  const bool all = cut >= 0 && need == sh.hist[cut];      // the cut falls between two bins
+  keep = 0;
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    const int j = n * kFusedThreads + tid;
+    if (j < r && (bin[n] < cut || (all && bin[n] == cut))) keep |= 1u << n;
+    if (!all && j < r && bin[n] == cut) {
+      const int at = atomicAdd(&sh.n_close, 1);
+      if (at < kCloseGates) sh.close[at] = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)j);
+    }
+  }
+  if (all || cut < 0) return true;
+  __syncthreads();
+  const int n_close = sh.n_close;
+  if (n_close > kCloseGates) return false;
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    const int j = n * kFusedThreads + tid;
+    if (j < r && bin[n] == cut) {
+      const unsigned long long mine = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)j);
+      int rank = 0;
+      for (int i = 0; i < n_close; ++i) rank += sh.close[i] > mine;
+      if (rank < need) keep |= 1u << n;
+    }
+  }
+  return true;
+}
 
 template <typename T>
-__global__ void __launch_bounds__(kFusedThreads)
+__global__ void __launch_bounds__(kFusedThreads, 2)
 compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, int32_t* __restrict__ idx, int32_t* __restrict__ k_dev,
                      float* __restrict__ z_det, const T* __restrict__ P, int64_t ldp, const T* __restrict__ Q, int64_t ldq, int d_in,
-                     int d_out, T* __restrict__ Pc, int64_t ldpc, T* __restrict__ Qc, int64_t ldqc, int vec_q, int pair_p, int pieces) {
-  constexpr int kWords = kKeys * kFusedWarps;
-  constexpr int kWordsPerLane = (kWords + 31) / 32;
-  __shared__ __align__(16) int hist[4][256];
-  __shared__ double red[kFusedWarps];
-  __shared__ uint32_t s_gt[kWords], s_eq[kWords];
-  __shared__ int s_base[kWords + 1];
-  __shared__ __align__(16) unsigned short s_idx[kKeys * kFusedThreads];
-  __shared__ float s_z[kKeys * kFusedThreads];
+                     int d_out, T* __restrict__ Pc, int64_t ldpc, T* __restrict__ Qc, int64_t ldqc, int vec_q, int vec_p, int pair_p, int pieces) {
+  __shared__ FusedShared sh;
+  extern __shared__ __align__(16) unsigned char rows[];      // [kFusedWarps][fused_row_bytes]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int warps = (int)gridDim.x * kFusedWarps, my_warp = (int)blockIdx.x * kFusedWarps + warp;
+  T* my_row = reinterpret_cast<T*>(rows + warp * fused_row_bytes<T>(r));
   // a hint only: nothing is read before the wait below
   for (int i = my_warp; i < d_out; i += warps)
     for (int b = lane * 128; b < r * (int)sizeof(T); b += 32 * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(P + (int64_t)i * ldp) + b));
-  for (int i = tid; i < 4 * 256; i += kFusedThreads) (&hist[0][0])[i] = 0;
+  for (int i = tid; i < kFineBins; i += kFusedThreads) sh.hist[i] = 0;
+  if (tid == 0) sh.n_close = 0;
   pdl_wait();
   pdl_launch_dependents();
 
   // gate n of this thread is n * kFusedThreads + tid: word n * kFusedWarps + warp of the ballots, bit lane
-  float v[kKeys], zv[kKeys];
-  double sum = 0.0;
+  float v[kKeys];
 #pragma unroll
-  for (int n = 0; n < kKeys; ++n) {
-    const int j = n * kFusedThreads + tid;
-    v[n] = j < r ? in[j] : 0.f;
-    zv[n] = v[n];
-    if (mode == 0 && j < r) {
-      const double pi = 1.0 / (1.0 + exp(-((double)v[n] - thr)));
-      sum += pi;
-      zv[n] = (float)pi;
-    }
+  for (int n = 0; n < kKeys; ++n) v[n] = n * kFusedThreads + tid < r ? in[n * kFusedThreads + tid] : 0.f;
+  // this warp's first row of P, known before the selection
+  const bool staged = vec_p && my_warp < d_out;
+  if (staged) {
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(P + (int64_t)my_warp * ldp);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(my_row);
+    const int bytes = r * (int)sizeof(T);
+    for (int b = lane * 16; b < bytes; b += 32 * 16)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)b), "l"(src + b), "r"(min(16, bytes - b)) : "memory");
   }
-  int k = 0, need_eq = 0;
-  uint32_t kth = 0;   // key of the k-th largest gate
+  unsigned keep = 0;     // bit n: gate n of this thread survives
   if (mode == 0) {
-    sum = warp_sum_f64(sum);
-    if (lane == 0) red[warp] = sum;
-    __syncthreads();   // histograms are zero, warp sums are there
-    sum = warp_sum_f64(lane < kFusedWarps ? red[lane] : 0.0);
-    k = max(0, min(r, (int)floor(sum + 0.5)));
-    uint32_t prefix = 0, pmask = 0;
-    int need = k;       // rank (1-based, from the top) still to be located inside the prefix class
+    if (!select_fast(sh, v, keep, (float)thr, r)) keep = select_general(sh, v[0], v[1], thr, r);
+  } else {
 #pragma unroll
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-#pragma unroll
-      for (int n = 0; n < kKeys; ++n) {
-        const uint32_t key = order_key(v[n]);
-        if (n * kFusedThreads + tid < r && (key & pmask) == prefix) atomicAdd(&hist[pass][(key >> shift) & 255], 1);
-      }
-      __syncthreads();
-      // lane l holds bins 255 - 8 l .. 248 - 8 l, so that a scan over the lanes counts from the top
-      const int4 hi = *reinterpret_cast<const int4*>(&hist[pass][252 - 8 * lane]), lo = *reinterpret_cast<const int4*>(&hist[pass][248 - 8 * lane]);
-      const int h[8] = {hi.w, hi.z, hi.y, hi.x, lo.w, lo.z, lo.y, lo.x};
-      int total = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) total += h[i];
-      int inc = total;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += up;
-      }
-      int above = inc - total, bin = -1, left = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (above < need && need <= above + h[i]) { bin = 255 - 8 * lane - i; left = need - above; }
-        above += h[i];
-      }
-      const unsigned who = __ballot_sync(0xffffffffu, bin >= 0);   // one lane (none when k is 0)
-      const int src = who ? __ffs(who) - 1 : 0;
-      bin = __shfl_sync(0xffffffffu, bin, src);
-      left = __shfl_sync(0xffffffffu, left, src);
-      if (who) { prefix |= (uint32_t)bin << shift; need = left; }
-      pmask |= 255u << shift;
-    }
-    kth = prefix;
-    need_eq = need;
+    for (int n = 0; n < kKeys; ++n)
+      if (n * kFusedThreads + tid < r && v[n] > 0.f) keep |= 1u << n;
   }
 #pragma unroll
   for (int n = 0; n < kKeys; ++n) {
-    const bool in_range = n * kFusedThreads + tid < r;
-    const uint32_t key = order_key(v[n]);
-    const bool gt = in_range && (mode == 0 ? k > 0 && key > kth : v[n] > 0.f);
-    const bool eq = in_range && mode == 0 && k > 0 && key == kth;
-    const uint32_t bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
-    if (lane == 0) { s_gt[n * kFusedWarps + warp] = bg; s_eq[n * kFusedWarps + warp] = be; }
+    const uint32_t word = __ballot_sync(0xffffffffu, (keep >> n) & 1u);
+    if (lane == 0) sh.words[n * kFusedWarps + warp] = word;
   }
   __syncthreads();
-  if (warp == 0) {
-    // of the gates equal to the k-th largest, the need_eq lowest indices are kept
-    uint32_t g[kWordsPerLane], e[kWordsPerLane];
-    int n_eq = 0;
+  int k;
+  {
+    const uint32_t word = sh.words[lane];
+    const int before = warp_exclusive_scan(__popc(word), lane, &k);
 #pragma unroll
-    for (int i = 0; i < kWordsPerLane; ++i) {
-      const int w = lane * kWordsPerLane + i;
-      g[i] = w < kWords ? s_gt[w] : 0u;
-      e[i] = w < kWords ? s_eq[w] : 0u;
-      n_eq += __popc(e[i]);
+    for (int n = 0; n < kKeys; ++n) {
+      const int j = n * kFusedThreads + tid, w = n * kFusedWarps + warp;
+      const int pos = __shfl_sync(0xffffffffu, before, w) + __popc(__shfl_sync(0xffffffffu, word, w) & ((1u << lane) - 1u));
+      if ((keep >> n) & 1u) {
+        sh.idx[pos] = (unsigned short)j;
+        sh.v[pos] = v[n];
+        if (blockIdx.x == 0) idx[pos] = j;
+      }
     }
-    int inc = n_eq;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += up;
-    }
-    int take = need_eq - (inc - n_eq), kept = 0;
-#pragma unroll
-    for (int i = 0; i < kWordsPerLane; ++i) {
-      const int have = __popc(e[i]);
-      uint32_t keep_eq = e[i];
-      for (int drop = have - max(0, min(have, take)); drop > 0; --drop) keep_eq &= ~(0x80000000u >> __clz(keep_eq));
-      take -= have;
-      g[i] |= keep_eq;
-      kept += __popc(g[i]);
-    }
-    inc = kept;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += up;
-    }
-    int base = inc - kept;
-#pragma unroll
-    for (int i = 0; i < kWordsPerLane; ++i) {
-      const int w = lane * kWordsPerLane + i;
-      if (w < kWords) { s_gt[w] = g[i]; s_base[w] = base; }
-      base += __popc(g[i]);
-    }
-    if (lane == 31) s_base[kWords] = base;
   }
-  __syncthreads();
-  k = s_base[kWords];
-  const bool writer = blockIdx.x == 0;
-#pragma unroll
-  for (int n = 0; n < kKeys; ++n) {
-    const int j = n * kFusedThreads + tid, w = n * kFusedWarps + warp;
-    const uint32_t bits = s_gt[w];
-    const bool keep = (bits >> lane) & 1u;
-    const int pos = s_base[w] + __popc(bits & ((1u << lane) - 1u));
-    if (keep) {
-      s_idx[pos] = (unsigned short)j;
-      s_z[pos] = zv[n];
-      if (writer) idx[pos] = j;
-    }
-    if (writer && z_det && j < r) z_det[j] = keep ? zv[n] : 0.f;
-  }
-  if (writer && tid == 0) *k_dev = k;
+  if (blockIdx.x == 0 && tid == 0) *k_dev = k;
+  if (staged) asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
 
   constexpr int V = Vec16<T>::n;
   const int piece = ((d_in + max(pieces, 1) - 1) / max(pieces, 1) + 63) & ~63;
   for (int t = my_warp; t < d_out + k * pieces; t += warps) {
     if (t < d_out) {                       // Pc[t, :] = P[t, idx]
-      const T* p = P + (int64_t)t * ldp;
+      const T* p = staged && t == my_warp ? my_row : P + (int64_t)t * ldp;
       T* o = Pc + (int64_t)t * ldpc;
       if (pair_p) {
 #pragma unroll 4
         for (int c = 2 * lane; c < k; c += 64) {
           if (c + 1 < k) {
-            const uint32_t ii = *reinterpret_cast<const uint32_t*>(s_idx + c);
+            const uint32_t ii = *reinterpret_cast<const uint32_t*>(sh.idx + c);
             Pair2<T> two;
             two.e[0] = p[ii & 0xFFFFu];
             two.e[1] = p[ii >> 16];
             *reinterpret_cast<Pair2<T>*>(o + c) = two;
           } else {
-            o[c] = p[s_idx[c]];
+            o[c] = p[sh.idx[c]];
           }
         }
       } else {
-        for (int c = lane; c < k; c += 32) o[c] = p[s_idx[c]];
+        for (int c = lane; c < k; c += 32) o[c] = p[sh.idx[c]];
       }
     } else {                               // Qc[c, :] = z[idx[c]] * Q[idx[c], :]
       const int c = (t - d_out) / pieces, j0 = (t - d_out - c * pieces) * piece, j1 = min(d_in, j0 + piece);
-      const float g = s_z[c];
-      const T* q = Q + (int64_t)s_idx[c] * ldq;
+      const T* q = Q + (int64_t)sh.idx[c] * ldq;
       T* o = Qc + (int64_t)c * ldqc;
       const int full = vec_q ? j1 / V * V : j0;
-#pragma unroll 4
-      for (int j = j0 + lane * V; j < full; j += 32 * V) {
-        uint4 raw = *reinterpret_cast<const uint4*>(q + j);
-        T* e = reinterpret_cast<T*>(&raw);
+      float g = 0.f;
+      for (int j = j0 + lane * V, first = 1; first || j - lane * V < full; j += 4 * 32 * V, first = 0) {
+        uint4 raw[4];
 #pragma unroll
-        for (int i = 0; i < V; ++i) e[i] = from_f32<T>(to_f32<T>(e[i]) * g);
-        *reinterpret_cast<uint4*>(o + j) = raw;
+        for (int u = 0; u < 4; ++u)
+          if (j + u * 32 * V < full) raw[u] = *reinterpret_cast<const uint4*>(q + j + u * 32 * V);
+        if (first) g = mode == 0 ? probability(sh.v[c], thr) : sh.v[c];         // while the first loads are on their way
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (j + u * 32 * V < full) {
+            T* e = reinterpret_cast<T*>(&raw[u]);
+#pragma unroll
+            for (int i = 0; i < V; ++i) e[i] = from_f32<T>(to_f32<T>(e[i]) * g);
+            *reinterpret_cast<uint4*>(o + j + u * 32 * V) = raw[u];
+          }
       }
       for (int j = max(full, j0) + lane; j < j1; j += 32) o[j] = from_f32<T>(to_f32<T>(q[j]) * g);
+    }
+  }
+  if (z_det) {       // a few gates per block: their fp64 probabilities hold nobody up here
+#pragma unroll
+    for (int n = 0; n < kKeys; ++n) {
+      const int j = n * kFusedThreads + tid;
+      if (j < r && j % (int)gridDim.x == (int)blockIdx.x) z_det[j] = !((keep >> n) & 1u) ? 0.f : mode == 0 ? probability(v[n], thr) : v[n];
     }
   }
 }

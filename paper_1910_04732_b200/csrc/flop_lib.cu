@@ -1060,12 +1060,17 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
                                 int64_t ldp, const void* Q, int64_t ldq, int64_t d_in, int64_t d_out, void* Pc, int64_t ldpc, void* Qc,
                                 int64_t ldqc, cudaStream_t st) {
   const int vec_q = aligned16(Q) && aligned16(Qc) && (ldq * sizeof(T)) % 16 == 0 && (ldqc * sizeof(T)) % 16 == 0;
+  const int vec_p = aligned16(P) && (ldp * sizeof(T)) % 16 == 0;
   const int pair_p = reinterpret_cast<uintptr_t>(Pc) % (2 * sizeof(T)) == 0 && ldpc % 2 == 0;
+  const size_t smem = d_out > 0 ? kFusedWarps * fused_row_bytes<T>(r) : 0;
+  static bool configured[kMaxDevices] = {};
+  if (first_use_on_device(configured))
+    FLOP_CUDA(cudaFuncSetAttribute(compact_fused_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kFusedWarps * fused_row_bytes<T>(kFusedMaxR))));
   const int pieces = fused_pieces(d_in);
   const int64_t rows = d_out + r * pieces;                                   // a warp each, at most two blocks per SM
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms() * 2));
-  launch_k(compact_fused_kernel<T>, dim3((unsigned)grid), dim3(kFusedThreads), (size_t)0, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
-           (const T*)Q, ldq, (int)d_in, (int)d_out, (T*)Pc, ldpc, (T*)Qc, ldqc, vec_q, pair_p, pieces);
+  launch_k(compact_fused_kernel<T>, dim3((unsigned)grid), dim3(kFusedThreads), smem, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
+           (const T*)Q, ldq, (int)d_in, (int)d_out, (T*)Pc, ldpc, (T*)Qc, ldqc, vec_q, vec_p, pair_p, pieces);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
