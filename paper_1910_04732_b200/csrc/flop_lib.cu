@@ -751,14 +751,15 @@ MergedShape plan_merged(const flop_bwd_problem_t* pr, int n) {
 // Whether the shared launches may stand in for the launches per product: the first writes dP while dH' still reads dY and P (and
 // X and Q are read after it), the second writes dX and dQ while the other of the two still reads X and Q.  One after another,
 // dX may take the place of X, and split weight gradients the place of anything but Q.
-bool merged_apart(const flop_bwd_problem_t* pr, int n, int wgrad_dt) {
+bool merged_apart(const flop_bwd_problem_t* pr, int n, int dt, int wgrad_dt) {
+  const size_t es = elt(dt);
   for (int i = 0; i < n; ++i) {
     const flop_bwd_problem_t& a = pr[i];
-    const Span dP(a.dP, a.d_out, a.r, a.lddp, elt(wgrad_dt)), dQ(a.dQ, a.r, a.d_in, a.lddq, elt(wgrad_dt)), dX(a.dX, a.T, a.d_in, a.lddx, 2);
+    const Span dP(a.dP, a.d_out, a.r, a.lddp, elt(wgrad_dt)), dQ(a.dQ, a.r, a.d_in, a.lddq, elt(wgrad_dt)), dX(a.dX, a.T, a.d_in, a.lddx, es);
     for (int j = 0; j < n; ++j) {
       const flop_bwd_problem_t& o = pr[j];
-      const Span X(o.X, o.T, o.d_in, o.ldx, 2), Q(o.Q, o.r, o.d_in, o.ldq, 2);
-      for (const Span& in : {Span(o.dY, o.T, o.d_out, o.lddy, 2), Span(o.P, o.d_out, o.r, o.ldp, 2), Span(o.H_save, o.T, o.r, o.ldh, 2)})
+      const Span X(o.X, o.T, o.d_in, o.ldx, es), Q(o.Q, o.r, o.d_in, o.ldq, es);
+      for (const Span& in : {Span(o.dY, o.T, o.d_out, o.lddy, es), Span(o.P, o.d_out, o.r, o.ldp, es), Span(o.H_save, o.T, o.r, o.ldh, es)})
         if (dP.meets(in)) return false;
       for (const Span& in : {X, Q})
         if (dP.meets(in) || dQ.meets(in) || dX.meets(in)) return false;
@@ -887,10 +888,8 @@ int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, v
 // An operand of an fp32 product: a row-major matrix read along its rows (k_fast) or down its columns.
 struct SimtOperand { const float* ptr; int64_t ld; bool k_fast; };
 
-template <bool A_K, bool B_K, bool SCALE_K>
-int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
-  auto kern = simt::gemm_kernel<A_K, B_K, SCALE_K>;
+template <typename... KArgs>
+int launch_simt_kernel(void (*kern)(KArgs...), bool (&configured)[kMaxDevices], dim3 grid, cudaStream_t st, const KArgs&... args) {
   if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kSmemBytes));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = dim3(simt::kThreads); cfg.dynamicSmemBytes = simt::kSmemBytes; cfg.stream = st;
@@ -901,33 +900,73 @@ int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl_on() ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, kern, a);
+  cudaLaunchKernelEx(&cfg, kern, args...);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
 }
+template <bool A_K, bool B_K, bool SCALE_K>
+int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
+  static bool configured[kMaxDevices] = {};
+  auto kern = simt::gemm_kernel<A_K, B_K, SCALE_K>;
+  return launch_simt_kernel(kern, configured, grid, st, a);
+}
 
-// fp32 product with the fields of `a` that the caller sets (outputs, gates, accumulate, row dot).  K is cut over a
-// cluster while the 64 x 64 tiles alone leave SMs idle and a CTA has two 32-wide k-blocks on average (they are rounded up, so the
-// last CTAs of a cluster can have fewer, or none, and add zeros).
+int simt_blocks(int64_t K) { return (int)((K + simt::BK - 1) / simt::BK); }
+int64_t simt_tiles(int64_t M, int64_t N) { return ((M + simt::BM - 1) / simt::BM) * ((N + simt::BN - 1) / simt::BN); }
+// K is cut over a cluster while the 64 x 64 tiles alone leave SMs idle and a CTA has two 32-wide k-blocks on average (they are
+// rounded up, so the last CTAs of a cluster can have fewer, or none, and add zeros).
+int simt_split(int64_t tiles, int num_kb) {
+  int split = 1;
+  while (split < simt::kMaxSplit && tiles * split < num_sms() && num_kb >= 4 * split) split *= 2;
+  return split;
+}
+void simt_operands(SimtGemmArgs& a, const SimtOperand& A, const SimtOperand& B, int64_t M, int64_t N, int64_t K, int split) {
+  a.A = A.ptr; a.lda = A.ld; a.B = B.ptr; a.ldb = B.ld;
+  a.M = (int)M; a.N = (int)N; a.K = (int)K;
+  a.kb_per_split = (simt_blocks(K) + split - 1) / split;
+  a.a_vec = aligned16(A.ptr) && A.ld % 4 == 0;
+  a.b_vec = aligned16(B.ptr) && B.ld % 4 == 0;
+}
+// fp32 product with the fields of `a` that the caller sets (outputs, gates, accumulate, row dot).
 int launch_simt(const SimtOperand& A, const SimtOperand& B, int64_t M, int64_t N, int64_t K, SimtGemmArgs a, cudaStream_t st) {
   if (M <= 0 || N <= 0) return FLOP_OK;
   if (M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return FLOP_ERR_UNSUPPORTED;
   const int64_t tiles_n = (N + simt::BN - 1) / simt::BN, tiles_m = (M + simt::BM - 1) / simt::BM;
   if (tiles_m > 65535) return FLOP_ERR_UNSUPPORTED;
-  const int num_kb = (int)((K + simt::BK - 1) / simt::BK);
-  int split = 1;
-  while (split < simt::kMaxSplit && tiles_m * tiles_n * split < num_sms() && num_kb >= 4 * split) split *= 2;
-  a.A = A.ptr; a.lda = A.ld; a.B = B.ptr; a.ldb = B.ld;
-  a.M = (int)M; a.N = (int)N; a.K = (int)K;
-  a.kb_per_split = (num_kb + split - 1) / split;
-  a.a_vec = aligned16(A.ptr) && A.ld % 4 == 0;
-  a.b_vec = aligned16(B.ptr) && B.ld % 4 == 0;
+  const int split = simt_split(tiles_m * tiles_n, simt_blocks(K));
+  simt_operands(a, A, B, M, N, K, split);
   const dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, (unsigned)split);
   if (A.k_fast && B.k_fast) return launch_simt_inst<true, true, false>(a, grid, st);
   if (A.k_fast) return a.k_scale ? launch_simt_inst<true, false, true>(a, grid, st) : launch_simt_inst<true, false, false>(a, grid, st);
   if (!B.k_fast) return launch_simt_inst<false, false, false>(a, grid, st);
   return FLOP_ERR_UNSUPPORTED;
+}
+
+// A product of the backward pass before its launch, and two of them in one: `act` has (K-fast, MN-fast) operands, `wgrad` contracts over
+// the tokens.
+struct SimtJob { SimtOperand A, B; int64_t M, N, K; SimtGemmArgs a; };
+int launch_simt(const SimtJob& j, cudaStream_t st) { return launch_simt(j.A, j.B, j.M, j.N, j.K, j.a, st); }
+bool simt_dual_ok(const SimtJob& act, const SimtJob& wgrad) {      // one work list: as many tiles, in either form, as the separate launches take
+  return std::max({act.M, act.N, act.K, wgrad.M, wgrad.N, wgrad.K}) <= INT32_MAX &&
+         std::max((act.M + simt::BM - 1) / simt::BM, (wgrad.M + simt::BM - 1) / simt::BM) <= 65535 &&
+         std::max(simt_tiles(act.M, act.N), simt_tiles(wgrad.M, wgrad.N)) <= INT32_MAX / 2;
+}
+int launch_simt_dual(const SimtJob& act, const SimtJob& wgrad, cudaStream_t st) {
+  const int64_t act_tiles = simt_tiles(act.M, act.N), wgrad_tiles = simt_tiles(wgrad.M, wgrad.N);
+  simt::DualArgs d{act.a, wgrad.a};
+  d.act_split = simt_split(act_tiles, simt_blocks(act.K));
+  d.wgrad_split = simt_split(wgrad_tiles, simt_blocks(wgrad.K));
+  simt_operands(d.act, act.A, act.B, act.M, act.N, act.K, d.act_split);
+  simt_operands(d.wgrad, wgrad.A, wgrad.B, wgrad.M, wgrad.N, wgrad.K, d.wgrad_split);
+  const int size = std::max(d.act_split, d.wgrad_split), act_per = size / d.act_split, wgrad_per = size / d.wgrad_split;   // splits are powers of two
+  d.act_clusters = (int)((act_tiles + act_per - 1) / act_per);
+  d.wgrad_clusters = (int)((wgrad_tiles + wgrad_per - 1) / wgrad_per);
+  d.wgrad_first = d.wgrad.kb_per_split > d.act.kb_per_split;
+  const dim3 grid((unsigned)(d.act_clusters + d.wgrad_clusters), 1, (unsigned)size);
+  static bool configured[2][kMaxDevices] = {};
+  return act.a.k_scale ? launch_simt_kernel(simt::gemm_dual_kernel<true>, configured[1], grid, st, d)
+                       : launch_simt_kernel(simt::gemm_dual_kernel<false>, configured[0], grid, st, d);
 }
 
 SimtGemmArgs simt_out(void* C, int64_t ldc, const float* col_scale = nullptr) {
@@ -1503,7 +1542,7 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     // (768 -> 3072 at 4096 tokens, dX and dlog_alpha: a launch per product 55 us, shared 65, estimated at 51 and 49).
     const double margin = need_m && !(dP && dX) ? 0.84 : 1.0;
     if (plan_merged(&one, 1).cycles < margin * separate && ws_bytes >= plan_bwd_ws(grouped, T, d_in, d_out, r, dt, true, true).bytes &&
-        merged_apart(&one, 1, wgrad_dt))
+        merged_apart(&one, 1, dt, wgrad_dt))
       return bwd_grouped_impl(&one, 1, accumulate, dt, wgrad_dt, nullptr, 0, stream, separate);
   }
   if (dt == FLOP_BF16) {
@@ -1556,33 +1595,37 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     const float* dYf = (const float*)dY; const float* Xf = (const float*)X; const float* Qf = (const float*)Q;
     const float* Pf = (const float*)P; const float* Hf = (const float*)H_save;
     float* dHf = (float*)w.dH;
-    // dH'[t,k] = sum_i dY[t,i] P[i,k]
-    FLOP_TRY(launch_simt({dYf, lddy, true}, {Pf, ldp, false}, T, r, d_out, simt_out(dHf, w.lddh), st));
-    // dP[i,k] = sum_t dY[t,i] H'[t,k]
-    if (dP) {
-      SimtGemmArgs a = simt_out(dP, lddp);
-      a.accumulate = accumulate;
-      FLOP_TRY(launch_simt({dYf, lddy, false}, {Hf, ldh, false}, d_out, r, T, a, st));
+    // dH'[t,k] = sum_i dY[t,i] P[i,k];  dP[i,k] = sum_t dY[t,i] H'[t,k]
+    const SimtJob dh{{dYf, lddy, true}, {Pf, ldp, false}, T, r, d_out, simt_out(dHf, w.lddh)};
+    SimtJob dp{{dYf, lddy, false}, {Hf, ldh, false}, d_out, r, T, simt_out(dP, lddp)};
+    dp.a.accumulate = accumulate;
+    // M[k,j] = sum_t dH'[t,k] X[t,j]; dQ = diag(z) M and the row dots <Q[k,:], M[k,:]> leave with the tile
+    SimtJob dq{{dHf, w.lddh, false}, {Xf, ldx, false}, r, d_in, T, simt_out(dQ, lddq)};
+    dq.a.row_scale = z; dq.a.accumulate = accumulate;
+    if (dlog_alpha) { dq.a.qdot = Qf; dq.a.ldq = ldq; dq.a.dz_part = (double*)w.dz_part; dq.a.dz_stride = r; }
+    // dX[t,j] = sum_k dH'[t,k] z[k] Q[k,j], the gate applied to the rows of Q as they are read
+    SimtJob dx{{dHf, w.lddh, true}, {Qf, ldq, false}, T, d_in, r, simt_out(dX, lddx)};
+    dx.a.k_scale = z;
+    // Products that wait for the same input share a launch.
+    const flop_bwd_problem_t one{dY, lddy, X, ldx, Q, ldq, P, ldp, z, dz_dla, H_save, ldh, dX, lddx, dP, lddp, dQ, lddq, dlog_alpha,
+                                 T, d_in, d_out, r, ws, ws_bytes, nullptr, nullptr, 0, 0};
+    const bool apart = merged_apart(&one, 1, dt, wgrad_dt);
+    if (dP && apart && simt_dual_ok(dh, dp)) {
+      FLOP_TRY(launch_simt_dual(dh, dp, st));
+    } else {
+      FLOP_TRY(launch_simt(dh, st));
+      if (dP) FLOP_TRY(launch_simt(dp, st));
     }
-    if (need_m) {
-      // M[k,j] = sum_t dH'[t,k] X[t,j]; dQ = diag(z) M and the row dots <Q[k,:], M[k,:]> leave with the tile
-      SimtGemmArgs a = simt_out(dQ, lddq);
-      a.row_scale = z; a.accumulate = accumulate;
-      if (dlog_alpha) { a.qdot = Qf; a.ldq = ldq; a.dz_part = (double*)w.dz_part; a.dz_stride = r; }
-      FLOP_TRY(launch_simt({dHf, w.lddh, false}, {Xf, ldx, false}, r, d_in, T, a, st));
-      if (dlog_alpha) {
-        const int n_part = (int)((d_in + simt::BN - 1) / simt::BN);
-        launch_k(dalpha_f64_kernel, dim3((unsigned)((r + 255) / 256)), dim3(256), (size_t)(0), st, (const double*)w.dz_part, n_part, r, dz_dla, (int)r, dlog_alpha, accumulate);
-        count_launch();
-        FLOP_CUDA(cudaGetLastError());
-      }
+    const bool shared = need_m && dX && apart && simt_dual_ok(dx, dq);
+    if (shared) FLOP_TRY(launch_simt_dual(dx, dq, st));
+    else if (need_m) FLOP_TRY(launch_simt(dq, st));
+    if (dlog_alpha) {
+      const int n_part = (int)((d_in + simt::BN - 1) / simt::BN);
+      launch_k(dalpha_f64_kernel, dim3((unsigned)((r + 255) / 256)), dim3(256), (size_t)(0), st, (const double*)w.dz_part, n_part, r, dz_dla, (int)r, dlog_alpha, accumulate);
+      count_launch();
+      FLOP_CUDA(cudaGetLastError());
     }
-    if (dX) {
-      // dX[t,j] = sum_k dH'[t,k] z[k] Q[k,j], the gate applied to the rows of Q as they are read
-      SimtGemmArgs a = simt_out(dX, lddx);
-      a.k_scale = z;
-      FLOP_TRY(launch_simt({dHf, w.lddh, true}, {Qf, ldq, false}, T, d_in, r, a, st));
-    }
+    if (dX && !shared) FLOP_TRY(launch_simt(dx, st));
   }
   return FLOP_OK;
 }
@@ -1750,7 +1793,7 @@ static int bwd_grouped_impl(const flop_bwd_problem_t* pr, int n, int accumulate,
   }
   MergedShape mg{0, 0, 0, 0, 1e300};
   if (sw.bn == 0 || sw.items < (sw.cta2 ? num_sms() / 2 : num_sms())) {
-    if (direct && n > 0 && !sync && 2 * n <= tc::kMaxGroup && merged_apart(pr, n, wgrad_dt)) {
+    if (direct && n > 0 && !sync && 2 * n <= tc::kMaxGroup && merged_apart(pr, n, dt, wgrad_dt)) {
       mg = plan_merged(pr, n);
       if (single_cycles <= 0.0) {     // the other form of this call: a launch per product, weight gradients split, a finishing pass
         LaunchCost h{s3.cta2}, p{0}, q{0}, x{s6.cta2};

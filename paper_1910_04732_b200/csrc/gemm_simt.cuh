@@ -14,7 +14,7 @@
 //   * a cluster of up to eight CTAs shares one 64 x 64 tile: each takes a slice of K, and every CTA adds up its rows of
 //     the tile from all slices through distributed shared memory, in rank order (the same bits on every run).
 // One 512 x 256 x 256 product took 26.6 us in the single-buffered unsplit form (64 x 64 x 16); forward and backward of that
-// matrix with its small launches went from 181.6 to 69.8 us.  4 x 4 results per thread: 64 FMAs per eight 16-byte
+// matrix with its small launches went from 181.6 to 69.8 us, and to 42.3 from 52.0 when the backward products came to share two launches.  4 x 4 results per thread: 64 FMAs per eight 16-byte
 // shared-memory reads, of which half are broadcasts.
 // The epilogue applies the gate of the column (H'), of the row (dQ) and the fused row dot <Q[m,:], C[m,:]> (dz), whose
 // partial sums stay in fp64; `k_scale` multiplies B(n,k) by z[k] as it is read, so that diag(z) Q is never written.
@@ -88,16 +88,15 @@ __device__ __forceinline__ void load_block(const float* __restrict__ p, int64_t 
   }
 }
 
+// The 64 x 64 tile (tile_m, tile_n) of one product: this CTA takes slice `split` of K, the other slices are with CTAs first ..
+// first + n_split - 1 of the cluster.  A CTA without a tile (live = false) only takes part in the cluster's barriers, which
+// `clustered` asks for also where this tile is not split.
 template <bool A_K, bool B_K, bool SCALE_K>
-__global__ void __launch_bounds__(kThreads, 2)
-gemm_kernel(const SimtGemmArgs p) {
-  pdl_wait();
-  pdl_launch_dependents();
+__device__ __forceinline__ void gemm_tile(const SimtGemmArgs& p, int tile_m, int tile_n, int split, int n_split, int first, bool live, bool clustered) {
   extern __shared__ __align__(16) float smem[];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int split = blockIdx.z, n_split = gridDim.z;      // the cluster spans z: split is the rank in it
-  const int kb0 = split * p.kb_per_split, kb1 = min((p.K + BK - 1) / BK, kb0 + p.kb_per_split);
+  const int m0 = tile_m * BM, n0 = tile_n * BN;
+  const int kb0 = split * p.kb_per_split, kb1 = live ? min((p.K + BK - 1) / BK, kb0 + p.kb_per_split) : kb0;
 
   auto load = [&](int kb) {
     if (kb < kb1) {
@@ -171,14 +170,14 @@ gemm_kernel(const SimtGemmArgs p) {
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       smem[(A_K ? ty + 16 * i : ty * 4 + i) * kRowP + (B_K ? tx + 16 * j : tx * 4 + j)] = acc[i][j];
-  if (n_split > 1) {
+  if (clustered) {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   } else {
     __syncthreads();
   }
   // this CTA finishes rows [split, split + 1) * BM / n_split of the tile, 16 lanes per row, 4 columns each
-  const int rows = BM / n_split;
+  const int rows = live ? BM / n_split : 0;
   const bool c_vec = (reinterpret_cast<uintptr_t>(p.C) & 15) == 0 && (p.ldc & 3) == 0;
   for (int lr = ty; lr < rows; lr += 16) {
     const int r = split * rows + lr, gm = m0 + r, gn = n0 + tx * 4;
@@ -187,7 +186,7 @@ gemm_kernel(const SimtGemmArgs p) {
     for (int s = 0; s < n_split; ++s) {
       uint32_t peer;
       float x, y, z, w;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(s));
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(first + s));
       asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x), "=f"(y), "=f"(z), "=f"(w) : "r"(peer) : "memory");
       v[0] += x; v[1] += y; v[2] += z; v[3] += w;
     }
@@ -198,7 +197,7 @@ gemm_kernel(const SimtGemmArgs p) {
           if (gn + j < p.N) dot += (double)v[j] * (double)p.qdot[(int64_t)gm * p.ldq + gn + j];
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);   // rows is 8..64: warps are in the loop as a whole
-      if (tx == 0 && gm < p.M) p.dz_part[(int64_t)blockIdx.x * p.dz_stride + gm] = dot;
+      if (tx == 0 && gm < p.M) p.dz_part[(int64_t)tile_n * p.dz_stride + gm] = dot;
     }
     if (p.C && gm < p.M) {
       const float rs = p.row_scale ? p.row_scale[gm] : 1.f;
@@ -219,10 +218,41 @@ gemm_kernel(const SimtGemmArgs p) {
       }
     }
   }
-  if (n_split > 1) {       // no CTA leaves while another still reads its shared memory
+  if (clustered) {         // no CTA leaves while another still reads its shared memory
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
+}
+
+template <bool A_K, bool B_K, bool SCALE_K>
+__global__ void __launch_bounds__(kThreads, 2)
+gemm_kernel(const SimtGemmArgs p) {
+  pdl_wait();
+  pdl_launch_dependents();
+  gemm_tile<A_K, B_K, SCALE_K>(p, blockIdx.y, blockIdx.x, blockIdx.z, gridDim.z, 0, true, gridDim.z > 1);      // the cluster spans z
+}
+
+// Two products that need only what is there before the launch: an activation gradient (dH' = dY P, or dX = dH' diag(z) Q with
+// SCALE_K) and the weight gradient that contracts over the tokens (dP, dQ).  Apart, each leaves SMs idle and waits for the other's
+// last tile.  Each keeps the split, and so the bits, of its own launch: a cluster has as many CTAs as the larger split, and
+// several tiles of the product with the smaller one.  The product with the longer slices comes first.
+struct DualArgs {
+  SimtGemmArgs act, wgrad;
+  int act_split, wgrad_split, act_clusters, wgrad_clusters, wgrad_first;
+};
+template <bool SCALE_K>
+__global__ void __launch_bounds__(kThreads, 2)
+gemm_dual_kernel(const DualArgs d) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int c = blockIdx.x, rank = blockIdx.z, size = gridDim.z;
+  const bool wgrad = d.wgrad_first ? c < d.wgrad_clusters : c >= d.act_clusters;
+  const SimtGemmArgs& p = wgrad ? d.wgrad : d.act;
+  const int split = wgrad ? d.wgrad_split : d.act_split, local = c - (wgrad == (d.wgrad_first != 0) ? 0 : wgrad ? d.act_clusters : d.wgrad_clusters);
+  const int t = local * (size / split) + rank / split, tiles_n = (p.N + BN - 1) / BN, tile_m = t / tiles_n, first = rank / split * split;
+  const bool live = tile_m < (p.M + BM - 1) / BM;
+  if (wgrad) gemm_tile<false, false, false>(d.wgrad, tile_m, t % tiles_n, rank % split, split, first, live, size > 1);
+  else gemm_tile<true, false, SCALE_K>(d.act, tile_m, t % tiles_n, rank % split, split, first, live, size > 1);
 }
 
 }  // namespace simt
