@@ -324,8 +324,9 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the selection, and in pieces it takes 16).  Surviving columns of further rows of P are read straight from global memory, two
 // per lane: neighbouring lanes read neighbouring survivors, so a load touches only a few lines.
 // Measured, the 72 matrices of a BERT-base-shaped model: three launches each 1364 us (13.0 + 4.0 + 5.8 us of GPU time per matrix);
-// one launch with four histogram passes and all probabilities in fp64 643 us; this form 444 us.  Held to 40 or 32 registers, so that
-// more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
+// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us.  Two blocks per SM, which repeat the selection twice,
+// 444 (66 MB of factors, r = 1021: 257 against 270); one block of 1024 threads 455 (longer barriers); held to 40 or 32 registers,
+// so that more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
 // saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74), and for long P the staged
 // gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
@@ -521,7 +522,7 @@ __device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kK
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kFusedThreads, 2)
+__global__ void __launch_bounds__(kFusedThreads, 1)
 compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, int32_t* __restrict__ idx, int32_t* __restrict__ k_dev,
                      float* __restrict__ z_det, const T* __restrict__ P, int64_t ldp, const T* __restrict__ Q, int64_t ldq, int d_in,
                      int d_out, T* __restrict__ Pc, int64_t ldpc, T* __restrict__ Qc, int64_t ldqc, int vec_q, int vec_p, int pair_p, int pieces) {

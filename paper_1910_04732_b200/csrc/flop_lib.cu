@@ -1106,8 +1106,8 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
   if (first_use_on_device(configured))
     FLOP_CUDA(cudaFuncSetAttribute(compact_fused_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kFusedWarps * fused_row_bytes<T>(kFusedMaxR))));
   const int pieces = fused_pieces(d_in);
-  const int64_t rows = d_out + r * pieces;                                   // a warp each, at most two blocks per SM
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms() * 2));
+  const int64_t rows = d_out + r * pieces;                                   // a warp each, at most one block per SM
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms()));
   launch_k(compact_fused_kernel<T>, dim3((unsigned)grid), dim3(kFusedThreads), smem, st, in, mode, thr, (int)r, idx, k_dev, z_det, (const T*)P, ldp,
            (const T*)Q, ldq, (int)d_in, (int)d_out, (T*)Pc, ldpc, (T*)Qc, ldqc, vec_q, vec_p, pair_p, pieces);
   count_launch();
