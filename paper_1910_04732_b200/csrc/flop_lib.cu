@@ -817,32 +817,52 @@ int launch_chain_fwd(const void* X, int64_t ldx, const void* Q, int64_t ldq, con
 
 // Forward product for few tokens (see gemm_few.cuh).  `second`: A is what the launch before on the stream wrote, and that
 // launch wrote nothing else.
-template <int MT, int NT, int KS>
-int launch_few_inst(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, bf16* C, int64_t ldc, const float* cs, int T, int N, int K,
-                    bool second, cudaStream_t st) {
+// `n_pad`: columns of C written, zeros from N on; `a_padded`: A has zeros from K to the next multiple of 8, in every row.
+struct FewArgs { const bf16* A; int64_t lda; const bf16* B; int64_t ldb; bf16* C; int64_t ldc; const float* cs; int T, N, K; bool second; int n_pad, a_padded; };
+template <int MT, int NT, int KS, bool EARLY, bool RAGGED>
+int launch_few_kernel(const FewArgs& a, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
   constexpr int smem = few::smem_bytes(MT, NT);
-  if (smem > 48 * 1024 && first_use_on_device(configured)) {
-    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, KS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FLOP_CUDA(cudaFuncSetAttribute(few::gemm_kernel<MT, NT, KS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  }
+  auto kern = few::gemm_kernel<MT, NT, KS, EARLY, RAGGED>;
+  if (smem > 48 * 1024 && first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   constexpr int rows = 16 * MT * (few::kWarps / KS);       // weight rows per block
-  const dim3 grid((unsigned)((N + rows - 1) / rows), (unsigned)((T + 8 * NT - 1) / (8 * NT)));
-  launch_k(second ? few::gemm_kernel<MT, NT, KS, true> : few::gemm_kernel<MT, NT, KS, false>, grid, dim3(few::kThreads), (size_t)smem, st, A, lda, B,
-           ldb, C, ldc, cs, T, N, K);
+  const dim3 grid((unsigned)((a.N + rows - 1) / rows), (unsigned)((a.T + 8 * NT - 1) / (8 * NT)));
+  launch_k(kern, grid, dim3(few::kThreads), (size_t)smem, st, a.A, a.lda, a.B, a.ldb, a.C, a.ldc, a.cs, a.T, a.N, a.K, a.n_pad, a.a_padded);
   count_launch();
   FLOP_CUDA(cudaGetLastError());
   return FLOP_OK;
 }
-template <int NT>
-int launch_few_cut(int ks, const bf16* a, int64_t lda, const bf16* b, int64_t ldb, bf16* c, int64_t ldc, const float* cs, int t, int n, int k, bool second,
-                   cudaStream_t st) {
-  if (ks == 8) return launch_few_inst<1, NT, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (ks == 4) return launch_few_inst<1, NT, 4>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (ks == 2) return launch_few_inst<1, NT, 2>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  return launch_few_inst<1, NT, 1>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+template <int MT, int NT, int KS>
+int launch_few_inst(const FewArgs& a, cudaStream_t st) {
+  if constexpr (NT > 2) {
+    if (a.K % 8) return a.second ? launch_few_kernel<MT, NT, KS, true, true>(a, st) : launch_few_kernel<MT, NT, KS, false, true>(a, st);
+  }
+  return a.second ? launch_few_kernel<MT, NT, KS, true, false>(a, st) : launch_few_kernel<MT, NT, KS, false, false>(a, st);
 }
-int64_t few_blocks(int64_t T, int64_t N) { return ((N + 31) / 32) * ((T + 63) / 64); }
+template <int NT>
+int launch_few_cut(int ks, const FewArgs& a, cudaStream_t st) {
+  if (ks == 8) return launch_few_inst<1, NT, 8>(a, st);
+  if (ks == 4) return launch_few_inst<1, NT, 4>(a, st);
+  if (ks == 2) return launch_few_inst<1, NT, 2>(a, st);
+  return launch_few_inst<1, NT, 1>(a, st);
+}
+// Blocks of `rows` weight rows by 64 tokens.
+int64_t few_blocks(int64_t T, int64_t N, int64_t rows = 32) { return ((N + rows - 1) / rows) * ((T + 63) / 64); }
+// Block shape for more than 32 tokens: 16 mt weight rows for each of 8 / ks groups of warps, K over ks warps; mt = 0: tcgen05 tiles.  One
+// round of blocks over the SMs, with as many rows (fewer reads of the tokens, no idle warps) as K is short: a block of all eight warps
+// on K has eight 32-long steps to deal out.  Second product of a pair with a first of K = 64, replayed, us, before (32 rows, or
+// tcgen05 beyond a round of them) / by this rule: K = 40: 100 x 4096 outputs 7.0 / 5.4, 256 x 2048 6.4 / 5.3; K = 100: 100 x 4096 7.2 / 5.6,
+// 512 x 512 7.0 / 5.6; K = 160: 150 x 1024 5.8 / 5.0, 150 x 2048 7.0 / 6.4; K = 256: 100 x 4096 7.8 / 7.2.  Lines, this kernel / tcgen05: K = 100,
+// 384 x 2048 7.6 / 7.6 (2 x 2), 512 x 1024 6.7 / 6.6; K = 160, 256 x 2048 7.2 / 6.7, 384 x 1024 7.2 / 6.8; K = 300, 150 x 2048 9.5 / 7.4.
+struct FewShape { int mt, ks; };
+FewShape few_shape(int64_t T, int64_t N, int64_t K) {
+  const int64_t sms = num_sms();
+  if (K > 256) return few_blocks(T, N) > sms ? FewShape{0, 0} : few_blocks(T, N) * 2 >= sms ? FewShape{2, 8} : FewShape{1, 8};
+  if (few_blocks(T, N, 16) <= sms) return {1, 8};
+  if (K <= 128) return few_blocks(T, N, 64) <= sms ? FewShape{1, 2} : K <= 64 && few_blocks(T, N, 128) <= sms ? FewShape{1, 1} : FewShape{0, 0};
+  if (few_blocks(T, N) <= sms) return {1, 4};
+  return T <= 256 && few_blocks(T, N, 64) * 4 <= sms * 3 ? FewShape{2, 4} : FewShape{0, 0};
+}
 // Warps that K is cut over for up to 32 tokens: as many as leave the blocks of 128 / ks weight rows one round on the SMs (three
 // resident blocks each, two with the registers of 16 tokens).  Second product of a pair, with its small first one, in a replayed
 // graph, us, ks = 8 / by this rule: 100 000 outputs, K = 32 at 1, 8, 16 tokens 18.8 / 4.7, 19.0 / 4.8, 30.3 / 7.5; 16 384 outputs, K = 150
@@ -855,33 +875,30 @@ int few_cut(int64_t T, int64_t N, int64_t K) {
   while (ks > 1 && (N * ks + 16 * few::kWarps - 1) / (16 * few::kWarps) > round) ks /= 2;
   return ks;
 }
-int launch_few(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
-               int64_t K, bool second, cudaStream_t st) {
-  const bf16* a = (const bf16*)A; const bf16* b = (const bf16*)B; bf16* c = (bf16*)C;
-  const int t = (int)T, n = (int)N, k = (int)K;
-  if (T <= 8) return launch_few_cut<1>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (T <= 16) return launch_few_cut<2>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  if (T <= 32) return launch_few_cut<4>(few_cut(T, N, K), a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  // 32 weight rows per block read half as many token rows in all; 16 where 32 would leave half of the SMs idle
-  if (few_blocks(T, N) * 2 >= num_sms()) return launch_few_inst<2, 8, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
-  return launch_few_inst<1, 8, 8>(a, lda, b, ldb, c, ldc, cs, t, n, k, second, st);
+int launch_few(const FewArgs& a, cudaStream_t st) {
+  if (a.T <= 8) return launch_few_cut<1>(few_cut(a.T, a.N, a.K), a, st);
+  if (a.T <= 16) return launch_few_cut<2>(few_cut(a.T, a.N, a.K), a, st);
+  if (a.T <= 32) return launch_few_cut<4>(few_cut(a.T, a.N, a.K), a, st);
+  const FewShape s = few_shape(a.T, a.N, a.K);
+  if (s.mt == 2) return s.ks == 8 ? launch_few_inst<2, 8, 8>(a, st) : launch_few_inst<2, 8, 4>(a, st);
+  return launch_few_cut<8>(s.ks, a, st);
 }
 // Whether a product takes the few-token kernel.  Up to 16 tokens always.  Up to 32 unless the weights are wide and large: every
 // group of 16 weight rows reads the tokens again, which a tcgen05 tile of 128 or 256 columns does not (32 tokens, K = 1024, us, this
-// kernel / tcgen05 tiles: 8192 outputs 8.1 / 11.2, 16 384 12.3 / 12.4, 32 768 20.0 / 15.1, 100 000 62.2 / 46.2).  Beyond, while its 32 x 64
-// blocks are one round over the SMs.  Both products of a pair in a replayed graph: 1024 -> 358 -> 4096 at 16, 64, 128 tokens
-// 4.7 / 11.9, 9.2 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024 tokens 16.2 / 26.6; at two rounds
-// it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
+// kernel / tcgen05 tiles: 8192 outputs 8.1 / 11.2, 16 384 12.3 / 12.4, 32 768 20.0 / 15.1, 100 000 62.2 / 46.2).  Beyond, by few_shape.  Both products of a pair in a replayed
+// graph: 1024 -> 358 -> 4096 at 16, 64, 128 tokens 4.7 / 11.9, 8.6 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024
+// tokens 16.2 / 26.6; at two rounds it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
 bool few_ok(int64_t T, int64_t N, int64_t K) {
   if (T < 1 || T > 1024 || N > INT32_MAX / 2 || K > INT32_MAX / 2 || tuning().no_few) return false;
   if (T <= 16) return true;
   if (T <= 32) return N < 16384 || N * K < 10000000;
-  return few_blocks(T, N) <= num_sms();
+  return few_shape(T, N, K).mt > 0;
 }
 // Forward product C = (A B^T) * col_scale of a layer, in the form the sizes call for.  `few`: the few-token kernel may serve it.
 int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, void* C, int64_t ldc, const float* cs, int64_t T, int64_t N,
-                       int64_t K, bool few, bool second, cudaStream_t st) {
-  if (few && few_ok(T, N, K)) return launch_few(A, lda, B, ldb, C, ldc, cs, T, N, K, second, st);
+                       int64_t K, bool few, bool second, cudaStream_t st, int64_t n_pad = 0, bool a_padded = false) {
+  if (few && few_ok(T, N, K))
+    return launch_few({(const bf16*)A, lda, (const bf16*)B, ldb, (bf16*)C, ldc, cs, (int)T, (int)N, (int)K, second, (int)std::max(N, n_pad), a_padded}, st);
   return launch_tc({A, lda, false}, {B, ldb, false}, T, N, K, plan_tc(T, N, K, false, false), store_epilogue(C, ldc, cs), st);
 }
 
@@ -1473,8 +1490,9 @@ int flop_compact_fwd(const void* X, int64_t ldx, const void* Qc, int64_t ldqc, c
   const FwdWs w = plan_fwd_ws(ar, T, k, dt);
   if (dt == FLOP_BF16) {
     if (!bf16_ok(Y, ldy) || !bf16_ok(X, ldx) || !bf16_ok(Qc, ldqc) || !bf16_ok(Pc, ldpc)) return FLOP_ERR_UNSUPPORTED;
-    FLOP_TRY(launch_fwd_product(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, true, false, st));
-    FLOP_TRY(launch_fwd_product(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, true, true, st));
+    // the rows of H' in the workspace are whole 16-byte pieces: the few-token kernel fills them up with zeros
+    FLOP_TRY(launch_fwd_product(X, ldx, Qc, ldqc, w.H, w.ldh, nullptr, T, k, d_in, true, false, st, w.ldh));
+    FLOP_TRY(launch_fwd_product(w.H, w.ldh, Pc, ldpc, Y, ldy, nullptr, T, d_out, k, true, true, st, 0, few_ok(T, k, d_in)));
   } else {
     FLOP_TRY(launch_simt({(const float*)X, ldx, true}, {(const float*)Qc, ldqc, true}, T, k, d_in, simt_out(w.H, w.ldh), st));
     FLOP_TRY(launch_simt({(const float*)w.H, w.ldh, true}, {(const float*)Pc, ldpc, true}, T, d_out, k, simt_out(Y, ldy), st));

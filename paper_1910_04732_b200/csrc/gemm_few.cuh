@@ -13,6 +13,11 @@
 //     rows enough, and with a short K the cut would leave warps without a step (the host picks KS);
 //   * a lane reads 16 contiguous bytes of a row per step: the k positions inside a step are permuted identically for both
 //     operands, so that those bytes serve two instructions without a shuffle;
+//   * with RAGGED (K no multiple of 8, more than 16 tokens) the 16 bytes across the end of a row are read whole and clipped in
+//     registers, but for the last row of a matrix, after which nothing need follow.  The first product of a pair fills the rows of
+//     H' in the workspace with zeros up to a piece (n_pad), so that the second clips its weights only (a_padded).  From single elements the end of a row costs a
+//     wait per row: 410 -> 150 -> 410 at 64 tokens 8.4 us, at 300 8.6, with RAGGED 5.9 and 6.8; up to 16 tokens there are few
+//     rows per lane and the extra registers and instructions cost more (one token: 3.4 against 3.7);
 //   * with EARLY the first weights are requested before the wait on the previous launch.  That is for the second product of
 //     a pair only: its predecessor on the stream is the first product, which waits for everything before it
 //     before it lets this launch start, and which writes H' and nothing else, so the weights are final.
@@ -33,10 +38,12 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// Eight elements of a row from k on, zero beyond K (rows are 16-byte aligned; nothing beyond K is read).
-__device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, int k, int K) {
+// Eight elements of a row from k on, zero beyond K (rows are 16-byte aligned), nothing beyond K being read unless `whole` says so:
+// then a piece across the end of the row is read with its padding, and the caller clips it when it is used.  (Putting a ragged
+// end together from single elements waits for them before the next load is issued.)
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, int k, int K, bool whole) {
   uint4 v = make_uint4(0, 0, 0, 0);
-  if (k + 8 <= K) {
+  if (k + 8 <= K || (whole && k < K)) {
     v = *reinterpret_cast<const uint4*>(row + k);
   } else if (k < K) {
     __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(&v);
@@ -46,14 +53,19 @@ __device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, in
   }
   return v;
 }
+// The first `left` of eight elements, zeros after them.
+__device__ __forceinline__ uint4 clip8(uint4 v, int left) {
+  auto word = [&](uint32_t w, int i) { return left >= i + 2 ? w : left == i + 1 ? w & 0xffffu : 0u; };
+  return make_uint4(word(v.x, 0), word(v.y, 2), word(v.z, 4), word(v.w, 6));
+}
 
 __host__ __device__ constexpr int part_stride(int mt) { return 16 * mt + 4; }   // floats per token of a warp's partial tile: conflict-free writes
 __host__ __device__ constexpr int smem_bytes(int mt, int nt) { return kWarps * 8 * nt * part_stride(mt) * 4; }
 
-template <int MT, int NT, int KS, bool EARLY>
+template <int MT, int NT, int KS, bool EARLY, bool RAGGED>
 __global__ void __launch_bounds__(kThreads)
 gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat16* __restrict__ B, int64_t ldb,
-            __nv_bfloat16* __restrict__ C, int64_t ldc, const float* __restrict__ col_scale, int T, int N, int K) {
+            __nv_bfloat16* __restrict__ C, int64_t ldc, const float* __restrict__ col_scale, int T, int N, int K, int n_pad, int a_padded) {
   constexpr int kDepth = 2 * MT + NT <= 4 ? 4 : 2;         // steps of loads in flight: up to 24 16-byte loads per lane
   constexpr int kGroups = kWarps / KS;                     // groups of weight rows side by side in the block, KS warps each
   extern __shared__ __align__(16) float part[];            // [kGroups][KS][8 NT][part_stride(MT)]
@@ -61,17 +73,24 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
   const int n0 = (blockIdx.x * kGroups + warp / KS) * 16 * MT, t0 = blockIdx.y * 8 * NT;
   const __nv_bfloat16* wrow[2 * MT];                       // rows past the end are read from the last row and not stored
   const __nv_bfloat16* trow[NT];
+  uint32_t wwhole = 0, twhole = 0;                         // RAGGED, bit i: another row follows row i in its matrix
 #pragma unroll
-  for (int i = 0; i < 2 * MT; ++i) wrow[i] = B + (int64_t)min(n0 + 8 * i + g, N - 1) * ldb;
+  for (int i = 0; i < 2 * MT; ++i) {
+    wrow[i] = B + (int64_t)min(n0 + 8 * i + g, N - 1) * ldb;
+    if (RAGGED && n0 + 8 * i + g < N - 1) wwhole |= 1u << i;
+  }
 #pragma unroll
-  for (int i = 0; i < NT; ++i) trow[i] = A + (int64_t)min(t0 + 8 * i + g, T - 1) * lda;
+  for (int i = 0; i < NT; ++i) {
+    trow[i] = A + (int64_t)min(t0 + 8 * i + g, T - 1) * lda;
+    if (RAGGED && (a_padded || t0 + 8 * i + g < T - 1)) twhole |= 1u << i;
+  }
   float acc[MT][NT][4] = {};
   uint4 wv[kDepth][2 * MT], tv[kDepth][NT];
   auto load_weights = [&](int s) {
 #pragma unroll
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
-      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * KS) * 32 + 8 * q, K);
+      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * KS) * 32 + 8 * q, K, RAGGED && ((wwhole >> i) & 1u));
   };
   if (!EARLY) pdl_wait();
   load_weights(k_warp);
@@ -82,9 +101,18 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
 #pragma unroll
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
-      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * KS) * 32 + 8 * q, K);
+      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * KS) * 32 + 8 * q, K, RAGGED && ((twhole >> i) & 1u));
 #pragma unroll
-    for (int d = 0; d < kDepth; ++d)
+    for (int d = 0; d < kDepth; ++d) {
+      const int at = (s + d * KS) * 32;
+      if (RAGGED && at + 32 > K) {                         // the whole warp: the row's end is here, or behind
+#pragma unroll
+        for (int i = 0; i < 2 * MT; ++i) wv[d][i] = clip8(wv[d][i], K - at - 8 * q);
+        if (!a_padded) {
+#pragma unroll
+          for (int i = 0; i < NT; ++i) tv[d][i] = clip8(tv[d][i], K - at - 8 * q);
+        }
+      }
 #pragma unroll
       for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -93,6 +121,7 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
           mma_bf16_16816(acc[m][n], lo.x, hi.x, lo.y, hi.y, t.x, t.y);
           mma_bf16_16816(acc[m][n], lo.z, hi.z, lo.w, hi.w, t.z, t.w);
         }
+    }
   }
   // lane (g, q) holds rows 16 m + g and + 8, tokens 8 n + 2 q and + 1
   constexpr int S = part_stride(MT);
@@ -114,10 +143,12 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
       x += v.x; y += v.y;
     }
     const int n = (blockIdx.x * kGroups + grp) * 16 * MT + c;
-    if (t0 + t < T && n < N) {
-      if (col_scale) { x *= __ldg(col_scale + n); if (n + 1 < N) y *= __ldg(col_scale + n + 1); }
+    if (t0 + t < T && n < n_pad) {
+      if (n >= N) x = 0.f;
+      if (n + 1 >= N) y = 0.f;
+      if (col_scale && n < N) { x *= __ldg(col_scale + n); if (n + 1 < N) y *= __ldg(col_scale + n + 1); }
       __nv_bfloat16* o = C + (int64_t)(t0 + t) * ldc + n;
-      if (n + 1 < N) *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(x, y);   // rows are 16-byte aligned, n is even
+      if (n + 1 < n_pad) *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(x, y);   // rows are 16-byte aligned, n is even
       else *o = __float2bfloat16_rn(x);
     }
   }
