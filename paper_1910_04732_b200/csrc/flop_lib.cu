@@ -853,7 +853,8 @@ int64_t few_blocks(int64_t T, int64_t N, int64_t rows = 32) { return ((N + rows 
 // on K has eight 32-long steps to deal out.  Second product of a pair with a first of K = 64, replayed, us, before (32 rows, or
 // tcgen05 beyond a round of them) / by this rule: K = 40: 100 x 4096 outputs 7.0 / 5.4, 256 x 2048 6.4 / 5.3; K = 100: 100 x 4096 7.2 / 5.6,
 // 512 x 512 7.0 / 5.6; K = 160: 150 x 1024 5.8 / 5.0, 150 x 2048 7.0 / 6.4; K = 256: 100 x 4096 7.8 / 7.2.  Lines, this kernel / tcgen05: K = 100,
-// 384 x 2048 7.6 / 7.6 (2 x 2), 512 x 1024 6.7 / 6.6; K = 160, 256 x 2048 7.2 / 6.7, 384 x 1024 7.2 / 6.8; K = 300, 150 x 2048 9.5 / 7.4.
+// 384 x 2048 7.6 / 7.6 (2 x 2), 512 x 1024 6.7 / 6.6; K = 160, 256 x 2048 7.2 / 6.7, 384 x 1024 7.2 / 6.8; K = 250, 200 x 1700 7.9 / 7.3;
+// K = 300, 150 x 2048 9.5 / 7.4.
 struct FewShape { int mt, ks; };
 FewShape few_shape(int64_t T, int64_t N, int64_t K) {
   const int64_t sms = num_sms();
@@ -861,7 +862,7 @@ FewShape few_shape(int64_t T, int64_t N, int64_t K) {
   if (few_blocks(T, N, 16) <= sms) return {1, 8};
   if (K <= 128) return few_blocks(T, N, 64) <= sms ? FewShape{1, 2} : K <= 64 && few_blocks(T, N, 128) <= sms ? FewShape{1, 1} : FewShape{0, 0};
   if (few_blocks(T, N) <= sms) return {1, 4};
-  return T <= 256 && few_blocks(T, N, 64) * 4 <= sms * 3 ? FewShape{2, 4} : FewShape{0, 0};
+  return T <= 256 && few_blocks(T, N, 64) * 10 <= sms * 7 ? FewShape{2, 4} : FewShape{0, 0};
 }
 // Warps that K is cut over for up to 32 tokens: as many as leave the blocks of 128 / ks weight rows one round on the SMs (three
 // resident blocks each, two with the registers of 16 tokens).  Second product of a pair, with its small first one, in a replayed

@@ -51,7 +51,7 @@ def test_block_shapes(b, T, k, d_out):
     """Every block shape above 32 tokens, ragged and whole."""
     d_in, g = 72, torch.Generator(device="cuda").manual_seed(T + k)
     X, Q, P = _matrix(g, T, d_in, 1.0), _matrix(g, k, d_in, d_in ** -0.5), _matrix(g, d_out, k, k ** -0.5)
-    Y = torch.full((T, d_out + 8), float("nan"), dtype=BF16, device="cuda")[:, :d_out]
+    Y = torch.full((T, (d_out + 15) // 8 * 8), float("nan"), dtype=BF16, device="cuda")[:, :d_out]
     b.compact_fwd(X, Q, P, Y, k, b.alloc_workspace(b.workspace_bytes(b.OP_COMPACT_FWD, T, d_in, d_out, k, b.BF16)))
     exact = X.double() @ Q.double().T
     want = exact.to(BF16).double() @ P.double().T
