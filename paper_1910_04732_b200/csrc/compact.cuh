@@ -324,7 +324,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the selection, and in pieces it takes 16).  Surviving columns of further rows of P are read straight from global memory, two
 // per lane: neighbouring lanes read neighbouring survivors, so a load touches only a few lines.
 // Measured, the 72 matrices of a BERT-base-shaped model: three launches each 1364 us (13.0 + 4.0 + 5.8 us of GPU time per matrix);
-// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us (399 with Q prefetched).  Two blocks per SM, which repeat the selection twice,
+// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us (399 with Q prefetched, 391 with the gates).  Two blocks per SM, which repeat the selection twice,
 // 444 (66 MB of factors, r = 1021: 257 against 270); one block of 1024 threads 455 (longer barriers); held to 40 or 32 registers,
 // so that more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
@@ -538,6 +538,7 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
       for (int64_t b = lane * 128; b < cols * (int64_t)sizeof(T); b += 32 * 128)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(m + (int64_t)i * ld) + b));
   };
+  if (warp == 0 && lane * 32 < r) asm volatile("prefetch.global.L2 [%0];" ::"l"(in + lane * 32));      // the gates: 128 bytes a lane
   prefetch(P, ldp, d_out, r);
   if (pieces == 1 && d_in > 0) prefetch(Q, ldq, r, d_in);
   for (int i = tid; i < kFineBins; i += kFusedThreads) sh.hist[i] = 0;
