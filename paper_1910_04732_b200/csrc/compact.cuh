@@ -316,7 +316,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // and goes straight on to its rows.  What makes the repetition cheap: gates stay in registers (kKeys per thread), ordinary
 // gates need no fp64 and one histogram (select_fast; the rest goes to select_general), and positions come from ballots and a scan
 // of the 32 words by every warp.  The fp64 probabilities are evaluated only where they are results: one per row of Q_c, by the warp
-// that scales it, and z_det spread over the blocks.
+// that scales it and writes it to z_det (a pass over z_det at the end of the block cost 850 cycles of about 8000).
 // A warp then takes one row at a time: P rows first (their number is known before the selection, so the rows are
 // prefetched into L2 while the previous launch on the stream still runs, and the warp's first one is staged in shared memory
 // during the selection), then the surviving rows of Q in pieces of at most
@@ -324,7 +324,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the selection, and in pieces it takes 16).  Surviving columns of further rows of P are read straight from global memory, two
 // per lane: neighbouring lanes read neighbouring survivors, so a load touches only a few lines.
 // Measured, the 72 matrices of a BERT-base-shaped model: three launches each 1364 us (13.0 + 4.0 + 5.8 us of GPU time per matrix);
-// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us (399 with Q prefetched, 391 with the gates).  Two blocks per SM, which repeat the selection twice,
+// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us (399 with Q prefetched, 391 with the gates, 381 with z_det written beside Q_c).  Two blocks per SM, which repeat the selection twice,
 // 444 (66 MB of factors, r = 1021: 257 against 270); one block of 1024 threads 455 (longer barriers); held to 40 or 32 registers,
 // so that more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
 // Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
@@ -514,6 +514,7 @@ __device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kK
     if (j < r && bin[n] == cut) {
       const unsigned long long mine = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)j);
       int rank = 0;
+#pragma unroll 8
       for (int i = 0; i < n_close; ++i) rank += sh.close[i] > mine;
       if (rank < need) keep |= 1u << n;
     }
@@ -625,7 +626,10 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (j + u * 32 * V < full) raw[u] = *reinterpret_cast<const uint4*>(q + j + u * 32 * V);
-        if (first) g = mode == 0 ? probability(sh.v[c], thr) : sh.v[c];         // while the first loads are on their way
+        if (first) {                                       // while the first loads are on their way
+          g = mode == 0 ? probability(sh.v[c], thr) : sh.v[c];
+          if (z_det && j0 == 0 && lane == 0) z_det[sh.idx[c]] = g;
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (j + u * 32 * V < full) {
@@ -638,11 +642,12 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
       for (int j = max(full, j0) + lane; j < j1; j += 32) o[j] = from_f32<T>(to_f32<T>(q[j]) * g);
     }
   }
-  if (z_det) {       // a few gates per block: their fp64 probabilities hold nobody up here
+  if (z_det) {       // the dropped gates, a few per block; the kept ones are written with their rows of Q (here when there are none)
 #pragma unroll
     for (int n = 0; n < kKeys; ++n) {
       const int j = n * kFusedThreads + tid;
-      if (j < r && j % (int)gridDim.x == (int)blockIdx.x) z_det[j] = !((keep >> n) & 1u) ? 0.f : mode == 0 ? probability(v[n], thr) : v[n];
+      const bool kept = (keep >> n) & 1u;
+      if (j < r && j % (int)gridDim.x == (int)blockIdx.x && (!kept || pieces == 0)) z_det[j] = !kept ? 0.f : mode == 0 ? probability(v[n], thr) : v[n];
     }
   }
 }
