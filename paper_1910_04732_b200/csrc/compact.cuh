@@ -342,6 +342,7 @@ constexpr int kKeys = kFusedMaxR / kFusedThreads;   // gates per thread
 constexpr int kFusedWords = kKeys * kFusedWarps;    // 32-gate words, one per lane of a warp that scans them
 static_assert(kFusedWords == 32, "a warp scans all words at once");
 constexpr int kFineBins = 1024, kCloseGates = 64;
+constexpr double kFastThr = 1 << 20;    // largest |thr| of select_fast
 // Shared memory for one row of P per warp, staged while the selection runs.
 template <typename T> __host__ __device__ constexpr size_t fused_row_bytes(int64_t r) { return ((size_t)r * sizeof(T) + 15) & ~(size_t)15; }
 
@@ -449,12 +450,15 @@ __device__ __noinline__ unsigned select_general(FusedShared& sh, float v0, float
 }
 
 // The same decision for ordinary gates in a third of the time; false (for the whole block) when it is not certain here.
-//   k: probabilities in fp32, added as 20-bit fixed point (order-free, one instruction per warp).  A gate is off by at most half a
-//      unit of rounding and 0.42 of fp32 error (|x| e^-|x| times a few 2^-24, and two units in the last place of the quotient), so
-//      the sum is off by less than r units, and floor(sum + 1/2) is that of fp64 unless the sum lies within r + 16 units of a half.
+//   k: probabilities p = 1 / (1 + e^x), x = thr - v, in fp32, added as 20-bit fixed point (order-free, one instruction per warp).  thr
+//      comes as the sum of two floats: rounded to one it would move every x the same way, by up to 2^-25 |thr| (at beta = 100 and gates
+//      near thr 2000 units for 1024 gates).  As (hi - v) + lo, x is off by 2^-23 |x|, and by less than 2^-27 up to kFastThr.  In
+//      units of 2^-20 that is at most 0.03 + 0.01 of p; __expf, good to 2 + 1.173 |x| units in its last place, adds 0.08, the sum
+//      1 + e^x 0.07 and the quotient, two units in its last place, 0.25: with the half unit of rounding a gate is off by less than
+//      one, the sum by less than r, and floor(sum + 1/2) is that of fp64 unless the sum lies within r + 16 units of a half.
 //   k-th largest: 1024 bins between the smallest and the largest gate (finite ones; the map to a bin is monotone in fp32 arithmetic),
 //      found through 32 coarse sums; the gates of its bin, a few, are ranked against one another on (value, lower index first).
-__device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kKeys], unsigned& keep, float thr, int r) {
+__device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kKeys], unsigned& keep, float thr, float thr_lo, int r) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint32_t lo = 0xffffffffu, hi = 0u, fixed = 0u;
 #pragma unroll
@@ -462,7 +466,7 @@ __device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kK
     if (n * kFusedThreads + tid < r) {
       const uint32_t key = order_key(v[n]);
       lo = min(lo, key); hi = max(hi, fabsf(v[n]) <= FLT_MAX ? key : 0xffffffffu);     // the key of no finite gate
-      fixed += __float2uint_rn(__fdividef(1048576.f, 1.f + __expf(thr - v[n])));
+      fixed += __float2uint_rn(__fdividef(1048576.f, 1.f + __expf((thr - v[n]) + thr_lo)));
     }
   lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi); fixed = __reduce_add_sync(0xffffffffu, fixed);
   if (lane == 0) { sh.lo[warp] = lo; sh.hi[warp] = hi; sh.fixed[warp] = fixed; }
@@ -562,7 +566,7 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
   }
   unsigned keep = 0;     // bit n: gate n of this thread survives
   if (mode == 0) {
-    if (!select_fast(sh, v, keep, (float)thr, r)) keep = select_general(sh, v[0], v[1], thr, r);
+    if (!(fabs(thr) <= kFastThr) || !select_fast(sh, v, keep, (float)thr, (float)(thr - (double)(float)thr), r)) keep = select_general(sh, v[0], v[1], thr, r);
   } else {
 #pragma unroll
     for (int n = 0; n < kKeys; ++n)

@@ -73,3 +73,31 @@ def test_survivors(b, kind, r):
         k, idx, _ = O.deterministic_mask(a, *HC)
         assert one[0] == k and np.array_equal(one[1][:k], idx)
     assert b.device_status() == b.OK
+
+
+def _count_gates(hc, r, units):
+    """fp32 gates around the constants' threshold whose fp64 probabilities sum to a half plus about `units` * 2^-20."""
+    thr = hc[0] * np.log(-hc[1] / hc[2])
+    p = lambda x: 1.0 / (1.0 + np.exp(-(x.astype(np.float64) - thr)))  # noqa: E731
+    a = (thr + np.random.default_rng([r, int(hc[0])]).normal(0.0, 0.3, r)).astype(np.float32)
+    rest = p(a[1:]).sum()
+    want = (0.5 + units * 2.0 ** -20 - rest) % 1.0
+    a[0] = thr + np.log(want / (1.0 - want))
+    return a
+
+
+# k = floor(sum + 1/2) must be the fp64 one wherever the fp32 sum is taken for certain: it declines within r + 16 units of 2^-20
+@pytest.mark.parametrize("beta,gamma,zeta", [HC, (1.0, -0.5, 1.5), (20.0, -0.1, 1.1), (100.0, -0.1, 1.1), (100.0, -1.1, 1.1), (1000.0, -0.1, 1.1),
+                                             (1e5, -0.1, 1.1), (1e7, -0.1, 1.1)])
+def test_count_near_a_half(b, beta, gamma, zeta):
+    hc = tuple(float(np.float32(v)) for v in (beta, gamma, zeta))
+    for r in (300, 1024):
+        for units in (0.0, 0.02 * r, 0.25 * r, 0.5 * r, 0.75 * r, r + 20.0, r + 200.0, 1.5 * r, 3.0 * r):
+            for sign in (1.0, -1.0):
+                a = _count_gates(hc, r, sign * units)
+                gates = torch.from_numpy(a).cuda()
+                idx, kd = torch.full((r,), -1, dtype=torch.int32, device="cuda"), torch.full((1,), -1, dtype=torch.int32, device="cuda")
+                b.compact_ranks(gates, 0, hc, idx, kd, torch.empty(r, device="cuda"))
+                k, want, _ = O.deterministic_mask(a, *hc)
+                assert int(kd.item()) == k and np.array_equal(idx.cpu().numpy()[:k], want), (r, sign * units)
+    assert b.device_status() == b.OK
