@@ -27,6 +27,7 @@
 #include "gemm_tc2_chain.cuh"
 #include "gemm_tc_chainfwd.cuh"
 #include "l0_lagrangian.cuh"
+#include "per_device.cuh"
 #include "wgrad.cuh"
 #include "active_ranks.cuh"
 #include "gemm_few.cuh"
@@ -131,19 +132,18 @@ inline bool valid_hc(const flop_hc_params_t& hc) { return hc.beta > 0.f && hc.ga
 
 // Per-device state (function attributes already set, SM count, built-in scratch address) is indexed by the
 // current device, so that a process that drives several GPUs configures each of them.
-constexpr int kMaxDevices = 64;
 inline int current_device() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return -1; }
   return (dev >= 0 && dev < kMaxDevices) ? dev : -1;
 }
-// True the first time it is called for (flag array, current device): the caller then sets its function attributes.
-inline bool first_use_on_device(bool (&done)[kMaxDevices]) {
-  const int dev = current_device();
-  if (dev < 0) return true;            // unknown device: configure every time
-  if (done[dev]) return false;
-  done[dev] = true;
-  return true;
+// Lets kernels be launched with up to `bytes` of dynamic shared memory on the current device.
+template <typename... Kernels>
+int allow_smem(OncePerDevice& once, size_t bytes, Kernels... kernels) {
+  return once(current_device(), [&]() -> int {
+    for (const void* k : {reinterpret_cast<const void*>(kernels)...}) FLOP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return FLOP_OK;
+  });
 }
 
 int num_sms() {
@@ -360,13 +360,10 @@ struct TcJob {
 
 template <bool A_MN, bool B_MN, int EPI>
 int launch_group_inst(const tc::GroupParams& gp, int cta2, double flops, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
+  static OncePerDevice configured;
   auto kern1 = tc::gemm_group_kernel<A_MN, B_MN, EPI>;
   auto kern2 = tc::gemm2_group_kernel<A_MN, B_MN, EPI>;
-  if (first_use_on_device(configured)) {
-    FLOP_CUDA(cudaFuncSetAttribute(kern1, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-    FLOP_CUDA(cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-  }
+  FLOP_TRY(allow_smem(configured, kSmemBudget, kern1, kern2));
   {
     GemmTimer timer(st, flops);
     if (!cta2) {
@@ -396,9 +393,9 @@ int launch_group_inst(const tc::GroupParams& gp, int cta2, double flops, cudaStr
 // gradients with both operands MN-major (the two steps of the grouped backward pass).  CTA pairs only.
 template <bool B0_MN, int E1>   // B operand of the stores; epilogue of the products that contract over tokens
 int launch_dual_inst(const tc::GroupParams& gp, double flops, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
+  static OncePerDevice configured;
   auto kern = tc::gemm2_dual_kernel<false, B0_MN, tc::EPI_STORE, true, true, E1>;
-  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+  FLOP_TRY(allow_smem(configured, kSmemBudget, kern));
   {
     GemmTimer timer(st, flops);
     const int smem = kSmemFixed + gp.stages * (int)tc::stage_bytes2(gp.bn_max);
@@ -537,9 +534,9 @@ constexpr size_t kSyncBytes = 64 * 1024;   // size of a sync area (flop_sync_byt
 
 template <bool A0, bool B0, int E0, bool A1, bool B1, int E1>
 int launch_chain_inst(const tc::GroupParams& gp, int pairs, double flops, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
+  static OncePerDevice configured;
   auto kern = tc::gemm2_chain_kernel<A0, B0, E0, A1, B1, E1>;
-  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+  FLOP_TRY(allow_smem(configured, kSmemBudget, kern));
   {
     GemmTimer timer(st, flops);
     const int smem = kSmemFixed + gp.stages * (int)tc::stage_bytes2(gp.bn_max);
@@ -787,9 +784,8 @@ int launch_chain_fwd(const void* X, int64_t ldx, const void* Q, int64_t ldq, con
     return FLOP_ERR_UNSUPPORTED;
   const int64_t row_blocks = (T + tc::BM - 1) / tc::BM;
   if (row_blocks > 65535) return FLOP_ERR_UNSUPPORTED;
-  static bool configured[kMaxDevices] = {};
-  if (first_use_on_device(configured))
-    FLOP_CUDA(cudaFuncSetAttribute(tc::chain_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kChainSmemBytes));
+  static OncePerDevice configured;
+  FLOP_TRY(allow_smem(configured, tc::kChainSmemBytes, tc::chain_fwd_kernel));
   tc::ChainFwdParams cp;
   memset(&cp, 0, sizeof(cp));
   FLOP_TRY(make_tmap(&cp.tx, X, T, d_in, ldx, tc::BK, tc::BM));
@@ -821,10 +817,10 @@ int launch_chain_fwd(const void* X, int64_t ldx, const void* Q, int64_t ldq, con
 struct FewArgs { const bf16* A; int64_t lda; const bf16* B; int64_t ldb; bf16* C; int64_t ldc; const float* cs; int T, N, K; bool second; int n_pad, a_padded; };
 template <int MT, int NT, int KS, bool EARLY, bool RAGGED>
 int launch_few_kernel(const FewArgs& a, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
+  static OncePerDevice configured;
   constexpr int smem = few::smem_bytes(MT, NT);
   auto kern = few::gemm_kernel<MT, NT, KS, EARLY, RAGGED>;
-  if (smem > 48 * 1024 && first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  if (smem > 48 * 1024) FLOP_TRY(allow_smem(configured, smem, kern));
   constexpr int rows = 16 * MT * (few::kWarps / KS);       // weight rows per block
   const dim3 grid((unsigned)((a.N + rows - 1) / rows), (unsigned)((a.T + 8 * NT - 1) / (8 * NT)));
   launch_k(kern, grid, dim3(few::kThreads), (size_t)smem, st, a.A, a.lda, a.B, a.ldb, a.C, a.ldc, a.cs, a.T, a.N, a.K, a.n_pad, a.a_padded);
@@ -907,8 +903,8 @@ int launch_fwd_product(const void* A, int64_t lda, const void* B, int64_t ldb, v
 struct SimtOperand { const float* ptr; int64_t ld; bool k_fast; };
 
 template <typename... KArgs>
-int launch_simt_kernel(void (*kern)(KArgs...), bool (&configured)[kMaxDevices], dim3 grid, cudaStream_t st, const KArgs&... args) {
-  if (first_use_on_device(configured)) FLOP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kSmemBytes));
+int launch_simt_kernel(void (*kern)(KArgs...), OncePerDevice& configured, dim3 grid, cudaStream_t st, const KArgs&... args) {
+  FLOP_TRY(allow_smem(configured, simt::kSmemBytes, kern));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = dim3(simt::kThreads); cfg.dynamicSmemBytes = simt::kSmemBytes; cfg.stream = st;
   cudaLaunchAttribute attr[2];
@@ -925,7 +921,7 @@ int launch_simt_kernel(void (*kern)(KArgs...), bool (&configured)[kMaxDevices], 
 }
 template <bool A_K, bool B_K, bool SCALE_K>
 int launch_simt_inst(const SimtGemmArgs& a, dim3 grid, cudaStream_t st) {
-  static bool configured[kMaxDevices] = {};
+  static OncePerDevice configured;
   auto kern = simt::gemm_kernel<A_K, B_K, SCALE_K>;
   return launch_simt_kernel(kern, configured, grid, st, a);
 }
@@ -982,7 +978,7 @@ int launch_simt_dual(const SimtJob& act, const SimtJob& wgrad, cudaStream_t st) 
   d.wgrad_clusters = (int)((wgrad_tiles + wgrad_per - 1) / wgrad_per);
   d.wgrad_first = d.wgrad.kb_per_split > d.act.kb_per_split;
   const dim3 grid((unsigned)(d.act_clusters + d.wgrad_clusters), 1, (unsigned)size);
-  static bool configured[2][kMaxDevices] = {};
+  static OncePerDevice configured[2];
   return act.a.k_scale ? launch_simt_kernel(simt::gemm_dual_kernel<true>, configured[1], grid, st, d)
                        : launch_simt_kernel(simt::gemm_dual_kernel<false>, configured[0], grid, st, d);
 }
@@ -1120,9 +1116,8 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
   const int vec_p = aligned16(P) && (ldp * sizeof(T)) % 16 == 0;
   const int pair_p = reinterpret_cast<uintptr_t>(Pc) % (2 * sizeof(T)) == 0 && ldpc % 2 == 0;
   const size_t smem = d_out > 0 ? kFusedWarps * fused_row_bytes<T>(r) : 0;
-  static bool configured[kMaxDevices] = {};
-  if (first_use_on_device(configured))
-    FLOP_CUDA(cudaFuncSetAttribute(compact_fused_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kFusedWarps * fused_row_bytes<T>(kFusedMaxR))));
+  static OncePerDevice configured;
+  FLOP_TRY(allow_smem(configured, kFusedWarps * fused_row_bytes<T>(kFusedMaxR), compact_fused_kernel<T>));
   const int pieces = fused_pieces(d_in);
   const int64_t rows = d_out + r * pieces;                                   // a warp each, at most one block per SM
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kFusedWarps - 1) / kFusedWarps, (int64_t)num_sms()));
@@ -2427,9 +2422,8 @@ int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t h
         while (nbuf > 2 && need(nbuf) > 100 * 1024) --nbuf;   // two blocks per SM where the rows allow it
         if (need(nbuf) <= (size_t)kSmemBudget) {
           const size_t sm = need(nbuf);
-          static bool configured[kMaxDevices] = {};
-          if (sm > 48 * 1024 && first_use_on_device(configured))
-            FLOP_CUDA(cudaFuncSetAttribute(gather_p_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget));
+          static OncePerDevice configured;
+          if (sm > 48 * 1024) FLOP_TRY(allow_smem(configured, kSmemBudget, gather_p_pipe_kernel));
           const int64_t groups = (d_out + rows_per_stage - 1) / rows_per_stage;
           const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(8, (size_t)(224 * 1024) / sm));
           const int grid = (int)std::min<int64_t>(groups, (int64_t)num_sms() * per_sm);
