@@ -137,7 +137,8 @@ inline int current_device() {
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return -1; }
   return (dev >= 0 && dev < kMaxDevices) ? dev : -1;
 }
-// Lets kernels be launched with up to `bytes` of dynamic shared memory on the current device.
+// Lets kernels be launched with up to `bytes` of dynamic shared memory on the current device: the most that any call asks for, since
+// the limit belongs to the kernel and a smaller call's would take it from a larger one on another thread.
 template <typename... Kernels>
 int allow_smem(OncePerDevice& once, size_t bytes, Kernels... kernels) {
   return once(current_device(), [&]() -> int {
@@ -1136,6 +1137,12 @@ static int launch_compact_fused(const float* in, int mode, double thr, int64_t r
   return FLOP_OK;
 }
 
+template <typename T>
+static int allow_gather_p() {
+  static OncePerDevice configured;
+  return allow_smem(configured, kSmemBudget, gather_p_kernel<T>);
+}
+
 // Room for the split-K slices of dO: the query knows the tokens and the cluster's width but not the output width d, so
 // it reserves 8 bytes per element of dH' (2 T / d slices of d_i x d floats), at most 64 MB; the call splits no finer.
 static size_t embedding_slice_bytes(int64_t T, int64_t d_i) {
@@ -1155,7 +1162,8 @@ template <int LPT>
 static int launch_embed_bwd(const int32_t* ids, int64_t T, const void* E, int64_t lde, int64_t n_rows, const float* z, int64_t d_i,
                             const bf16* dH, int64_t lddh, float* dE, int64_t ldde, float* part, int runs, cudaStream_t st) {
   const size_t smem = (size_t)kEmbWarps * d_i * 4;
-  if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(embed_bwd_kernel<LPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static OncePerDevice configured;
+  if (smem > 48 * 1024) FLOP_TRY(allow_smem(configured, kSmemBudget, embed_bwd_kernel<LPT>));
   launch_k(embed_bwd_kernel<LPT>, dim3((unsigned)embedding_blocks(T, runs)), dim3(32 * kEmbWarps), smem, st, ids, (int)T, (const bf16*)E, lde,
            (int)n_rows, z, (int)d_i, dH, lddh, dE, ldde, part, runs);
   return FLOP_OK;
@@ -2120,7 +2128,8 @@ int flop_active_ranks_gather(const flop_active_gather_t* pr, int n, int dt, void
     launch_k(active_select_kernel, dim3(g.n), dim3(1024), (size_t)0, st, g);
     const int row_elems = (max_r + 7) & ~7;   // per-warp staging row, 16-byte aligned
     const size_t smem = (size_t)row_elems * 2 * kActiveWarps;
-    if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(active_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static OncePerDevice configured;
+    if (smem > 48 * 1024) FLOP_TRY(allow_smem(configured, kSmemBudget, active_gather_kernel));
     launch_k(active_gather_kernel, dim3((max_blocks + kActiveWarps - 1) / kActiveWarps, g.n), dim3(32 * kActiveWarps), smem, st, g, row_elems);
     count_launch(2);
     FLOP_CUDA(cudaGetLastError());
@@ -2438,19 +2447,19 @@ int flop_compact_ranks(const float* log_alpha_or_z, int mode, flop_hc_params_t h
           launch_k(gather_p_pipe_kernel, dim3((unsigned)grid), dim3(256), sm, st, (const bf16*)P, ldp, idx, k_dev, (int)r, (int)d_out,
                    (bf16*)Pc, ldpc, rows_per_stage, nbuf);
         } else {
-          if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(gather_p_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+          if (smem > 48 * 1024) FLOP_TRY(allow_gather_p<bf16>());
           launch_k(gather_p_kernel<bf16>, dim3((unsigned)((d_out + rows_per_block - 1) / rows_per_block)), dim3(256), (size_t)(smem), st,
               (const bf16*)P, ldp, idx, k_dev, (int)r, (int)d_out, (bf16*)Pc, ldpc, rows_per_block, vp);
         }
       } else if (d_out > 0) {
-        if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(gather_p_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem > 48 * 1024) FLOP_TRY(allow_gather_p<bf16>());
         launch_k(gather_p_kernel<bf16>, dim3((unsigned)((d_out + rows_per_block - 1) / rows_per_block)), dim3(256), (size_t)(smem), st, 
             (const bf16*)P, ldp, idx, k_dev, (int)r, (int)d_out, (bf16*)Pc, ldpc, rows_per_block, vp);
       }
     } else {
       if (d_in > 0) launch_k(gather_q_kernel<float>, dim3((unsigned)r), dim3(256), (size_t)(0), st, (const float*)Q, ldq, idx, k_dev, zsrc, (int)d_in, (float*)Qc, ldqc, vq);
       if (d_out > 0) {
-        if (smem > 48 * 1024) FLOP_CUDA(cudaFuncSetAttribute(gather_p_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem > 48 * 1024) FLOP_TRY(allow_gather_p<float>());
         launch_k(gather_p_kernel<float>, dim3((unsigned)((d_out + rows_per_block - 1) / rows_per_block)), dim3(256), (size_t)(smem), st, 
             (const float*)P, ldp, idx, k_dev, (int)r, (int)d_out, (float*)Pc, ldpc, rows_per_block, vp);
       }
