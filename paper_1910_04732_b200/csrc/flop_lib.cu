@@ -840,7 +840,10 @@ int launch_few_kernel(const FewArgs& a, cudaStream_t st) {
 template <int MT, int NT, int KS>
 int launch_few_inst(const FewArgs& a, cudaStream_t st) {
   if constexpr (NT > 2) {
-    if (a.K % 8) return a.second ? launch_few_kernel<MT, NT, KS, true, true>(a, st) : launch_few_kernel<MT, NT, KS, false, true>(a, st);
+    // With NT = 4 the clipping takes the registers of a third resident block, which outputs of more than two rounds of blocks lose
+    // more by: second product at 17 tokens, 348 x 5478, 4.7 us without RAGGED, 5.3 with; 18 tokens, 73 x 4855, 4.2 and 5.0.
+    constexpr int rows = 16 * MT * (few::kWarps / KS);
+    if (a.K % 8 && (NT > 4 || (a.N + rows - 1) / rows <= 2 * num_sms())) return a.second ? launch_few_kernel<MT, NT, KS, true, true>(a, st) : launch_few_kernel<MT, NT, KS, false, true>(a, st);
   }
   return a.second ? launch_few_kernel<MT, NT, KS, true, false>(a, st) : launch_few_kernel<MT, NT, KS, false, false>(a, st);
 }

@@ -15,9 +15,12 @@
 //     operands, so that those bytes serve two instructions without a shuffle;
 //   * with RAGGED (K no multiple of 8, more than 16 tokens) the 16 bytes across the end of a row are read whole and clipped in
 //     registers, but for the last row of a matrix, after which nothing need follow.  The first product of a pair fills the rows of
-//     H' in the workspace with zeros up to a piece (n_pad), so that the second clips its weights only (a_padded).  From single elements the end of a row costs a
-//     wait per row: 410 -> 150 -> 410 at 64 tokens 8.4 us, at 300 8.6, with RAGGED 5.9 and 6.8; up to 16 tokens there are few
-//     rows per lane and the extra registers and instructions cost more (one token: 3.4 against 3.7);
+//     H' in the workspace with zeros up to a piece (n_pad), so that the second clips its weights only (a_padded).  From single elements
+//     the end of a row costs a wait per row.  Kernel times of the two products, us, single elements / RAGGED: 300 tokens,
+//     410 -> 150 -> 410 5.2 + 6.0 / 4.1 + 3.8; 100 tokens, 3001 -> 100 -> 500 11.3 + 4.2 / 8.7 + 3.6; 64 tokens, K = 358, 4096 outputs
+//     5.6 / 5.4.  What cost RAGGED its gain before: rows past the end taken for the last row, whose end came from single elements
+//     as well (37 tokens, 38 -> 203, 4.2 us), and a look at each row in every step (36 tokens, K = 3098, 12.6; now 3.5 and 9.8).
+//     Up to 16 tokens there are few rows per lane and the extra registers and instructions cost more (one token: 3.4 against 3.7);
 //   * with EARLY the first weights are requested before the wait on the previous launch.  That is for the second product of
 //     a pair only: its predecessor on the stream is the first product, which waits for everything before it
 //     before it lets this launch start, and which writes H' and nothing else, so the weights are final.
@@ -40,11 +43,27 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
 }
 // Eight elements of a row from k on, zero beyond K (rows are 16-byte aligned), nothing beyond K being read unless `whole` says so:
 // then a piece across the end of the row is read with its padding, and the caller clips it when it is used.  (Putting a ragged
-// end together from single elements waits for them before the next load is issued.)
+// end together from single elements waits for them before the next load is issued.)  With RAGGED the end of a row that is not read
+// whole comes in up to three aligned loads, each straight to its registers: K % 8 is the same for all rows, and nothing waits.
+template <bool RAGGED>
 __device__ __forceinline__ uint4 load8(const __nv_bfloat16* __restrict__ row, int k, int K, bool whole) {
   uint4 v = make_uint4(0, 0, 0, 0);
   if (k + 8 <= K || (whole && k < K)) {
     v = *reinterpret_cast<const uint4*>(row + k);
+  } else if (RAGGED && k < K) {
+    const int left = K & 7;                                // (k is a multiple of 8)
+    const __nv_bfloat16* p = row + k;
+    auto u16 = [](const __nv_bfloat16* a) { return (uint32_t)*reinterpret_cast<const unsigned short*>(a); };
+    auto u32 = [](const __nv_bfloat16* a) { return *reinterpret_cast<const uint32_t*>(a); };
+    if (left & 4) {
+      const uint2 two = *reinterpret_cast<const uint2*>(p);
+      v.x = two.x; v.y = two.y;
+      if (left & 2) { v.z = u32(p + 4); if (left & 1) v.w = u16(p + 6); }
+      else if (left & 1) v.z = u16(p + 4);
+    } else {
+      if (left & 2) { v.x = u32(p); if (left & 1) v.y = u16(p + 2); }
+      else if (left & 1) v.x = u16(p);
+    }
   } else if (k < K) {
     __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(&v);
 #pragma unroll
@@ -74,23 +93,40 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
   const __nv_bfloat16* wrow[2 * MT];                       // rows past the end are read from the last row and not stored
   const __nv_bfloat16* trow[NT];
   uint32_t wwhole = 0, twhole = 0;                         // RAGGED, bit i: another row follows row i in its matrix
+  // with RAGGED from the last row but one, which is read whole: at 17 tokens a group's rows past the end are half of them
+  auto row_read = [](int row, int rows) { return RAGGED ? (row < rows ? row : max(rows - 2, 0)) : min(row, rows - 1); };
 #pragma unroll
   for (int i = 0; i < 2 * MT; ++i) {
-    wrow[i] = B + (int64_t)min(n0 + 8 * i + g, N - 1) * ldb;
-    if (RAGGED && n0 + 8 * i + g < N - 1) wwhole |= 1u << i;
+    const int row = row_read(n0 + 8 * i + g, N);
+    wrow[i] = B + (int64_t)row * ldb;
+    if (RAGGED && row < N - 1) wwhole |= 1u << i;
   }
 #pragma unroll
   for (int i = 0; i < NT; ++i) {
-    trow[i] = A + (int64_t)min(t0 + 8 * i + g, T - 1) * lda;
-    if (RAGGED && (a_padded || t0 + 8 * i + g < T - 1)) twhole |= 1u << i;
+    const int row = row_read(t0 + 8 * i + g, T);
+    trow[i] = A + (int64_t)row * lda;
+    if (RAGGED && (a_padded || row < T - 1)) twhole |= 1u << i;
   }
   float acc[MT][NT][4] = {};
   uint4 wv[kDepth][2 * MT], tv[kDepth][NT];
+  // this lane's part of the step at column `at` of some rows; only the step across the end of the rows, in the warps that have a last
+  // row, looks at each of them
+  auto load_step = [&](auto& v, const auto& rows, uint32_t whole, int at) {
+    constexpr int n = sizeof(v) / sizeof(v[0]);
+    if (RAGGED && at + 32 > K && __all_sync(0xffffffffu, whole == (1u << n) - 1u)) {
+#pragma unroll
+      for (int i = 0; i < n; ++i) v[i] = at + 8 * q < K ? *reinterpret_cast<const uint4*>(rows[i] + at + 8 * q) : make_uint4(0, 0, 0, 0);
+    } else if (RAGGED && at + 32 > K) {
+#pragma unroll
+      for (int i = 0; i < n; ++i) v[i] = load8<true>(rows[i], at + 8 * q, K, (whole >> i) & 1u);
+    } else {
+#pragma unroll
+      for (int i = 0; i < n; ++i) v[i] = RAGGED ? *reinterpret_cast<const uint4*>(rows[i] + at + 8 * q) : load8<false>(rows[i], at + 8 * q, K, false);
+    }
+  };
   auto load_weights = [&](int s) {
 #pragma unroll
-    for (int d = 0; d < kDepth; ++d)
-#pragma unroll
-      for (int i = 0; i < 2 * MT; ++i) wv[d][i] = load8(wrow[i], (s + d * KS) * 32 + 8 * q, K, RAGGED && ((wwhole >> i) & 1u));
+    for (int d = 0; d < kDepth; ++d) load_step(wv[d], wrow, wwhole, (s + d * KS) * 32);
   };
   if (!EARLY) pdl_wait();
   load_weights(k_warp);
@@ -99,9 +135,7 @@ gemm_kernel(const __nv_bfloat16* __restrict__ A, int64_t lda, const __nv_bfloat1
   for (int s = k_warp; s * 32 < K; s += kDepth * KS) {
     if (s != k_warp) load_weights(s);
 #pragma unroll
-    for (int d = 0; d < kDepth; ++d)
-#pragma unroll
-      for (int i = 0; i < NT; ++i) tv[d][i] = load8(trow[i], (s + d * KS) * 32 + 8 * q, K, RAGGED && ((twhole >> i) & 1u));
+    for (int d = 0; d < kDepth; ++d) load_step(tv[d], trow, twhole, (s + d * KS) * 32);
 #pragma unroll
     for (int d = 0; d < kDepth; ++d) {
       const int at = (s + d * KS) * 32;
