@@ -314,7 +314,7 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // of dependent steps, and as a launch of its own (one block of 1024 threads, 13 us) it kept 147 SMs waiting.  Here
 // every block repeats the selection in its own shared memory -- r gates are 4 KB, L2-resident after the first block --
 // and goes straight on to its rows.  What makes the repetition cheap: gates stay in registers (kKeys per thread), ordinary
-// gates need no fp64 and one histogram (select_fast; the rest goes to select_general), and positions come from ballots and a scan
+// gates need no fp64 and one histogram (select_largest), and positions come from ballots and a scan
 // of the 32 words by every warp.  The fp64 probabilities are evaluated only where they are results: one per row of Q_c, by the warp
 // that scales it and writes it to z_det (a pass over z_det at the end of the block cost 850 cycles of about 8000).
 // A warp then takes one row at a time: P rows first (their number is known before the selection, so the rows are
@@ -342,7 +342,7 @@ constexpr int kKeys = kFusedMaxR / kFusedThreads;   // gates per thread
 constexpr int kFusedWords = kKeys * kFusedWarps;    // 32-gate words, one per lane of a warp that scans them
 static_assert(kFusedWords == 32, "a warp scans all words at once");
 constexpr int kFineBins = 1024, kCloseGates = 64;
-constexpr double kFastThr = 1 << 20;    // largest |thr| of select_fast
+constexpr double kFastThr = 1 << 20;    // largest |thr| for which k is taken from fp32 probabilities
 // Shared memory for one row of P per warp, staged while the selection runs.
 template <typename T> __host__ __device__ constexpr size_t fused_row_bytes(int64_t r) { return ((size_t)r * sizeof(T) + 15) & ~(size_t)15; }
 
@@ -369,7 +369,7 @@ __device__ __forceinline__ int warp_find(int count, int lane, int* need) {
 }
 
 struct FusedShared {
-  __align__(16) int hist[kFineBins];           // fine bins of the fast selection, or four times 256 of the general one
+  __align__(16) int hist[kFineBins];
   int coarse[32];
   unsigned long long close[kCloseGates];
   double red[kFusedWarps];
@@ -382,57 +382,99 @@ struct FusedShared {
 // P(z > 0) as the deterministic gate, evaluated in fp64 (out of line: it is needed once per row and must not cost the kernel registers).
 __device__ __noinline__ float probability(float a, double thr) { return (float)(1.0 / (1.0 + exp(-((double)a - thr)))); }
 
-// Which of this thread's gates are among the k = floor(sum of probabilities + 1/2) largest, for any input (NaN, infinities, all
-// equal, sums next to a half): k from fp64 probabilities, the k-th largest by four histogram passes over the gates' bits.
-// Bit n of the result: gate n is kept.
-__device__ __noinline__ unsigned select_general(FusedShared& sh, float v0, float v1, double thr, int r) {
+// k = floor(sum of the probabilities + 1/2) from fp64 probabilities.
+__device__ __noinline__ int count_f64(FusedShared& sh, float v0, float v1, double thr, int r) {
   static_assert(kKeys == 2, "two gates per thread");
-  const float v[kKeys] = {v0, v1};
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  __syncthreads();
-  for (int i = tid; i < kFineBins; i += kFusedThreads) sh.hist[i] = 0;
+  const int tid = threadIdx.x, lane = tid & 31;
   double sum = 0.0;
-#pragma unroll
-  for (int n = 0; n < kKeys; ++n)
-    if (n * kFusedThreads + tid < r) sum += 1.0 / (1.0 + exp(-((double)v[n] - thr)));
+  if (tid < r) sum += 1.0 / (1.0 + exp(-((double)v0 - thr)));
+  if (kFusedThreads + tid < r) sum += 1.0 / (1.0 + exp(-((double)v1 - thr)));
   sum = warp_sum_f64(sum);
-  if (lane == 0) sh.red[warp] = sum;
-  __syncthreads();   // histograms are zero, warp sums are there
+  if (lane == 0) sh.red[tid >> 5] = sum;
+  __syncthreads();
   sum = warp_sum_f64(lane < kFusedWarps ? sh.red[lane] : 0.0);
-  const int k = max(0, min(r, (int)floor(sum + 0.5)));
-  uint32_t prefix = 0, pmask = 0;
-  int need = k;       // rank (1-based, from the top) still to be located inside the prefix class
-#pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
-    int* hist = sh.hist + 256 * pass;
-#pragma unroll
-    for (int n = 0; n < kKeys; ++n) {
-      const uint32_t key = order_key(v[n]);
-      if (n * kFusedThreads + tid < r && (key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255], 1);
-    }
-    __syncthreads();
-    // lane l holds bins 255 - 8 l .. 248 - 8 l, so that a scan over the lanes counts from the top
-    int total = 0;
-    for (int i = 0; i < 8; ++i) total += hist[255 - 8 * lane - i];
-    int left = need;
-    const int at = warp_find(total, lane, &left);      // (none when k is 0)
-    if (at >= 0) {
-      int bin = 255 - 8 * at;
-      for (; left > hist[bin]; --bin) left -= hist[bin];
-      prefix |= (uint32_t)bin << shift;
-      need = left;
-    }
-    pmask |= 255u << shift;
-  }
-  // of the gates equal to the k-th largest, the `need` lowest indices are kept
-  unsigned keep = 0, eq = 0;
+  return max(0, min(r, (int)floor(sum + 0.5)));
+}
+
+__device__ __forceinline__ float key_value(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
+
+// One step towards the `need` largest of the active gates (bit n: gate n of this thread), whose keys lie in lo .. hi: they are counted
+// in 1024 bins, linear in the gate or in its key (both monotone; in fp32 arithmetic too, and with infinities in the end bins).  Gates
+// above the bin of the cut are kept, those of the bin stay active; up to kCloseGates of them are ranked against one another
+// on (value, lower index first).  True when all is decided.  The bins and n_close are zero before.
+__device__ __forceinline__ bool cut_pass(FusedShared& sh, const float (&v)[kKeys], unsigned& active, unsigned& keep, int& need, uint32_t lo,
+                                         uint32_t hi, bool linear) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float low = key_value(lo), scale = (kFineBins - 0.25f) / (key_value(hi) - low);
+  const int shift = max(0, 32 - __clz(hi - lo) - 10);
+  static_assert(kFineBins == 1 << 10, "ten bits of the keys' differences");
+  int bin[kKeys];      // counted from the largest gate down
 #pragma unroll
   for (int n = 0; n < kKeys; ++n) {
-    const bool in_range = n * kFusedThreads + tid < r && k > 0;
-    if (in_range && order_key(v[n]) > prefix) keep |= 1u << n;
-    if (in_range && order_key(v[n]) == prefix) eq |= 1u << n;
-    const uint32_t word = __ballot_sync(0xffffffffu, (eq >> n) & 1u);
+    const int up = linear ? (int)((v[n] - low) * scale) : (int)((order_key(v[n]) - lo) >> shift);
+    bin[n] = kFineBins - 1 - max(0, min(kFineBins - 1, up));
+    if ((active >> n) & 1u) atomicAdd(&sh.hist[bin[n]], 1);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 32 / kFusedWarps; ++i) {
+    const int c = warp * (32 / kFusedWarps) + i, sum = __reduce_add_sync(0xffffffffu, sh.hist[32 * c + lane]);
+    if (lane == 0) sh.coarse[c] = sum;
+  }
+  __syncthreads();
+  const int c = warp_find(sh.coarse[lane], lane, &need), cut = 32 * c + warp_find(sh.hist[32 * c + lane], lane, &need), count = sh.hist[cut];
+  const bool all = need == count;      // the cut falls between two bins
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    if (!((active >> n) & 1u)) continue;
+    if (bin[n] < cut || (all && bin[n] == cut)) keep |= 1u << n;
+    if (bin[n] != cut) active &= ~(1u << n);
+    else if (!all && count <= kCloseGates) sh.close[atomicAdd(&sh.n_close, 1)] = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)(n * kFusedThreads + tid));
+  }
+  if (all) return true;
+  if (count > kCloseGates) return false;
+  __syncthreads();
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n)
+    if ((active >> n) & 1u) {
+      const unsigned long long mine = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)(n * kFusedThreads + tid));
+      int rank = 0;
+#pragma unroll 8
+      for (int i = 0; i < count; ++i) rank += sh.close[i] > mine;
+      if (rank < need) keep |= 1u << n;
+    }
+  return true;
+}
+
+// The rest of the decision for many active gates close together or equal: bins between their own extremes, linear once and then on
+// the keys, whose range shrinks by 2^10 a pass, until the gates left are few or equal; of equal ones the lowest indices are kept.
+// Such gates are no exception (all equal after initialisation, two classes after clamping, one gate that ran away).  768 -> 768
+// at r = 768, us, ordinary gates 4.4: clamped 4.65, all equal 4.8, an outlier 5.4, a sum next to a half (count_f64) 4.9.  A selection
+// from the start for them (fp64 probabilities and four passes over the bits, after the attempt at the short way) took 8.7, 9.3, 9.1
+// and 8.2, more than before there was a short way at small ranks (256 -> 768: clamped 7.7 against 5.4, now 3.9).
+__device__ __noinline__ unsigned cut_again(FusedShared& sh, float v0, float v1, unsigned active, int need) {
+  const float v[kKeys] = {v0, v1};
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned keep = 0;
+#pragma unroll 1
+  for (bool linear = true;; linear = false) {
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+    for (int n = 0; n < kKeys; ++n)
+      if ((active >> n) & 1u) { lo = min(lo, order_key(v[n])); hi = max(hi, order_key(v[n])); }
+    lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi);
+    __syncthreads();     // the bins and extremes of the pass before have been read
+    if (lane == 0) { sh.lo[warp] = lo; sh.hi[warp] = hi; }
+    for (int i = tid; i < kFineBins; i += kFusedThreads) sh.hist[i] = 0;
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, sh.lo[lane % kFusedWarps]);
+    hi = __reduce_max_sync(0xffffffffu, sh.hi[lane % kFusedWarps]);
+    if (lo == hi) break;
+    if (cut_pass(sh, v, active, keep, need, lo, hi, linear && fabsf(key_value(lo)) <= FLT_MAX && fabsf(key_value(hi)) <= FLT_MAX)) return keep;
+  }
+#pragma unroll
+  for (int n = 0; n < kKeys; ++n) {
+    const uint32_t word = __ballot_sync(0xffffffffu, (active >> n) & 1u);
     if (lane == 0) sh.words[n * kFusedWarps + warp] = word;
   }
   __syncthreads();
@@ -443,30 +485,35 @@ __device__ __noinline__ unsigned select_general(FusedShared& sh, float v0, float
   for (int n = 0; n < kKeys; ++n) {
     const int w = n * kFusedWarps + warp;
     const int rank = __shfl_sync(0xffffffffu, before, w) + __popc(__shfl_sync(0xffffffffu, word, w) & ((1u << lane) - 1u));
-    if (((eq >> n) & 1u) && rank < need) keep |= 1u << n;
+    if (((active >> n) & 1u) && rank < need) keep |= 1u << n;
   }
   __syncthreads();   // the words are written again
   return keep;
 }
 
-// The same decision for ordinary gates in a third of the time; false (for the whole block) when it is not certain here.
+// Which of this thread's gates are among the k = floor(sum of probabilities + 1/2) largest (bit n of the result: gate n).
 //   k: probabilities p = 1 / (1 + e^x), x = thr - v, in fp32, added as 20-bit fixed point (order-free, one instruction per warp).  thr
 //      comes as the sum of two floats: rounded to one it would move every x the same way, by up to 2^-25 |thr| (at beta = 100 and gates
 //      near thr 2000 units for 1024 gates).  As (hi - v) + lo, x is off by 2^-23 |x|, and by less than 2^-27 up to kFastThr.  In
 //      units of 2^-20 that is at most 0.03 + 0.01 of p; __expf, good to 2 + 1.173 |x| units in its last place, adds 0.08, the sum
 //      1 + e^x 0.07 and the quotient, two units in its last place, 0.25: with the half unit of rounding a gate is off by less than
-//      one, the sum by less than r, and floor(sum + 1/2) is that of fp64 unless the sum lies within r + 16 units of a half.
-//   k-th largest: 1024 bins between the smallest and the largest gate (finite ones; the map to a bin is monotone in fp32 arithmetic),
-//      found through 32 coarse sums; the gates of its bin, a few, are ranked against one another on (value, lower index first).
-__device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kKeys], unsigned& keep, float thr, float thr_lo, int r) {
+//      one, the sum by less than r, and floor(sum + 1/2) is that of fp64 unless the sum lies within r + 16 units of a half.  Only
+//      then, and beyond kFastThr, the fp64 probabilities are evaluated.
+//   k-th largest: bins between the smallest and the largest finite gate, and again between the gates of the cut's bin while those are
+//      many (a class of equal gates, a distant gate that stretches the bins).
+__device__ __forceinline__ unsigned select_largest(FusedShared& sh, const float (&v)[kKeys], double thr, int r) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const float thr_hi = (float)thr, thr_lo = (float)(thr - (double)thr_hi);
   uint32_t lo = 0xffffffffu, hi = 0u, fixed = 0u;
+  unsigned active = 0, keep = 0;
 #pragma unroll
   for (int n = 0; n < kKeys; ++n)
     if (n * kFusedThreads + tid < r) {
       const uint32_t key = order_key(v[n]);
-      lo = min(lo, key); hi = max(hi, fabsf(v[n]) <= FLT_MAX ? key : 0xffffffffu);     // the key of no finite gate
-      fixed += __float2uint_rn(__fdividef(1048576.f, 1.f + __expf((thr - v[n]) + thr_lo)));
+      active |= 1u << n;
+      if (fabsf(v[n]) <= FLT_MAX) { lo = min(lo, key); hi = max(hi, key); }
+      if (v[n] != v[n]) hi = 0xffffffffu;     // NaN: the key of no finite gate
+      fixed += __float2uint_rn(__fdividef(1048576.f, 1.f + __expf((thr_hi - v[n]) + thr_lo)));
     }
   lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi); fixed = __reduce_add_sync(0xffffffffu, fixed);
   if (lane == 0) { sh.lo[warp] = lo; sh.hi[warp] = hi; sh.fixed[warp] = fixed; }
@@ -474,56 +521,13 @@ __device__ __forceinline__ bool select_fast(FusedShared& sh, const float (&v)[kK
   lo = __reduce_min_sync(0xffffffffu, sh.lo[lane % kFusedWarps]);
   hi = __reduce_max_sync(0xffffffffu, sh.hi[lane % kFusedWarps]);
   fixed = __reduce_add_sync(0xffffffffu, lane < kFusedWarps ? sh.fixed[lane] : 0u) + (1u << 19);
+  if (hi == 0xffffffffu) return 0;            // the sum is NaN, which counts as none
   const uint32_t part = fixed & 0xfffffu, margin = (uint32_t)r + 16u;
-  if (r == 0 || hi == 0xffffffffu || part <= margin || part >= 0x100000u - margin) return false;
-  int need = min(r, (int)(fixed >> 20));
-  auto value = [](uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); };
-  const float low = value(lo), scale = (kFineBins - 0.25f) / (value(hi) - low);
-  int bin[kKeys];      // counted from the largest gate down
-#pragma unroll
-  for (int n = 0; n < kKeys; ++n) {
-    bin[n] = kFineBins - 1 - max(0, min(kFineBins - 1, (int)((v[n] - low) * scale)));
-    if (n * kFusedThreads + tid < r) atomicAdd(&sh.hist[bin[n]], 1);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 32 / kFusedWarps; ++i) {
-    const int c = warp * (32 / kFusedWarps) + i, sum = __reduce_add_sync(0xffffffffu, sh.hist[32 * c + lane]);
-    if (lane == 0) sh.coarse[c] = sum;
-  }
-  __syncthreads();
-  int cut = -1;        // bin of the k-th largest; none when k is 0
-  if (need > 0) {
-    const int c = warp_find(sh.coarse[lane], lane, &need);
-    cut = 32 * c + warp_find(sh.hist[32 * c + lane], lane, &need);
-  }
-  const bool all = cut >= 0 && need == sh.hist[cut];      // the cut falls between two bins
-  keep = 0;
-#pragma unroll
-  for (int n = 0; n < kKeys; ++n) {
-    const int j = n * kFusedThreads + tid;
-    if (j < r && (bin[n] < cut || (all && bin[n] == cut))) keep |= 1u << n;
-    if (!all && j < r && bin[n] == cut) {
-      const int at = atomicAdd(&sh.n_close, 1);
-      if (at < kCloseGates) sh.close[at] = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)j);
-    }
-  }
-  if (all || cut < 0) return true;
-  __syncthreads();
-  const int n_close = sh.n_close;
-  if (n_close > kCloseGates) return false;
-#pragma unroll
-  for (int n = 0; n < kKeys; ++n) {
-    const int j = n * kFusedThreads + tid;
-    if (j < r && bin[n] == cut) {
-      const unsigned long long mine = ((unsigned long long)order_key(v[n]) << 32) | (0xffffffffu - (uint32_t)j);
-      int rank = 0;
-#pragma unroll 8
-      for (int i = 0; i < n_close; ++i) rank += sh.close[i] > mine;
-      if (rank < need) keep |= 1u << n;
-    }
-  }
-  return true;
+  const bool sure = fabs(thr) <= kFastThr && part > margin && part < 0x100000u - margin;
+  int need = sure ? min(r, (int)(fixed >> 20)) : count_f64(sh, v[0], v[1], thr, r);
+  if (need == 0) return 0;
+  if (!cut_pass(sh, v, active, keep, need, lo, hi, true)) keep |= cut_again(sh, v[0], v[1], active, need);
+  return keep;
 }
 
 template <typename T>
@@ -566,7 +570,7 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
   }
   unsigned keep = 0;     // bit n: gate n of this thread survives
   if (mode == 0) {
-    if (!(fabs(thr) <= kFastThr) || !select_fast(sh, v, keep, (float)thr, (float)(thr - (double)(float)thr), r)) keep = select_general(sh, v[0], v[1], thr, r);
+    keep = select_largest(sh, v, thr, r);
   } else {
 #pragma unroll
     for (int n = 0; n < kKeys; ++n)

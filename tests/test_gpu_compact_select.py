@@ -1,5 +1,5 @@
-"""Survivors chosen inside the one-launch compaction: the binned selection and the general one it hands over to, against the
-oracle and against the separate launches (which a call takes when z_det overwrites the gates).  Indices and values are exact."""
+"""Survivors chosen inside the one-launch compaction, whatever the gates ask of its bins (one pass over them or several, gates ranked or
+equal, k from fp32 or fp64 probabilities), against the oracle and against the separate launches (which a call takes when z_det overwrites the gates).  Indices and values are exact."""
 import numpy as np
 import pytest
 import torch
@@ -46,12 +46,23 @@ def _gates(kind, r):
         a = np.where(g.random(r) < 0.5, 3e38, -3e38) * g.random(r)
     elif kind == "infinite":
         a[:: 5], a[1:: 7] = np.inf, -np.inf
+    elif kind == "clamped":         # two classes of equal gates
+        a = np.where(g.random(r) < 0.4, 4.0, -4.0)
+    elif kind == "scales":          # distances over 76 decades: several passes over the bins
+        a = np.sign(a) * 10.0 ** g.uniform(-38.0, 38.0, r)
+    elif kind == "steps":           # neighbouring numbers, many of them equal
+        a = 1.0 + np.round(40.0 * g.random(r)) * 2.0 ** -23
+    elif kind == "masked":          # hard-pruned gates
+        a = np.where(g.random(r) < 0.5, -np.inf, a)
+    elif kind == "signs":           # equal to the selection
+        a = np.where(g.random(r) < 0.5, 0.0, -0.0)
     elif kind == "nan":
         a[r // 3] = np.nan
     return a.astype(np.float32)
 
 
-@pytest.mark.parametrize("kind", ["normal", "bimodal", "far", "ties", "equal", "half", "none", "every", "wide", "infinite", "nan"])
+@pytest.mark.parametrize("kind", ["normal", "bimodal", "far", "ties", "equal", "half", "none", "every", "wide", "infinite", "clamped", "scales", "steps", "masked",
+                                  "signs", "nan"])
 @pytest.mark.parametrize("r", [1, 2, 65, 511, 513, 768, 1024])
 def test_survivors(b, kind, r):
     a, d_in, d_out = _gates(kind, r), 24, 40
@@ -69,7 +80,7 @@ def test_survivors(b, kind, r):
     assert one[0] == three[0]
     for x, y in zip(one[1:], three[1:]):
         assert np.array_equal(x, y, equal_nan=x.dtype.kind == "f")
-    if kind not in ("infinite", "nan"):
+    if kind != "nan":
         k, idx, _ = O.deterministic_mask(a, *HC)
         assert one[0] == k and np.array_equal(one[1][:k], idx)
     assert b.device_status() == b.OK
