@@ -978,6 +978,17 @@ bool simt_dual_ok(const SimtJob& act, const SimtJob& wgrad) {      // one work l
          std::max((act.M + simt::BM - 1) / simt::BM, (wgrad.M + simt::BM - 1) / simt::BM) <= 65535 &&
          std::max(simt_tiles(act.M, act.N), simt_tiles(wgrad.M, wgrad.N)) <= INT32_MAX / 2;
 }
+// Sharing fills places (two CTAs per SM) that a product alone leaves idle.  Not where both take nearly all of them in clusters of one or
+// two (larger clusters leave some): backward pass, us, five launches / three: 2048 tokens of 768 -> 768 312 / 315; 554 tokens of
+// 483 -> 532, clusters of four, 79 / 64.  Nor where the one cut in two does, in the eight-CTA clusters of the other, four of its
+// tiles at a time: 128 tokens of 768 -> 768 39.3 / 40.0, 160 tokens 57.0 / 59.1 (just below the line, 128 of 700 -> 700, 39.9 / 39.5).
+bool simt_dual_faster(const SimtJob& act, const SimtJob& wgrad) {
+  const int64_t act_tiles = simt_tiles(act.M, act.N), wgrad_tiles = simt_tiles(wgrad.M, wgrad.N), nearly_all = (int64_t)num_sms() * 2 * 15 / 16;
+  const int act_split = simt_split(act_tiles, simt_blocks(act.K)), wgrad_split = simt_split(wgrad_tiles, simt_blocks(wgrad.K));
+  const bool act_fills = act_tiles * act_split >= nearly_all, wgrad_fills = wgrad_tiles * wgrad_split >= nearly_all;
+  if (act_fills && wgrad_fills && std::max(act_split, wgrad_split) <= 2) return false;
+  return !(act_fills && act_split == 2 && wgrad_split == 8) && !(wgrad_fills && wgrad_split == 2 && act_split == 8);
+}
 int launch_simt_dual(const SimtJob& act, const SimtJob& wgrad, cudaStream_t st) {
   const int64_t act_tiles = simt_tiles(act.M, act.N), wgrad_tiles = simt_tiles(wgrad.M, wgrad.N);
   simt::DualArgs d{act.a, wgrad.a};
@@ -1643,13 +1654,13 @@ int flop_gated_lowrank_bwd(const void* dY, int64_t lddy, const void* X, int64_t 
     const flop_bwd_problem_t one{dY, lddy, X, ldx, Q, ldq, P, ldp, z, dz_dla, H_save, ldh, dX, lddx, dP, lddp, dQ, lddq, dlog_alpha,
                                  T, d_in, d_out, r, ws, ws_bytes, nullptr, nullptr, 0, 0};
     const bool apart = merged_apart(&one, 1, dt, wgrad_dt);
-    if (dP && apart && simt_dual_ok(dh, dp)) {
+    if (dP && apart && simt_dual_ok(dh, dp) && simt_dual_faster(dh, dp)) {
       FLOP_TRY(launch_simt_dual(dh, dp, st));
     } else {
       FLOP_TRY(launch_simt(dh, st));
       if (dP) FLOP_TRY(launch_simt(dp, st));
     }
-    const bool shared = need_m && dX && apart && simt_dual_ok(dx, dq);
+    const bool shared = need_m && dX && apart && simt_dual_ok(dx, dq) && simt_dual_faster(dx, dq);
     if (shared) FLOP_TRY(launch_simt_dual(dx, dq, st));
     else if (need_m) FLOP_TRY(launch_simt(dq, st));
     if (dlog_alpha) {

@@ -45,3 +45,14 @@ def test_shared_launch_has_the_bits_of_separate_ones(b, T, d_in, d_out, r, accum
     for a, c in zip(shared, separate):
         assert torch.equal(a, c)
     assert b.device_status() == b.OK
+
+
+@pytest.mark.parametrize("T,d,launches", [(100, 768, 5), (160, 768, 5), (2048, 768, 5), (128, 700, 3), (200, 768, 3), (554, 512, 3)])
+def test_products_that_fill_the_sms_keep_their_launches(b, T, d, launches):
+    """The line of the shared launches on 148 SMs: each alone with nearly two blocks per SM (5) or not (3)."""
+    rand = lambda *s: torch.randn(*s, device="cuda")  # noqa: E731
+    ws = b.alloc_workspace(b.workspace_bytes(b.OP_BWD, T, d, d, d, b.F32))
+    before = b.launch_count()
+    b.gated_lowrank_bwd(rand(T, d), rand(T, d), rand(d, d), rand(d, d), rand(d), rand(d), rand(T, d), rand(T, d), rand(d, d), rand(d, d), rand(d), ws)
+    assert b.launch_count() - before == launches
+    assert b.device_status() == b.OK
