@@ -755,8 +755,9 @@ MergedShape plan_merged(const flop_bwd_problem_t* pr, int n) {
 }
 
 // Whether the shared launches may stand in for the launches per product: the first writes dP while dH' still reads dY and P (and
-// X and Q are read after it), the second writes dX and dQ while the other of the two still reads X and Q.  One after another,
-// dX may take the place of X, and split weight gradients the place of anything but Q.
+// X and Q are read after it), the second writes dX and dQ while the other of the two still reads X, Q and the gates, and before the
+// gates' derivatives are read.  One after another, dX may take the place of X or of these, and split weight gradients the place of
+// anything but Q.
 bool merged_apart(const flop_bwd_problem_t* pr, int n, int dt, int wgrad_dt) {
   const size_t es = elt(dt);
   for (int i = 0; i < n; ++i) {
@@ -769,6 +770,7 @@ bool merged_apart(const flop_bwd_problem_t* pr, int n, int dt, int wgrad_dt) {
         if (dP.meets(in)) return false;
       for (const Span& in : {X, Q})
         if (dP.meets(in) || dQ.meets(in) || dX.meets(in)) return false;
+      if (dX.meets(Span(o.z, 1, o.r, o.r, 4)) || dX.meets(Span(o.dz_dla, 1, o.r, o.r, 4))) return false;
     }
   }
   return true;

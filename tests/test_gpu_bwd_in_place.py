@@ -44,3 +44,29 @@ def test_dx_on_x_and_dp_on_p(b, T, d, r, n):
             assert_close(P, G["dP"], "bf16", "dP")
             assert_close(dQ, G["dQ"], "bf16", "dQ")
     assert b.device_status() == b.OK
+
+
+@pytest.mark.parametrize("kind,T,d,r", [("f32", 200, 96, 64), ("bf16", 200, 96, 64), ("bf16", 1000, 768, 768)])
+def test_dx_on_the_gates_derivatives(b, kind, T, d, r):
+    """dX takes the place of d z / d log_alpha, which a launch per product has read by then."""
+    dt, f32 = (torch.float32, True) if kind == "f32" else (torch.bfloat16, False)
+    g = np.random.default_rng(T + d)
+    X, dY = to_dev(g.standard_normal((T, d)), kind), to_dev(g.standard_normal((T, d)), kind)
+    Q, P = to_dev(g.standard_normal((r, d)) * d ** -0.5, kind), to_dev(g.standard_normal((d, r)) * r ** -0.5, kind)
+    z = torch.from_numpy(g.uniform(0.1, 1.0, r).astype(np.float32)).cuda()
+    H, Y = empty_dev(T, r, dt), empty_dev(T, d, dt)
+    b.gated_lowrank_fwd(X, Q, P, z, Y, H, None)
+    dX = empty_dev(T, d, dt)
+    dz = dX.flatten().view(torch.float32)[:r]
+    assert dz.data_ptr() == dX.data_ptr()
+    dz.copy_(torch.from_numpy(g.uniform(0.5, 1.5, r).astype(np.float32)))
+    dz_host = host(dz)
+    G = O.gated_lowrank_bwd(host(dY), host(X), host(Q), host(P), host(z), dz_host)
+    dP, dQ, dla = empty_dev(d, r, dt), empty_dev(r, d, dt), torch.zeros(r, device="cuda")
+    b.gated_lowrank_bwd(dY, X, Q, P, z, dz, H, dX, dP, dQ, dla, b.alloc_workspace(b.workspace_bytes(b.OP_BWD, T, d, d, r, b.F32 if f32 else b.BF16)))
+    for got, name in ((dX, "dX"), (dP, "dP"), (dQ, "dQ")):
+        assert_close(got, G[name], kind, name)
+    # dlog_alpha sums products of both signs: its error is measured against the sum of their magnitudes
+    size = np.sum(np.abs(host(Q)) * (np.abs(host(dY) @ host(P)).T @ np.abs(host(X))), axis=1) * dz_host
+    assert np.all(np.abs(host(dla) - G["dlog_alpha"]) <= (1e-5 if f32 else 2.0 ** -6) * size + 1e-6)
+    assert b.device_status() == b.OK
