@@ -15,14 +15,16 @@ def b():
     return binding
 
 
-# 64 x 64 tiles and slices of (dH', dP, dX, dQ) for 148 SMs in the comments
+# 64 x 64 tiles x slices of (dH', dP, dX, dQ) for 148 SMs in the comments
 @pytest.mark.parametrize("T,d_in,d_out,r", [
     (64, 64, 768, 64),       # 1 x 8, 12 x 1, 1 x 1, 1 x 1
     (1100, 100, 60, 60),     # 18 x 1, 1 x 8, 36 x 1, 2 x 8
-    (200, 320, 256, 192),    # 12 x 2, 12 x 2, 20 x 2, 15 x 2
-    (520, 128, 256, 128),    # 18 x 2, 8 x 4, 18 x 1, 4 x 4
-    (2048, 200, 700, 130),   # 96 x 2, 33 x 8, 128 x 1, 12 x 8
-    (1500, 640, 640, 640),   # more tiles than SMs
+    (200, 320, 256, 192),    # 12 x 4, 12 x 2, 20 x 2, 15 x 2
+    (200, 320, 300, 192),    # 12 x 4, 15 x 2 in clusters of four (half of the last one empty), 20 x 2, 15 x 2
+    (300, 130, 1400, 130),   # 15 x 8, 66 x 4 in clusters of eight, 15 x 2 in clusters of four (half of the last one empty), 9 x 4
+    (520, 128, 256, 128),    # 18 x 4, 8 x 8, 18 x 2, 4 x 8
+    (2048, 200, 700, 130),   # 96 x 2, 33 x 8, 128 x 2, 12 x 8
+    (1500, 640, 640, 640),   # 240 x 1, 100 x 2 of both: more tiles than SMs
 ])
 @pytest.mark.parametrize("accumulate", [False, True])
 def test_shared_launch_has_the_bits_of_separate_ones(b, T, d_in, d_out, r, accumulate):
