@@ -20,6 +20,9 @@
  *     accumulation and needs every bf16 leading dimension to be a multiple of
  *     8 elements and every bf16 base pointer to be 16-byte aligned
  *     (FLOP_ERR_UNSUPPORTED otherwise).  FLOP_F32 computes in fp32 FMA.
+ *   - Columns of an input between a row's end and its leading dimension do not
+ *     reach any result, but up to the next multiple of 16 bytes they may be read
+ *     (not behind the last row).
  *   - Errors are return codes.  Arguments are checked on the host before
  *     anything is launched.  A device-side wait that runs out (a pipeline
  *     barrier that never completes) makes the kernel stop cleanly and record
@@ -395,8 +398,8 @@ int flop_agp_gates(const float* g, int64_t n, const int64_t* seg_off, int32_t n_
                    float l1, float* z, uint8_t* mask, float* dz_dg, float* seg_l1, float* dg, void* stream);
 
 /* Deterministic gates and compaction of one weight matrix (Sections 4.4, 4.1).
- * mode 0: log_alpha_or_z holds log_alpha; k = floor(sum_j pi_j + 1/2); the k
- *         gates with the largest log_alpha are kept (ties: lower index) with
+ * mode 0: log_alpha_or_z holds log_alpha; k = floor(sum_j pi_j + 1/2), as the
+ *         sum in fp64 gives it; the k gates with the largest log_alpha are kept (ties: lower index) with
  *         value pi_j, the rest are 0.
  * mode 1: log_alpha_or_z holds a gate vector z; component j is kept iff z_j > 0.
  * Writes idx[r] (first k entries valid, ascending), k_dev[1], z_det[r]

@@ -324,12 +324,14 @@ gather_p_pipe_kernel(const __nv_bfloat16* __restrict__ P, int64_t ldp, const int
 // the selection, and in pieces it takes 16).  Surviving columns of further rows of P are read straight from global memory, two
 // per lane: neighbouring lanes read neighbouring survivors, so a load touches only a few lines.
 // Measured, the 72 matrices of a BERT-base-shaped model: three launches each 1364 us (13.0 + 4.0 + 5.8 us of GPU time per matrix);
-// one launch with four histogram passes and all probabilities in fp64 643 us; this form 423 us (399 with Q prefetched, 391 with the gates, 381 with z_det written beside Q_c).  Two blocks per SM, which repeat the selection twice,
-// 444 (66 MB of factors, r = 1021: 257 against 270); one block of 1024 threads 455 (longer barriers); held to 40 or 32 registers,
-// so that more of the next launch's blocks could be resident early, 578 and 782 us (spills in the chain).
-// Ranks up to 1024 and P up to 16 MB: with more gates per thread the repeated selection costs more than the launches it
-// saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74), and for long P the staged
-// gather above streams better (1024 x 40 000: 54 against 49 us; 1024 x 4096: 17.6 against 26.1).
+// one launch with four histogram passes and all probabilities in fp64 643-694 us; this form 383 us, with clamped gates 400, all equal 448.
+// Against an earlier form of it that took 423: two blocks per SM, which repeat the selection twice, 444 (66 MB of factors, r = 1021:
+// 257 against 270); one block of 1024 threads 455 (longer barriers); held to 40 or 32 registers, so that more of the next
+// launch's blocks could be resident early, 578 and 782 us (spills in the chain).
+// Ranks up to 1024: two gates per thread and a word per lane.  With four (the former selection) repeating it cost more than the
+// launches it saves (2048 -> 6144 at r = 2048: 37.5 against 28.6 us; 4096 x 4096 x 16384: 127 against 74).  P up to 16 MB: for long P
+// the staged gather above streams better.  The line was drawn for the former selection; with this one, us, one launch / three:
+// 1024 x 4096 bf16 8.1 / 20.9, at the line 1024 x 8192 14.1 / 24.0, beyond it 1024 x 16 384 26.8 / 30.5, 1024 x 40 000 65.5 / 44.0.
 constexpr int kFusedMaxR = 1024;
 constexpr int64_t kFusedMaxBytes = 16 << 20;
 constexpr int kFusedPiece = 4096;
@@ -540,8 +542,10 @@ compact_fused_kernel(const float* __restrict__ in, int mode, double thr, int r, 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int warps = (int)gridDim.x * kFusedWarps, my_warp = (int)blockIdx.x * kFusedWarps + warp;
   T* my_row = reinterpret_cast<T*>(rows + warp * fused_row_bytes<T>(r));
-  // a hint only: nothing is read before the wait below.  Which rows of Q survive is not known yet; all of them are asked for (the
-  // third that is read of them came from HBM at the end of the chain: 72 matrices in 420 us without, 399 with)
+  // a hint only: nothing is read before the wait below.  Which rows of Q survive is not known yet; all of them are asked for (what
+  // is read of them came from HBM at the end of the chain).  us, without / with, 4096 columns at r = 1024 with 1024 rows of P: 90 % of
+  // the gates open bf16 8.6 / 7.0, fp32 12.6 / 11.6; 30 % 8.1 / 7.1, 11.1 / 10.2; 5 % 7.3 / 7.3, 10.4 / 10.0; 0.5 % 7.1 / 7.3, 9.9 / 10.3; the
+  // most it can cost, 0.5 % of 16 MB of Q and 64 rows of P: 9.4 / 10.5
   auto prefetch = [&](const T* m, int64_t ld, int n, int cols) {
     for (int i = my_warp; i < n; i += warps)
       for (int64_t b = lane * 128; b < cols * (int64_t)sizeof(T); b += 32 * 128)

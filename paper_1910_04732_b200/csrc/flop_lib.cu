@@ -861,10 +861,10 @@ int64_t few_blocks(int64_t T, int64_t N, int64_t rows = 32) { return ((N + rows 
 // Block shape for more than 32 tokens: 16 mt weight rows for each of 8 / ks groups of warps, K over ks warps; mt = 0: tcgen05 tiles.  One
 // round of blocks over the SMs, with as many rows (fewer reads of the tokens, no idle warps) as K is short: a block of all eight warps
 // on K has eight 32-long steps to deal out.  Second product of a pair with a first of K = 64, replayed, us, before (32 rows, or
-// tcgen05 beyond a round of them) / by this rule: K = 40: 100 x 4096 outputs 7.0 / 5.4, 256 x 2048 6.4 / 5.3; K = 100: 100 x 4096 7.2 / 5.6,
-// 512 x 512 7.0 / 5.6; K = 160: 150 x 1024 5.8 / 5.0, 150 x 2048 7.0 / 6.4; K = 256: 100 x 4096 7.8 / 7.2.  Lines, this kernel / tcgen05: K = 100,
-// 384 x 2048 7.6 / 7.6 (2 x 2), 512 x 1024 6.7 / 6.6; K = 160, 256 x 2048 7.2 / 6.7, 384 x 1024 7.2 / 6.8; K = 250, 200 x 1700 7.9 / 7.3;
-// K = 300, 150 x 2048 9.5 / 7.4.
+// tcgen05 beyond a round of them) / by this rule: K = 40: 100 x 4096 outputs 7.2 / 5.7, 256 x 2048 7.2 / 5.7; K = 100: 100 x 4096 7.7 / 5.7,
+// 512 x 512 7.7 / 6.2, 512 x 1024 7.2 / 6.2; K = 160: 150 x 1024 6.2 / 5.6, 150 x 2048 7.2 / 6.7; K = 256: 100 x 4096 8.4 / 8.3.  Lines, this
+// kernel / tcgen05: K = 160, 256 x 2048 7.2 / 6.7, 384 x 1024 7.2 / 6.8; where K is ragged as measured while every step looked at its
+// rows: K = 100, 384 x 2048 7.6 / 7.6 (2 x 2); K = 250, 200 x 1700 7.9 / 7.3; K = 300, 150 x 2048 9.5 / 7.4.
 struct FewShape { int mt, ks; };
 FewShape few_shape(int64_t T, int64_t N, int64_t K) {
   const int64_t sms = num_sms();
@@ -897,8 +897,8 @@ int launch_few(const FewArgs& a, cudaStream_t st) {
 // Whether a product takes the few-token kernel.  Up to 16 tokens always.  Up to 32 unless the weights are wide and large: every
 // group of 16 weight rows reads the tokens again, which a tcgen05 tile of 128 or 256 columns does not (32 tokens, K = 1024, us, this
 // kernel / tcgen05 tiles: 8192 outputs 8.1 / 11.2, 16 384 12.3 / 12.4, 32 768 20.0 / 15.1, 100 000 62.2 / 46.2).  Beyond, by few_shape.  Both products of a pair in a replayed
-// graph: 1024 -> 358 -> 4096 at 16, 64, 128 tokens 4.7 / 11.9, 8.6 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024
-// tokens 16.2 / 26.6; at two rounds it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
+// graph: 1024 -> 358 -> 4096 at 16, 64, 128 tokens 4.6 / 11.9, 8.6 / 14.6, (first product only) 11.4 / 14.3; 4096 -> 100 -> 256 at 1024
+// tokens 14.9 / 26.6; at two rounds it loses (4096 -> 1600 -> 4096 at 192 tokens 58.6 / 34.1).
 bool few_ok(int64_t T, int64_t N, int64_t K) {
   if (T < 1 || T > 1024 || N > INT32_MAX / 2 || K > INT32_MAX / 2 || tuning().no_few) return false;
   if (T <= 16) return true;

@@ -24,9 +24,10 @@
 //   * with EARLY the first weights are requested before the wait on the previous launch.  That is for the second product of
 //     a pair only: its predecessor on the stream is the first product, which waits for everything before it
 //     before it lets this launch start, and which writes H' and nothing else, so the weights are final.
-// Both products of 1024 -> 358 -> 4096, replayed: 3.7 us at one token and 4.7 at 16, where a warp per output column on the
+// Both products of 1024 -> 358 -> 4096, replayed: 3.5 us at one token and 4.6 at 16, where a warp per output column on the
 // CUDA cores (up to 4 tokens) took 5.3 and a warp per 8 columns walking all of K, on 7 SMs for the first product, 11.9.
-// At 64 tokens 9.2 against 14.6 with tcgen05 tiles.  A 64 x 64 block per CTA (fewer bytes read in all) was never faster.
+// At 64 tokens 8.6 against 14.6 with tcgen05 tiles.  64 x 64 outputs per block (fewer bytes read in all) were never faster with all eight
+// warps on K; with two or four of them on a short K they are (few_shape).
 #pragma once
 #include "common.cuh"
 
